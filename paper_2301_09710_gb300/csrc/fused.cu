@@ -299,39 +299,49 @@ __global__ void __launch_bounds__(kRotThreads, 2) k_rot_fwd8(Geometry g, FusedDi
         }
         return;
     }
-    float* dst = wsl + ((size_t)v * ny + j) * d.parea;
-    if (d.nT == 1) {
-        if (threadIdx.x == 0) {
-            fence_proxy_async_smem();
-            tma_store_1d(dst, S, (unsigned)d.parea * 4u);
-            tma_store_wait_read<0>();  // the block may leave once its shared memory is read
-        }
-        return;
-    }
-    for (int r = warp; r < d.nT * nz; r += NW) {
-        const int t = r / nz, k = r - t * nz;
-        const int tw = min(d.TI + 2 * C, wcols - t * d.TI);
-        const float* src = S + k * wp + t * d.TI;
-        float* out = dst + (size_t)t * d.warea + (size_t)k * d.wp;
-        for (int c = lane; c < tw; c += 32) out[c] = src[c];
+    if (threadIdx.x == 0) {
+        fence_proxy_async_smem();
+        tma_store_1d(wsl + ((size_t)v * ny + j) * d.farea, S, (unsigned)d.farea * 4u);
+        tma_store_wait_read<0>();  // the block may leave once its shared memory is read
     }
 }
 
 // ----------------------------------------------------------------------------
-// Forward blur + depth sum: one block per (depth group of J planes, view,
-// column tile).
-// Rotated planes arrive by TMA into a double buffer (plane j+2 is requested as
-// soon as plane j's i-pass has read its buffer); per plane the i-pass writes U
-// (k halos by warp shuffles), the k-pass accumulates into ACC.
+// Forward blur + depth sum: one block per (column tile, depth group of J planes,
+// view), the tiles of a plane adjacent, so their overlapping boxes hit L2.
 // ----------------------------------------------------------------------------
-template <int P, bool TILED>
-__global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_sep_fused(Geometry g, FusedDims d,
-                                                                     const float* __restrict__ wsl,
-                                                                     const float* __restrict__ fx,
-                                                                     const float* __restrict__ fz,
+template <int P, bool RACC>
+__global__ void __launch_bounds__(FwdBlock<P>::T, FwdBlock<P>::B) k_fwd_sep_fused(const __grid_constant__ CUtensorMap tmap,
+                                                                     Geometry g, FwdDims d,
+                                                                     const float* __restrict__ rec,
                                                                      float* __restrict__ part, int l0, int* err)
 {
-    fwd_sep_body<P, TILED>(g, d, wsl, fx, fz, part, l0, err, blockIdx.x, blockIdx.y, blockIdx.z);
+    const int grp = blockIdx.x / d.nT;
+    fwd_sep_body<P, RACC>(g, d, &tmap, rec, part, l0, err, grp, blockIdx.y, blockIdx.x - grp * d.nT);
+}
+
+// Plan time: the tap records of the forward blur (layout: fwd_rec_floats), one
+// block per PSF plane; the folds are summed in FP64 and rounded once.
+__global__ void k_fwd_records(Geometry g, int P, int PT, int nkb, const float* __restrict__ fx,
+                              const float* __restrict__ fz, float* __restrict__ rec)
+{
+    const int row = blockIdx.x, C = (P - 1) / 2, ox = (P - g.px) / 2, oz = (P - g.pz) / 2;
+    const float* f = fz + (size_t)row * g.pz;
+    float* r = rec + (size_t)row * fwd_rec_floats(PT, nkb);
+    for (int a = threadIdx.x; a < PT; a += blockDim.x) {
+        r[a] = (a >= ox && a < ox + g.px) ? fx[(size_t)row * g.px + a - ox] : 0.f;
+        r[PT + a] = (a >= oz && a < oz + g.pz) ? f[a - oz] : 0.f;
+    }
+    for (int k = threadIdx.x; k < 16 * nkb; k += blockDim.x) {
+        double lo = 0.0, hi = 0.0;
+        if (k < g.nz)
+            for (int b = 0; b < g.pz; ++b) {
+                if (b + oz > k + C) lo += f[b];
+                if (b + oz < k + C - g.nz + 1) hi += f[b];
+            }
+        r[2 * PT + k] = (float)lo;
+        r[2 * PT + 16 * nkb + k] = (float)hi;
+    }
 }
 
 // v(i,k,l) = sum over depth groups of the partials (fixed order), optionally
@@ -415,16 +425,16 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_dir_fused(Geometry g, 
     const int j_begin = grp * d.J, j_end = min(ny, j_begin + d.J);
     const int ox = (P - g.px) / 2, oz = (P - g.pz) / 2;
     const int pln = nx * nz;
-    const float* wv = wsl + (size_t)v * ny * d.parea;
+    const float* wv = wsl + (size_t)v * ny * d.farea;
 
     for (int e = tid; e < d.urows * d.apc; e += T) ACC[e] = 0.f;
     if (tid == 0) {
         mbar_init(bar, 1);
         mbar_init(bar + 1, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        tma_load_1d(WB + ZH * d.wp, wv + (size_t)j_begin * d.parea, (unsigned)d.warea * 4u, bar);
+        tma_load_1d(WB + ZH * d.wp, wv + (size_t)j_begin * d.farea, (unsigned)d.warea * 4u, bar);
         if (j_begin + 1 < j_end)
-            tma_load_1d(WB + xarea + ZH * d.wp, wv + (size_t)(j_begin + 1) * d.parea, (unsigned)d.warea * 4u,
+            tma_load_1d(WB + xarea + ZH * d.wp, wv + (size_t)(j_begin + 1) * d.farea, (unsigned)d.warea * 4u,
                         bar + 1);
     }
     __syncthreads();
@@ -484,7 +494,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_dir_fused(Geometry g, 
         __syncthreads();  // buffer b and the taps are free
         if (tid == 0 && j + 2 < j_end) {
             fence_proxy_async_smem();
-            tma_load_1d(W + ZH * d.wp, wv + (size_t)(j + 2) * d.parea, (unsigned)d.warea * 4u, bar + b);
+            tma_load_1d(W + ZH * d.wp, wv + (size_t)(j + 2) * d.farea, (unsigned)d.warea * 4u, bar + b);
         }
     }
     float* pout = part + ((size_t)grp * g.nview + l) * pln;
@@ -736,7 +746,7 @@ int tiles_that_fit(const Geometry& g, size_t limit, int min_tiles)
         const FusedDims d = dims_for<P>(g, 8, t);
         if (d.nT == last_nt) continue;  // same tile width as a smaller request
         last_nt = d.nT;
-        if (smem_fwd<P>(g, d) <= limit && smem_adj<P>(g, d) <= limit && rot_smem_min(d) <= limit &&
+        if (smem_fwd_bound<P>(g, d) <= limit && smem_adj<P>(g, d) <= limit && rot_smem_min(d) <= limit &&
             (size_t)d.marea * 4 < (1u << 20))
             return d.nT;
     }
@@ -747,19 +757,19 @@ template <int P>
 cudaError_t fwd_launch(const spect_plan_s& Pl, const float* /*xt: the blur reads the work slab*/, int l0, int nv,
                        cudaStream_t st)
 {
-    const FusedDims d = dims_for<P>(Pl.g, Pl.fused_J, Pl.fused_nT);
-    const size_t smem = smem_fwd<P>(Pl.g, d);
-    auto kern = d.nT > 1 ? k_fwd_sep_fused<P, true> : k_fwd_sep_fused<P, false>;
+    const FwdDims d = fwd_dims<P>(Pl.g, Pl.fused_J, Pl.fwd_nT, (size_t)Pl.smem_optin);
+    const size_t smem = smem_fwd<P>(d);
+    auto kern = d.racc ? k_fwd_sep_fused<P, true> : k_fwd_sep_fused<P, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(d.G, nv, d.nT), kFusedThreads, smem, st>>>(Pl.g, d, Pl.slab, Pl.fx, Pl.fz, Pl.part, l0, Pl.err);
+    kern<<<dim3(d.G * d.nT, nv), d.T, smem, st>>>(Pl.fmap, Pl.g, d, Pl.frec, Pl.part, l0, Pl.err);
     return cudaGetLastError();
 }
 
 template <int P>
 cudaError_t rot_launch(const spect_plan_s& Pl, const float* xt, int l0, int nv, cudaStream_t st)
 {
-    const FusedDims d = dims_for<P>(Pl.g, Pl.fused_J, Pl.fused_nT);
+    const FusedDims d = dims_for<P>(Pl.g, Pl.fused_J, 1);
     // the three-pass rotation: eight taps per output from its own table
     const size_t smin = Pl.rot3 ? ((size_t)d.farea + (size_t)rot3_ts8(Pl.g.nx)) * sizeof(float) : rot_smem_min(d);
     const size_t smem_mu = smin + (size_t)d.ps * sizeof(float) + 16;
@@ -777,7 +787,7 @@ cudaError_t rot_launch(const spect_plan_s& Pl, const float* xt, int l0, int nv, 
 template <int P>
 cudaError_t adj_launch(const spect_plan_s& Pl, const float* v, int l0, int nv, cudaStream_t st)
 {
-    const FusedDims d = dims_for<P>(Pl.g, Pl.adj_J, Pl.fused_nT);
+    const FusedDims d = dims_for<P>(Pl.g, Pl.adj_J, Pl.adj_nT);
     const size_t smem = smem_adj<P>(Pl.g, d);
     auto kern = d.nT > 1 ? k_adj_sep_fused<P, true> : k_adj_sep_fused<P, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -887,7 +897,7 @@ int fused_tiles_fit(const Geometry& g, int bucket, int J, int adj_J, int tiles, 
     auto check = [&](auto tag) -> int {
         constexpr int B = decltype(tag)::value;
         const FusedDims df = dims_for<B>(g, J, tiles), da = dims_for<B>(g, adj_J, tiles);
-        const bool ok = smem_fwd<B>(g, df) <= smem_limit && smem_adj<B>(g, da) <= smem_limit &&
+        const bool ok = smem_fwd_bound<B>(g, df) <= smem_limit && smem_adj<B>(g, da) <= smem_limit &&
                         rot_smem_min(df) <= smem_limit && (size_t)df.marea * 4 < (1u << 20);
         return ok ? df.nT : 0;
     };
@@ -944,8 +954,8 @@ cudaError_t launch_fused_forward(const spect_plan_s& P, const float* xt, int l0,
 
 cudaError_t launch_fused_rotate(const spect_plan_s& P, const float* xt, int l0, int nv, cudaStream_t st)
 {
-    // untiled planes read from the plan's own x_t: the patch-staged rotation (rotpatch.cu)
-    if (P.rotpatch && P.rotpatch_on && P.fused_nT == 1 && xt == P.xt) return launch_rot_patch(P, l0, nv, st);
+    // read from the plan's own x_t: the patch-staged rotation (rotpatch.cu)
+    if (P.rotpatch && P.rotpatch_on && xt == P.xt) return launch_rot_patch(P, l0, nv, st);
     SPECT_DISPATCH(rot_launch, P, xt, l0, nv, st)
 }
 
@@ -953,9 +963,83 @@ namespace {
 template <int P>
 size_t plane_area(const spect_plan_s& Pl)
 {
-    return (size_t)dims_for<P>(Pl.g, Pl.fused_J, Pl.fused_nT).parea;
+    return (size_t)dims_for<P>(Pl.g, Pl.fused_J, 1).farea;
+}
+
+// The plane images of the work slab as a tensor map -- column (wpf) x k (nz) x
+// plane (chunk * ny) -- with the forward blur's tile as its box.
+template <int P>
+cudaError_t encode_fwd_map(spect_plan_s& Pl)
+{
+    const Geometry& g = Pl.g;
+    const FusedDims im = dims_for<P>(g, Pl.fused_J, 1);
+    const FwdDims d = fwd_dims<P>(g, Pl.fused_J, Pl.fwd_nT, (size_t)Pl.smem_optin);
+    const cuuint64_t dims[3] = {(cuuint64_t)im.wpf, (cuuint64_t)g.nz, (cuuint64_t)Pl.chunk * g.ny};
+    const cuuint64_t strides[2] = {(cuuint64_t)im.wpf * 4, (cuuint64_t)im.farea * 4};
+    const cuuint32_t box[3] = {(cuuint32_t)d.wp, (cuuint32_t)d.br, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    if (!encode_fn() ||
+        encode_fn()(&Pl.fmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, Pl.slab, dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return cudaSuccess;
 }
 }  // namespace
+
+// Floats of the forward blur's tap records of a plan.
+size_t fwd_records_floats(const spect_plan_s& P)
+{
+    const int PT = (P.bucket + 3) & ~3, nkb = (P.g.nz + 15) / 16;
+    return (size_t)P.g.nvp * P.g.ny * fwd_rec_floats(PT, nkb);
+}
+
+cudaError_t launch_fwd_records(const spect_plan_s& P, cudaStream_t st)
+{
+    const int PT = (P.bucket + 3) & ~3, nkb = (P.g.nz + 15) / 16;
+    k_fwd_records<<<P.g.nvp * P.g.ny, 128, 0, st>>>(P.g, P.bucket, PT, nkb, P.fx, P.fz, P.frec);
+    return cudaGetLastError();
+}
+
+cudaError_t build_fwd_map(spect_plan_s& P)
+{
+    if (!P.separable) return cudaSuccess;
+    SPECT_DISPATCH(encode_fwd_map, P)
+}
+
+// Default launch shape of the forward blur.  Tiles of 32 columns: a block is then
+// 2 nkb warps, and four to sixteen such blocks share an SM, so one block's
+// barriers, plane loads and set-up are covered by the others' FMAs (128x80, 128 views,
+// 37 taps: 458 us against 502 for whole planes, 470 for 64 columns; 160x96, 120
+// views, 29 taps: 659 against 812 for 80 columns; 192x128, 64 views, 37 taps: 815
+// against 939 for 64; 16 columns give the overlap of neighbouring boxes more to
+// read: 561 at 128x80).  J = 8 planes per block, fewer when that leaves the chip short
+// of blocks: at 64x32, 64 views J = 4 takes 18.6 us against 20.4, at 32x16, 32 views
+// J = 2 takes 8.0 against 12.2.
+void default_fwd_shape(spect_plan_s& P, int sms)
+{
+    const Geometry& g = P.g;
+    P.fused_J = 8;
+    if (!P.separable) return;
+    const int nib = (g.nx + 15) / 16;
+    P.fwd_nT = std::max(P.fwd_nT, (nib + 1) / 2);
+    P.fwd_nT = fwd_tiles(P);
+    const auto blocks = [&](int J) { return (long long)((g.ny + J - 1) / J) * P.fwd_nT * g.nview; };
+    if (blocks(8) < 10ll * sms) P.fused_J = blocks(4) >= 4ll * sms ? 4 : 2;
+}
+
+// Column tiles of the forward blur at its launch shape (what fwd_dims makes of the request).
+int fwd_tiles(const spect_plan_s& P)
+{
+    switch (P.bucket) {
+#define SPECT_FT(B) \
+    case B: return fwd_dims<B>(P.g, P.fused_J, P.fwd_nT, (size_t)P.smem_optin).nT;
+        SPECT_FT(3) SPECT_FT(5) SPECT_FT(7) SPECT_FT(9) SPECT_FT(11) SPECT_FT(13) SPECT_FT(15)
+        SPECT_FT(17) SPECT_FT(21) SPECT_FT(25) SPECT_FT(29) SPECT_FT(33) SPECT_FT(37)
+#undef SPECT_FT
+        default: return 1;
+    }
+}
 
 // floats per view of the work slab the fused path needs (rotated tile images or t planes)
 size_t fused_slab_per_view(const spect_plan_s& P)

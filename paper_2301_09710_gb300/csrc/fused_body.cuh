@@ -64,7 +64,7 @@ __device__ __forceinline__ void transpose_body(const float* __restrict__ in, flo
 // (view, depth) plane into the work slab, already in the blur kernel's
 // shared-memory image; k_fwd_sep_fused (one block per view and depth group)
 // streams those images in by TMA and blurs them.  Its shared memory:
-//   W   two plane buffers, nz rows x wp columns: W[k][C + i] with replicate
+//   W   one or two tile buffers, nz rows x wp columns: W[k][C + i] with replicate
 //       halo columns; wp is a multiple of 4 with wp/4 odd, so the i-pass
 //       windows (lanes over k) load as bank-conflict-free float4s.
 //   U   nx rows x kpu: i-pass output, U[i][ZH + k], with zero halo columns;
@@ -72,8 +72,7 @@ __device__ __forceinline__ void transpose_body(const float* __restrict__ in, flo
 //       bank-conflict free.  Replicate padding along k enters as folded edge
 //       taps: output k adds U(0) sum_{b>k+C} fz(b) + U(nz-1) sum_{b<k+C-nz+1} fz(b).
 //   taps and folded edge taps of every plane of the group, staged once.
-//   ACC nx x apc depth-sum accumulators of the group, [i][k] (apc/4 odd, so
-//       the k-pass float4 read-modify-writes are bank-conflict free).
+// The depth sums stay in registers.
 // Per plane there are two block barriers: after the i-pass (which also agrees
 // on the bounded TMA wait) and after the k-pass.
 // ============================================================================
@@ -89,6 +88,16 @@ struct Sep {
 
 constexpr int kFusedThreads = 640;
 
+// Largest block of the forward blur and the resident blocks its registers are bounded
+// for.  Short FIRs (P <= 11) wait more on shared memory and barriers than on FMAs, so
+// they get 64 registers (two blocks of 512, or four of 256) instead of about 80.
+template <int P>
+struct FwdBlock {
+    static constexpr int T = P <= 11 ? 512 : kFusedThreads;
+    static constexpr int B = P <= 11 ? 2 : 1;
+    static constexpr int regs = P <= 11 ? 64 : 80;
+};
+
 // Shared-memory plan of a fused kernel, computed identically on host and device.
 // Planes wider than shared memory allows are cut into nT column tiles of TI
 // detector columns (TI a multiple of CX); a tile carries C halo columns on
@@ -97,14 +106,13 @@ constexpr int kFusedThreads = 640;
 struct FusedDims {
     int wp;     // W row pitch of one tile image (pitch4odd(TI + 2*C))
     int warea;  // floats of one tile image, nz x wp (multiple of 4, keeps U 16-byte aligned)
-    int parea;  // floats of one plane's tile images in the slab, nT x warea
     int kpu;    // U row pitch (>= nkb*CZ + 2*ZH, multiple of 4, pitch/4 odd)
     int nib, nkb;
     int TI, nT; // tile width in columns (multiple of CX), tiles per plane
     int wpf;    // row pitch of the untiled plane image (pitch4odd(nib*CX + 2*C))
     int wz;     // row pitch of the adjoint's Zb (multiple of 4, wz/4 odd: conflict-free float4 windows)
     int zarea;  // floats of Zb, nz x wz
-    int farea;  // floats of the untiled plane image (the rotation kernel's shared memory)
+    int farea;  // floats of a plane image in the slab (and the rotation kernel's shared memory)
     int urows;  // rows of U / ACC / MB per tile: min(TI, nx)
     int vrows;  // detector rows a tile's k-adjoint needs: min(nx, TI + 2*C)
     int marea;  // floats of an attenuation tile, urows*nz rounded up to 4
@@ -113,14 +121,6 @@ struct FusedDims {
     int ts;     // rotation table block per (view, row): 5*nx rounded up to 4
     int apc;    // accumulator row pitch (>= nkb*CZ, multiple of 4, pitch/4 odd)
 };
-
-__host__ __device__ inline size_t fwd_smem_floats(const FusedDims& d, int nz, int PT)
-{
-    // W x2 | U | taps J x (FX,FZ) | ACC | folded edge taps J x 2 x (nkb*16) | 2 mbarriers
-    (void)nz;
-    return 2 * (size_t)d.warea + (size_t)d.urows * d.kpu + 2 * (size_t)PT * d.J + (size_t)d.urows * d.apc +
-           2 * (size_t)d.J * d.nkb * 16 + 8;
-}
 
 __host__ __device__ inline size_t adj_smem_floats(const FusedDims& d, int PT)
 {
@@ -229,10 +229,8 @@ __device__ __forceinline__ void flag_timeout(int* err)
 // are warp-uniform and every gather is a coalesced run along k (96 k per
 // pass, 30 independent loads per lane in flight).  The plane is
 // assembled in shared memory as the blur kernel wants it -- W[k][C+i] with
-// replicate halo columns and pitch4odd pitch -- and leaves with one TMA bulk store,
-// so the blur kernel can bring it back with one bulk load.  A plane cut into
-// column tiles leaves instead as nT tile images W_t[k][c] = W[k][t*TI + c],
-// c < TI + 2C, written with coalesced stores.
+// replicate halo columns and pitch4odd pitch -- and leaves with one TMA bulk store;
+// the blur kernel brings its column tiles back as boxes of the image.
 // ----------------------------------------------------------------------------
 
 constexpr int kRotThreads = 512;
@@ -349,91 +347,107 @@ __device__ __forceinline__ void rot_fwd_body(const Geometry& g, const FusedDims&
         }
         return;
     }
-    float* dst = wsl + ((size_t)v * ny + j) * d.parea;
-    if (d.nT == 1) {
-        if (threadIdx.x == 0) {
-            fence_proxy_async_smem();
-            tma_store_1d(dst, S, (unsigned)d.parea * 4u);
-            tma_store_wait_read<0>();  // the block may leave once its shared memory is read
-        }
-        return;
-    }
-    // tile images: row k of tile t is W[k][t*TI .. t*TI + TI + 2C), cut at
-    // the end of the plane's row (the blur never reads past it)
-    for (int r = warp; r < d.nT * nz; r += NW) {
-        const int t = r / nz, k = r - t * nz;
-        const int tw = min(d.TI + 2 * C, wcols - t * d.TI);
-        const float* src = S + k * wp + t * d.TI;
-        float* out = dst + (size_t)t * d.warea + (size_t)k * d.wp;
-        for (int c = lane; c < tw; c += 32) out[c] = src[c];
+    if (threadIdx.x == 0) {
+        fence_proxy_async_smem();
+        tma_store_1d(wsl + ((size_t)v * ny + j) * d.farea, S, (unsigned)d.farea * 4u);
+        tma_store_wait_read<0>();  // the block may leave once its shared memory is read
     }
 }
 
-template <int P, bool TILED>
-__device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FusedDims& d, const float* __restrict__ wsl,
-                                             const float* __restrict__ fx, const float* __restrict__ fz,
-                                             float* __restrict__ part, int l0, int* err, const int grp, const int v,
-                                             const int tile)
+// Launch shape of the forward blur: one block per depth group of J planes, view
+// and column tile of TI detector columns.  A tile is a TMA box (wp x br rows,
+// nbox of them) of the rotated plane image, its C halo columns on each side
+// included, so every tile is blurred independently from one image.
+struct FwdDims {
+    int TI, nT;        // tile width in columns (multiple of CX), tiles per plane
+    int wp;            // row pitch of a tile buffer = box width: pitch4odd(TI + 2C), at most 252
+    int br, nbox;      // rows per box (at most 256), boxes per plane
+    int warea;         // floats of a tile buffer (nbox * br * wp, rounded up to 128 bytes)
+    int nbuf;          // tile buffers (1 or 2): planes in flight per block
+    int kpu, nkb, nib; // U row pitch; k runs; column runs of the whole plane
+    int urows;         // rows of U: min(TI, nx)
+    int J, G;          // depth planes per block, depth groups
+    int T;             // threads per block
+    int racc;          // depth sums in registers (every k-pass item has its own thread)
+    int apc;           // row pitch of the shared accumulators (racc == 0)
+};
+
+// Tap record of one PSF plane (view, depth) for the forward blur, built at plan
+// time (k_fwd_records): FX and FZ zero-padded to P and centred (PT floats each),
+// then the folded edge taps of replicate padding along k, lo and hi (nkb * 16
+// floats each): output k adds U(0) lo(k) + U(nz-1) hi(k), lo(k) = sum_{b > k+C} fz(b),
+// hi(k) = sum_{b < k+C-nz+1} fz(b).  A group's records are contiguous, so a block
+// fetches them with one bulk copy instead of building them.
+__host__ __device__ inline int fwd_rec_floats(int PT, int nkb) { return 2 * PT + 2 * 16 * nkb; }
+
+__host__ __device__ inline size_t fwd_smem_floats(const FwdDims& d, int PT)
+{
+    // W x nbuf | U | tap records of J planes | ACC (racc == 0) | 3 mbarriers
+    return (size_t)d.nbuf * d.warea + (size_t)d.urows * d.kpu + (size_t)d.J * fwd_rec_floats(PT, d.nkb) +
+           (d.racc ? 0 : (size_t)d.urows * d.apc) + 8;
+}
+
+// RACC: a thread keeps the depth sums of its one k-pass item (16 k of a column)
+// in registers over all planes of the group, so the k-pass touches shared memory
+// only to read U; otherwise (planes of more than 640 items) they are in ACC.
+template <int P, bool RACC>
+__device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FwdDims& d, const CUtensorMap* tmap,
+                                             const float* __restrict__ rec, float* __restrict__ part, int l0, int* err,
+                                             const int grp, const int v, const int tile)
 {
     using S = Sep<P>;
     constexpr int C = S::C, CX = S::CX, CZ = S::CZ, ZH = S::ZH, WZ = S::WZ, PT = S::PT;
-    extern __shared__ __align__(16) float sm[];
+    extern __shared__ __align__(128) float smf[];
     const int nx = g.nx, ny = g.ny, nz = g.nz;
-    float* WB = sm;                                    // [2][warea]
-    float* U = WB + 2 * (size_t)d.warea;
-    float* TAP = U + (size_t)d.urows * d.kpu;          // [J][FX PT | FZ PT], every plane of the group
-    float* ACC = TAP + 2 * PT * (size_t)d.J;           // urows x apc, [i - i0][k]
-    const int fs = d.nkb * CZ;                          // folded-tap row length (zero beyond nz)
-    float* FOLD = ACC + (size_t)d.urows * d.apc;        // [J][2][fs] folded edge taps of the k-pass
-    uint64_t* bar = reinterpret_cast<uint64_t*>(FOLD + 2 * (size_t)d.J * fs);
-    const int tid = threadIdx.x;
-    constexpr int T = kFusedThreads;
+    float* WB = smf;                                   // [nbuf][warea]
+    float* U = WB + (size_t)d.nbuf * d.warea;
+    float* TAP = U + (size_t)d.urows * d.kpu;          // the records of every plane of the group
+    const int rf = fwd_rec_floats(PT, d.nkb);
+    float* ACC = TAP + (size_t)d.J * rf;               // urows x apc, [i - i0][k] (!RACC)
+    uint64_t* bar = reinterpret_cast<uint64_t*>(ACC + (RACC ? 0 : (size_t)d.urows * d.apc));  // buffers, records
+    const int tid = threadIdx.x, T = blockDim.x;
     const int l = l0 + v;
-    // this tile's columns (untiled: the whole plane, constants folded at compile time)
-    const int i0 = TILED ? (int)tile * d.TI : 0;
-    const int ti = TILED ? min(d.TI, nx - i0) : nx;
-    const int nibt = TILED ? (ti + CX - 1) / CX : d.nib;
+    const int i0 = tile * d.TI, ti = min(d.TI, nx - i0), nibt = (ti + CX - 1) / CX;
     const int lp = g.nvp == 1 ? 0 : l;
-    const int j_begin = grp * d.J, j_end = min(ny, j_begin + d.J);
-    const int ox = (P - g.px) / 2, oz = (P - g.pz) / 2;  // zero-padding offsets of the taps
+    const int j_begin = grp * d.J, nj = min(ny - j_begin, d.J);
     const int pln = nx * nz;
-    // tile `tile` of plane j sits at wv + j * parea
-    const float* wv = wsl + (size_t)v * ny * d.parea + (size_t)tile * d.warea;
 
-    // the first two plane images are requested before anything else, so their
-    // loads overlap the set-up below
+    // tensor copies want 128-byte aligned shared memory: refuse (error word) rather than fault
+    if ((smem_u32(smf) & 127u) != 0) {
+        if (tid == 0 && err) atomicExch(err, (int)SPECT_ECUDA);
+        return;
+    }
+    auto request = [&](int n) {  // plane j_begin + n into its buffer
+        const int b = d.nbuf == 1 ? 0 : n & 1;
+        float* dst = WB + (size_t)b * d.warea;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar + b)),
+                     "r"((unsigned)(d.nbox * d.br * d.wp) * 4u)
+                     : "memory");
+        for (int q = 0; q < d.nbox; ++q)
+            tma_load_3d(dst + (size_t)q * d.br * d.wp, tmap, i0, q * d.br, v * ny + j_begin + n, bar + b);
+    };
+    // the first planes are requested before anything else, so their loads overlap the set-up below
     if (tid == 0) {
         mbar_init(bar, 1);
         mbar_init(bar + 1, 1);
+        mbar_init(bar + 2, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        tma_load_1d(WB, wv + (size_t)j_begin * d.parea, (unsigned)d.warea * 4u, bar);
-        if (j_begin + 1 < j_end)
-            tma_load_1d(WB + d.warea, wv + (size_t)(j_begin + 1) * d.parea, (unsigned)d.warea * 4u, bar + 1);
+        tma_load_1d(TAP, rec + ((size_t)lp * ny + j_begin) * rf, (unsigned)(nj * rf) * 4u, bar + 2);
+        for (int n = 0; n < d.nbuf && n < nj; ++n) request(n);
     }
-    // taps of every plane of the group (zero-padded to P, centred)
-    for (int e = tid; e < (j_end - j_begin) * PT; e += T) {
-        const int jj = e / PT, a = e - jj * PT, j = j_begin + jj;
-        const int ax = a - ox, az = a - oz;
-        TAP[jj * 2 * PT + a] = (ax >= 0 && ax < g.px) ? __ldg(fx + ((size_t)lp * ny + j) * g.px + ax) : 0.f;
-        TAP[jj * 2 * PT + PT + a] = (az >= 0 && az < g.pz) ? __ldg(fz + ((size_t)lp * ny + j) * g.pz + az) : 0.f;
+    if (!RACC)
+        for (int e = tid; e < d.urows * d.apc; e += T) ACC[e] = 0.f;
+    // zero k-halo columns of U (never written again): [0, ZH) and [ZH + nz, kpu) of each row
+    for (int r = tid; r < d.urows; r += T) {
+        float* ur = U + r * d.kpu;
+#pragma unroll
+        for (int c = 0; c < ZH; c += 4) *reinterpret_cast<float4*>(ur + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+        int c = ZH + nz;
+        for (; c & 3; ++c) ur[c] = 0.f;
+        for (; c < d.kpu; c += 4) *reinterpret_cast<float4*>(ur + c) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    for (int e = tid; e < d.urows * d.apc; e += T) ACC[e] = 0.f;
-    for (int e = tid; e < d.urows * d.kpu; e += T) U[e] = 0.f;  // zero k-halo columns (never written again)
-    __syncthreads();
-    // replicate padding along k, folded: output k takes U(0) * sum_{b > k+C} fz(b)
-    // and U(nz-1) * sum_{b < k+C-nz+1} fz(b) on top of the zero-padded k-pass
-    for (int e = tid; e < (j_end - j_begin) * fs; e += T) {
-        const int jj = e / fs, k = e - jj * fs;
-        const float* f = TAP + jj * 2 * PT + PT;
-        float lo = 0.f, hi = 0.f;
-        if (k < nz) {
-            for (int bq = k + C + 1; bq < P; ++bq) lo += f[bq];
-            for (int bq = 0; bq < k + C - nz + 1 && bq < P; ++bq) hi += f[bq];
-        }
-        FOLD[(jj * 2) * fs + k] = lo;
-        FOLD[(jj * 2 + 1) * fs + k] = hi;
-    }
-    __syncthreads();
+    __syncthreads();  // the barriers are initialised and U's halos are zero
+    bool ok = mbar_wait_bounded(bar + 2, 0u);
 
     // the thread's first work item of each pass and the step to its next one
     // (the same for every plane: the divisions stay out of the plane loop)
@@ -441,14 +455,17 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FusedDims&
     const int kp_kb = tid / ti, kp_i = tid - kp_kb * ti;    // k-pass: (k run, column)
     const int ip_dib = T / nz, ip_dk = T - ip_dib * nz;
     const int kp_dkb = T / ti, kp_di = T - kp_dkb * ti;
-    unsigned phases = 0u;                                   // bit b: parity of buffer b's barrier
-    for (int j = j_begin; j < j_end; ++j) {
-        const int b = (j - j_begin) & 1;
-        const float* FX = TAP + (j - j_begin) * 2 * PT;
+    float acc[CZ];  // RACC: the depth sums of item (kp_kb, kp_i)
+#pragma unroll
+    for (int c = 0; c < CZ; ++c) acc[c] = 0.f;
+
+    for (int n = 0; n < nj; ++n) {
+        const int b = d.nbuf == 1 ? 0 : n & 1;
+        const unsigned parity = (unsigned)(d.nbuf == 1 ? n : n >> 1) & 1u;
+        const float* FX = TAP + n * rf;
         const float* FZ = FX + PT;
-        const float* W = WB + b * (size_t)d.warea;
-        const bool ok = mbar_wait_bounded(bar + b, (phases >> b) & 1u);
-        phases ^= 1u << b;
+        const float* W = WB + (size_t)b * d.warea;
+        ok = mbar_wait_bounded(bar + b, parity) && ok;
 
         // i-pass: U(i,k) = sum_a fx(a) w(clamp(i-a+cx), k); lanes over k
         if (ok) {
@@ -475,30 +492,28 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FusedDims&
             }
         }
         if (__syncthreads_or(!ok)) {
-            if (tid == 0) {
+            if (tid == 0) {  // a last chance for the copies in flight to land
                 flag_timeout(err);
-                mbar_wait_bounded(bar + b, ((phases >> b) & 1u) ^ 1u);  // a last chance for the copies in flight
-                mbar_wait_bounded(bar + (b ^ 1), (phases >> (b ^ 1)) & 1u);
+                mbar_wait_bounded(bar + 2, 0u);
+                for (int m = n; m < n + d.nbuf && m < nj; ++m)
+                    mbar_wait_bounded(bar + (d.nbuf == 1 ? 0 : m & 1), (unsigned)(d.nbuf == 1 ? m : m >> 1) & 1u);
             }
             return;
         }
-        // buffer b has been read: request plane j+2 into it (from the last warp,
-        // which has the fewest halo rows below)
-        if (tid == T - 32 && j + 2 < j_end) {
+        // buffer b has been read: request its next plane (from the last warp, which has the fewest halo rows below)
+        if (tid == T - 32 && n + d.nbuf < nj) {
             fence_proxy_async_smem();
-            tma_load_1d(WB + b * (size_t)d.warea, wv + (size_t)(j + 2) * d.parea, (unsigned)d.warea * 4u, bar + b);
+            request(n + d.nbuf);
         }
 
-        // k-pass into the depth-sum accumulators: lanes over i; zero-padded
-        // FIR plus the folded replicate-padding terms on the edge rows
-        const float* fold_lo = FOLD + (j - j_begin) * 2 * fs;
-        const float* fold_hi = fold_lo + fs;
-        int kb = kp_kb, i = kp_i;  // i relative to the tile
-        for (int it = tid; it < ti * d.nkb; it += T) {
+        // k-pass into the depth sums: lanes over i; zero-padded FIR plus the
+        // folded replicate-padding terms on the edge rows
+        const float* fold_lo = FZ + PT;  // zero outside the first (lo) and last (hi) C rows
+        const float* fold_hi = fold_lo + d.nkb * CZ;
+        auto kpass = [&](int kb, int i, float (&o)[CZ]) {
             const float* ur = U + i * d.kpu;
             float win[WZ];
             load_window_f4<P>(ur + kb * CZ, win);
-            float o[CZ];
             fir<P, CZ, -1, C + ZH>(FZ, win, o);
             const int k0 = kb * CZ;
             // folded taps are zero outside the first and last C rows
@@ -526,28 +541,52 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FusedDims&
                     o[4 * c4 + 3] = fmaf(ulo, f.w, o[4 * c4 + 3]);
                 }
             }
-            float4* acc4 = reinterpret_cast<float4*>(ACC + i * d.apc + kb * CZ);
+        };
+        if (RACC) {
+            if (tid < ti * d.nkb) {
+                float o[CZ];
+                kpass(kp_kb, kp_i, o);
 #pragma unroll
-            for (int c4 = 0; c4 < CZ / 4; ++c4) {
-                float4 a = acc4[c4];
-                a.x += o[4 * c4];
-                a.y += o[4 * c4 + 1];
-                a.z += o[4 * c4 + 2];
-                a.w += o[4 * c4 + 3];
-                acc4[c4] = a;
+                for (int c = 0; c < CZ; ++c) acc[c] += o[c];
             }
-            kb += kp_dkb;  // next item: it + T
-            i += kp_di;
-            if (i >= ti) i -= ti, ++kb;
+        } else {
+            int kb = kp_kb, i = kp_i;  // i relative to the tile
+            for (int it = tid; it < ti * d.nkb; it += T) {
+                float o[CZ];
+                kpass(kb, i, o);
+                float4* acc4 = reinterpret_cast<float4*>(ACC + i * d.apc + kb * CZ);
+#pragma unroll
+                for (int c4 = 0; c4 < CZ / 4; ++c4) {
+                    float4 a = acc4[c4];
+                    a.x += o[4 * c4];
+                    a.y += o[4 * c4 + 1];
+                    a.z += o[4 * c4 + 2];
+                    a.w += o[4 * c4 + 3];
+                    acc4[c4] = a;
+                }
+                kb += kp_dkb;  // next item: it + T
+                i += kp_di;
+                if (i >= ti) i -= ti, ++kb;
+            }
         }
         __syncthreads();
     }
 
     // partial depth sums of this group: part[grp][l][k][i], this tile's columns
     float* pout = part + ((size_t)grp * g.nview + l) * pln + i0;
-    for (int e = tid; e < nz * ti; e += T) {
-        const int k = e / ti, i = e - k * ti;
-        pout[(size_t)k * nx + i] = ACC[i * d.apc + k];
+    if (RACC) {
+        if (tid < ti * d.nkb) {
+#pragma unroll
+            for (int c = 0; c < CZ; ++c) {
+                const int k = kp_kb * CZ + c;
+                if (k < nz) pout[(size_t)k * nx + kp_i] = acc[c];
+            }
+        }
+    } else {
+        for (int e = tid; e < nz * ti; e += T) {
+            const int k = e / ti, i = e - k * ti;
+            pout[(size_t)k * nx + i] = ACC[i * d.apc + k];
+        }
     }
 }
 
@@ -760,7 +799,6 @@ FusedDims dims_for(const Geometry& g, int J, int tiles)
     d.marea = (d.urows * g.nz + 3) & ~3;
     d.wp = pitch4odd(d.TI + 2 * S::C);
     d.warea = (g.nz * d.wp + 3) & ~3;
-    d.parea = d.nT * d.warea;
     d.wpf = pitch4odd(d.nib * S::CX + 2 * S::C);
     d.wz = pitch4odd(d.TI + 2 * S::C);
     d.zarea = g.nz * d.wz;
@@ -780,10 +818,74 @@ FusedDims dims_for(const Geometry& g, int J, int tiles)
 // Rotation kernel without the attenuation plane staged: plane image + table.
 inline size_t rot_smem_min(const FusedDims& d) { return ((size_t)d.farea + d.ts) * sizeof(float); }
 
-template <int P>
-size_t smem_fwd(const Geometry& g, const FusedDims& d)
+// Launch shape of the forward blur for `tiles` column tiles (the nearest count
+// whose box fits the tensor map's 256 columns) and J planes per block.
+//   threads: one per work item where the tile has at most 640 (the depth sums
+//     then live in registers), so small planes run as small blocks, several
+//     per SM, instead of one block of mostly idle warps;
+//   tile buffers: two, or one when that lets more blocks run on an SM (the other
+//     blocks then cover the load) or is all that fits.
+constexpr size_t kSmSharedBytes = 233472;  // shared memory of an SM (1 KB of it per resident block)
+
+inline int blocks_per_sm(size_t smem_bytes, int T, int regs)
 {
-    return fwd_smem_floats(d, g.nz, Sep<P>::PT) * sizeof(float);
+    const int by_smem = (int)(kSmSharedBytes / (smem_bytes + 1024));
+    const int by_regs = 65536 / (((T + 31) / 32) * 32 * regs);
+    const int by_thr = 2048 / T;
+    const int b = by_smem < by_regs ? by_smem : by_regs;
+    return b < by_thr ? b : by_thr;
+}
+
+template <int P>
+FwdDims fwd_dims(const Geometry& g, int J, int tiles, size_t smem_limit)
+{
+    using S = Sep<P>;
+    FwdDims d;
+    d.nib = (g.nx + S::CX - 1) / S::CX;
+    d.nkb = (g.nz + S::CZ - 1) / S::CZ;
+    tiles = tiles < 1 ? 1 : (tiles > d.nib ? d.nib : tiles);
+    d.TI = ((d.nib + tiles - 1) / tiles) * S::CX;
+    while (pitch4odd(d.TI + 2 * S::C) > 252) d.TI -= S::CX;
+    d.nT = (g.nx + d.TI - 1) / d.TI;
+    d.wp = pitch4odd(d.TI + 2 * S::C);
+    d.nbox = (g.nz + 255) / 256;
+    d.br = (g.nz + d.nbox - 1) / d.nbox;
+    // every box starts on 128 bytes of shared memory: wp is 4 * odd, so 8 rows are a multiple of 128 bytes
+    if (d.nbox > 1) d.br = (d.br + 7) & ~7;
+    d.warea = (d.nbox * d.br * d.wp + 31) & ~31;
+    d.urows = d.TI < g.nx ? d.TI : g.nx;
+    d.kpu = pitch4odd(d.nkb * S::CZ + 2 * S::ZH);
+    d.apc = pitch4odd(d.nkb * S::CZ);
+    d.J = J;
+    d.G = (g.ny + J - 1) / J;
+    const int kitems = d.urows * d.nkb, iitems = g.nz * ((d.urows + S::CX - 1) / S::CX);
+    constexpr int kT = FwdBlock<P>::T;
+    d.racc = kitems <= kT;
+    const int want = kitems > iitems ? kitems : iitems;
+    d.T = d.racc && want <= kT ? (want + 31) & ~31 : kT;
+    d.nbuf = 2;
+    const size_t two = fwd_smem_floats(d, S::PT) * sizeof(float);
+    d.nbuf = 1;
+    const size_t one = fwd_smem_floats(d, S::PT) * sizeof(float);
+    const int b1 = blocks_per_sm(one, d.T, FwdBlock<P>::regs), b2 = blocks_per_sm(two, d.T, FwdBlock<P>::regs);
+    if (two <= smem_limit && b2 >= 1 && (b1 <= b2 || b2 * d.T >= 768)) d.nbuf = 2;
+    return d;
+}
+
+template <int P>
+size_t smem_fwd(const FwdDims& d)
+{
+    return fwd_smem_floats(d, Sep<P>::PT) * sizeof(float);
+}
+
+// The geometries and shapes that the fused kernels take: two tile buffers, U,
+// accumulators, taps and folds of a block in shared memory.  (The forward kernel needs
+// less: its sums are in registers and one buffer may do.)
+template <int P>
+size_t smem_fwd_bound(const Geometry& g, const FusedDims& d)
+{
+    return (2 * (size_t)d.warea + (size_t)d.urows * d.kpu + 2 * (size_t)Sep<P>::PT * d.J + (size_t)d.urows * d.apc +
+            2 * (size_t)d.J * d.nkb * 16 + 8) * sizeof(float);
 }
 
 template <int P>

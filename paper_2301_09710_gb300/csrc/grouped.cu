@@ -24,14 +24,14 @@ namespace {
 
 struct GroupPlan {
     Geometry g;
-    FusedDims df, da;  // forward / adjoint launch shapes
+    FusedDims im, da;  // plane images (rotation), adjoint launch shape
+    FwdDims df;        // forward launch shape
     int cls_z;
     const float* rtab;
     const float* xt;
     const float* mubar;
     float* slab;
-    const float* fx;
-    const float* fz;
+    const float* frec;
     float* part;
     const float* fx_adj;
     const float* fz_adj;
@@ -43,6 +43,7 @@ struct GroupPlan {
 };
 struct GroupPlans {
     GroupPlan p[kGroupMax];
+    CUtensorMap fmap[kGroupMax];  // the slabs' plane images (forward blur)
     GroupGrid grid;
 };
 
@@ -61,15 +62,16 @@ __global__ void __launch_bounds__(kRotThreads, 2) k_rot_fwd_grp(const __grid_con
 {
     const int4 w = group_item(gp.grid);
     const GroupPlan q = gp.p[w.x];  // by value: the fields live in registers, not re-read from parameter space
-    rot_fwd_body<P, MUS>(q.g, q.df, q.rtab, q.xt, q.mubar, q.slab, 0, q.err, w.y, w.z);
+    rot_fwd_body<P, MUS>(q.g, q.im, q.rtab, q.xt, q.mubar, q.slab, 0, q.err, w.y, w.z);
 }
 
-template <int P, bool TILED>
-__global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_sep_grp(const __grid_constant__ GroupPlans gp)
+template <int P, bool RACC>
+__global__ void __launch_bounds__(FwdBlock<P>::T, FwdBlock<P>::B) k_fwd_sep_grp(const __grid_constant__ GroupPlans gp)
 {
     const int4 w = group_item(gp.grid);
     const GroupPlan q = gp.p[w.x];  // by value: the fields live in registers, not re-read from parameter space
-    fwd_sep_body<P, TILED>(q.g, q.df, q.slab, q.fx, q.fz, q.part, 0, q.err, w.y, w.z, w.w);
+    const int grp = w.y / q.df.nT;
+    fwd_sep_body<P, RACC>(q.g, q.df, &gp.fmap[w.x], q.frec, q.part, 0, q.err, grp, w.z, w.y - grp * q.df.nT);
 }
 
 template <int P, bool TILED>
@@ -122,15 +124,15 @@ template <int P>
 void fill_plan(GroupPlan& q, const spect_plan_s* Pl, const float* y, const float* rbar)
 {
     q.g = Pl->g;
-    q.df = dims_for<P>(Pl->g, Pl->fused_J, Pl->fused_nT);
-    q.da = dims_for<P>(Pl->g, Pl->adj_J, Pl->fused_nT);
+    q.im = dims_for<P>(Pl->g, Pl->fused_J, 1);
+    q.df = fwd_dims<P>(Pl->g, Pl->fused_J, Pl->fwd_nT, (size_t)Pl->smem_optin);
+    q.da = dims_for<P>(Pl->g, Pl->adj_J, Pl->adj_nT);
     q.cls_z = Pl->cls_z;
     q.rtab = Pl->rtab;
     q.xt = Pl->xt;
     q.mubar = Pl->mubar;
     q.slab = Pl->slab;
-    q.fx = Pl->fx;
-    q.fz = Pl->fz;
+    q.frec = Pl->frec;
     q.part = Pl->part;
     q.fx_adj = Pl->fx_adj;
     q.fz_adj = Pl->fz_adj;
@@ -146,7 +148,7 @@ void fill_plan(GroupPlan& q, const spect_plan_s* Pl, const float* y, const float
 template <int P>
 size_t rot_smem(const spect_plan_s& Pl, bool* mus)
 {
-    const FusedDims d = dims_for<P>(Pl.g, Pl.fused_J, Pl.fused_nT);
+    const FusedDims d = dims_for<P>(Pl.g, Pl.fused_J, 1);
     const size_t smin = rot_smem_min(d);
     const size_t smem_mu = smin + (size_t)d.ps * sizeof(float) + 16;
     *mus = smem_mu <= (size_t)Pl.smem_optin;
@@ -183,18 +185,22 @@ cudaError_t stage_launches(int stage, const std::vector<int>& idx, const std::ve
                            const float* const* y, const float* const* rbar, GroupedBatch& /*B*/,
                            std::vector<GroupLaunch>& out)
 {
-    // sub-groups by kernel variant: attenuation staged (rotation) / tiled (blurs)
+    // sub-groups by kernel variant: attenuation staged (rotation), sums in registers (blur), tiled (adjoint)
     std::vector<int> var[2];
     for (int i : idx) {
         bool flag = false;
         if (stage == 0) rot_smem<P>(*plans[i], &flag);
-        else flag = dims_for<P>(plans[i]->g, plans[i]->fused_J, plans[i]->fused_nT).nT > 1;
+        else if (stage == 1)
+            flag = fwd_dims<P>(plans[i]->g, plans[i]->fused_J, plans[i]->fwd_nT, (size_t)plans[i]->smem_optin).racc;
+        else
+            flag = dims_for<P>(plans[i]->g, plans[i]->adj_J, plans[i]->adj_nT).nT > 1;
         var[flag ? 1 : 0].push_back(i);
     }
     for (int f = 0; f < 2; ++f) {
         for (const std::vector<int>& ch : chunks_of(var[f], plans)) {
             GroupPlans gp{};
             size_t smem = 0;
+            int thr = 0;  // the forward blur's block: the largest of its plans'
             for (int m = 0; m < (int)ch.size(); ++m) {
                 const spect_plan_s* Pl = plans[ch[m]];
                 fill_plan<P>(gp.p[m], Pl, y[ch[m]], rbar ? rbar[ch[m]] : nullptr);
@@ -203,10 +209,14 @@ cudaError_t stage_launches(int stage, const std::vector<int>& idx, const std::ve
                     bool mus = false;
                     smem = std::max(smem, rot_smem<P>(*Pl, &mus));
                     add_grid(gp.grid, m, q.g.ny, q.g.nview, 1);
-                } else {           // the blurs' grid: (depth group, view, column tile)
-                    const FusedDims& d = stage == 1 ? q.df : q.da;
-                    smem = std::max(smem, stage == 1 ? smem_fwd<P>(q.g, d) : smem_adj<P>(q.g, d));
-                    add_grid(gp.grid, m, d.G, q.g.nview, d.nT);
+                } else if (stage == 1) {  // the forward blur's grid: (depth group and column tile, view)
+                    smem = std::max(smem, smem_fwd<P>(q.df));
+                    thr = std::max(thr, q.df.T);
+                    gp.fmap[m] = Pl->fmap;
+                    add_grid(gp.grid, m, q.df.G * q.df.nT, q.g.nview, 1);
+                } else {           // the adjoint's grid: (depth group, view, column tile)
+                    smem = std::max(smem, smem_adj<P>(q.g, q.da));
+                    add_grid(gp.grid, m, q.da.G, q.g.nview, q.da.nT);
                 }
             }
             if (ch.empty()) continue;
@@ -214,8 +224,8 @@ cudaError_t stage_launches(int stage, const std::vector<int>& idx, const std::ve
                 out.push_back(f ? make_launch(k_rot_fwd_grp<P, true>, gp, dim3(kRotThreads), smem)
                                 : make_launch(k_rot_fwd_grp<P, false>, gp, dim3(kRotThreads), smem));
             else if (stage == 1)
-                out.push_back(f ? make_launch(k_fwd_sep_grp<P, true>, gp, dim3(kFusedThreads), smem)
-                                : make_launch(k_fwd_sep_grp<P, false>, gp, dim3(kFusedThreads), smem));
+                out.push_back(f ? make_launch(k_fwd_sep_grp<P, true>, gp, dim3(thr), smem)
+                                : make_launch(k_fwd_sep_grp<P, false>, gp, dim3(thr), smem));
             else
                 out.push_back(f ? make_launch(k_adj_sep_grp<P, true>, gp, dim3(kFusedThreads), smem)
                                 : make_launch(k_adj_sep_grp<P, false>, gp, dim3(kFusedThreads), smem));

@@ -134,7 +134,7 @@ void free_plan(spect_plan_s* P, cudaStream_t st)
     }
     for (cudaEvent_t e : P->evpool) cudaEventDestroy(e);
     void* ptrs[] = {P->mu, P->psf, P->psf_adj, P->fx, P->fz, P->fx_adj, P->fz_adj, P->rot, P->adj_off, P->adj,
-                    P->slab, P->e, P->ratio, P->s, P->mubar, P->xt, P->et, P->st, P->part, P->adjf, P->err, P->rtab, P->ut,
+                    P->frec, P->slab, P->e, P->ratio, P->s, P->mubar, P->xt, P->et, P->st, P->part, P->adjf, P->err, P->rtab, P->ut,
                     P->gboxes, P->gent, P->rboxes, P->r3_tab, P->mut};
     for (void* p : ptrs) raw_free(P, p, st);
     delete P;
@@ -390,6 +390,7 @@ size_t plan_bytes_bound(const spect_plan_s& P)
     const size_t chunk = std::max<size_t>(1, std::min<size_t>((size_t)g.nview, budget / view_bytes(P, per_view)));
     b += per_view * chunk * F;
     b += (2 * vol + nproj) * F;
+    if (P.fast && P.separable) b += spect::fwd_records_floats(P) * F;
     if (P.fast) {
         // attenuation factors of every view, or of one chunk plus mu in the internal layout
         b += P.recompute ? ((size_t)g.ny * P.ps * chunk + vol) * F : (size_t)g.ny * P.ps * g.nview * F;
@@ -433,14 +434,23 @@ spect_status spect_plan_bytes(int nx, int ny, int nz, int nview, int px, int pz,
     P.cls_z = nz >= 2 ? 3 : 1;
     P.rot3 = (flags & SPECT_PLAN_ROTATION_3PASS) != 0;
     if (P.separable && !(flags & SPECT_PLAN_LOW_MEMORY)) {
-        P.bucket = spect::fused_bucket(g, (size_t)smem_optin, &P.fused_nT);
+        P.bucket = spect::fused_bucket(g, (size_t)smem_optin, &P.fwd_nT);
         P.fast = P.bucket > 0;
     } else if (!(flags & SPECT_PLAN_LOW_MEMORY)) {
         P.bucket = spect::fused_dir_bucket(g, (size_t)smem_optin);
         P.fast = P.bucket > 0;
-        P.fused_nT = 1;
+        P.fwd_nT = 1;
     }
     P.recompute = (flags & SPECT_PLAN_RECOMPUTE_ATTENUATION) != 0 && P.fast && !P.rot3;
+    P.smem_optin = smem_optin;
+    if (P.fast) {
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(SPECT_ECUDA, "device query failed");
+        }
+        spect::default_fwd_shape(P, sms);
+    }
     *bytes = plan_bytes_bound(P);
     return SPECT_OK;
 }
@@ -518,14 +528,18 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         P->pooled = pools != 0;
     }
     if (P->separable && !(flags & SPECT_PLAN_LOW_MEMORY)) {
-        P->bucket = spect::fused_bucket(g, (size_t)smem_optin, &P->fused_nT);
+        P->bucket = spect::fused_bucket(g, (size_t)smem_optin, &P->fwd_nT);
+        P->adj_nT = P->fwd_nT;
         P->fast = P->bucket > 0;
     } else if (!(flags & SPECT_PLAN_LOW_MEMORY)) {
         // full PSF: the fused full-PSF blur kernels, untiled planes only
         P->bucket = spect::fused_dir_bucket(g, (size_t)smem_optin);
         P->fast = P->bucket > 0;
-        P->fused_nT = 1;
+        P->fwd_nT = P->adj_nT = 1;
     }
+    int sms = 0;
+    PLAN_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device query");
+    if (P->fast) spect::default_fwd_shape(*P, sms);
     P->rot3 = (flags & SPECT_PLAN_ROTATION_3PASS) != 0;
     if (P->rot3 && !P->fast) {
         free_plan(P);
@@ -638,6 +652,16 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         PLAN_TRY(cudaStreamSynchronize(st), "adjacency fill");
     }
 
+    // the forward blur's tap records; the factors themselves are not read again
+    if (P->fast && P->separable) {
+        PLAN_ALLOC(P->frec, spect::fwd_records_floats(*P), "tap records");
+        PLAN_TRY(spect::launch_fwd_records(*P, st), "tap record launch");
+        raw_free(P, P->fx, st);
+        raw_free(P, P->fz, st);
+        P->fx = P->fz = nullptr;
+        P->bytes -= (size_t)(px + pz) * nrows * sizeof(float);
+    }
+
     // work slab and EM buffers
     const size_t budget = P->recompute ? recompute_budget_bytes() : slab_budget_bytes(P->fast);
     // the fused path stores padded planes (rotated image planes or adjoint planes)
@@ -645,6 +669,7 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
     P->chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)nview, budget / (view_bytes(*P, per_view))));
     PLAN_ALLOC(P->slab, per_view * (size_t)P->chunk, "work slab");
     P->slab_cap = per_view * (size_t)P->chunk;
+    if (P->fast) PLAN_TRY(spect::build_fwd_map(*P), "tensor map of the plane images");
     // fused adjoint: all views of the slab in one pass by default (measured
     // faster than L2-sized passes); SPECT_ADJ_CHUNK sets fewer views per pass,
     // with a depth-group size that keeps about two blocks per SM (tuning)
@@ -654,8 +679,6 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         if (atoi(env) > 0) {
             P->adj_chunk_req = atoi(env);
             P->adj_chunk = std::min(std::min(atoi(env), nview), P->chunk);
-            int sms = 0;
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             const int want_groups = std::max(1, (2 * std::max(sms, 1) + P->adj_chunk - 1) / P->adj_chunk);
             P->adj_J = std::max(1, std::min(8, (ny + want_groups - 1) / want_groups));
         }
@@ -983,13 +1006,21 @@ spect_status realloc_floats(spect_plan_s* P, float** p, size_t* cap, size_t need
     return SPECT_OK;
 }
 
-// Set the fused kernels' depth-group sizes and column-tile count, growing the
-// work slab and the partial-sum buffer when the new shape needs more room.
-spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, cudaStream_t st)
+// The forward blur's tensor map for the plan's present slab, chunk and launch shape.
+spect_status refresh_maps(spect_plan_s* P)
+{
+    SPECT_CUDA_TRY(spect::build_fwd_map(*P), "tensor map of the plane images");
+    return SPECT_OK;
+}
+
+// Set the fused kernels' depth-group sizes and column-tile counts (forward blur,
+// blur adjoint), growing the work slab and the partial-sum buffer when the new
+// shape needs more room.
+spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, int adj_tiles, cudaStream_t st)
 {
     if (!P->fast) return fail(SPECT_EUNSUPPORTED, "launch-shape tuning applies to the fused kernels only");
     const Geometry& g = P->g;
-    if (J < 1 || J > 32 || adj_J < 1 || adj_J > 32 || tiles < 1)
+    if (J < 1 || J > 32 || adj_J < 1 || adj_J > 32 || tiles < 1 || adj_tiles < 1)
         return fail(SPECT_EINVAL, "fused_J and adj_J must be in [1, 32], tiles >= 1");
     int dev = 0, smem = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -997,13 +1028,18 @@ spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, cudaStrea
         cudaGetLastError();
         return fail(SPECT_ECUDA, "device query failed");
     }
-    const int nt = P->separable ? spect::fused_tiles_fit(g, P->bucket, J, adj_J, tiles, (size_t)smem)
-                                : (tiles == 1 && spect::fused_dir_fit(g, P->bucket, J, adj_J, (size_t)smem) ? 1 : 0);
-    if (nt == 0) return fail(SPECT_EUNSUPPORTED, "this launch shape does not fit shared memory");
-    const int oJ = P->fused_J, oaJ = P->adj_J, ont = P->fused_nT;
+    auto fit = [&](int t) {
+        if (P->separable) return spect::fused_tiles_fit(g, P->bucket, J, adj_J, t, (size_t)smem);
+        return t == 1 && spect::fused_dir_fit(g, P->bucket, J, adj_J, (size_t)smem) ? 1 : 0;
+    };
+    const int nt = fit(tiles), ant = adj_tiles == tiles ? nt : fit(adj_tiles);
+    if (nt == 0 || ant == 0) return fail(SPECT_EUNSUPPORTED, "this launch shape does not fit shared memory");
+    const int oJ = P->fused_J, oaJ = P->adj_J, ont = P->fwd_nT, oant = P->adj_nT;
     P->fused_J = J;
     P->adj_J = adj_J;
-    P->fused_nT = nt;
+    P->fwd_nT = nt;
+    P->adj_nT = ant;
+    P->fwd_nT = P->separable ? spect::fwd_tiles(*P) : 1;
     const size_t vol = (size_t)g.nx * g.ny * g.nz, nproj = (size_t)g.nx * g.nz * g.nview;
     const size_t per_view = std::max(vol, spect::fused_slab_per_view(*P));
     const size_t budget = P->recompute ? recompute_budget_bytes() : slab_budget_bytes(true);
@@ -1017,12 +1053,15 @@ spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, cudaStrea
     if (r != SPECT_OK) {
         P->fused_J = oJ;
         P->adj_J = oaJ;
-        P->fused_nT = ont;
-        return r;
+        P->fwd_nT = ont;
+        P->adj_nT = oant;
+        const std::string msg = g_err;
+        refresh_maps(P);  // the slab may have moved
+        return fail(r, msg);
     }
     P->chunk = chunk;
     P->adj_chunk = P->adj_chunk_req > 0 ? std::min(P->adj_chunk_req, chunk) : chunk;
-    return SPECT_OK;
+    return refresh_maps(P);
 }
 
 // One pass over every view, as the grouped batch launches need: grow the work
@@ -1039,7 +1078,7 @@ spect_status single_pass(spect_plan_s* P, cudaStream_t st)
     if (r != SPECT_OK) return r;
     P->chunk = g.nview;
     P->adj_chunk = g.nview;
-    return SPECT_OK;
+    return refresh_maps(P);
 }
 
 // Device time of one call of fn (best of `reps` after one warm-up run).
@@ -1070,7 +1109,7 @@ spect_status time_best(cudaStream_t st, int reps, float* best, F&& fn)
 }
 
 struct Tuned {
-    int J, adj_J, tiles, rotpatch;
+    int J, adj_J, tiles, adj_tiles, rotpatch;
 };
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int, int, int, int, int>, Tuned> g_tuned;  // per geometry, mode and device
@@ -1082,7 +1121,7 @@ extern "C" {
 spect_status spect_plan_set_tuning(spect_plan P, int fused_J, int adj_J, int tiles, spect_stream stream)
 {
     if (!P) return fail(SPECT_EINVAL, "plan is NULL");
-    return reconfigure(P, fused_J, adj_J, tiles, (cudaStream_t)stream);
+    return reconfigure(P, fused_J, adj_J, tiles, tiles, (cudaStream_t)stream);
 }
 
 spect_status spect_plan_get_tuning(spect_plan P, int* fused_J, int* adj_J, int* tiles)
@@ -1090,7 +1129,7 @@ spect_status spect_plan_get_tuning(spect_plan P, int* fused_J, int* adj_J, int* 
     if (!P) return fail(SPECT_EINVAL, "plan is NULL");
     if (fused_J) *fused_J = P->fused_J;
     if (adj_J) *adj_J = P->adj_J;
-    if (tiles) *tiles = P->fused_nT;
+    if (tiles) *tiles = P->fwd_nT;
     return SPECT_OK;
 }
 
@@ -1102,13 +1141,14 @@ spect_status spect_plan_autotune(spect_plan P, spect_stream stream)
     const Geometry& g = P->g;
     int dev = 0;
     cudaGetDevice(&dev);
-    const auto key = std::make_tuple(dev, g.nx, g.nz, g.nview, g.nvp, P->bucket, (int)P->g.has_mu, P->recompute);
+    const auto key = std::make_tuple(dev, g.nx, g.nz, g.nview, g.nvp, P->bucket, (int)P->g.has_mu,
+                                     P->recompute | P->separable << 1 | P->rot3 << 2);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tuned.find(key);
         if (it != g_tuned.end()) {
             P->rotpatch_on = P->rotpatch && it->second.rotpatch;
-            return reconfigure(P, it->second.J, it->second.adj_J, it->second.tiles, st);
+            return reconfigure(P, it->second.J, it->second.adj_J, it->second.tiles, it->second.adj_tiles, st);
         }
     }
     // inputs of the timed calls: the plan's own scratch (x_t = 1, v = 1)
@@ -1118,46 +1158,40 @@ spect_status spect_plan_autotune(spect_plan P, spect_stream stream)
         return fail(SPECT_ECUDA, "fill launch failed");
     const int prof = P->prof;
     P->prof = 0;
-    const int base = P->fused_nT;
+    const int base = P->fwd_nT, abase = P->adj_nT;
     const int nib = (g.nx + 15) / 16;
-    std::vector<int> tile_cands;
-    for (int t : {base, base + 1, 2 * base, 4 * base})
-        if (t <= nib && std::find(tile_cands.begin(), tile_cands.end(), t) == tile_cands.end()) tile_cands.push_back(t);
-    if (!P->separable) tile_cands.assign(1, 1);  // the full-PSF kernels run untiled
+    auto cands = [&](int b) {
+        std::vector<int> c;
+        for (int t : {b, b / 2, b + 1, 2 * b, 4 * b})
+            if (t >= 1 && t <= nib && std::find(c.begin(), c.end(), t) == c.end()) c.push_back(t);
+        if (!P->separable) c.assign(1, 1);  // the full-PSF kernels run untiled
+        return c;
+    };
     std::vector<int> Js;
     for (int J : {4, 8, 12, 16, 20, 24, 32})
         if (J <= std::max(g.ny, 4)) Js.push_back(J);
-    Tuned best{P->fused_J, P->adj_J, base, 0};
+    Tuned best{P->fused_J, P->adj_J, base, abase, 0};
     P->rotpatch_on = 0;
-    float best_ms = 1e30f;
     spect_status r = SPECT_OK;
-    for (int t : tile_cands) {
-        float fbest = 1e30f, abest = 1e30f;
-        int fJ = 0, aJ = 0;
+    // the two blur kernels' shapes are independent of each other
+    float fbest = 1e30f, abest = 1e30f;
+    for (int t : cands(base))
         for (int J : Js) {
-            if (reconfigure(P, J, Js.front(), t, st) != SPECT_OK) continue;
+            if (r != SPECT_OK || reconfigure(P, J, best.adj_J, t, abase, st) != SPECT_OK) continue;
             float ms = 0.f;
             r = time_best(st, 3, &ms, [&] { return fast_forward(P, P->xt, P->ratio, nullptr, nullptr, st); });
-            if (r != SPECT_OK) break;
-            if (ms < fbest) fbest = ms, fJ = J;
+            if (r == SPECT_OK && ms < fbest) fbest = ms, best.J = J, best.tiles = t;
         }
-        if (r != SPECT_OK) break;
+    for (int t : cands(abase))
         for (int J : Js) {
-            if (!fJ || reconfigure(P, fJ, J, t, st) != SPECT_OK) continue;
+            if (r != SPECT_OK || reconfigure(P, best.J, J, best.tiles, t, st) != SPECT_OK) continue;
             float ms = 0.f;
             r = time_best(st, 3, &ms, [&] { return fast_back(P, P->ratio, P->et, spect::EmArgs(), st); });
-            if (r != SPECT_OK) break;
-            if (ms < abest) abest = ms, aJ = J;
+            if (r == SPECT_OK && ms < abest) abest = ms, best.adj_J = J, best.adj_tiles = t;
         }
-        if (r != SPECT_OK) break;
-        if (fJ && aJ && fbest + abest < best_ms) {
-            best_ms = fbest + abest;
-            best = {fJ, aJ, t, 0};
-        }
-    }
-    if (r == SPECT_OK) r = reconfigure(P, best.J, best.adj_J, best.tiles, st);
-    // the rotation kernel: plane gathers or patch-staged boxes (untiled planes only)
-    if (r == SPECT_OK && P->rotpatch && P->fused_nT == 1) {
+    if (r == SPECT_OK) r = reconfigure(P, best.J, best.adj_J, best.tiles, best.adj_tiles, st);
+    // the rotation kernel: plane gathers or patch-staged boxes
+    if (r == SPECT_OK && P->rotpatch) {
         float ms_plane = 0.f, ms_patch = 0.f;
         r = time_best(st, 3, &ms_plane, [&] { return fast_forward(P, P->xt, P->ratio, nullptr, nullptr, st); });
         P->rotpatch_on = 1;

@@ -63,6 +63,7 @@ struct spect_plan_s {
     float* psf_adj = nullptr;    // direct: nvar * px*pz*ny*nvp edge-class variants for A'
     float* fx = nullptr;         // separable: px*ny*nvp
     float* fz = nullptr;         // separable: pz*ny*nvp
+    float* frec = nullptr;       // fused separable: tap records of the forward blur (then fx, fz are not kept)
     float* fx_adj = nullptr;     // separable: cls_x * px*ny*nvp
     float* fz_adj = nullptr;     // separable: cls_z * pz*ny*nvp
     spect::ViewRot* rot = nullptr;  // nview
@@ -84,7 +85,9 @@ struct spect_plan_s {
     int fast = 0;                // 1 when the fused kernels serve this plan
     int bucket = 0;              // padded tap count of the fused kernels
     int fused_J = 8;             // depth planes per fused forward block
-    int fused_nT = 1;            // column tiles per plane in the fused kernels
+    int fwd_nT = 1;              // column tiles per plane of the fused forward blur
+    int adj_nT = 1;              // column tiles per plane of the fused blur adjoint
+    CUtensorMap fmap;            // the slab's plane images, boxed as the forward blur's tiles (build_fwd_map)
     int adj_J = 8;               // depth planes per fused adjoint block
     int adj_chunk = 0;           // views per adjoint pass (t slab sized to stay in L2)
     int adj_chunk_req = 0;       // views per adjoint pass asked for (SPECT_ADJ_CHUNK), 0: all
@@ -423,6 +426,12 @@ int choose_sep_tile(const Geometry& g, int cls_z, size_t smem_limit);
 // they do not fit; *tiles receives the column-tile count they need.
 int fused_bucket(const Geometry& g, size_t smem_limit, int* tiles);
 int fused_groups(const spect_plan_s& P);
+// (re)encode P.fmap after the slab, the view chunk or the forward launch shape changed
+cudaError_t build_fwd_map(spect_plan_s& P);
+size_t fwd_records_floats(const spect_plan_s& P);
+cudaError_t launch_fwd_records(const spect_plan_s& P, cudaStream_t st);
+int fwd_tiles(const spect_plan_s& P);
+void default_fwd_shape(spect_plan_s& P, int sms);
 // Bucket of the fused full-PSF kernels (untiled planes), 0 when they do not fit.
 int fused_dir_bucket(const Geometry& g, size_t smem_limit);
 bool fused_dir_fit(const Geometry& g, int bucket, int J, int adj_J, size_t smem_limit);
