@@ -35,15 +35,15 @@ namespace spect {
 // ============================================================================
 
 // out[c][r] = in[r][c] for an R x C matrix (tiled through shared memory).
-__global__ void k_transpose(const float* __restrict__ in, float* __restrict__ out, int R, int C)
+__global__ void k_transpose(const float* __restrict__ in, float* __restrict__ out, int R, int C, int ip, int op)
 {
-    transpose_body(in, out, R, C, blockIdx.x, blockIdx.y);
+    transpose_body(in, out, R, C, ip, op, blockIdx.x, blockIdx.y);
 }
 
-cudaError_t launch_transpose(const float* in, float* out, int R, int C, cudaStream_t st)
+cudaError_t launch_transpose(const float* in, float* out, int R, int C, int ip, int op, cudaStream_t st)
 {
     dim3 grid((C + 31) / 32, (R + 31) / 32);
-    k_transpose<<<grid, dim3(32, 8), 0, st>>>(in, out, R, C);
+    k_transpose<<<grid, dim3(32, 8), 0, st>>>(in, out, R, C, ip, op);
     return cudaGetLastError();
 }
 
@@ -77,9 +77,13 @@ __global__ void __launch_bounds__(kMuThreads) k_mubar_cache(Geometry g, int ps, 
         TB[j] = __ldg(reinterpret_cast<const int*>(tab + 4 * g.nx) + i);
     }
     __syncthreads();
-    if (k >= g.nz) return;
-    const size_t rs = (size_t)g.nx * g.nz;
-    float* out = mubar + (size_t)v * g.ny * ps + (size_t)i * g.nz + k;
+    if (k >= g.kp) return;
+    const size_t rs = (size_t)g.nx * g.kp;
+    float* out = mubar + (size_t)v * g.ny * ps + (size_t)i * g.kp + k;
+    if (k >= g.nz) {  // padding
+        for (int j = 0; j < g.ny; ++j) out[(size_t)j * ps] = 0.f;
+        return;
+    }
     if (!g.has_mu) {
         for (int j = 0; j < g.ny; ++j) out[(size_t)j * ps] = 1.f;
         return;
@@ -88,12 +92,12 @@ __global__ void __launch_bounds__(kMuThreads) k_mubar_cache(Geometry g, int ps, 
 #pragma unroll 8
     for (int j = g.ny - 1; j >= 0; --j) {
         const float4 w = TW[j];
-        const float* m = mu_t + (size_t)TB[j] * g.nz + k;
+        const float* m = mu_t + (size_t)TB[j] * g.kp + k;
         float mv = 0.f;
         mv = __fmaf_rn(w.x, __ldg(m), mv);
-        mv = __fmaf_rn(w.y, __ldg(m + g.nz), mv);
+        mv = __fmaf_rn(w.y, __ldg(m + g.kp), mv);
         mv = __fmaf_rn(w.z, __ldg(m + rs), mv);
-        mv = __fmaf_rn(w.w, __ldg(m + rs + g.nz), mv);
+        mv = __fmaf_rn(w.w, __ldg(m + rs + g.kp), mv);
         out[(size_t)j * ps] = sc.step(mv, g.dy);
     }
 }
@@ -106,9 +110,9 @@ cudaError_t mubar_launch(const spect_plan_s& P, const float* mu_t, int l0, int n
         cudaError_t e = cudaFuncSetAttribute(k_mubar_cache, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    // a run of columns k per block: nz rounded up to whole warps, at most kMuThreads
-    const int thr = std::min(kMuThreads, (P.g.nz + 31) & ~31);
-    const dim3 grid((P.g.nz + thr - 1) / thr, P.g.nx, nv);
+    // a run of columns k per block: kp rounded up to whole warps, at most kMuThreads
+    const int thr = std::min(kMuThreads, (P.g.kp + 31) & ~31);
+    const dim3 grid((P.g.kp + thr - 1) / thr, P.g.nx, nv);
     k_mubar_cache<<<grid, thr, smem, st>>>(P.g, P.ps, P.ts, P.rtab, mu_t, P.mubar, l0);
     return cudaGetLastError();
 }
@@ -152,7 +156,7 @@ cudaError_t launch_rot_tables(const spect_plan_s& P, cudaStream_t st)
 }
 
 // Fixed-length adjacency lists for the transposed rotation: for destination
-// q and view l, up to `maxe` (source column offset j*ps + i*nz, weight) pairs,
+// q and view l, up to `maxe` (source column offset j*ps + i*kp, weight) pairs,
 // zero-padded, laid out [q][l][e].  The candidate search and weights are those
 // of k_build_adjacency (rotate.cu).
 __global__ void k_build_adjacency_fixed(Geometry g, int ps, const ViewRot* __restrict__ rot, int maxe, AdjEntry* adj)
@@ -182,7 +186,7 @@ __global__ void k_build_adjacency_fixed(Geometry g, int ps, const ViewRot* __res
             const float w = bilinear_w(s, di, dj);
             if (w == 0.f || cnt >= maxe) continue;
             AdjEntry e;
-            e.p = pj * ps + pi * g.nz;  // offset of the source column in a [j][i][k] slab with plane stride ps
+            e.p = pj * ps + pi * g.kp;  // offset of the source column in a [j][i][k] slab with plane stride ps
             e.w = w;
             out[cnt++] = e;
         }
@@ -266,7 +270,7 @@ __global__ void __launch_bounds__(kRotThreads, 2) k_rot_fwd8(Geometry g, FusedDi
                 if (k < nz) {
 #pragma unroll
                     for (int m = 0; m < 8; ++m) xs[q][m] = __ldg(xt + o[m] + k);
-                    if (!MUS) ma[q] = __ldg(mb + i * nz + k);
+                    if (!MUS) ma[q] = __ldg(mb + i * g.kp + k);
                 }
             }
             if (!waited) {
@@ -277,7 +281,7 @@ __global__ void __launch_bounds__(kRotThreads, 2) k_rot_fwd8(Geometry g, FusedDi
             for (int q = 0; q < 3; ++q) {
                 const int k = k0 + 32 * q + lane;
                 if (k < nz) {
-                    if (MUS) ma[q] = MU[i * nz + k];
+                    if (MUS) ma[q] = MU[i * g.kp + k];
                     float* wr = S + k * wp + C;
                     float va = w[0] * xs[q][0];
 #pragma unroll
@@ -396,11 +400,12 @@ __host__ __device__ inline size_t dir_fwd_smem_floats(const FusedDims& d, int nz
     return 2 * xarea + (size_t)P * PT + (size_t)d.urows * d.apc + 8;
 }
 
-__host__ __device__ inline size_t dir_adj_smem_floats(const FusedDims& d, int nz, int P, int PT, int ZH, int ncls)
+__host__ __device__ inline size_t dir_adj_smem_floats(const FusedDims& d, int nz, int P, int PT, int ZH, int ncls,
+                                                      int nmb)
 {
     const size_t xarea = ((size_t)dir_rows(nz, ZH) * d.wp + 3) & ~(size_t)3;
-    // Vx | MB x2 | taps ncls x P x PT | 2 mbarriers
-    return xarea + 2 * (size_t)d.marea + (size_t)ncls * P * PT + 8;
+    // Vx | MB x nmb | taps ncls x P x PT | 2 mbarriers
+    return xarea + (size_t)nmb * d.marea + (size_t)ncls * P * PT + 8;
 }
 
 template <int P>
@@ -505,7 +510,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_dir_fused(Geometry g, 
 }
 
 template <int P>
-__global__ void __launch_bounds__(kFusedThreads, 1) k_adj_dir_fused(Geometry g, FusedDims d, int cls_z,
+__global__ void __launch_bounds__(kFusedThreads, 1) k_adj_dir_fused(Geometry g, FusedDims d, int cls_z, int nmb,
                                                                      const float* __restrict__ vin,
                                                                      const float* __restrict__ mubar,
                                                                      const float* __restrict__ psf_adj,
@@ -518,8 +523,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_adj_dir_fused(Geometry g, 
     const int xarea = (dir_rows(nz, ZH) * d.wp + 3) & ~3;
     const int ncls = 3 * cls_z;                    // edge classes (ci, ck)
     float* Vx = sm;                                // zero-padded detector plane, Vx[ZH + k][C + i]
-    float* MB = Vx + xarea;                        // [2][marea]
-    float* TAP = MB + 2 * (size_t)d.marea;         // [ci * cls_z + ck][P][PT], this plane
+    float* MB = Vx + xarea;                        // [nmb][marea]: two, or one where two do not fit
+    float* TAP = MB + (size_t)nmb * d.marea;       // [ci * cls_z + ck][P][PT], this plane
     uint64_t* bar = reinterpret_cast<uint64_t*>(TAP + (size_t)ncls * P * PT);
     const int tid = threadIdx.x;
     constexpr int T = kFusedThreads;
@@ -548,7 +553,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_adj_dir_fused(Geometry g, 
 
     unsigned phases = 0u;
     for (int j = j_begin; j < j_end; ++j) {
-        const int b = (j - j_begin) & 1;
+        const int b = nmb == 1 ? 0 : (j - j_begin) & 1;
         // taps of every edge class of this plane
         for (int e = tid; e < ncls * P * PT; e += T) {
             const int cls = e / (P * PT), r = e - cls * P * PT, bb = r / PT, a = r - bb * PT;
@@ -559,7 +564,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_adj_dir_fused(Geometry g, 
         }
         __syncthreads();
         // the other buffer receives the next plane's attenuation once its store has read it
-        if (tid == 0 && j + 1 < j_end) {
+        if (nmb == 1 && tid == 0 && j > j_begin) {  // the one buffer: this plane's, once the last store has read it
+            tma_store_wait_read<0>();
+            tma_load_1d(MB, mub + (size_t)j * d.ps, mbytes, bar);
+        }
+        if (nmb == 2 && tid == 0 && j + 1 < j_end) {
             tma_store_wait_read<0>();
             tma_load_1d(MB + (b ^ 1) * (size_t)d.marea, mub + (size_t)(j + 1) * d.ps, mbytes, bar + (b ^ 1));
         }
@@ -607,10 +616,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_adj_dir_fused(Geometry g, 
                             if (c == cl) o[c] = edge(c, nx == 1 ? 0 : 2);
                     }
                 }
-                float* mp = mb + li * nz + k;
+                float* mp = mb + li * g.kp + k;
 #pragma unroll
                 for (int c = 0; c < CX; ++c)
-                    if (li + c < nx) mp[c * nz] = o[c] * mp[c * nz];
+                    if (li + c < nx) mp[c * g.kp] = o[c] * mp[c * g.kp];
             }
         }
         if (__syncthreads_or(!ok)) {
@@ -632,29 +641,18 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_adj_dir_fused(Geometry g, 
 // x_t(q,k) (+)= sum_{v in chunk} sum_{e < MAXE} w_e t[v][p_e][k]
 // with the EM update (em_update) on the last chunk when em.x is set.  The
 // lists are laid out [q][l][e] so one destination's entries for all views are
-// contiguous; each entry holds the premultiplied offset p*nz of its source
-// column in the slab.  A thread owns VEC consecutive k of one destination (float4 loads
-// when nz % 4 == 0).  Per view the few terms are summed plainly, the views
+// contiguous; each entry holds the premultiplied offset p*kp of its source
+// column in the slab.  A thread owns four consecutive k of one destination (float4 loads).  Per view the few terms are summed plainly, the views
 // with Kahan compensation.
-template <int VEC>
-struct VecT;
-template <>
-struct VecT<1> {
-    using type = float;
-};
-template <>
-struct VecT<4> {
-    using type = float4;
-};
-
-template <int MAXE, int VEC>
+template <int MAXE>
 __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const AdjEntry* __restrict__ adj,
                                                    const float* __restrict__ slab, int l0, int nv, float* out,
                                                    int accumulate, EmArgs em)
 {
-    using VT = typename VecT<VEC>::type;
+    using VT = float4;
+    constexpr int VEC = 4;
     const int nxy = g.nx * g.ny;
-    const int nzv = g.nz / VEC;
+    const int nzv = g.kp / VEC;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= nxy * nzv) return;
     const int qq = idx / nzv;
@@ -723,7 +721,7 @@ __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const Adj
         e += MAXE;
         t += vstride;
     }
-    const size_t o = (size_t)q * g.nz + k;
+    const size_t o = (size_t)q * g.kp + k;
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
         float val = acc[u].value();
@@ -746,7 +744,7 @@ int tiles_that_fit(const Geometry& g, size_t limit, int min_tiles)
         const FusedDims d = dims_for<P>(g, 8, t);
         if (d.nT == last_nt) continue;  // same tile width as a smaller request
         last_nt = d.nT;
-        if (smem_fwd_bound<P>(g, d) <= limit && smem_adj<P>(g, d) <= limit && rot_smem_min(d) <= limit &&
+        if (smem_fwd_bound<P>(g, d) <= limit && smem_adj_bound<P>(g, d) <= limit && rot_smem_min(d) <= limit &&
             (size_t)d.marea * 4 < (1u << 20))
             return d.nT;
     }
@@ -806,9 +804,9 @@ size_t dir_smem_fwd(const Geometry& g, const FusedDims& d)
 }
 
 template <int P>
-size_t dir_smem_adj(const Geometry& g, const FusedDims& d, int cls_z)
+size_t dir_smem_adj(const Geometry& g, const FusedDims& d, int cls_z, int nmb)
 {
-    return dir_adj_smem_floats(d, g.nz, P, Sep<P>::PT, Sep<P>::ZH, 3 * cls_z) * sizeof(float);
+    return dir_adj_smem_floats(d, g.nz, P, Sep<P>::PT, Sep<P>::ZH, 3 * cls_z, nmb) * sizeof(float);
 }
 
 template <int P>
@@ -816,8 +814,11 @@ bool dir_fits(const Geometry& g, size_t limit, int J, int adj_J)
 {
     const int cls_z = g.nz >= 2 ? 3 : 1;
     const FusedDims df = dims_for<P>(g, J, 1), da = dims_for<P>(g, adj_J, 1);
-    return df.nT == 1 && dir_smem_fwd<P>(g, df) <= limit && dir_smem_adj<P>(g, da, cls_z) <= limit &&
-           rot_smem_min(df) <= limit && (size_t)df.ps * 4 < (1u << 20);
+    // attenuation planes counted without their k padding: where that leaves no room for
+    // two padded ones, the adjoint runs with one
+    const size_t pad = 2 * ((size_t)da.marea - (((size_t)g.nx * g.nz + 3) & ~(size_t)3)) * sizeof(float);
+    return df.nT == 1 && dir_smem_fwd<P>(g, df) <= limit && dir_smem_adj<P>(g, da, cls_z, 2) - pad <= limit &&
+           dir_smem_adj<P>(g, da, cls_z, 1) <= limit && rot_smem_min(df) <= limit && (size_t)df.ps * 4 < (1u << 20);
 }
 
 template <int P>
@@ -835,11 +836,12 @@ template <int P>
 cudaError_t dir_adj_launch(const spect_plan_s& Pl, const float* v, int l0, int nv, cudaStream_t st)
 {
     const FusedDims d = dims_for<P>(Pl.g, Pl.adj_J, 1);
-    const size_t smem = dir_smem_adj<P>(Pl.g, d, Pl.cls_z);
+    const int nmb = dir_smem_adj<P>(Pl.g, d, Pl.cls_z, 2) <= (size_t)Pl.smem_optin ? 2 : 1;
+    const size_t smem = dir_smem_adj<P>(Pl.g, d, Pl.cls_z, nmb);
     cudaError_t e = cudaFuncSetAttribute(k_adj_dir_fused<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_adj_dir_fused<P><<<dim3(d.G, nv), kFusedThreads, smem, st>>>(Pl.g, d, Pl.cls_z, v, mubar_for(Pl, l0), Pl.psf_adj,
-                                                                    Pl.slab, l0, Pl.err);
+    k_adj_dir_fused<P><<<dim3(d.G, nv), kFusedThreads, smem, st>>>(Pl.g, d, Pl.cls_z, nmb, v, mubar_for(Pl, l0),
+                                                                    Pl.psf_adj, Pl.slab, l0, Pl.err);
     return cudaGetLastError();
 }
 }  // namespace
@@ -897,7 +899,7 @@ int fused_tiles_fit(const Geometry& g, int bucket, int J, int adj_J, int tiles, 
     auto check = [&](auto tag) -> int {
         constexpr int B = decltype(tag)::value;
         const FusedDims df = dims_for<B>(g, J, tiles), da = dims_for<B>(g, adj_J, tiles);
-        const bool ok = smem_fwd_bound<B>(g, df) <= smem_limit && smem_adj<B>(g, da) <= smem_limit &&
+        const bool ok = smem_fwd_bound<B>(g, df) <= smem_limit && smem_adj_bound<B>(g, da) <= smem_limit &&
                         rot_smem_min(df) <= smem_limit && (size_t)df.marea * 4 < (1u << 20);
         return ok ? df.nT : 0;
     };
@@ -1028,6 +1030,27 @@ void default_fwd_shape(spect_plan_s& P, int sms)
     if (blocks(8) < 10ll * sms) P.fused_J = blocks(4) >= 4ll * sms ? 4 : 2;
 }
 
+// Column tiles of the blur adjoint: the fewest, at least adj_nT, that fit with adj_J planes per block.
+int adj_tiles(const spect_plan_s& P)
+{
+    auto find = [&](auto tag) -> int {
+        constexpr int B = decltype(tag)::value;
+        for (int t = P.adj_nT; t <= (P.g.nx + 15) / 16; ++t) {
+            const FusedDims d = dims_for<B>(P.g, P.adj_J, t);
+            if (smem_adj<B>(P.g, d) <= (size_t)P.smem_optin) return d.nT;
+        }
+        return P.adj_nT;
+    };
+    switch (P.bucket) {
+#define SPECT_AT(B) \
+    case B: return find(std::integral_constant<int, B>());
+        SPECT_AT(3) SPECT_AT(5) SPECT_AT(7) SPECT_AT(9) SPECT_AT(11) SPECT_AT(13) SPECT_AT(15)
+        SPECT_AT(17) SPECT_AT(21) SPECT_AT(25) SPECT_AT(29) SPECT_AT(33) SPECT_AT(37)
+#undef SPECT_AT
+        default: return P.adj_nT;
+    }
+}
+
 // Column tiles of the forward blur at its launch shape (what fwd_dims makes of the request).
 int fwd_tiles(const spect_plan_s& P)
 {
@@ -1053,7 +1076,7 @@ size_t fused_slab_per_view(const spect_plan_s& P)
 #undef SPECT_AREA
         default: break;
     }
-    const size_t ps = ((size_t)P.g.nx * P.g.nz + 3) & ~(size_t)3;
+    const size_t ps = (size_t)P.g.nx * P.g.kp;
     return (size_t)P.g.ny * (parea > ps ? parea : ps);
 }
 
@@ -1077,18 +1100,12 @@ cudaError_t launch_fwd_reduce(const spect_plan_s& P, float* v, const float* em_y
 cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, int accumulate, EmArgs em,
                              cudaStream_t st)
 {
-    const bool vec4 = (P.g.nz % 4) == 0;
-    const size_t n = (size_t)P.g.nx * P.g.ny * (vec4 ? P.g.nz / 4 : P.g.nz);
+    const size_t n = (size_t)P.g.nx * P.g.ny * (P.g.kp / 4);
     const unsigned blocks = (unsigned)((n + 255) / 256);
     const float* src = P.slab;
     switch (P.adj_max) {
 #define SPECT_ADJ(M)                                                                                                 \
-    case M:                                                                                                          \
-        if (vec4)                                                                                                    \
-            k_adj_rot_t<M, 4><<<blocks, 256, 0, st>>>(P.g, P.ps, P.adjf, src, l0, nv, out, accumulate, em);    \
-        else                                                                                                         \
-            k_adj_rot_t<M, 1><<<blocks, 256, 0, st>>>(P.g, P.ps, P.adjf, src, l0, nv, out, accumulate, em);    \
-        break;
+    case M: k_adj_rot_t<M><<<blocks, 256, 0, st>>>(P.g, P.ps, P.adjf, src, l0, nv, out, accumulate, em); break;
         SPECT_ADJ(1) SPECT_ADJ(2) SPECT_ADJ(3) SPECT_ADJ(4) SPECT_ADJ(5) SPECT_ADJ(6) SPECT_ADJ(7) SPECT_ADJ(8)
 #undef SPECT_ADJ
         default: return cudaErrorInvalidValue;

@@ -39,21 +39,21 @@ __device__ __forceinline__ void rot_table_entry(int i, int j, const ViewRot r, c
 
 }  // namespace
 
-// out[c][r] = in[r][c] for the 32x32 tile (bx, by) of an R x C matrix (tiled
-// through shared memory; blocks of 32 x 8 threads).
+// out[c][r] = in[r][c] for the 32x32 tile (bx, by) of an R x C matrix with row
+// pitches ip and op (tiled through shared memory; blocks of 32 x 8 threads).
 __device__ __forceinline__ void transpose_body(const float* __restrict__ in, float* __restrict__ out, int R, int C,
-                                               int bx, int by)
+                                               int ip, int op, int bx, int by)
 {
     __shared__ float tile[32][33];
     const int c0 = bx * 32, r0 = by * 32;
     for (int dy = threadIdx.y; dy < 32; dy += blockDim.y) {
         const int r = r0 + dy, c = c0 + threadIdx.x;
-        if (r < R && c < C) tile[dy][threadIdx.x] = in[(size_t)r * C + c];
+        if (r < R && c < C) tile[dy][threadIdx.x] = in[(size_t)r * ip + c];
     }
     __syncthreads();
     for (int dy = threadIdx.y; dy < 32; dy += blockDim.y) {
         const int c = c0 + dy, r = r0 + threadIdx.x;
-        if (r < R && c < C) out[(size_t)c * R + r] = tile[threadIdx.x][dy];
+        if (r < R && c < C) out[(size_t)c * op + r] = tile[threadIdx.x][dy];
     }
 }
 
@@ -115,9 +115,9 @@ struct FusedDims {
     int farea;  // floats of a plane image in the slab (and the rotation kernel's shared memory)
     int urows;  // rows of U / ACC / MB per tile: min(TI, nx)
     int vrows;  // detector rows a tile's k-adjoint needs: min(nx, TI + 2*C)
-    int marea;  // floats of an attenuation tile, urows*nz rounded up to 4
+    int marea;  // floats of an attenuation tile, urows*kp
     int J, G;   // depth planes per block, depth groups
-    int ps;     // plane stride of the attenuation cache / slab (nx*nz rounded up to 4)
+    int ps;     // plane stride of the attenuation cache / slab (nx*kp)
     int ts;     // rotation table block per (view, row): 5*nx rounded up to 4
     int apc;    // accumulator row pitch (>= nkb*CZ, multiple of 4, pitch/4 odd)
 };
@@ -249,11 +249,11 @@ __device__ __forceinline__ void rot_fwd_body(const Geometry& g, const FusedDims&
     float* TBL = sm + d.farea;  // the (view, row) rotation table: nx float4 weights, then nx bases
     float* MU = TBL + d.ts;     // [i][k] attenuation plane (MUS)
     uint64_t* bar = reinterpret_cast<uint64_t*>(MU + d.ps);
-    const int nx = g.nx, ny = g.ny, nz = g.nz;
+    const int nx = g.nx, ny = g.ny, nz = g.nz, kp = g.kp;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int NW = kRotThreads / 32;
     const int l = l0 + v;
-    const int pln = nx * nz;
+    const int pln = nx * kp;
     const int wp = d.wpf;
     const int wcols = d.nib * Sep<P>::CX + 2 * C;
     const float* tab = rtab + ((size_t)l * ny + j) * d.ts;
@@ -275,8 +275,8 @@ __device__ __forceinline__ void rot_fwd_body(const Geometry& g, const FusedDims&
         const bool two = i + 1 < nx;
         const float4 wa = TW[i];
         const float4 wb = two ? TW[i + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float* pa = xt + (size_t)TB[i] * nz;
-        const float* pb = xt + (size_t)TB[two ? i + 1 : i] * nz;
+        const float* pa = xt + (size_t)TB[i] * kp;
+        const float* pb = xt + (size_t)TB[two ? i + 1 : i] * kp;
         for (int k0 = 0; k0 < nz; k0 += 96) {
             float xa[3][4], xb[3][4], ma[3], mc[3];
 #pragma unroll
@@ -284,16 +284,16 @@ __device__ __forceinline__ void rot_fwd_body(const Geometry& g, const FusedDims&
                 const int k = k0 + 32 * q + lane;
                 if (k < nz) {
                     xa[q][0] = __ldg(pa + k);
-                    xa[q][1] = __ldg(pa + nz + k);
+                    xa[q][1] = __ldg(pa + kp + k);
                     xa[q][2] = __ldg(pa + pln + k);
-                    xa[q][3] = __ldg(pa + pln + nz + k);
+                    xa[q][3] = __ldg(pa + pln + kp + k);
                     xb[q][0] = __ldg(pb + k);
-                    xb[q][1] = __ldg(pb + nz + k);
+                    xb[q][1] = __ldg(pb + kp + k);
                     xb[q][2] = __ldg(pb + pln + k);
-                    xb[q][3] = __ldg(pb + pln + nz + k);
+                    xb[q][3] = __ldg(pb + pln + kp + k);
                     if (!MUS) {
-                        ma[q] = __ldg(mb + i * nz + k);
-                        mc[q] = two ? __ldg(mb + (i + 1) * nz + k) : 0.f;
+                        ma[q] = __ldg(mb + i * kp + k);
+                        mc[q] = two ? __ldg(mb + (i + 1) * kp + k) : 0.f;
                     }
                 }
             }
@@ -306,8 +306,8 @@ __device__ __forceinline__ void rot_fwd_body(const Geometry& g, const FusedDims&
                 const int k = k0 + 32 * q + lane;
                 if (k < nz) {
                     if (MUS) {
-                        ma[q] = MU[i * nz + k];
-                        mc[q] = two ? MU[(i + 1) * nz + k] : 0.f;
+                        ma[q] = MU[i * kp + k];
+                        mc[q] = two ? MU[(i + 1) * kp + k] : 0.f;
                     }
                     float* wr = S + k * wp + C;
                     float va = wa.x * xa[q][0];
@@ -628,14 +628,15 @@ __device__ __forceinline__ void adj_sep_body(const Geometry& g, const FusedDims&
     const int last_col = nx - 1 - i0;    // tile-relative position of column nx-1
     const bool first_tile = i0 == 0;
     // attenuation / t tile: columns [i0, i0 + ti) of a plane are one contiguous run
-#define SPECT_MBYTES ((unsigned)(((size_t)ti * nz + 3) & ~(size_t)3) * 4u)
+#define SPECT_MBYTES ((unsigned)(ti * kp) * 4u)
     const int lp = g.nvp == 1 ? 0 : l;
     const int j_begin = grp * d.J, j_end = min(ny, j_begin + d.J);
     const int ox = (P - g.px) / 2, oz = (P - g.pz) / 2;
     const size_t nrow = (size_t)g.nvp * ny;
     const int pln = nx * nz;
-    const float* mub = mubar + ((size_t)l * ny) * d.ps + (size_t)i0 * nz;
-    float* tsl = slab + ((size_t)v * ny) * d.ps + (size_t)i0 * nz;
+    const int kp = g.kp;
+    const float* mub = mubar + ((size_t)l * ny) * d.ps + (size_t)i0 * kp;
+    float* tsl = slab + ((size_t)v * ny) * d.ps + (size_t)i0 * kp;
 
     // the first plane's attenuation is requested before anything else
     if (tid == 0) {
@@ -749,14 +750,14 @@ __device__ __forceinline__ void adj_sep_body(const Geometry& g, const FusedDims&
                 const int cl = last_col - li;  // position of column nx-1 in this run
                 const bool last = cl < CX;
                 const float e_last = last ? edge_tap_dot<P>(FX + 2 * PT, zr - li, li + cl) : 0.f;
-                float* mp = mb + li * nz + k;
+                float* mp = mb + li * kp + k;
                 if (!last) {
 #pragma unroll
-                    for (int c = 0; c < CX; ++c) mp[c * nz] = o[c] * mp[c * nz];
+                    for (int c = 0; c < CX; ++c) mp[c * kp] = o[c] * mp[c * kp];
                 } else {
 #pragma unroll
                     for (int c = 0; c < CX; ++c)
-                        if (c <= cl) mp[c * nz] = (c == cl ? e_last : o[c]) * mp[c * nz];
+                        if (c <= cl) mp[c * kp] = (c == cl ? e_last : o[c]) * mp[c * kp];
                 }
             }
         }
@@ -787,7 +788,7 @@ FusedDims dims_for(const Geometry& g, int J, int tiles)
 {
     using S = Sep<P>;
     FusedDims d;
-    d.ps = (g.nx * g.nz + 3) & ~3;
+    d.ps = g.nx * g.kp;
     d.ts = (5 * g.nx + 3) & ~3;
     d.nib = (g.nx + S::CX - 1) / S::CX;
     d.nkb = (g.nz + S::CZ - 1) / S::CZ;
@@ -796,7 +797,7 @@ FusedDims dims_for(const Geometry& g, int J, int tiles)
     d.nT = (g.nx + d.TI - 1) / d.TI;
     d.urows = d.TI < g.nx ? d.TI : g.nx;
     d.vrows = d.TI + 2 * S::C < g.nx ? d.TI + 2 * S::C : g.nx;
-    d.marea = (d.urows * g.nz + 3) & ~3;
+    d.marea = d.urows * g.kp;
     d.wp = pitch4odd(d.TI + 2 * S::C);
     d.warea = (g.nz * d.wp + 3) & ~3;
     d.wpf = pitch4odd(d.nib * S::CX + 2 * S::C);
@@ -878,6 +879,20 @@ size_t smem_fwd(const FwdDims& d)
     return fwd_smem_floats(d, Sep<P>::PT) * sizeof(float);
 }
 
+template <int P>
+size_t smem_adj(const Geometry& g, const FusedDims& d)
+{
+    (void)g;
+    return adj_smem_floats(d, Sep<P>::PT) * sizeof(float);
+}
+
+// The same for the blur adjoint, its attenuation planes counted without their k padding.
+template <int P>
+size_t smem_adj_bound(const Geometry& g, const FusedDims& d)
+{
+    return smem_adj<P>(g, d) - 2 * ((size_t)d.marea - (((size_t)d.urows * g.nz + 3) & ~(size_t)3)) * sizeof(float);
+}
+
 // The geometries and shapes that the fused kernels take: two tile buffers, U,
 // accumulators, taps and folds of a block in shared memory.  (The forward kernel needs
 // less: its sums are in registers and one buffer may do.)
@@ -886,13 +901,6 @@ size_t smem_fwd_bound(const Geometry& g, const FusedDims& d)
 {
     return (2 * (size_t)d.warea + (size_t)d.urows * d.kpu + 2 * (size_t)Sep<P>::PT * d.J + (size_t)d.urows * d.apc +
             2 * (size_t)d.J * d.nkb * 16 + 8) * sizeof(float);
-}
-
-template <int P>
-size_t smem_adj(const Geometry& g, const FusedDims& d)
-{
-    (void)g;
-    return adj_smem_floats(d, Sep<P>::PT) * sizeof(float);
 }
 
 // The fewest column tiles with which the rotation, blur and adjoint kernels

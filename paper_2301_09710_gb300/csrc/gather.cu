@@ -45,7 +45,7 @@ __global__ void k_patch_boxes(Geometry g, int ps, int maxe, const AdjEntry* __re
         const AdjEntry* e = adjf + ((size_t)(qj * g.nx + qi) * g.nview + l) * maxe;
         for (int m = 0; m < maxe; ++m) {
             if (e[m].w == 0.f) continue;
-            const int pj = e[m].p / ps, pi = (e[m].p - pj * ps) / g.nz;
+            const int pj = e[m].p / ps, pi = (e[m].p - pj * ps) / g.kp;
             atomicMin(&mn_i, pi);
             atomicMin(&mn_j, pj);
             atomicMax(&mx_i, pi);
@@ -76,7 +76,7 @@ __global__ void k_patch_entries(Geometry g, int ps, int maxe, const AdjEntry* __
         o.p = 0;
         o.w = 0.f;
         if (inside && e[m].w != 0.f) {
-            const int pj = e[m].p / ps, pi = (e[m].p - pj * ps) / g.nz;
+            const int pj = e[m].p / ps, pi = (e[m].p - pj * ps) / g.kp;
             o.p = ((pj - b.y) * bw + (pi - b.x)) * kc;
             o.w = e[m].w;
         }
@@ -163,8 +163,8 @@ __device__ __forceinline__ void adj_gather_body(const CUtensorMap* tmap, const G
     const int qi = (patch % a.npx) * kPatch + (ql % kPatch), qj = (patch / a.npx) * kPatch + (ql / kPatch);
     // the EM epilogue's operands, fetched before the view loop so their latency hides behind it
     const int k = kc0 + 4 * k4;
-    const bool mine = qi < g.nx && qj < g.ny && k < g.nz;
-    const size_t o = mine ? (size_t)(qj * g.nx + qi) * g.nz + k : 0;
+    const bool mine = qi < g.nx && qj < g.ny && k < g.kp;
+    const size_t o = mine ? (size_t)(qj * g.nx + qi) * g.kp + k : 0;
     float4 ex = make_float4(0.f, 0.f, 0.f, 0.f), es = ex, eu = ex;
     if (mine && em.x) {
         ex = *reinterpret_cast<const float4*>(em.x + o);
@@ -286,13 +286,13 @@ EncodeTiled encode_fn()
 int gather_kc() { return 16; }
 
 // Plan time: boxes, box extents and patch entries.  Leaves P.gather = 0 when
-// the geometry does not suit the kernel (k rows not a whole number of 16-byte
-// units, boxes too large for the tensor map or shared memory, no encoder).
+// the geometry does not suit the kernel (boxes too large for the tensor map or
+// shared memory, no encoder).
 cudaError_t build_gather(spect_plan_s& P, cudaStream_t st)
 {
     P.gather = 0;
     const Geometry& g = P.g;
-    if (!P.fast || (g.nz % 4) != 0 || !encode_fn()) return cudaSuccess;
+    if (!P.fast || !encode_fn()) return cudaSuccess;
     const char* env = getenv("SPECT_GATHER");  // 0: use the list gather k_adj_rot_t (testing)
     if (env && atoi(env) == 0) return cudaSuccess;
     const int npx = (g.nx + kPatch - 1) / kPatch, npy = (g.ny + kPatch - 1) / kPatch;
@@ -349,15 +349,15 @@ cudaError_t build_gather(spect_plan_s& P, cudaStream_t st)
 }
 
 namespace {
-// The t slab as a 3D tensor map -- k (nz, contiguous) x i (nx, stride nz) x
+// The t slab as a 3D tensor map -- k (kp, contiguous) x i (nx, stride kp) x
 // plane (chunk * ny, stride ps) -- and the gather's arguments for views
 // [l0, l0 + nv).
 cudaError_t gather_setup(const spect_plan_s& P, int l0, int nv, CUtensorMap* map, GatherArgs* a)
 {
     const Geometry& g = P.g;
     const int kc = gather_kc();
-    const cuuint64_t dims[3] = {(cuuint64_t)g.nz, (cuuint64_t)g.nx, (cuuint64_t)P.chunk * g.ny};
-    const cuuint64_t strides[2] = {(cuuint64_t)g.nz * 4, (cuuint64_t)P.ps * 4};
+    const cuuint64_t dims[3] = {(cuuint64_t)g.kp, (cuuint64_t)g.nx, (cuuint64_t)P.chunk * g.ny};
+    const cuuint64_t strides[2] = {(cuuint64_t)g.kp * 4, (cuuint64_t)P.ps * 4};
     const cuuint32_t box[3] = {(cuuint32_t)kc, (cuuint32_t)P.gbw, (cuuint32_t)P.gbh};
     const cuuint32_t estr[3] = {1, 1, 1};
     if (encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, P.slab, dims, strides, box, estr,
@@ -374,7 +374,7 @@ cudaError_t gather_setup(const spect_plan_s& P, int l0, int nv, CUtensorMap* map
     a->stage_floats = stage_floats(a->box_floats, a->ent_bytes);
     a->l0 = l0;
     a->nv = nv;
-    a->nkc = (g.nz + kc - 1) / kc;
+    a->nkc = (g.kp + kc - 1) / kc;
     return cudaSuccess;
 }
 }  // namespace

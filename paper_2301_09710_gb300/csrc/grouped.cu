@@ -50,7 +50,7 @@ struct GroupPlans {
 struct GroupT {
     const float* in;
     float* out;
-    int R, C;
+    int R, C, ip, op;
 };
 struct GroupTs {
     GroupT p[kGroupMax];
@@ -101,7 +101,7 @@ __global__ void k_transpose_grp(const __grid_constant__ GroupTs gt)
 {
     const int4 w = group_item(gt.grid);
     const GroupT& q = gt.p[w.x];
-    transpose_body(q.in, q.out, q.R, q.C, w.y, w.z);
+    transpose_body(q.in, q.out, q.R, q.C, q.ip, q.op, w.y, w.z);
 }
 
 size_t plan_work(const spect_plan_s* P)
@@ -298,6 +298,8 @@ cudaError_t transpose_launches(const std::vector<spect_plan_s*>& plans, float* c
             q.out = to_internal ? Pl->xt : x[ch[m]];
             q.R = to_internal ? nz : nxy;
             q.C = to_internal ? nxy : nz;
+            q.ip = to_internal ? nxy : Pl->g.kp;
+            q.op = to_internal ? Pl->g.kp : nxy;
             add_grid(gt.grid, m, (q.C + 31) / 32, (q.R + 31) / 32, 1);
         }
         out.push_back(make_launch(k_transpose_grp, gt, dim3(32, 8), 0));

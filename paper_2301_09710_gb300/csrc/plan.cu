@@ -264,7 +264,7 @@ spect_status run_back(spect_plan_s* P, const float* v, float* out, spect::EmArgs
 spect_status to_internal(spect_plan_s* P, const float* x, float* xt, cudaStream_t st)
 {
     const int nxy = P->g.nx * P->g.ny;
-    SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_transpose(x, xt, P->g.nz, nxy, st); }),
+    SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_transpose(x, xt, P->g.nz, nxy, nxy, P->g.kp, st); }),
                    "transpose launch");
     return SPECT_OK;
 }
@@ -272,7 +272,7 @@ spect_status to_internal(spect_plan_s* P, const float* x, float* xt, cudaStream_
 spect_status from_internal(spect_plan_s* P, const float* xt, float* x, cudaStream_t st)
 {
     const int nxy = P->g.nx * P->g.ny;
-    SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_transpose(xt, x, nxy, P->g.nz, st); }),
+    SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_transpose(xt, x, nxy, P->g.nz, P->g.kp, nxy, st); }),
                    "transpose launch");
     return SPECT_OK;
 }
@@ -378,6 +378,7 @@ size_t plan_bytes_bound(const spect_plan_s& P)
     const size_t F = sizeof(float);
     const size_t vol = (size_t)g.nx * g.ny * g.nz, nproj = (size_t)g.nx * g.nz * g.nview;
     const size_t nxy = (size_t)g.nx * g.ny, nrows = (size_t)g.nvp * g.ny, nlist = nxy * g.nview;
+    const size_t volt = nxy * g.kp;  // an internal volume
     size_t b = sizeof(int) + vol * F;
     if (P.separable) b += ((size_t)g.px * 4 + (size_t)g.pz * (1 + P.cls_z)) * nrows * F;
     else b += (size_t)g.px * g.pz * nrows * (1 + (size_t)P.cls_x * P.cls_z) * F;
@@ -393,8 +394,8 @@ size_t plan_bytes_bound(const spect_plan_s& P)
     if (P.fast && P.separable) b += spect::fwd_records_floats(P) * F;
     if (P.fast) {
         // attenuation factors of every view, or of one chunk plus mu in the internal layout
-        b += P.recompute ? ((size_t)g.ny * P.ps * chunk + vol) * F : (size_t)g.ny * P.ps * g.nview * F;
-        b += 4 * vol * F;
+        b += P.recompute ? ((size_t)g.ny * P.ps * chunk + volt) * F : (size_t)g.ny * P.ps * g.nview * F;
+        b += 4 * volt * F;
         b += nproj * (size_t)spect::fused_groups(P) * F + (size_t)g.nview * g.ny * P.ts * F;
         // patch gather: boxes and box-local entries (at most 8 per list)
         const size_t np = (size_t)((g.nx + 7) / 8) * ((g.ny + 7) / 8) * g.nview;
@@ -428,7 +429,8 @@ spect_status spect_plan_bytes(int nx, int ny, int nz, int nview, int px, int pz,
     g.nx = nx; g.ny = ny; g.nz = nz; g.nview = nview;
     g.px = px; g.pz = pz; g.nvp = nview_psf;
     P.separable = separable != 0;
-    P.ps = (nx * nz + 3) & ~3;
+    g.kp = (nz + 3) & ~3;
+    P.ps = nx * g.kp;
     P.ts = (5 * nx + 3) & ~3;
     P.cls_x = 3;
     P.cls_z = nz >= 2 ? 3 : 1;
@@ -494,7 +496,8 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
     g.dy = dy;
     g.has_mu = mu != nullptr;
     P->separable = psf_fx && (!psf || (flags & SPECT_PLAN_PREFER_SEPARABLE));
-    P->ps = (nx * nz + 3) & ~3;
+    g.kp = (nz + 3) & ~3;
+    P->ps = nx * g.kp;
     P->ts = (5 * nx + 3) & ~3;
     P->cls_x = 3;
     P->cls_z = nz >= 2 ? 3 : 1;
@@ -540,6 +543,7 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
     int sms = 0;
     PLAN_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device query");
     if (P->fast) spect::default_fwd_shape(*P, sms);
+    if (P->fast && P->separable) P->adj_nT = spect::adj_tiles(*P);
     P->rot3 = (flags & SPECT_PLAN_ROTATION_3PASS) != 0;
     if (P->rot3 && !P->fast) {
         free_plan(P);
@@ -565,6 +569,7 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
 
     const size_t vol = (size_t)nx * ny * nz, nproj = (size_t)nx * nz * nview;
     const size_t nxy = (size_t)nx * ny, nrows = (size_t)nview_psf * ny;
+    const size_t volt = nxy * g.kp;  // an internal volume
 
     PLAN_ALLOC(P->err, 1, "error word");
     PLAN_TRY(cudaMemsetAsync(P->err, 0, sizeof(int), st), "clear error word");
@@ -693,21 +698,23 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         const int mu_views = P->recompute ? P->chunk : nview;
         PLAN_ALLOC(P->mubar, (size_t)ny * P->ps * mu_views, "attenuation cache");
         P->mubar_cap = (size_t)ny * P->ps * mu_views;
-        PLAN_ALLOC(P->xt, vol, "internal image");
-        PLAN_ALLOC(P->et, vol, "internal back-projection");
-        PLAN_ALLOC(P->st, vol, "internal sensitivity");
-        PLAN_ALLOC(P->ut, vol, "internal regulariser target");
+        PLAN_ALLOC(P->xt, volt, "internal image");
+        PLAN_ALLOC(P->et, volt, "internal back-projection");
+        PLAN_ALLOC(P->st, volt, "internal sensitivity");
+        PLAN_ALLOC(P->ut, volt, "internal regulariser target");
+        for (float* p : {P->xt, P->et, P->st, P->ut})  // defines their padding
+            PLAN_TRY(cudaMemsetAsync(p, 0, volt * sizeof(float), st), "clear internal volume");
         PLAN_ALLOC(P->part, nproj * (size_t)spect::fused_groups(*P), "depth-group partial sums");
         P->part_cap = nproj * (size_t)spect::fused_groups(*P);
         // mu in the [j][i][k] layout (temporary, the slab serves as scratch)
-        PLAN_TRY(spect::launch_transpose(P->mu, P->slab, nz, (int)nxy, st), "mu transpose launch");
+        PLAN_TRY(spect::launch_transpose(P->mu, P->slab, nz, (int)nxy, (int)nxy, g.kp, st), "mu transpose launch");
         if (P->rot3) {
             // three passes: the eight-tap table of the forward rotation kernel, the
             // eight-entry lists of the adjoint gather (in adjf), and the attenuation
             // cache from mu turned the same way (one volume of scratch)
             PLAN_ALLOC(P->r3_tab, (size_t)nview * ny * spect::rot3_ts8(nx), "three-pass table");
             float* scratch = nullptr;
-            PLAN_TRY(raw_alloc(P, (void**)&scratch, vol * sizeof(float), st), "three-pass scratch");
+            PLAN_TRY(raw_alloc(P, (void**)&scratch, volt * sizeof(float), st), "three-pass scratch");
             cudaError_t e3 = spect::build_rot3(*P, angles, P->slab, scratch, st);
             raw_free(P, scratch, st);
             PLAN_TRY(e3, "three-pass rotation set-up");
@@ -715,8 +722,8 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
             drop_fixed_lists(P, st);
         } else if (P->recompute) {
             // mu stays in the [j][i][k] layout; the factors are made per view chunk
-            PLAN_ALLOC(P->mut, vol, "attenuation map (internal layout)");
-            PLAN_TRY(cudaMemcpyAsync(P->mut, P->slab, vol * sizeof(float), cudaMemcpyDeviceToDevice, st),
+            PLAN_ALLOC(P->mut, volt, "attenuation map (internal layout)");
+            PLAN_TRY(cudaMemcpyAsync(P->mut, P->slab, volt * sizeof(float), cudaMemcpyDeviceToDevice, st),
                      "attenuation map copy");
             PLAN_ALLOC(P->rtab, (size_t)nview * ny * P->ts, "rotation tables");
             PLAN_TRY(spect::launch_rot_tables(*P, st), "rotation table launch");
@@ -1039,6 +1046,7 @@ spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, int adj_t
     P->adj_J = adj_J;
     P->fwd_nT = nt;
     P->adj_nT = ant;
+    if (P->separable) P->adj_nT = spect::adj_tiles(*P);
     P->fwd_nT = P->separable ? spect::fwd_tiles(*P) : 1;
     const size_t vol = (size_t)g.nx * g.ny * g.nz, nproj = (size_t)g.nx * g.nz * g.nview;
     const size_t per_view = std::max(vol, spect::fused_slab_per_view(*P));
@@ -1152,8 +1160,8 @@ spect_status spect_plan_autotune(spect_plan P, spect_stream stream)
         }
     }
     // inputs of the timed calls: the plan's own scratch (x_t = 1, v = 1)
-    const size_t vol = (size_t)g.nx * g.ny * g.nz, nproj = (size_t)g.nx * g.nz * g.nview;
-    if (spect::launch_fill(P->xt, vol, 1.f, st) != cudaSuccess ||
+    const size_t volt = (size_t)g.nx * g.ny * g.kp, nproj = (size_t)g.nx * g.nz * g.nview;
+    if (spect::launch_fill(P->xt, volt, 1.f, st) != cudaSuccess ||
         spect::launch_fill(P->ratio, nproj, 1.f, st) != cudaSuccess)
         return fail(SPECT_ECUDA, "fill launch failed");
     const int prof = P->prof;

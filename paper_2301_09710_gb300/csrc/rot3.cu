@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) k_gather_taps(Geometry g, int tsn, const 
     const int j = blockIdx.x;
     const float* blk = tab + ((size_t)l * g.ny + j) * tsn;
     const int* off = reinterpret_cast<const int*>(blk + N * g.nx);
-    float* dst = out + (size_t)j * g.nx * g.nz;
+    float* dst = out + (size_t)j * g.nx * g.kp;
     const int n = g.nx * g.nz;
     for (int e = threadIdx.x; e < n; e += blockDim.x) {
         const int i = e / g.nz, k = e - i * g.nz;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(256) k_gather_taps(Geometry g, int tsn, const 
         float acc = w[0] * __ldg(in + o[0] + k);
 #pragma unroll
         for (int m = 1; m < N; ++m) acc = fmaf(w[m], __ldg(in + o[m] + k), acc);
-        dst[(size_t)i * g.nz + k] = acc;
+        dst[(size_t)i * g.kp + k] = acc;
     }
 }
 
@@ -132,8 +132,12 @@ __global__ void k_mubar_rotated(Geometry g, int ps, const float* __restrict__ mu
                                 float* __restrict__ mubar)
 {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int per = g.nx * g.nz;
+    const int per = g.nx * g.kp;
     if (idx >= per) return;
+    if (idx % g.kp >= g.nz) {  // padding
+        for (int j = 0; j < g.ny; ++j) mubar[((size_t)l * g.ny + j) * ps + idx] = 0.f;
+        return;
+    }
     const size_t pln = (size_t)per;
     AttenScan sc;
     for (int j = g.ny - 1; j >= 0; --j) {
@@ -151,10 +155,10 @@ int rot3_ts8(int nx) { return 16 * nx; }
 cudaError_t build_rot3(spect_plan_s& P, const double* angles, const float* mu_t, float* scratch, cudaStream_t st)
 {
     const Geometry& g = P.g;
-    const int n = g.nx, nz = g.nz, nview = g.nview, ts8 = rot3_ts8(n), ps = P.ps, E = P.adj_max;
+    const int n = g.nx, kp = g.kp, nview = g.nview, ts8 = rot3_ts8(n), ps = P.ps, E = P.adj_max;
     if (E < 8) return cudaErrorInvalidValue;  // the lists hold eight entries per (voxel, view)
     const double c = 0.5 * (double)(n - 1);
-    const size_t pln = (size_t)n * nz, nxy = (size_t)n * n;
+    const size_t pln = (size_t)n * kp, nxy = (size_t)n * n;
     std::vector<float> tab((size_t)nview * n * ts8, 0.f);
     std::vector<AdjEntry> lists(nxy * nview * (size_t)E);
     std::vector<Shift> rows(n), cols(n);
@@ -185,7 +189,7 @@ cudaError_t build_rot3(spect_plan_s& P, const double* angles, const float* mu_t,
                             int si, sj;
                             quarter_from(n, rv.q, hi, r, &si, &sj);
                             w[8 * i + cnt] = (float)((cs.w[mp] * rows[r].w[m]) * rows[j].w[m3]);
-                            o[8 * i + cnt] = sj * (int)pln + si * nz;
+                            o[8 * i + cnt] = sj * (int)pln + si * kp;
                             ++cnt;
                         }
                     }
@@ -215,7 +219,7 @@ cudaError_t build_rot3(spect_plan_s& P, const double* angles, const float* mu_t,
                             const int c3 = c1 - rows[r].o - m3;  // pass-3 output column that read (c1, r)
                             const float wt = (float)((cs.w[mp] * rows[hj].w[m]) * rows[r].w[m3]);
                             if (c3 < 0 || c3 >= n || wt == 0.f) continue;
-                            e[cnt].p = r * ps + c3 * nz;  // the t plane r, column c3 (plane stride ps)
+                            e[cnt].p = r * ps + c3 * kp;  // the t plane r, column c3 (plane stride ps)
                             e[cnt].w = wt;
                             ++cnt;
                         }

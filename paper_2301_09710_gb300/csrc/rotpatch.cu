@@ -166,13 +166,12 @@ size_t rot_smem(int box_floats) { return 2 * (size_t)rot_stage_floats(box_floats
 
 // Plan time: per-(patch, view) boxes from the rotation tables and the two
 // tensor maps.  Leaves P.rotpatch = 0 when the geometry does not suit the
-// kernel (k rows not a whole number of 16-byte units, boxes too large, no
-// tensor-map encoder).
+// kernel (boxes too large, no tensor-map encoder).
 cudaError_t build_rotpatch(spect_plan_s& P, cudaStream_t st)
 {
     P.rotpatch = 0;
     const Geometry& g = P.g;
-    if (!P.fast || (g.nz % 4) != 0 || !encode_fn()) return cudaSuccess;
+    if (!P.fast || !encode_fn()) return cudaSuccess;
     // SPECT_ROTPATCH (testing): 0 = not built; 1 = built and used from the start;
     // unset = built, used once the autotuner finds it faster
     const char* env = getenv("SPECT_ROTPATCH");
@@ -198,13 +197,13 @@ cudaError_t build_rotpatch(spect_plan_s& P, cudaStream_t st)
     CUtensorMap mx, mm;
     bool ok = e == cudaSuccess && bw <= 256 && bh <= 256 && rot_smem(box_floats) <= (size_t)P.smem_optin;
     if (ok) {
-        // x_t: k (nz, contiguous) x i (nx) x j (ny)
-        const cuuint64_t dx[3] = {(cuuint64_t)g.nz, (cuuint64_t)g.nx, (cuuint64_t)g.ny};
-        const cuuint64_t sx[2] = {(cuuint64_t)g.nz * 4, (cuuint64_t)g.nx * g.nz * 4};
+        // x_t: k (kp, contiguous) x i (nx) x j (ny)
+        const cuuint64_t dx[3] = {(cuuint64_t)g.kp, (cuuint64_t)g.nx, (cuuint64_t)g.ny};
+        const cuuint64_t sx[2] = {(cuuint64_t)g.kp * 4, (cuuint64_t)g.nx * g.kp * 4};
         const cuuint32_t bx[3] = {(cuuint32_t)kRK, (cuuint32_t)bw, (cuuint32_t)bh};
-        // attenuation cache: k (nz) x i (nx) x (view, row) plane (nview * ny, stride ps)
-        const cuuint64_t dm[3] = {(cuuint64_t)g.nz, (cuuint64_t)g.nx, (cuuint64_t)g.nview * g.ny};
-        const cuuint64_t sm_[2] = {(cuuint64_t)g.nz * 4, (cuuint64_t)P.ps * 4};
+        // attenuation cache: k (kp) x i (nx) x (view, row) plane (nview * ny, stride ps)
+        const cuuint64_t dm[3] = {(cuuint64_t)g.kp, (cuuint64_t)g.nx, (cuuint64_t)g.nview * g.ny};
+        const cuuint64_t sm_[2] = {(cuuint64_t)g.kp * 4, (cuuint64_t)P.ps * 4};
         const cuuint32_t bm[3] = {(cuuint32_t)kRK, (cuuint32_t)kRP, (cuuint32_t)kRP};
         const cuuint32_t es[3] = {1, 1, 1};
         ok = encode_fn()(&mx, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, P.xt, dx, sx, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE,

@@ -41,6 +41,7 @@ struct Geometry {
     float cfrac;      // (nx-1)/2 - cint  (0 or 0.5)
     float dy;
     int has_mu;
+    int kp;           // k pitch of the internal [j][i][k] volumes and [i][k] planes: nz rounded up to 4
 };
 
 // One adjacency entry of the transposed rotation: source pixel p (i + nx*j
@@ -91,11 +92,13 @@ struct spect_plan_s {
     int adj_J = 8;               // depth planes per fused adjoint block
     int adj_chunk = 0;           // views per adjoint pass (t slab sized to stay in L2)
     int adj_chunk_req = 0;       // views per adjoint pass asked for (SPECT_ADJ_CHUNK), 0: all
-    float* mubar = nullptr;      // nview * ny*nx*nz, [l][j][i][k]
-    float* xt = nullptr;         // nx*ny*nz, [j][i][k] image
-    float* et = nullptr;         // nx*ny*nz, [j][i][k] back-projection accumulator
-    float* st = nullptr;         // nx*ny*nz, [j][i][k] sensitivity
-    float* ut = nullptr;         // nx*ny*nz, [j][i][k] regulariser target of the regularised EM
+    // internal volumes: k pitch kp (a multiple of 4, so columns are 16-byte aligned);
+    // entries k >= nz are padding that no result reads
+    float* mubar = nullptr;      // nview * ny*nx*kp, [l][j][i][k]
+    float* xt = nullptr;         // nx*ny*kp, [j][i][k] image
+    float* et = nullptr;         // nx*ny*kp, [j][i][k] back-projection accumulator
+    float* st = nullptr;         // nx*ny*kp, [j][i][k] sensitivity
+    float* ut = nullptr;         // nx*ny*kp, [j][i][k] regulariser target of the regularised EM
     float* part = nullptr;       // G * nx*nz*nview forward partial sums
     spect::AdjEntry* adjf = nullptr;  // nview*nx*ny*adj_max fixed-length lists
     // patch-staged adjoint gather (gather.cu); gather == 0: the list gather k_adj_rot_t
@@ -121,7 +124,7 @@ struct spect_plan_s {
     int4* rboxes = nullptr;      // [patch][l] source box of x_t (i0, j0, width, height)
     int rbw = 0, rbh = 0;
     CUtensorMap rmap_x, rmap_mu; // x_t (k, i, j) and the attenuation cache (k, i, plane)
-    int ps = 0;                  // plane stride of the attenuation cache and slab: nx*nz rounded up to 4
+    int ps = 0;                  // plane stride of the attenuation cache and slab: nx*kp
     int ts = 0;                  // rotation table block per (view, row): 5*nx rounded up to 4
     float* rtab = nullptr;       // nview*ny*ts rotation tables of the fused forward
     int* err = nullptr;          // device error word (SPECT_ETIMEOUT when a bounded wait ran out)
@@ -431,12 +434,14 @@ cudaError_t build_fwd_map(spect_plan_s& P);
 size_t fwd_records_floats(const spect_plan_s& P);
 cudaError_t launch_fwd_records(const spect_plan_s& P, cudaStream_t st);
 int fwd_tiles(const spect_plan_s& P);
+int adj_tiles(const spect_plan_s& P);
 void default_fwd_shape(spect_plan_s& P, int sms);
 // Bucket of the fused full-PSF kernels (untiled planes), 0 when they do not fit.
 int fused_dir_bucket(const Geometry& g, size_t smem_limit);
 bool fused_dir_fit(const Geometry& g, int bucket, int J, int adj_J, size_t smem_limit);
 int fused_tiles_fit(const Geometry& g, int bucket, int J, int adj_J, int tiles, size_t smem_limit);
-cudaError_t launch_transpose(const float* in, float* out, int R, int C, cudaStream_t st);
+// out[c][r] = in[r][c], R x C; row pitches of in and out (at least C and R)
+cudaError_t launch_transpose(const float* in, float* out, int R, int C, int ip, int op, cudaStream_t st);
 cudaError_t launch_mubar_cache(const spect_plan_s& P, const float* mu_t, cudaStream_t st);
 cudaError_t launch_build_adjacency_fixed(const spect_plan_s& P, cudaStream_t st);
 cudaError_t launch_rot_tables(const spect_plan_s& P, cudaStream_t st);
