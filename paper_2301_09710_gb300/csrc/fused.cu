@@ -11,14 +11,12 @@
 //    view, [l][j][i][k] (nview * nx*ny*nz floats; HBM is plentiful), so the hot
 //    kernels multiply by a streamed, coalesced value instead of re-rotating mu.
 //  * Forward: a rotation kernel rotates and attenuates every (view, depth)
-//    plane into the work slab, already laid out as the blur kernel's shared-
-//    memory image (replicate halo columns, conflict-free pitch).  The blur
-//    kernel (one block per view and group of J depth planes) streams those
-//    images in by TMA, runs the separable PSF blur as two register-blocked
-//    sliding-window passes (i, then k; replicate padding along k folded into
-//    edge taps), and accumulates the group's depth sum in shared memory; the
-//    groups' partials are added in a fixed order by a small reduce kernel
-//    (deterministic, no atomics).
+//    plane into a plane image [i][k] of the work slab.  The blur kernel (one block
+//    per view, group of J depth planes and 32-column tile) streams the tiles in
+//    as tensor boxes, runs the separable PSF blur as two register-blocked
+//    sliding-window passes (i, then k; replicate padding folded into edge
+//    taps), and keeps the group's depth sum in registers; the groups' partials
+//    are added in a fixed order by a small reduce kernel (deterministic, no atomics).
 //  * Transpose: one block per (view, depth group) expands the detector plane
 //    into blurred-adjoint planes times mubar (the t slab, [v][j][i][k]); a
 //    gather kernel then sums sum_l sum_p W_l(p;q) t_l(p,k) per destination voxel
@@ -205,109 +203,16 @@ cudaError_t launch_build_adjacency_fixed(const spect_plan_s& P, cudaStream_t st)
     return cudaGetLastError();
 }
 
-template <int P, bool MUS>
-__global__ void __launch_bounds__(kRotThreads, 2) k_rot_fwd(Geometry g, FusedDims d, const float* __restrict__ rtab,
-                                                         const float* __restrict__ xt,
-                                                         const float* __restrict__ mubar, float* __restrict__ wsl,
-                                                         int l0, int* err)
+// Rotation + attenuation of every (view, plane) into the plane images: bilinear
+// (TAPS = 4) or the three-pass rotation's eight-tap products (rot3.cu, TAPS = 8).
+template <int TAPS>
+__global__ void __launch_bounds__(kRotThreads, TAPS == 4 ? 5 : 3) k_rot_fwd(Geometry g, RotDims d,
+                                                                            const float* __restrict__ tabs,
+                                                                            const float* __restrict__ xt,
+                                                                            const float* __restrict__ mubar,
+                                                                            float* __restrict__ wsl, int l0)
 {
-    rot_fwd_body<P, MUS>(g, d, rtab, xt, mubar, wsl, l0, err, blockIdx.x, blockIdx.y);
-}
-
-// ----------------------------------------------------------------------------
-// Forward rotation with the three-pass rotation (rot3.cu): the same block, plane
-// image, attenuation and output as k_rot_fwd, but every output (i, k) of plane
-// j is the eight-tap sum  sum_m w_m x_t[off_m + k]  of its table row (the three
-// passes' products; unused taps have weight 0, offset 0).  The (view, row)
-// table -- nx x 8 weights, then nx x 8 offsets -- is staged in shared memory
-// once; warps take one row i per step with lanes over k (24 gathers in
-// flight per lane, as k_rot_fwd's row pairs).
-// ----------------------------------------------------------------------------
-template <int P, bool MUS>
-__global__ void __launch_bounds__(kRotThreads, 2) k_rot_fwd8(Geometry g, FusedDims d, const float* __restrict__ tab8,
-                                                          const float* __restrict__ xt,
-                                                          const float* __restrict__ mubar, float* __restrict__ wsl,
-                                                          int l0, int* err)
-{
-    constexpr int C = Sep<P>::C;
-    extern __shared__ __align__(16) float sm[];
-    const int nx = g.nx, ny = g.ny, nz = g.nz;
-    const int ts8 = 16 * nx;
-    float* S = sm;
-    float* TBL = sm + d.farea;  // nx x 8 weights, then nx x 8 int offsets
-    float* MU = TBL + ts8;      // [i][k] attenuation plane (MUS)
-    uint64_t* bar = reinterpret_cast<uint64_t*>(MU + d.ps);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int NW = kRotThreads / 32;
-    const int j = blockIdx.x, v = blockIdx.y, l = l0 + v;
-    const int wp = d.wpf;
-    const int wcols = d.nib * Sep<P>::CX + 2 * C;
-    const float* tab = tab8 + ((size_t)l * ny + j) * ts8;
-    const float* mb = mubar + ((size_t)l * ny + j) * d.ps;
-    if (MUS && threadIdx.x == 0) {
-        mbar_init(bar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        tma_load_1d(MU, mb, (unsigned)d.ps * 4u, bar);
-    }
-    for (int e = threadIdx.x; e < ts8 / 4; e += kRotThreads)
-        reinterpret_cast<float4*>(TBL)[e] = __ldg(reinterpret_cast<const float4*>(tab) + e);
-    __syncthreads();  // table staged; the barrier is initialised before anyone waits on it
-    const int* OFF = reinterpret_cast<const int*>(TBL + 8 * nx);
-    bool ok = true, waited = !MUS;
-
-    for (int i = warp; i < nx; i += NW) {
-        const float4 wl = reinterpret_cast<const float4*>(TBL)[2 * i];
-        const float4 wh = reinterpret_cast<const float4*>(TBL)[2 * i + 1];
-        const int4 ol = reinterpret_cast<const int4*>(OFF)[2 * i];
-        const int4 oh = reinterpret_cast<const int4*>(OFF)[2 * i + 1];
-        const float w[8] = {wl.x, wl.y, wl.z, wl.w, wh.x, wh.y, wh.z, wh.w};
-        const int o[8] = {ol.x, ol.y, ol.z, ol.w, oh.x, oh.y, oh.z, oh.w};
-        for (int k0 = 0; k0 < nz; k0 += 96) {
-            float xs[3][8], ma[3];
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const int k = k0 + 32 * q + lane;
-                if (k < nz) {
-#pragma unroll
-                    for (int m = 0; m < 8; ++m) xs[q][m] = __ldg(xt + o[m] + k);
-                    if (!MUS) ma[q] = __ldg(mb + i * g.kp + k);
-                }
-            }
-            if (!waited) {
-                ok = mbar_wait_bounded(bar, 0u);
-                waited = true;
-            }
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const int k = k0 + 32 * q + lane;
-                if (k < nz) {
-                    if (MUS) ma[q] = MU[i * g.kp + k];
-                    float* wr = S + k * wp + C;
-                    float va = w[0] * xs[q][0];
-#pragma unroll
-                    for (int m = 1; m < 8; ++m) va = fmaf(w[m], xs[q][m], va);
-                    va *= ma[q];
-                    wr[i] = va;
-                    if (i == 0)  // replicate padding along i: left halo columns
-                        for (int h = -C; h < 0; ++h) wr[h] = va;
-                    if (i == nx - 1)  // right halo columns
-                        for (int h = nx; h < wcols - C; ++h) wr[h] = va;
-                }
-            }
-        }
-    }
-    if (__syncthreads_or(!ok)) {  // the attenuation plane never arrived
-        if (threadIdx.x == 0) {
-            flag_timeout(err);
-            mbar_wait_bounded(bar, 0u);  // a last chance for the copy in flight to land
-        }
-        return;
-    }
-    if (threadIdx.x == 0) {
-        fence_proxy_async_smem();
-        tma_store_1d(wsl + ((size_t)v * ny + j) * d.farea, S, (unsigned)d.farea * 4u);
-        tma_store_wait_read<0>();  // the block may leave once its shared memory is read
-    }
+    rot_body<TAPS>(g, d, tabs, xt, mubar, wsl, l0, blockIdx.x, blockIdx.y);
 }
 
 // ----------------------------------------------------------------------------
@@ -346,6 +251,16 @@ __global__ void k_fwd_records(Geometry g, int P, int PT, int nkb, const float* _
         r[2 * PT + k] = (float)lo;
         r[2 * PT + 16 * nkb + k] = (float)hi;
     }
+    const float* h = fx + (size_t)row * g.px;
+    float* xf = r + 2 * PT + 32 * nkb;
+    for (int e = threadIdx.x; e < kFoldLo + kFoldHi; e += blockDim.x) {
+        const int i = e < kFoldLo ? e : fold_hi0(g.nx, C) + e - kFoldLo;
+        double s = 0.0;
+        if (i < g.nx)
+            for (int a = 0; a < g.px; ++a)
+                if (e < kFoldLo ? a + ox > i + C : a + ox < i + C - g.nx + 1) s += h[a];
+        xf[e] = (float)s;
+    }
 }
 
 // v(i,k,l) = sum over depth groups of the partials (fixed order), optionally
@@ -382,10 +297,12 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_adj_sep_fused(Geometry g, 
 // (taps p(:, b)) applied to row k - b + cz: every term of a row runs through
 // the register-blocked FIR of the separable kernels, and the rows add up per
 // output (a row partial per b, then the sum over b: short FP32 chains).
-//   forward: the rotated planes come from k_rot_fwd (same images as the
-//     separable path: W[k][C + i] with replicate halo columns); ZH replicate
-//     halo rows above and below are filled in shared memory after each TMA
-//     load; outputs accumulate over the group's planes in ACC[i][k].
+//   forward: with the roles of the axes exchanged -- FIRs along k (taps p(a, :)) of
+//     column i - a + cx, so lanes run over i and the windows are float4s along the
+//     images' k.  Column tiles as in the separable path, W[C + i][ZH + k]; replicate
+//     padding along i is a clamped column index, along k the blocks at the plane's
+//     ends copy its first / last row into their halo; a thread owns 16 k of one
+//     column and keeps their depth sums in registers.
 //   adjoint: the detector plane is staged once per block, zero-padded
 //     (Vx[ZH + k][C + i]); per plane the taps of the k edge class of each
 //     output row are used for the whole run, and the first / last detector
@@ -393,11 +310,19 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_adj_sep_fused(Geometry g, 
 // ============================================================================
 __host__ __device__ inline int dir_rows(int nz, int ZH) { return nz + 2 * ZH; }
 
-__host__ __device__ inline size_t dir_fwd_smem_floats(const FusedDims& d, int nz, int P, int PT, int ZH)
+// Launch shape of the forward full-PSF blur.
+struct DirDims {
+    int TI, nT;   // columns per tile, tiles per plane
+    int KR, nkr;  // k per block (a multiple of 16), k ranges per plane
+    int wr, wp;   // box: wr = TI + 2C columns of wp = pitch4odd(KR + 2ZH) <= 252 k
+    int warea;    // floats of a tile buffer (rounded up to 128 bytes)
+    int nbuf;     // tile buffers, each followed by the taps of its plane
+    int J, G, T;  // planes per block, depth groups, threads (one per work item)
+};
+
+__host__ __device__ inline size_t dir_fwd_smem_floats(const DirDims& d, int P, int PT)
 {
-    const size_t xarea = ((size_t)dir_rows(nz, ZH) * d.wp + 3) & ~(size_t)3;
-    // Wext x2 | taps P x PT | ACC | 2 mbarriers
-    return 2 * xarea + (size_t)P * PT + (size_t)d.urows * d.apc + 8;
+    return (size_t)d.nbuf * (d.warea + (((size_t)P * PT + 31) & ~(size_t)31)) + 8;  // + 2 mbarriers
 }
 
 __host__ __device__ inline size_t dir_adj_smem_floats(const FusedDims& d, int nz, int P, int PT, int ZH, int ncls,
@@ -408,104 +333,120 @@ __host__ __device__ inline size_t dir_adj_smem_floats(const FusedDims& d, int nz
     return xarea + (size_t)nmb * d.marea + (size_t)ncls * P * PT + 8;
 }
 
+// Plan time: the taps of every PSF plane as rows along k, [a][b], zero-padded to
+// P x PT and centred.
+__global__ void k_dir_records(Geometry g, int P, int PT, const float* __restrict__ psf, float* __restrict__ rec)
+{
+    const size_t row = blockIdx.x;
+    const int ox = (P - g.px) / 2, oz = (P - g.pz) / 2;
+    for (int e = threadIdx.x; e < P * PT; e += blockDim.x) {
+        const int a = e / PT - ox, b = e % PT - oz;
+        rec[row * P * PT + e] =
+            (a >= 0 && a < g.px && b >= 0 && b < g.pz) ? psf[row * g.px * g.pz + (size_t)b * g.px + a] : 0.f;
+    }
+}
+
+// One block per (column tile, k range, depth group of J planes, view).
 template <int P>
-__global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_dir_fused(Geometry g, FusedDims d,
-                                                                     const float* __restrict__ wsl,
-                                                                     const float* __restrict__ psf,
+__global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_dir_fused(const __grid_constant__ CUtensorMap tmap,
+                                                                     Geometry g, DirDims d,
+                                                                     const float* __restrict__ rec,
                                                                      float* __restrict__ part, int l0, int* err)
 {
     using S = Sep<P>;
-    constexpr int C = S::C, CX = S::CX, ZH = S::ZH, PT = S::PT;
-    extern __shared__ __align__(16) float sm[];
+    constexpr int C = S::C, CZ = S::CZ, ZH = S::ZH, WZ = S::WZ, PT = S::PT;
+    constexpr int TAPS = (P * PT + 31) & ~31;
+    extern __shared__ __align__(128) float smf[];
     const int nx = g.nx, ny = g.ny, nz = g.nz;
-    const int xarea = (dir_rows(nz, ZH) * d.wp + 3) & ~3;
-    float* WB = sm;                                 // [2][xarea]: rows -ZH .. nz+ZH-1 of a plane image
-    float* TAP = WB + 2 * (size_t)xarea;            // [P][PT], this plane's taps (zero-padded, centred)
-    float* ACC = TAP + (size_t)P * PT;              // [i][k], apc pitch
-    uint64_t* bar = reinterpret_cast<uint64_t*>(ACC + (size_t)d.urows * d.apc);
-    const int tid = threadIdx.x;
-    constexpr int T = kFusedThreads;
-    const int grp = blockIdx.x, v = blockIdx.y, l = l0 + v;
+    const int tid = threadIdx.x, T = blockDim.x;
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smf + (size_t)d.nbuf * (d.warea + TAPS));
+    int bx = blockIdx.x;
+    const int tile = bx % d.nT;
+    bx /= d.nT;
+    const int k_lo = (bx % d.nkr) * d.KR, grp = bx / d.nkr;
+    const int v = blockIdx.y, l = l0 + v;
+    const int i0 = tile * d.TI, ti = min(d.TI, nx - i0), nkb = (min(d.KR, nz - k_lo) + CZ - 1) / CZ;
     const int lp = g.nvp == 1 ? 0 : l;
-    const int j_begin = grp * d.J, j_end = min(ny, j_begin + d.J);
-    const int ox = (P - g.px) / 2, oz = (P - g.pz) / 2;
+    const int j_begin = grp * d.J, nj = min(ny - j_begin, d.J);
+    const int ox = (P - g.px) / 2;  // tap columns outside [ox, ox + px) are zero
     const int pln = nx * nz;
-    const float* wv = wsl + (size_t)v * ny * d.farea;
 
-    for (int e = tid; e < d.urows * d.apc; e += T) ACC[e] = 0.f;
+    // tensor copies want 128-byte aligned shared memory: refuse (error word) rather than fault
+    if ((smem_u32(smf) & 127u) != 0) {
+        if (tid == 0 && err) atomicExch(err, (int)SPECT_ECUDA);
+        return;
+    }
+    auto request = [&](int n) {  // plane j_begin + n and its taps into their buffer
+        const int b = d.nbuf == 1 ? 0 : n & 1;
+        float* dst = smf + (size_t)b * (d.warea + TAPS);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar + b)),
+                     "r"((unsigned)(d.wr * d.wp + P * PT) * 4u)
+                     : "memory");
+        tma_load_3d(dst, &tmap, k_lo - ZH, i0 - C, v * ny + j_begin + n, bar + b);
+        tma_copy_1d(dst + d.warea, rec + ((size_t)lp * ny + j_begin + n) * (P * PT), (unsigned)(P * PT) * 4u, bar + b);
+    };
     if (tid == 0) {
         mbar_init(bar, 1);
         mbar_init(bar + 1, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        tma_load_1d(WB + ZH * d.wp, wv + (size_t)j_begin * d.farea, (unsigned)d.warea * 4u, bar);
-        if (j_begin + 1 < j_end)
-            tma_load_1d(WB + xarea + ZH * d.wp, wv + (size_t)(j_begin + 1) * d.farea, (unsigned)d.warea * 4u,
-                        bar + 1);
+        for (int n = 0; n < d.nbuf && n < nj; ++n) request(n);
     }
     __syncthreads();
 
-    unsigned phases = 0u;
-    for (int j = j_begin; j < j_end; ++j) {
-        const int b = (j - j_begin) & 1;
-        float* W = WB + b * (size_t)xarea;
-        const bool ok = mbar_wait_bounded(bar + b, (phases >> b) & 1u);
-        phases ^= 1u << b;
-        // this plane's taps, and the replicate halo rows (copies of rows 0 and nz-1)
-        const float* pp = psf + ((size_t)lp * ny + j) * g.px * g.pz;
-        for (int e = tid; e < P * PT; e += T) {
-            const int bb = e / PT, a = e - bb * PT, ax = a - ox, bz = bb - oz;
-            TAP[e] = (ax >= 0 && ax < g.px && bz >= 0 && bz < g.pz) ? __ldg(pp + (size_t)bz * g.px + ax) : 0.f;
-        }
-        if (ok)
-            for (int e = tid; e < 2 * C * d.wp; e += T) {
-                const int r = e / d.wp, c = e - r * d.wp;
-                if (r < C) W[(ZH - C + r) * d.wp + c] = W[ZH * d.wp + c];
-                else W[(ZH + nz + r - C) * d.wp + c] = W[(ZH + nz - 1) * d.wp + c];
-            }
+    const int kb = tid / ti, i = tid - kb * ti;  // the thread's item: 16 k of column i0 + i
+    const bool mine = kb < nkb;
+    const int kz = nz - 1 - k_lo + ZH;           // position of row nz - 1 in a column of W
+    float acc[CZ];
+#pragma unroll
+    for (int c = 0; c < CZ; ++c) acc[c] = 0.f;
+    for (int n = 0; n < nj; ++n) {
+        const int b = d.nbuf == 1 ? 0 : n & 1;
+        float* W = smf + (size_t)b * (d.warea + TAPS);
+        const float* TAP = W + d.warea;
+        const bool ok = mbar_wait_bounded(bar + b, (unsigned)(d.nbuf == 1 ? n : n >> 1) & 1u);
+        if (ok && k_lo < C)  // rows -C .. -1 that this block holds
+            for (int r = tid; r < d.wr; r += T)
+                for (int c = max(0, ZH - k_lo - C); c < ZH - k_lo; ++c) W[r * d.wp + c] = W[r * d.wp + ZH - k_lo];
+        if (ok && kz < ZH + d.KR + C)  // rows nz .. nz + C - 1
+            for (int r = tid; r < d.wr; r += T)
+                for (int c = kz + 1; c <= min(kz + C, d.wp - 1); ++c) W[r * d.wp + c] = W[r * d.wp + kz];
         if (__syncthreads_or(!ok)) {
-            if (tid == 0) {
+            if (tid == 0) {  // a last chance for the copies in flight to land
                 flag_timeout(err);
-                mbar_wait_bounded(bar + b, ((phases >> b) & 1u) ^ 1u);
-                mbar_wait_bounded(bar + (b ^ 1), (phases >> (b ^ 1)) & 1u);
+                for (int m = n; m < n + d.nbuf && m < nj; ++m)
+                    mbar_wait_bounded(bar + (d.nbuf == 1 ? 0 : m & 1), (unsigned)(d.nbuf == 1 ? m : m >> 1) & 1u);
             }
             return;
         }
-        // c_j(i, k) = sum_b FIR_i(taps p(:, b), row k - b + cz); lanes over k
-        for (int it = tid; it < nz * d.nib; it += T) {
-            const int ib = it / nz, k = it - ib * nz;
-            const int li = ib * CX;
-            float o[CX];
+        // c_j(i, k) = sum_a FIR_k(taps p(a, :), column clamp(i - a + cx)); lanes over i
+        if (mine) {
+            float o[CZ];
 #pragma unroll
-            for (int c = 0; c < CX; ++c) o[c] = 0.f;
-            for (int bb = 0; bb < P; ++bb) {
-                const float* wr = W + (ZH + k - bb + C) * d.wp + li;
-                float win[4 * ((CX + P - 1 + 3) / 4)];
-                load_row_f4(wr, win);
-                float ob[CX];
-                fir<P, CX, -1, P - 1>(TAP + bb * PT, win, ob);
+            for (int c = 0; c < CZ; ++c) o[c] = 0.f;
+            for (int a = ox; a < ox + g.px; ++a) {
+                const int col = clampi(i0 + i - a + C, 0, nx - 1) - i0 + C;
+                float win[WZ];
+                load_window_f4<P>(W + col * d.wp + kb * CZ, win);
+                float ob[CZ];
+                fir<P, CZ, -1, C + ZH>(TAP + a * PT, win, ob);
 #pragma unroll
-                for (int c = 0; c < CX; ++c) o[c] += ob[c];
+                for (int c = 0; c < CZ; ++c) o[c] += ob[c];
             }
-            float* ac = ACC + li * d.apc + k;
-            if (li + CX <= nx) {
 #pragma unroll
-                for (int c = 0; c < CX; ++c) ac[c * d.apc] += o[c];
-            } else {
-#pragma unroll
-                for (int c = 0; c < CX; ++c)
-                    if (li + c < nx) ac[c * d.apc] += o[c];
-            }
+            for (int c = 0; c < CZ; ++c) acc[c] += o[c];
         }
-        __syncthreads();  // buffer b and the taps are free
-        if (tid == 0 && j + 2 < j_end) {
+        __syncthreads();  // buffer b and its taps are free
+        if (tid == 0 && n + d.nbuf < nj) {
             fence_proxy_async_smem();
-            tma_load_1d(W + ZH * d.wp, wv + (size_t)(j + 2) * d.farea, (unsigned)d.warea * 4u, bar + b);
+            request(n + d.nbuf);
         }
     }
-    float* pout = part + ((size_t)grp * g.nview + l) * pln;
-    for (int e = tid; e < pln; e += T) {
-        const int k = e / nx, i = e - k * nx;
-        pout[e] = ACC[i * d.apc + k];
+    if (mine) {
+        const int k0 = k_lo + kb * CZ;
+        float* pout = part + ((size_t)grp * g.nview + l) * pln + i0 + i;
+#pragma unroll
+        for (int c = 0; c < CZ; ++c)
+            if (k0 + c < nz) pout[(size_t)(k0 + c) * nx] = acc[c];
     }
 }
 
@@ -744,7 +685,7 @@ int tiles_that_fit(const Geometry& g, size_t limit, int min_tiles)
         const FusedDims d = dims_for<P>(g, 8, t);
         if (d.nT == last_nt) continue;  // same tile width as a smaller request
         last_nt = d.nT;
-        if (smem_fwd_bound<P>(g, d) <= limit && smem_adj_bound<P>(g, d) <= limit && rot_smem_min(d) <= limit &&
+        if (smem_fwd_bound<P>(g, d) <= limit && smem_adj_bound<P>(g, d) <= limit && rot_smem_bound(d) <= limit &&
             (size_t)d.marea * 4 < (1u << 20))
             return d.nT;
     }
@@ -765,24 +706,6 @@ cudaError_t fwd_launch(const spect_plan_s& Pl, const float* /*xt: the blur reads
 }
 
 template <int P>
-cudaError_t rot_launch(const spect_plan_s& Pl, const float* xt, int l0, int nv, cudaStream_t st)
-{
-    const FusedDims d = dims_for<P>(Pl.g, Pl.fused_J, 1);
-    // the three-pass rotation: eight taps per output from its own table
-    const size_t smin = Pl.rot3 ? ((size_t)d.farea + (size_t)rot3_ts8(Pl.g.nx)) * sizeof(float) : rot_smem_min(d);
-    const size_t smem_mu = smin + (size_t)d.ps * sizeof(float) + 16;
-    const bool mus = smem_mu <= (size_t)Pl.smem_optin;
-    const size_t smem = mus ? smem_mu : smin;
-    auto kern = Pl.rot3 ? (mus ? k_rot_fwd8<P, true> : k_rot_fwd8<P, false>)
-                        : (mus ? k_rot_fwd<P, true> : k_rot_fwd<P, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<dim3(Pl.g.ny, nv), kRotThreads, smem, st>>>(Pl.g, d, Pl.rot3 ? Pl.r3_tab : Pl.rtab, xt, mubar_for(Pl, l0),
-                                                       Pl.slab, l0, Pl.err);
-    return cudaGetLastError();
-}
-
-template <int P>
 cudaError_t adj_launch(const spect_plan_s& Pl, const float* v, int l0, int nv, cudaStream_t st)
 {
     const FusedDims d = dims_for<P>(Pl.g, Pl.adj_J, Pl.adj_nT);
@@ -797,10 +720,40 @@ cudaError_t adj_launch(const spect_plan_s& Pl, const float* v, int l0, int nv, c
 }  // namespace
 
 namespace {
+// The bound of the full-PSF geometries taken: two whole planes with halo rows,
+// accumulators and taps (the forward kernel's tiles need less).
 template <int P>
-size_t dir_smem_fwd(const Geometry& g, const FusedDims& d)
+size_t dir_smem_fwd_bound(const Geometry& g, const FusedDims& d)
 {
-    return dir_fwd_smem_floats(d, g.nz, P, Sep<P>::PT, Sep<P>::ZH) * sizeof(float);
+    const size_t xarea = ((size_t)dir_rows(g.nz, Sep<P>::ZH) * d.wp + 3) & ~(size_t)3;
+    return (2 * xarea + (size_t)P * Sep<P>::PT + (size_t)d.urows * d.apc + 8) * sizeof(float);
+}
+
+// Forward launch shape: 32-column tiles, at most 192 k per block (the tensor map's
+// 256 with the halos), a thread per work item, as the separable blur.  Two buffers
+// unless one lets more blocks run on an SM.
+template <int P>
+DirDims dir_fwd_dims(const Geometry& g, int J, size_t smem_limit)
+{
+    using S = Sep<P>;
+    DirDims d;
+    d.TI = g.nx > 16 ? 32 : 16;
+    d.nT = (g.nx + d.TI - 1) / d.TI;
+    d.nkr = (g.nz + 191) / 192;
+    d.KR = ((g.nz + d.nkr - 1) / d.nkr + 15) & ~15;
+    d.nkr = (g.nz + d.KR - 1) / d.KR;
+    d.wr = d.TI + 2 * S::C;
+    d.wp = pitch4odd(d.KR + 2 * S::ZH);
+    d.warea = (d.wr * d.wp + 31) & ~31;
+    d.J = J;
+    d.G = (g.ny + J - 1) / J;
+    d.T = (std::min(d.TI, g.nx) * (d.KR / 16) + 31) & ~31;
+    d.nbuf = 2;
+    const size_t two = dir_fwd_smem_floats(d, P, S::PT) * sizeof(float);
+    d.nbuf = 1;
+    const size_t one = dir_fwd_smem_floats(d, P, S::PT) * sizeof(float);
+    if (two <= smem_limit && blocks_per_sm(one, d.T, 96) <= blocks_per_sm(two, d.T, 96)) d.nbuf = 2;
+    return d;
 }
 
 template <int P>
@@ -817,18 +770,18 @@ bool dir_fits(const Geometry& g, size_t limit, int J, int adj_J)
     // attenuation planes counted without their k padding: where that leaves no room for
     // two padded ones, the adjoint runs with one
     const size_t pad = 2 * ((size_t)da.marea - (((size_t)g.nx * g.nz + 3) & ~(size_t)3)) * sizeof(float);
-    return df.nT == 1 && dir_smem_fwd<P>(g, df) <= limit && dir_smem_adj<P>(g, da, cls_z, 2) - pad <= limit &&
-           dir_smem_adj<P>(g, da, cls_z, 1) <= limit && rot_smem_min(df) <= limit && (size_t)df.ps * 4 < (1u << 20);
+    return df.nT == 1 && dir_smem_fwd_bound<P>(g, df) <= limit && dir_smem_adj<P>(g, da, cls_z, 2) - pad <= limit &&
+           dir_smem_adj<P>(g, da, cls_z, 1) <= limit && rot_smem_bound(df) <= limit && (size_t)df.ps * 4 < (1u << 20);
 }
 
 template <int P>
 cudaError_t dir_fwd_launch(const spect_plan_s& Pl, int l0, int nv, cudaStream_t st)
 {
-    const FusedDims d = dims_for<P>(Pl.g, Pl.fused_J, 1);
-    const size_t smem = dir_smem_fwd<P>(Pl.g, d);
+    const DirDims d = dir_fwd_dims<P>(Pl.g, Pl.fused_J, (size_t)Pl.smem_optin);
+    const size_t smem = dir_fwd_smem_floats(d, P, Sep<P>::PT) * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(k_fwd_dir_fused<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_fwd_dir_fused<P><<<dim3(d.G, nv), kFusedThreads, smem, st>>>(Pl.g, d, Pl.slab, Pl.psf, Pl.part, l0, Pl.err);
+    k_fwd_dir_fused<P><<<dim3(d.nT * d.nkr * d.G, nv), d.T, smem, st>>>(Pl.fmap, Pl.g, d, Pl.frec, Pl.part, l0, Pl.err);
     return cudaGetLastError();
 }
 
@@ -900,7 +853,7 @@ int fused_tiles_fit(const Geometry& g, int bucket, int J, int adj_J, int tiles, 
         constexpr int B = decltype(tag)::value;
         const FusedDims df = dims_for<B>(g, J, tiles), da = dims_for<B>(g, adj_J, tiles);
         const bool ok = smem_fwd_bound<B>(g, df) <= smem_limit && smem_adj_bound<B>(g, da) <= smem_limit &&
-                        rot_smem_min(df) <= smem_limit && (size_t)df.marea * 4 < (1u << 20);
+                        rot_smem_bound(df) <= smem_limit && (size_t)df.marea * 4 < (1u << 20);
         return ok ? df.nT : 0;
     };
     switch (bucket) {
@@ -958,27 +911,32 @@ cudaError_t launch_fused_rotate(const spect_plan_s& P, const float* xt, int l0, 
 {
     // read from the plan's own x_t: the patch-staged rotation (rotpatch.cu)
     if (P.rotpatch && P.rotpatch_on && xt == P.xt) return launch_rot_patch(P, l0, nv, st);
-    SPECT_DISPATCH(rot_launch, P, xt, l0, nv, st)
+    const RotDims d = rot_dims(P.g, P.ps, P.rot3 ? rot3_ts8(P.g.nx) : P.ts, nv, P.sms);
+    const dim3 grid(d.nb * ((P.g.ny + d.JP - 1) / d.JP), nv);
+    if (P.rot3) k_rot_fwd<8><<<grid, kRotThreads, 0, st>>>(P.g, d, P.r3_tab, xt, mubar_for(P, l0), P.slab, l0);
+    else k_rot_fwd<4><<<grid, kRotThreads, 0, st>>>(P.g, d, P.rtab, xt, mubar_for(P, l0), P.slab, l0);
+    return cudaGetLastError();
 }
 
 namespace {
-template <int P>
-size_t plane_area(const spect_plan_s& Pl)
-{
-    return (size_t)dims_for<P>(Pl.g, Pl.fused_J, 1).farea;
-}
-
-// The plane images of the work slab as a tensor map -- column (wpf) x k (nz) x
-// plane (chunk * ny) -- with the forward blur's tile as its box.
+// The plane images of the work slab as a tensor map -- k (nz; zeros beyond) x column
+// (nx) x plane (chunk * ny) -- with the forward blur's tile as its box.
 template <int P>
 cudaError_t encode_fwd_map(spect_plan_s& Pl)
 {
     const Geometry& g = Pl.g;
-    const FusedDims im = dims_for<P>(g, Pl.fused_J, 1);
-    const FwdDims d = fwd_dims<P>(g, Pl.fused_J, Pl.fwd_nT, (size_t)Pl.smem_optin);
-    const cuuint64_t dims[3] = {(cuuint64_t)im.wpf, (cuuint64_t)g.nz, (cuuint64_t)Pl.chunk * g.ny};
-    const cuuint64_t strides[2] = {(cuuint64_t)im.wpf * 4, (cuuint64_t)im.farea * 4};
-    const cuuint32_t box[3] = {(cuuint32_t)d.wp, (cuuint32_t)d.br, 1};
+    cuuint32_t box[3] = {0, 0, 1};
+    if (Pl.separable) {
+        const FwdDims d = fwd_dims<P>(g, Pl.fused_J, Pl.fwd_nT, (size_t)Pl.smem_optin);
+        box[0] = kWK;
+        box[1] = (cuuint32_t)d.wr;
+    } else {
+        const DirDims d = dir_fwd_dims<P>(g, Pl.fused_J, (size_t)Pl.smem_optin);
+        box[0] = (cuuint32_t)d.wp;
+        box[1] = (cuuint32_t)d.wr;
+    }
+    const cuuint64_t dims[3] = {(cuuint64_t)g.nz, (cuuint64_t)g.nx, (cuuint64_t)Pl.chunk * g.ny};
+    const cuuint64_t strides[2] = {(cuuint64_t)g.kp * 4, (cuuint64_t)Pl.ps * 4};
     const cuuint32_t estr[3] = {1, 1, 1};
     if (!encode_fn() ||
         encode_fn()(&Pl.fmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, Pl.slab, dims, strides, box, estr,
@@ -993,41 +951,43 @@ cudaError_t encode_fwd_map(spect_plan_s& Pl)
 size_t fwd_records_floats(const spect_plan_s& P)
 {
     const int PT = (P.bucket + 3) & ~3, nkb = (P.g.nz + 15) / 16;
-    return (size_t)P.g.nvp * P.g.ny * fwd_rec_floats(PT, nkb);
+    return (size_t)P.g.nvp * P.g.ny * (P.separable ? fwd_rec_floats(PT, nkb) : P.bucket * PT);
 }
 
 cudaError_t launch_fwd_records(const spect_plan_s& P, cudaStream_t st)
 {
     const int PT = (P.bucket + 3) & ~3, nkb = (P.g.nz + 15) / 16;
-    k_fwd_records<<<P.g.nvp * P.g.ny, 128, 0, st>>>(P.g, P.bucket, PT, nkb, P.fx, P.fz, P.frec);
+    if (P.separable) k_fwd_records<<<P.g.nvp * P.g.ny, 128, 0, st>>>(P.g, P.bucket, PT, nkb, P.fx, P.fz, P.frec);
+    else k_dir_records<<<P.g.nvp * P.g.ny, 256, 0, st>>>(P.g, P.bucket, PT, P.psf, P.frec);
     return cudaGetLastError();
 }
 
 cudaError_t build_fwd_map(spect_plan_s& P)
 {
-    if (!P.separable) return cudaSuccess;
     SPECT_DISPATCH(encode_fwd_map, P)
 }
 
 // Default launch shape of the forward blur.  Tiles of 32 columns: a block is then
 // 2 nkb warps, and four to sixteen such blocks share an SM, so one block's
 // barriers, plane loads and set-up are covered by the others' FMAs (128x80, 128 views,
-// 37 taps: 458 us against 502 for whole planes, 470 for 64 columns; 160x96, 120
-// views, 29 taps: 659 against 812 for 80 columns; 192x128, 64 views, 37 taps: 815
-// against 939 for 64; 16 columns give the overlap of neighbouring boxes more to
-// read: 561 at 128x80).  J = 8 planes per block, fewer when that leaves the chip short
-// of blocks: at 64x32, 64 views J = 4 takes 18.6 us against 20.4, at 32x16, 32 views
-// J = 2 takes 8.0 against 12.2.
-void default_fwd_shape(spect_plan_s& P, int sms)
+// 37 taps: 485 us, 542 with 48 columns; 160x96, 120 views, 29 taps: 698 against 846
+// with 48; whole planes in one block of 640 threads took 513 and 880).  J = 8
+// planes per block, fewer when that leaves the chip short of blocks: at 64x32, 64
+// views J = 4 takes 19 us against 21, at 32x16, 32 views J = 2 takes 8.0 against 12.2.
+void default_fwd_shape(spect_plan_s& P)
 {
     const Geometry& g = P.g;
     P.fused_J = 8;
-    if (!P.separable) return;
+    if (!P.separable) {  // as below, with blocks of the full-PSF kernel
+        const long long blocks = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * g.nview;
+        if (blocks < 24ll * P.sms) P.fused_J = blocks >= 4ll * P.sms ? 4 : 2;
+        return;
+    }
     const int nib = (g.nx + 15) / 16;
     P.fwd_nT = std::max(P.fwd_nT, (nib + 1) / 2);
     P.fwd_nT = fwd_tiles(P);
     const auto blocks = [&](int J) { return (long long)((g.ny + J - 1) / J) * P.fwd_nT * g.nview; };
-    if (blocks(8) < 10ll * sms) P.fused_J = blocks(4) >= 4ll * sms ? 4 : 2;
+    if (blocks(8) < 10ll * P.sms) P.fused_J = blocks(4) >= 4ll * P.sms ? 4 : 2;
 }
 
 // Column tiles of the blur adjoint: the fewest, at least adj_nT, that fit with adj_J planes per block.
@@ -1064,20 +1024,10 @@ int fwd_tiles(const spect_plan_s& P)
     }
 }
 
-// floats per view of the work slab the fused path needs (rotated tile images or t planes)
+// floats per view of the work slab the fused path needs (rotated plane images or t planes)
 size_t fused_slab_per_view(const spect_plan_s& P)
 {
-    size_t parea = 0;
-    switch (P.bucket) {
-#define SPECT_AREA(B) \
-    case B: parea = plane_area<B>(P); break;
-        SPECT_AREA(3) SPECT_AREA(5) SPECT_AREA(7) SPECT_AREA(9) SPECT_AREA(11) SPECT_AREA(13) SPECT_AREA(15)
-        SPECT_AREA(17) SPECT_AREA(21) SPECT_AREA(25) SPECT_AREA(29) SPECT_AREA(33) SPECT_AREA(37)
-#undef SPECT_AREA
-        default: break;
-    }
-    const size_t ps = (size_t)P.g.nx * P.g.kp;
-    return (size_t)P.g.ny * (parea > ps ? parea : ps);
+    return (size_t)P.g.ny * P.g.nx * P.g.kp;
 }
 
 cudaError_t launch_fused_adjoint(const spect_plan_s& P, const float* v, int l0, int nv, cudaStream_t st)

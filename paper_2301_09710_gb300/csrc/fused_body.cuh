@@ -64,13 +64,15 @@ __device__ __forceinline__ void transpose_body(const float* __restrict__ in, flo
 // (view, depth) plane into the work slab, already in the blur kernel's
 // shared-memory image; k_fwd_sep_fused (one block per view and depth group)
 // streams those images in by TMA and blurs them.  Its shared memory:
-//   W   one or two tile buffers, nz rows x wp columns: W[k][C + i] with replicate
-//       halo columns; wp is a multiple of 4 with wp/4 odd, so the i-pass
-//       windows (lanes over k) load as bank-conflict-free float4s.
+//   W   one or two tile buffers, as runs of 32 k: W[k / 32][C + i][k % 32], zero
+//       outside the plane (the tensor copy's fill); the i-pass windows (lanes over
+//       k) are conflict-free loads at immediate offsets.
 //   U   nx rows x kpu: i-pass output, U[i][ZH + k], with zero halo columns;
 //       kpu/4 is odd so the k-pass float4 windows (lanes over i) are
-//       bank-conflict free.  Replicate padding along k enters as folded edge
-//       taps: output k adds U(0) sum_{b>k+C} fz(b) + U(nz-1) sum_{b<k+C-nz+1} fz(b).
+//       bank-conflict free.
+//   Replicate padding enters both passes as folded edge taps on top of the
+//   zero-padded FIR: output k adds U(0) sum_{b>k+C} fz(b) + U(nz-1) sum_{b<k+C-nz+1} fz(b),
+//   and likewise along i.
 //   taps and folded edge taps of every plane of the group, staged once.
 // The depth sums stay in registers.
 // Per plane there are two block barriers: after the i-pass (which also agrees
@@ -90,12 +92,12 @@ constexpr int kFusedThreads = 640;
 
 // Largest block of the forward blur and the resident blocks its registers are bounded
 // for.  Short FIRs (P <= 11) wait more on shared memory and barriers than on FMAs, so
-// they get 64 registers (two blocks of 512, or four of 256) instead of about 80.
+// they get at most 72 registers (two blocks of 448, seven of 128) instead of about 80.
 template <int P>
 struct FwdBlock {
-    static constexpr int T = P <= 11 ? 512 : kFusedThreads;
+    static constexpr int T = P <= 11 ? 448 : kFusedThreads;
     static constexpr int B = P <= 11 ? 2 : 1;
-    static constexpr int regs = P <= 11 ? 64 : 80;
+    static constexpr int regs = P <= 11 ? 72 : 80;
 };
 
 // Shared-memory plan of a fused kernel, computed identically on host and device.
@@ -109,10 +111,9 @@ struct FusedDims {
     int kpu;    // U row pitch (>= nkb*CZ + 2*ZH, multiple of 4, pitch/4 odd)
     int nib, nkb;
     int TI, nT; // tile width in columns (multiple of CX), tiles per plane
-    int wpf;    // row pitch of the untiled plane image (pitch4odd(nib*CX + 2*C))
     int wz;     // row pitch of the adjoint's Zb (multiple of 4, wz/4 odd: conflict-free float4 windows)
     int zarea;  // floats of Zb, nz x wz
-    int farea;  // floats of a plane image in the slab (and the rotation kernel's shared memory)
+    int farea;  // floats of a whole plane with halo columns (bound of the shapes taken, rot_smem_bound)
     int urows;  // rows of U / ACC / MB per tile: min(TI, nx)
     int vrows;  // detector rows a tile's k-adjoint needs: min(nx, TI + 2*C)
     int marea;  // floats of an attenuation tile, urows*kp
@@ -217,6 +218,20 @@ __device__ __forceinline__ float edge_tap_dot(const float* taps, const float* ro
     }
 }
 
+// o[c] += u * f[c] (f 16-byte aligned)
+template <int N>
+__device__ __forceinline__ void fold_taps(float u, const float* f, float (&o)[N])
+{
+#pragma unroll
+    for (int c4 = 0; c4 < N / 4; ++c4) {
+        const float4 t = reinterpret_cast<const float4*>(f)[c4];
+        o[4 * c4] = fmaf(u, t.x, o[4 * c4]);
+        o[4 * c4 + 1] = fmaf(u, t.y, o[4 * c4 + 1]);
+        o[4 * c4 + 2] = fmaf(u, t.z, o[4 * c4 + 2]);
+        o[4 * c4 + 3] = fmaf(u, t.w, o[4 * c4 + 3]);
+    }
+}
+
 // Record a timed-out bounded wait in the plan's error word.
 __device__ __forceinline__ void flag_timeout(int* err)
 {
@@ -224,145 +239,118 @@ __device__ __forceinline__ void flag_timeout(int* err)
 }
 
 // ----------------------------------------------------------------------------
-// Forward rotation: one block per (depth plane j, view).  Warps take pairs of
-// rows i with lanes over k, so the table entry and the four corner pointers
-// are warp-uniform and every gather is a coalesced run along k (96 k per
-// pass, 30 independent loads per lane in flight).  The plane is
-// assembled in shared memory as the blur kernel wants it -- W[k][C+i] with
-// replicate halo columns and pitch4odd pitch -- and leaves with one TMA bulk store;
-// the blur kernel brings its column tiles back as boxes of the image.
+// Forward rotation and attenuation into plane images [j][i][k], the layout of x_t, of
+// the attenuation factors and of the adjoint's t planes, so nothing is transposed:
+// a thread takes four consecutive k of a column i (16-byte corner loads, attenuation
+// read and store, coalesced over the lanes at any nz) through JP planes of a view;
+// neighbouring planes share source columns in L1, and the next plane's table entry is
+// loaded while this one is gathered.  No shared memory and no barriers.
+//   Bound by DRAM: 8 bytes per voxel-view, attenuation in and image out (128x128x80,
+// 128 views: 238 us, 5.6 TB/s; 160x160x96, 120 views: 418 us; 192x192x128, 128 views:
+// 863 us, all of 6.7 TB/s copy rate at most).  Assembling whole [k][i] planes in shared
+// memory took 392, 1274 and 3063 us (one block per SM from 160x96 on), 32-column tiles
+// transposed through shared memory 418, 642 and 1246 (a barrier per plane before
+// each round of gathers).
+//   TAPS = 4: bilinear, table block (l, j) = nx float4 weights, then nx base voxels;
+//   TAPS = 8: three-pass rotation, nx x 8 weights, then nx x 8 element offsets.
 // ----------------------------------------------------------------------------
+constexpr int kRotThreads = 256;
 
-constexpr int kRotThreads = 512;
+struct RotDims {
+    int ps, ts;  // plane stride of images and attenuation factors; table block of a (view, plane)
+    int nb, JP;  // blocks per plane; planes per block
+};
 
-// MUS: the plane's attenuation factors arrive by one TMA bulk load into shared
-// memory (issued first, waited for after the first gathers are in flight)
-// instead of as per-element global loads, when the two planes fit.
-template <int P, bool MUS>
-__device__ __forceinline__ void rot_fwd_body(const Geometry& g, const FusedDims& d, const float* __restrict__ rtab,
-                                             const float* __restrict__ xt, const float* __restrict__ mubar,
-                                             float* __restrict__ wsl, int l0, int* err, const int j, const int v)
+__device__ __forceinline__ float4 ld_stream4(const float* p)
 {
-    constexpr int C = Sep<P>::C;
-    extern __shared__ __align__(16) float sm[];
-    float* S = sm;
-    float* TBL = sm + d.farea;  // the (view, row) rotation table: nx float4 weights, then nx bases
-    float* MU = TBL + d.ts;     // [i][k] attenuation plane (MUS)
-    uint64_t* bar = reinterpret_cast<uint64_t*>(MU + d.ps);
-    const int nx = g.nx, ny = g.ny, nz = g.nz, kp = g.kp;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int NW = kRotThreads / 32;
-    const int l = l0 + v;
-    const int pln = nx * kp;
-    const int wp = d.wpf;
-    const int wcols = d.nib * Sep<P>::CX + 2 * C;
-    const float* tab = rtab + ((size_t)l * ny + j) * d.ts;
-    const float* mb = mubar + ((size_t)l * ny + j) * d.ps;
-    if (MUS && threadIdx.x == 0) {
-        mbar_init(bar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        tma_load_1d(MU, mb, (unsigned)d.ps * 4u, bar);
-    }
-    // the table is staged once, so no row step waits on a table load before its gathers
-    for (int e = threadIdx.x; e < d.ts / 4; e += kRotThreads)
-        reinterpret_cast<float4*>(TBL)[e] = __ldg(reinterpret_cast<const float4*>(tab) + e);
-    __syncthreads();  // table staged; the barrier is initialised before anyone waits on it
-    const float4* TW = reinterpret_cast<const float4*>(TBL);
-    const int* TB = reinterpret_cast<const int*>(TBL + 4 * nx);
-    bool ok = true, waited = !MUS;
+    float4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p));
+    return v;
+}
 
-    for (int i = 2 * warp; i < nx; i += 2 * NW) {
-        const bool two = i + 1 < nx;
-        const float4 wa = TW[i];
-        const float4 wb = two ? TW[i + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float* pa = xt + (size_t)TB[i] * kp;
-        const float* pb = xt + (size_t)TB[two ? i + 1 : i] * kp;
-        for (int k0 = 0; k0 < nz; k0 += 96) {
-            float xa[3][4], xb[3][4], ma[3], mc[3];
+template <int TAPS>
+__device__ __forceinline__ void rot_body(const Geometry& g, const RotDims& d, const float* __restrict__ tabs,
+                                         const float* __restrict__ xt, const float* __restrict__ mubar,
+                                         float* __restrict__ wsl, int l0, const int bx, const int v)
+{
+    const int nx = g.nx, kp = g.kp, k4 = kp >> 2;
+    const int jb = bx / d.nb, e = (bx - jb * d.nb) * kRotThreads + (int)threadIdx.x;
+    if (e >= nx * k4) return;
+    const int i = e / k4, l = l0 + v;
+    const int j0 = jb * d.JP, j_end = min(g.ny, j0 + d.JP);
+    const int pln = nx * kp;
+    const float* x = xt + 4 * (e - i * k4);
+    constexpr int NO = TAPS == 4 ? 1 : TAPS;  // bilinear: the base column, its neighbours follow from it
+    float w[TAPS], wn[TAPS] = {};
+    int o[NO], on[NO] = {};
+    auto table = [&](int j, float (&tw)[TAPS], int (&to)[NO]) {
+        const float* tab = tabs + ((size_t)l * g.ny + j) * d.ts;
+        if (TAPS == 4) {
+            const float4 t = __ldg(reinterpret_cast<const float4*>(tab) + i);
+            tw[0] = t.x, tw[1] = t.y, tw[2] = t.z, tw[3] = t.w;
+            to[0] = __ldg(reinterpret_cast<const int*>(tab + 4 * nx) + i) * kp;
+        } else {
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const int k = k0 + 32 * q + lane;
-                if (k < nz) {
-                    xa[q][0] = __ldg(pa + k);
-                    xa[q][1] = __ldg(pa + kp + k);
-                    xa[q][2] = __ldg(pa + pln + k);
-                    xa[q][3] = __ldg(pa + pln + kp + k);
-                    xb[q][0] = __ldg(pb + k);
-                    xb[q][1] = __ldg(pb + kp + k);
-                    xb[q][2] = __ldg(pb + pln + k);
-                    xb[q][3] = __ldg(pb + pln + kp + k);
-                    if (!MUS) {
-                        ma[q] = __ldg(mb + i * kp + k);
-                        mc[q] = two ? __ldg(mb + (i + 1) * kp + k) : 0.f;
-                    }
-                }
-            }
-            if (!waited) {
-                ok = mbar_wait_bounded(bar, 0u);
-                waited = true;
-            }
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const int k = k0 + 32 * q + lane;
-                if (k < nz) {
-                    if (MUS) {
-                        ma[q] = MU[i * kp + k];
-                        mc[q] = two ? MU[(i + 1) * kp + k] : 0.f;
-                    }
-                    float* wr = S + k * wp + C;
-                    float va = wa.x * xa[q][0];
-                    va = fmaf(wa.y, xa[q][1], va);
-                    va = fmaf(wa.z, xa[q][2], va);
-                    va = fmaf(wa.w, xa[q][3], va);
-                    va *= ma[q];
-                    if (two) {
-                        float vb = wb.x * xb[q][0];
-                        vb = fmaf(wb.y, xb[q][1], vb);
-                        vb = fmaf(wb.z, xb[q][2], vb);
-                        vb = fmaf(wb.w, xb[q][3], vb);
-                        vb *= mc[q];
-                        if (C % 2 == 0) {  // i even: one 8-byte store (half the bank conflicts of two)
-                            *reinterpret_cast<float2*>(wr + i) = make_float2(va, vb);
-                        } else {
-                            wr[i] = va;
-                            wr[i + 1] = vb;
-                        }
-                        if (i + 1 == nx - 1)
-                            for (int h = nx; h < wcols - C; ++h) wr[h] = vb;
-                    } else {
-                        wr[i] = va;
-                    }
-                    if (i == 0)  // replicate padding along i: left halo columns
-                        for (int h = -C; h < 0; ++h) wr[h] = va;
-                    if (i == nx - 1)  // right halo columns
-                        for (int h = nx; h < wcols - C; ++h) wr[h] = va;
-                }
+            for (int h = 0; h < NO / 4; ++h) {
+                const float4 t = __ldg(reinterpret_cast<const float4*>(tab) + (TAPS / 4) * i + h);
+                const int4 b = __ldg(reinterpret_cast<const int4*>(tab + TAPS * nx) + (TAPS / 4) * i + h);
+                tw[4 * h] = t.x, tw[4 * h + 1] = t.y, tw[4 * h + 2] = t.z, tw[4 * h + 3] = t.w;
+                to[4 * h] = b.x, to[4 * h + 1] = b.y, to[4 * h + 2] = b.z, to[4 * h + 3] = b.w;
             }
         }
-    }
-    if (__syncthreads_or(!ok)) {  // the attenuation plane never arrived
-        if (threadIdx.x == 0) {
-            flag_timeout(err);
-            mbar_wait_bounded(bar, 0u);  // a last chance for the copy in flight to land
+    };
+    table(j0, w, o);
+    const float* mb = mubar + ((size_t)l * g.ny + j0) * d.ps + 4 * (size_t)e;
+    float* out = wsl + ((size_t)v * g.ny + j0) * d.ps + 4 * (size_t)e;
+#pragma unroll 1
+    for (int j = j0; j < j_end; ++j, mb += d.ps, out += d.ps) {
+        const float4 m = ld_stream4(mb);
+        float4 c[TAPS];
+#pragma unroll
+        for (int t = 0; t < TAPS; ++t)
+            c[t] = __ldg(reinterpret_cast<const float4*>(
+                x + (TAPS == 4 ? o[0] + (t & 1) * kp + (t >> 1) * pln : o[t < NO ? t : 0])));
+        if (j + 1 < j_end) table(j + 1, wn, on);
+        float4 a = make_float4(w[0] * c[0].x, w[0] * c[0].y, w[0] * c[0].z, w[0] * c[0].w);
+#pragma unroll
+        for (int t = 1; t < TAPS; ++t) {
+            a.x = fmaf(w[t], c[t].x, a.x);
+            a.y = fmaf(w[t], c[t].y, a.y);
+            a.z = fmaf(w[t], c[t].z, a.z);
+            a.w = fmaf(w[t], c[t].w, a.w);
         }
-        return;
-    }
-    if (threadIdx.x == 0) {
-        fence_proxy_async_smem();
-        tma_store_1d(wsl + ((size_t)v * ny + j) * d.farea, S, (unsigned)d.farea * 4u);
-        tma_store_wait_read<0>();  // the block may leave once its shared memory is read
+        *reinterpret_cast<float4*>(out) = make_float4(a.x * m.x, a.y * m.y, a.z * m.z, a.w * m.w);
+#pragma unroll
+        for (int t = 0; t < TAPS; ++t) w[t] = wn[t];
+#pragma unroll
+        for (int t = 0; t < NO; ++t) o[t] = on[t];
     }
 }
 
+inline RotDims rot_dims(const Geometry& g, int ps, int ts, int nv, int sms)
+{
+    RotDims d;
+    d.ps = ps;
+    d.ts = ts;
+    d.nb = (g.nx * (g.kp / 4) + kRotThreads - 1) / kRotThreads;
+    // eight planes per block, fewer where that would leave SMs without eight blocks
+    d.JP = 8;
+    while (d.JP > 1 && (long long)d.nb * ((g.ny + d.JP - 1) / d.JP) * nv < 8ll * sms) d.JP /= 2;
+    return d;
+}
+
 // Launch shape of the forward blur: one block per depth group of J planes, view
-// and column tile of TI detector columns.  A tile is a TMA box (wp x br rows,
-// nbox of them) of the rotated plane image, its C halo columns on each side
-// included, so every tile is blurred independently from one image.
+// and column tile of TI detector columns.  A tile is nbox TMA boxes (32 k x wr
+// columns) of the rotated plane image, C halo columns on each side included, so
+// every tile is blurred independently from one image.
+constexpr int kWK = 32;  // k of a box
+
 struct FwdDims {
     int TI, nT;        // tile width in columns (multiple of CX), tiles per plane
-    int wp;            // row pitch of a tile buffer = box width: pitch4odd(TI + 2C), at most 252
-    int br, nbox;      // rows per box (at most 256), boxes per plane
-    int warea;         // floats of a tile buffer (nbox * br * wp, rounded up to 128 bytes)
+    int wr, nbox;      // columns of a box: TI + 2C (at most 256); boxes per plane: ceil(nz / 32)
+    int warea;         // floats of a tile buffer: nbox * wr * 32
     int nbuf;          // tile buffers (1 or 2): planes in flight per block
     int kpu, nkb, nib; // U row pitch; k runs; column runs of the whole plane
     int urows;         // rows of U: min(TI, nx)
@@ -374,11 +362,15 @@ struct FwdDims {
 
 // Tap record of one PSF plane (view, depth) for the forward blur, built at plan
 // time (k_fwd_records): FX and FZ zero-padded to P and centred (PT floats each),
-// then the folded edge taps of replicate padding along k, lo and hi (nkb * 16
-// floats each): output k adds U(0) lo(k) + U(nz-1) hi(k), lo(k) = sum_{b > k+C} fz(b),
-// hi(k) = sum_{b < k+C-nz+1} fz(b).  A group's records are contiguous, so a block
-// fetches them with one bulk copy instead of building them.
-__host__ __device__ inline int fwd_rec_floats(int PT, int nkb) { return 2 * PT + 2 * 16 * nkb; }
+// then the folded edge taps of replicate padding: along k lo and hi (nkb * 16
+// floats each; output k adds U(0) lo(k) + U(nz-1) hi(k), lo(k) = sum_{b > k+C} fz(b),
+// hi(k) = sum_{b < k+C-nz+1} fz(b)), along i likewise, lo for the columns
+// [0, kFoldLo) and hi for the kFoldHi columns from fold_hi0(nx).  A group's records
+// are contiguous, so a block fetches them with one bulk copy instead of building them.
+constexpr int kFoldLo = 32;  // runs of 16 columns that start before C <= 18
+constexpr int kFoldHi = 48;  // the same at the other end: C + 15 + 15 columns at most
+__host__ __device__ inline int fold_hi0(int nx, int C) { return nx > C ? (nx - C) & ~15 : 0; }
+__host__ __device__ inline int fwd_rec_floats(int PT, int nkb) { return 2 * PT + 2 * 16 * nkb + kFoldLo + kFoldHi; }
 
 __host__ __device__ inline size_t fwd_smem_floats(const FwdDims& d, int PT)
 {
@@ -421,10 +413,10 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FwdDims& d
         const int b = d.nbuf == 1 ? 0 : n & 1;
         float* dst = WB + (size_t)b * d.warea;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar + b)),
-                     "r"((unsigned)(d.nbox * d.br * d.wp) * 4u)
+                     "r"((unsigned)d.warea * 4u)
                      : "memory");
         for (int q = 0; q < d.nbox; ++q)
-            tma_load_3d(dst + (size_t)q * d.br * d.wp, tmap, i0, q * d.br, v * ny + j_begin + n, bar + b);
+            tma_load_3d(dst + q * d.wr * kWK, tmap, q * kWK, i0 - C, v * ny + j_begin + n, bar + b);
     };
     // the first planes are requested before anything else, so their loads overlap the set-up below
     if (tid == 0) {
@@ -449,6 +441,7 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FwdDims& d
     __syncthreads();  // the barriers are initialised and U's halos are zero
     bool ok = mbar_wait_bounded(bar + 2, 0u);
 
+    const int hi0 = fold_hi0(nx, C);
     // the thread's first work item of each pass and the step to its next one
     // (the same for every plane: the divisions stay out of the plane loop)
     const int ip_ib = tid / nz, ip_k = tid - ip_ib * nz;    // i-pass: (column run, k)
@@ -464,6 +457,8 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FwdDims& d
         const unsigned parity = (unsigned)(d.nbuf == 1 ? n : n >> 1) & 1u;
         const float* FX = TAP + n * rf;
         const float* FZ = FX + PT;
+        const float* xlo = FZ + PT + 2 * d.nkb * CZ;
+        const float* xhi = xlo + kFoldLo;
         const float* W = WB + (size_t)b * d.warea;
         ok = mbar_wait_bounded(bar + b, parity) && ok;
 
@@ -472,11 +467,15 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FwdDims& d
             int ib = ip_ib, k = ip_k;
             for (int it = tid; it < nz * nibt; it += T) {
                 const int li = ib * CX;  // first column of this run, relative to the tile
-                const float* wr = W + k * d.wp + li;
-                float win[4 * ((CX + P - 1 + 3) / 4)];
-                load_row_f4(wr, win);
+                const float* wr = W + (k / kWK) * (d.wr * kWK) + k % kWK;
+                float win[CX + P - 1];
+#pragma unroll
+                for (int m = 0; m < CX + P - 1; ++m) win[m] = wr[(li + m) * kWK];
                 float o[CX];
                 fir<P, CX, -1, P - 1>(FX, win, o);
+                // folded taps of the plane's first and last columns (zero elsewhere)
+                if (i0 + li < C) fold_taps(wr[(C - i0) * kWK], xlo + i0 + li, o);
+                if (i0 + li >= hi0) fold_taps(wr[(C + nx - 1 - i0) * kWK], xhi + i0 + li - hi0, o);
                 float* ur = U + li * d.kpu + ZH + k;
                 if (li + CX <= ti) {
 #pragma unroll
@@ -517,30 +516,8 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FwdDims& d
             fir<P, CZ, -1, C + ZH>(FZ, win, o);
             const int k0 = kb * CZ;
             // folded taps are zero outside the first and last C rows
-            if (k0 + CZ > nz - C) {
-                const float uhi = ur[ZH + nz - 1];
-                const float4* f4 = reinterpret_cast<const float4*>(fold_hi + k0);
-#pragma unroll
-                for (int c4 = 0; c4 < CZ / 4; ++c4) {
-                    const float4 f = f4[c4];
-                    o[4 * c4] = fmaf(uhi, f.x, o[4 * c4]);
-                    o[4 * c4 + 1] = fmaf(uhi, f.y, o[4 * c4 + 1]);
-                    o[4 * c4 + 2] = fmaf(uhi, f.z, o[4 * c4 + 2]);
-                    o[4 * c4 + 3] = fmaf(uhi, f.w, o[4 * c4 + 3]);
-                }
-            }
-            if (k0 < C) {
-                const float ulo = ur[ZH];
-                const float4* f4 = reinterpret_cast<const float4*>(fold_lo + k0);
-#pragma unroll
-                for (int c4 = 0; c4 < CZ / 4; ++c4) {
-                    const float4 f = f4[c4];
-                    o[4 * c4] = fmaf(ulo, f.x, o[4 * c4]);
-                    o[4 * c4 + 1] = fmaf(ulo, f.y, o[4 * c4 + 1]);
-                    o[4 * c4 + 2] = fmaf(ulo, f.z, o[4 * c4 + 2]);
-                    o[4 * c4 + 3] = fmaf(ulo, f.w, o[4 * c4 + 3]);
-                }
-            }
+            if (k0 + CZ > nz - C) fold_taps(ur[ZH + nz - 1], fold_hi + k0, o);
+            if (k0 < C) fold_taps(ur[ZH], fold_lo + k0, o);
         };
         if (RACC) {
             if (tid < ti * d.nkb) {
@@ -800,10 +777,9 @@ FusedDims dims_for(const Geometry& g, int J, int tiles)
     d.marea = d.urows * g.kp;
     d.wp = pitch4odd(d.TI + 2 * S::C);
     d.warea = (g.nz * d.wp + 3) & ~3;
-    d.wpf = pitch4odd(d.nib * S::CX + 2 * S::C);
     d.wz = pitch4odd(d.TI + 2 * S::C);
     d.zarea = g.nz * d.wz;
-    d.farea = (g.nz * d.wpf + 3) & ~3;
+    d.farea = (g.nz * pitch4odd(d.nib * S::CX + 2 * S::C) + 3) & ~3;
     int kpu = d.nkb * S::CZ + 2 * S::ZH;
     kpu = (kpu + 3) & ~3;
     if (((kpu / 4) & 1) == 0) kpu += 4;
@@ -816,8 +792,8 @@ FusedDims dims_for(const Geometry& g, int J, int tiles)
     return d;
 }
 
-// Rotation kernel without the attenuation plane staged: plane image + table.
-inline size_t rot_smem_min(const FusedDims& d) { return ((size_t)d.farea + d.ts) * sizeof(float); }
+// Part of the bound of the geometries taken: a plane with its halos and a rotation table in shared memory.
+inline size_t rot_smem_bound(const FusedDims& d) { return ((size_t)d.farea + d.ts) * sizeof(float); }
 
 // Launch shape of the forward blur for `tiles` column tiles (the nearest count
 // whose box fits the tensor map's 256 columns) and J planes per block.
@@ -846,14 +822,11 @@ FwdDims fwd_dims(const Geometry& g, int J, int tiles, size_t smem_limit)
     d.nkb = (g.nz + S::CZ - 1) / S::CZ;
     tiles = tiles < 1 ? 1 : (tiles > d.nib ? d.nib : tiles);
     d.TI = ((d.nib + tiles - 1) / tiles) * S::CX;
-    while (pitch4odd(d.TI + 2 * S::C) > 252) d.TI -= S::CX;
+    while (d.TI + 2 * S::C > 256) d.TI -= S::CX;
     d.nT = (g.nx + d.TI - 1) / d.TI;
-    d.wp = pitch4odd(d.TI + 2 * S::C);
-    d.nbox = (g.nz + 255) / 256;
-    d.br = (g.nz + d.nbox - 1) / d.nbox;
-    // every box starts on 128 bytes of shared memory: wp is 4 * odd, so 8 rows are a multiple of 128 bytes
-    if (d.nbox > 1) d.br = (d.br + 7) & ~7;
-    d.warea = (d.nbox * d.br * d.wp + 31) & ~31;
+    d.wr = d.TI + 2 * S::C;
+    d.nbox = (g.nz + kWK - 1) / kWK;
+    d.warea = d.nbox * d.wr * kWK;  // every box is a multiple of 128 bytes
     d.urows = d.TI < g.nx ? d.TI : g.nx;
     d.kpu = pitch4odd(d.nkb * S::CZ + 2 * S::ZH);
     d.apc = pitch4odd(d.nkb * S::CZ);

@@ -2,8 +2,8 @@
 // interface spect_batch_*): one launch per stage and kernel variant over a work
 // list that spans every plan of the batch, instead of one launch per stage and
 // plan.  Stages of one EM iteration (Eqs. (7)-(8), beta = 0):
-//   rotation + attenuation (per PSF bucket, attenuation staged or not),
-//   blur + depth-group sums (per bucket, tiled or not), depth-group reduce with
+//   rotation + attenuation (all plans),
+//   blur + depth-group sums (per bucket), depth-group reduce with
 //   the EM ratio (all plans), blur adjoint + attenuation (per bucket, tiled or
 //   not), adjoint rotation + view sum + MLEM update (gather.cu, per list length),
 // plus the layout transposes of the iterates before the first and after the
@@ -24,7 +24,8 @@ namespace {
 
 struct GroupPlan {
     Geometry g;
-    FusedDims im, da;  // plane images (rotation), adjoint launch shape
+    RotDims dr;        // rotation launch shape
+    FusedDims da;      // adjoint launch shape
     FwdDims df;        // forward launch shape
     int cls_z;
     const float* rtab;
@@ -57,12 +58,11 @@ struct GroupTs {
     GroupGrid grid;
 };
 
-template <int P, bool MUS>
-__global__ void __launch_bounds__(kRotThreads, 2) k_rot_fwd_grp(const __grid_constant__ GroupPlans gp)
+__global__ void __launch_bounds__(kRotThreads, 5) k_rot_fwd_grp(const __grid_constant__ GroupPlans gp)
 {
     const int4 w = group_item(gp.grid);
     const GroupPlan q = gp.p[w.x];  // by value: the fields live in registers, not re-read from parameter space
-    rot_fwd_body<P, MUS>(q.g, q.im, q.rtab, q.xt, q.mubar, q.slab, 0, q.err, w.y, w.z);
+    rot_body<4>(q.g, q.dr, q.rtab, q.xt, q.mubar, q.slab, 0, w.y, w.z);
 }
 
 template <int P, bool RACC>
@@ -124,12 +124,9 @@ template <int P>
 void fill_plan(GroupPlan& q, const spect_plan_s* Pl, const float* y, const float* rbar)
 {
     q.g = Pl->g;
-    q.im = dims_for<P>(Pl->g, Pl->fused_J, 1);
     q.df = fwd_dims<P>(Pl->g, Pl->fused_J, Pl->fwd_nT, (size_t)Pl->smem_optin);
     q.da = dims_for<P>(Pl->g, Pl->adj_J, Pl->adj_nT);
     q.cls_z = Pl->cls_z;
-    q.rtab = Pl->rtab;
-    q.xt = Pl->xt;
     q.mubar = Pl->mubar;
     q.slab = Pl->slab;
     q.frec = Pl->frec;
@@ -141,18 +138,6 @@ void fill_plan(GroupPlan& q, const spect_plan_s* Pl, const float* y, const float
     q.rbar = rbar;
     q.nproj = (size_t)Pl->g.nx * Pl->g.nz * Pl->g.nview;
     q.err = Pl->err;
-}
-
-// the shared memory the rotation kernel takes for this plan, and whether the
-// attenuation plane is staged (the choice rot_launch makes)
-template <int P>
-size_t rot_smem(const spect_plan_s& Pl, bool* mus)
-{
-    const FusedDims d = dims_for<P>(Pl.g, Pl.fused_J, 1);
-    const size_t smin = rot_smem_min(d);
-    const size_t smem_mu = smin + (size_t)d.ps * sizeof(float) + 16;
-    *mus = smem_mu <= (size_t)Pl.smem_optin;
-    return *mus ? smem_mu : smin;
 }
 
 // append plan m's grid (gx x gy x gz blocks) to a grouped launch's block ranges
@@ -185,12 +170,11 @@ cudaError_t stage_launches(int stage, const std::vector<int>& idx, const std::ve
                            const float* const* y, const float* const* rbar, GroupedBatch& /*B*/,
                            std::vector<GroupLaunch>& out)
 {
-    // sub-groups by kernel variant: attenuation staged (rotation), sums in registers (blur), tiled (adjoint)
+    // sub-groups by kernel variant: sums in registers (blur), tiled (adjoint)
     std::vector<int> var[2];
     for (int i : idx) {
         bool flag = false;
-        if (stage == 0) rot_smem<P>(*plans[i], &flag);
-        else if (stage == 1)
+        if (stage == 1)
             flag = fwd_dims<P>(plans[i]->g, plans[i]->fused_J, plans[i]->fwd_nT, (size_t)plans[i]->smem_optin).racc;
         else
             flag = dims_for<P>(plans[i]->g, plans[i]->adj_J, plans[i]->adj_nT).nT > 1;
@@ -205,11 +189,7 @@ cudaError_t stage_launches(int stage, const std::vector<int>& idx, const std::ve
                 const spect_plan_s* Pl = plans[ch[m]];
                 fill_plan<P>(gp.p[m], Pl, y[ch[m]], rbar ? rbar[ch[m]] : nullptr);
                 const GroupPlan& q = gp.p[m];
-                if (stage == 0) {  // the rotation's grid: (plane j, view)
-                    bool mus = false;
-                    smem = std::max(smem, rot_smem<P>(*Pl, &mus));
-                    add_grid(gp.grid, m, q.g.ny, q.g.nview, 1);
-                } else if (stage == 1) {  // the forward blur's grid: (depth group and column tile, view)
+                if (stage == 1) {  // the forward blur's grid: (depth group and column tile, view)
                     smem = std::max(smem, smem_fwd<P>(q.df));
                     thr = std::max(thr, q.df.T);
                     gp.fmap[m] = Pl->fmap;
@@ -220,10 +200,7 @@ cudaError_t stage_launches(int stage, const std::vector<int>& idx, const std::ve
                 }
             }
             if (ch.empty()) continue;
-            if (stage == 0)
-                out.push_back(f ? make_launch(k_rot_fwd_grp<P, true>, gp, dim3(kRotThreads), smem)
-                                : make_launch(k_rot_fwd_grp<P, false>, gp, dim3(kRotThreads), smem));
-            else if (stage == 1)
+            if (stage == 1)
                 out.push_back(f ? make_launch(k_fwd_sep_grp<P, true>, gp, dim3(thr), smem)
                                 : make_launch(k_fwd_sep_grp<P, false>, gp, dim3(thr), smem));
             else
@@ -282,6 +259,29 @@ cudaError_t reduce_launches(const std::vector<spect_plan_s*>& plans, const float
     return cudaSuccess;
 }
 
+// rotation + attenuation, all plans (any bucket): the grid is (planes and column run, view)
+cudaError_t rotate_launches(const std::vector<spect_plan_s*>& plans, std::vector<GroupLaunch>& out)
+{
+    std::vector<int> all(plans.size());
+    std::iota(all.begin(), all.end(), 0);
+    for (const std::vector<int>& ch : chunks_of(all, plans)) {
+        GroupPlans gp{};
+        for (int m = 0; m < (int)ch.size(); ++m) {
+            const spect_plan_s* Pl = plans[ch[m]];
+            GroupPlan& q = gp.p[m];
+            q.g = Pl->g;
+            q.dr = rot_dims(Pl->g, Pl->ps, Pl->ts, Pl->g.nview, Pl->sms);
+            q.rtab = Pl->rtab;
+            q.xt = Pl->xt;
+            q.mubar = Pl->mubar;
+            q.slab = Pl->slab;
+            add_grid(gp.grid, m, q.dr.nb * ((q.g.ny + q.dr.JP - 1) / q.dr.JP), q.g.nview, 1);
+        }
+        out.push_back(make_launch(k_rot_fwd_grp, gp, dim3(kRotThreads), 0));
+    }
+    return cudaSuccess;
+}
+
 // x (image layout) <-> x_t ([j][i][k]) for every plan: to_internal / from_internal
 cudaError_t transpose_launches(const std::vector<spect_plan_s*>& plans, float* const* x, bool to_internal,
                                GroupedBatch& /*B*/, std::vector<GroupLaunch>& out)
@@ -319,7 +319,7 @@ cudaError_t build_grouped(const std::vector<spect_plan_s*>& plans, float* const*
                           const float* const* rbar, GroupedBatch& B)
 {
     cudaError_t e = transpose_launches(plans, x, true, B, B.head);
-    if (e == cudaSuccess) e = stage_by_bucket(0, plans, y, rbar, B, B.iter);
+    if (e == cudaSuccess) e = rotate_launches(plans, B.iter);
     if (e == cudaSuccess) e = stage_by_bucket(1, plans, y, rbar, B, B.iter);
     if (e == cudaSuccess) e = reduce_launches(plans, y, rbar, B, B.iter);
     if (e == cudaSuccess) e = stage_by_bucket(2, plans, y, rbar, B, B.iter);

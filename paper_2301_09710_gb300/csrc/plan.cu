@@ -173,6 +173,16 @@ size_t view_bytes(const spect_plan_s& P, size_t slab_floats_per_view)
     return f * sizeof(float);
 }
 
+// Views per pass: what the budget holds, then evened out over the passes, so that
+// no pass is left with a few views (and the buffers are no larger than that takes).
+int view_chunk(const spect_plan_s& P, size_t slab_floats_per_view, size_t budget)
+{
+    const size_t nview = (size_t)P.g.nview;
+    const size_t most = std::max<size_t>(1, std::min<size_t>(nview, budget / view_bytes(P, slab_floats_per_view)));
+    const size_t passes = (nview + most - 1) / most;
+    return (int)((nview + passes - 1) / passes);
+}
+
 // The patch gather reads its own box-local copy of the adjacency entries, so
 // once it is set up the fixed-length lists were set-up input only: free them.
 void drop_fixed_lists(spect_plan_s* P, cudaStream_t st)
@@ -379,7 +389,8 @@ size_t plan_bytes_bound(const spect_plan_s& P)
     const size_t vol = (size_t)g.nx * g.ny * g.nz, nproj = (size_t)g.nx * g.nz * g.nview;
     const size_t nxy = (size_t)g.nx * g.ny, nrows = (size_t)g.nvp * g.ny, nlist = nxy * g.nview;
     const size_t volt = nxy * g.kp;  // an internal volume
-    size_t b = sizeof(int) + vol * F;
+    size_t b = sizeof(int);
+    if (!P.fast) b += 2 * vol * F;  // mu and the EM accumulator in the image layout
     if (P.separable) b += ((size_t)g.px * 4 + (size_t)g.pz * (1 + P.cls_z)) * nrows * F;
     else b += (size_t)g.px * g.pz * nrows * (1 + (size_t)P.cls_x * P.cls_z) * F;
     b += (size_t)g.nview * sizeof(ViewRot);
@@ -388,10 +399,10 @@ size_t plan_bytes_bound(const spect_plan_s& P)
     b += P.fast ? std::max(fixed, csr) : csr;
     const size_t per_view = std::max(vol, P.fast ? spect::fused_slab_per_view(P) : vol);
     const size_t budget = P.recompute ? recompute_budget_bytes() : slab_budget_bytes(P.fast);
-    const size_t chunk = std::max<size_t>(1, std::min<size_t>((size_t)g.nview, budget / view_bytes(P, per_view)));
+    const size_t chunk = view_chunk(P, per_view, budget);
     b += per_view * chunk * F;
-    b += (2 * vol + nproj) * F;
-    if (P.fast && P.separable) b += spect::fwd_records_floats(P) * F;
+    b += (vol + nproj) * F;
+    if (P.fast) b += spect::fwd_records_floats(P) * F;
     if (P.fast) {
         // attenuation factors of every view, or of one chunk plus mu in the internal layout
         b += P.recompute ? ((size_t)g.ny * P.ps * chunk + volt) * F : (size_t)g.ny * P.ps * g.nview * F;
@@ -446,12 +457,11 @@ spect_status spect_plan_bytes(int nx, int ny, int nz, int nview, int px, int pz,
     P.recompute = (flags & SPECT_PLAN_RECOMPUTE_ATTENUATION) != 0 && P.fast && !P.rot3;
     P.smem_optin = smem_optin;
     if (P.fast) {
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        if (cudaDeviceGetAttribute(&P.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
             cudaGetLastError();
             return fail(SPECT_ECUDA, "device query failed");
         }
-        spect::default_fwd_shape(P, sms);
+        spect::default_fwd_shape(P);
     }
     *bytes = plan_bytes_bound(P);
     return SPECT_OK;
@@ -540,9 +550,8 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         P->fast = P->bucket > 0;
         P->fwd_nT = P->adj_nT = 1;
     }
-    int sms = 0;
-    PLAN_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device query");
-    if (P->fast) spect::default_fwd_shape(*P, sms);
+    PLAN_TRY(cudaDeviceGetAttribute(&P->sms, cudaDevAttrMultiProcessorCount, dev), "device query");
+    if (P->fast) spect::default_fwd_shape(*P);
     if (P->fast && P->separable) P->adj_nT = spect::adj_tiles(*P);
     P->rot3 = (flags & SPECT_PLAN_ROTATION_3PASS) != 0;
     if (P->rot3 && !P->fast) {
@@ -657,21 +666,22 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         PLAN_TRY(cudaStreamSynchronize(st), "adjacency fill");
     }
 
-    // the forward blur's tap records; the factors themselves are not read again
-    if (P->fast && P->separable) {
+    // the forward blur's tap records; the factors (or the stack) themselves are not read again
+    if (P->fast) {
         PLAN_ALLOC(P->frec, spect::fwd_records_floats(*P), "tap records");
         PLAN_TRY(spect::launch_fwd_records(*P, st), "tap record launch");
-        raw_free(P, P->fx, st);
-        raw_free(P, P->fz, st);
-        P->fx = P->fz = nullptr;
-        P->bytes -= (size_t)(px + pz) * nrows * sizeof(float);
+        for (float** p : {&P->fx, &P->fz, &P->psf}) {
+            raw_free(P, *p, st);
+            *p = nullptr;
+        }
+        P->bytes -= (P->separable ? (size_t)(px + pz) : (size_t)px * pz) * nrows * sizeof(float);
     }
 
     // work slab and EM buffers
     const size_t budget = P->recompute ? recompute_budget_bytes() : slab_budget_bytes(P->fast);
     // the fused path stores padded planes (rotated image planes or adjoint planes)
     const size_t per_view = std::max(vol, P->fast ? spect::fused_slab_per_view(*P) : vol);
-    P->chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)nview, budget / (view_bytes(*P, per_view))));
+    P->chunk = view_chunk(*P, per_view, budget);
     PLAN_ALLOC(P->slab, per_view * (size_t)P->chunk, "work slab");
     P->slab_cap = per_view * (size_t)P->chunk;
     if (P->fast) PLAN_TRY(spect::build_fwd_map(*P), "tensor map of the plane images");
@@ -684,11 +694,11 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         if (atoi(env) > 0) {
             P->adj_chunk_req = atoi(env);
             P->adj_chunk = std::min(std::min(atoi(env), nview), P->chunk);
-            const int want_groups = std::max(1, (2 * std::max(sms, 1) + P->adj_chunk - 1) / P->adj_chunk);
+            const int want_groups = std::max(1, (2 * std::max(P->sms, 1) + P->adj_chunk - 1) / P->adj_chunk);
             P->adj_J = std::max(1, std::min(8, (ny + want_groups - 1) / want_groups));
         }
     }
-    PLAN_ALLOC(P->e, vol, "EM accumulator");
+    if (!P->fast) PLAN_ALLOC(P->e, vol, "EM accumulator");
     PLAN_ALLOC(P->ratio, nproj, "EM ratio");
     PLAN_ALLOC(P->s, vol, "sensitivity");
 
@@ -737,6 +747,10 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
             drop_fixed_lists(P, st);
             PLAN_TRY(spect::build_rotpatch(*P, st), "patch rotation set-up");
         }
+        // the image-layout map was set-up input only
+        raw_free(P, P->mu, st);
+        P->mu = nullptr;
+        P->bytes -= vol * sizeof(float);
     }
     PLAN_TRY(cudaStreamSynchronize(st), "plan set-up");
     *out = P;
@@ -1051,7 +1065,7 @@ spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, int adj_t
     const size_t vol = (size_t)g.nx * g.ny * g.nz, nproj = (size_t)g.nx * g.nz * g.nview;
     const size_t per_view = std::max(vol, spect::fused_slab_per_view(*P));
     const size_t budget = P->recompute ? recompute_budget_bytes() : slab_budget_bytes(true);
-    const int chunk = (int)std::max<size_t>(1, std::min<size_t>((size_t)g.nview, budget / view_bytes(*P, per_view)));
+    const int chunk = view_chunk(*P, per_view, budget);
     spect_status r = realloc_floats(P, &P->slab, &P->slab_cap, per_view * (size_t)chunk, st, "work slab");
     if (r == SPECT_OK)
         r = realloc_floats(P, &P->part, &P->part_cap, nproj * (size_t)spect::fused_groups(*P), st,

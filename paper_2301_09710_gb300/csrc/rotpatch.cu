@@ -8,7 +8,7 @@
 // double-buffered, so the four corner reads of a sample are shared-memory
 // reads instead of L2 gathers.  Weights, corner order and arithmetic are those
 // of k_rot_fwd (same rotation tables), and the output is the same plane image
-// W[k][C + i] with replicate halo columns: the results are bitwise the same.
+// [i][k]: the results are bitwise the same.
 #include <algorithm>
 #include <climits>
 #include <cstdlib>
@@ -59,8 +59,7 @@ struct RotPatchArgs {
     int bw, bh;          // x_t box extents (the tensor map's box: 16 x bw x bh)
     int box_floats;      // bw * bh * 16
     int stage_floats;    // attenuation tile (64 * 16) + box, 128-byte multiple
-    int C, wp, parea;    // plane image: halo width, row pitch, floats per plane
-    int wcols;           // columns of an image row that are written (nib*16 + 2C)
+    int ps;              // floats per plane image
     int ts;              // rotation table block per (view, row)
     int l0, nkc;         // first view of the launch; k runs
 };
@@ -111,7 +110,7 @@ __global__ void __launch_bounds__(kRT) k_rot_patch(const __grid_constant__ CUten
         o = ((bj - box.y) * a.bw + (bi - box.x)) * kRK + 4 * k4;
     }
     const int row = a.bw * kRK;
-    float* img = wsl + ((size_t)v * g.ny + j) * a.parea + a.C;
+    float* img = wsl + ((size_t)v * g.ny + j) * a.ps + (size_t)i * g.kp + 4 * k4;
     __syncthreads();
 
     for (int kc = 0; kc < a.nkc; ++kc) {
@@ -127,22 +126,17 @@ __global__ void __launch_bounds__(kRT) k_rot_patch(const __grid_constant__ CUten
             const float x00[4] = {c00.x, c00.y, c00.z, c00.w}, x10[4] = {c10.x, c10.y, c10.z, c10.w};
             const float x01[4] = {c01.x, c01.y, c01.z, c01.w}, x11[4] = {c11.x, c11.y, c11.z, c11.w};
             const float mv[4] = {m.x, m.y, m.z, m.w};
+            float va[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int k = kc * kRK + 4 * k4 + u;
-                if (k >= g.nz) break;
-                float va = w.x * x00[u];
-                va = fmaf(w.y, x10[u], va);
-                va = fmaf(w.z, x01[u], va);
-                va = fmaf(w.w, x11[u], va);
-                va *= mv[u];
-                float* wr = img + (size_t)k * a.wp;
-                wr[i] = va;
-                if (i == 0)  // replicate padding along i: left halo columns
-                    for (int h = -a.C; h < 0; ++h) wr[h] = va;
-                if (i == g.nx - 1)  // right halo columns
-                    for (int h = g.nx; h < a.wcols - a.C; ++h) wr[h] = va;
+                va[u] = w.x * x00[u];
+                va[u] = fmaf(w.y, x10[u], va[u]);
+                va[u] = fmaf(w.z, x01[u], va[u]);
+                va[u] = fmaf(w.w, x11[u], va[u]);
+                va[u] *= mv[u];
             }
+            if (kc * kRK + 4 * k4 < g.kp)
+                *reinterpret_cast<float4*>(img + kc * kRK) = make_float4(va[0], va[1], va[2], va[3]);
         }
         if (__syncthreads_or(!ok)) {  // a copy never landed: give the ones in flight a last chance, then stop
             if (tid == 0) {
@@ -239,15 +233,10 @@ cudaError_t launch_rot_patch(const spect_plan_s& P, int l0, int nv, cudaStream_t
     a.bh = P.rbh;
     a.box_floats = P.rbw * P.rbh * kRK;
     a.stage_floats = rot_stage_floats(a.box_floats);
-    const int C = (P.bucket - 1) / 2;
-    const int nib = (g.nx + 15) / 16;
-    a.C = C;
-    a.wp = pitch4odd(nib * 16 + 2 * C);  // as the fused kernels' untiled plane image
-    a.parea = (g.nz * a.wp + 3) & ~3;
-    a.wcols = nib * 16 + 2 * C;
+    a.ps = P.ps;
     a.ts = P.ts;
     a.l0 = l0;
-    a.nkc = (g.nz + kRK - 1) / kRK;
+    a.nkc = (g.kp + kRK - 1) / kRK;
     const size_t smem = rot_smem(a.box_floats);
     cudaError_t e = cudaFuncSetAttribute(k_rot_patch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

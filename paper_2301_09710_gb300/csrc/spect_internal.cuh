@@ -83,6 +83,7 @@ struct spect_plan_s {
     cudaStream_t home = nullptr; // creation stream (stream-ordered allocations)
     bool pooled = false;         // memory from cudaMallocAsync (freed with cudaFreeAsync)
     int smem_optin = 0;          // shared memory a block may opt in to (bytes)
+    int sms = 0;                 // multiprocessors of the device
     int fast = 0;                // 1 when the fused kernels serve this plan
     int bucket = 0;              // padded tap count of the fused kernels
     int fused_J = 8;             // depth planes per fused forward block
@@ -435,7 +436,7 @@ size_t fwd_records_floats(const spect_plan_s& P);
 cudaError_t launch_fwd_records(const spect_plan_s& P, cudaStream_t st);
 int fwd_tiles(const spect_plan_s& P);
 int adj_tiles(const spect_plan_s& P);
-void default_fwd_shape(spect_plan_s& P, int sms);
+void default_fwd_shape(spect_plan_s& P);
 // Bucket of the fused full-PSF kernels (untiled planes), 0 when they do not fit.
 int fused_dir_bucket(const Geometry& g, size_t smem_limit);
 bool fused_dir_fit(const Geometry& g, int bucket, int J, int adj_J, size_t smem_limit);

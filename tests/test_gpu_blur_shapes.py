@@ -41,3 +41,29 @@ def test_blur_launch_shapes(case):
     assert_close(host(plan.back(dev(yy))), oracle.back(yy, prob.mu, psf, prob.dy, ang), what="A' y")
     plan.check()
     plan.close()
+
+
+# nx, nz, nview, px, pz, nview_psf, seed: the full-PSF kernels' tiles
+DIRECT = [
+    (33, 17, 5, 21, 9, 5, 3),   # last tile: one column; zero tap rows of the bucket
+    (50, 5, 7, 13, 13, 1, 4),   # PSF taller than the plane
+    (16, 300, 2, 5, 5, 1, 5),   # two boxes per plane
+    (19, 40, 3, 37, 37, 1, 6),  # PSF wider than the plane: both halos in one tile
+]
+
+
+@pytest.mark.parametrize("case", DIRECT, ids=[f"{c[0]}x{c[1]}p{c[3]}x{c[4]}" for c in DIRECT])
+def test_full_psf_launch_shapes(case):
+    need_gpu()
+    nx, nz, nview, px, pz, nvp, seed = case
+    prob = synthetic.random_problem(seed, nx=nx, nz=nz, nview=nview, px=px, pz=pz, nview_psf=nvp, mu_scale=0.05)
+    rng = np.random.default_rng(seed)
+    ang = rng.uniform(0, 2 * np.pi, nview)
+    plan = make_plan(prob, ang, "direct")
+    assert plan.info()["fused"]
+    psf = prob.full_psf().astype(np.float64)
+    assert_close(host(plan.forward(dev(prob.x))), oracle.forward(prob.x, prob.mu, psf, prob.dy, ang), what="A x")
+    yy = rng.uniform(0, 1, plan.proj_shape).astype(np.float32)
+    assert_close(host(plan.back(dev(yy))), oracle.back(yy, prob.mu, psf, prob.dy, ang), what="A' y")
+    plan.check()
+    plan.close()
