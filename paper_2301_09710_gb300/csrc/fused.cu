@@ -22,6 +22,7 @@
 //    gather kernel then sums sum_l sum_p W_l(p;q) t_l(p,k) per destination voxel
 //    q over fixed-length adjacency lists (weights bitwise those of A).
 #include <algorithm>
+#include <cmath>
 
 #include "fused_body.cuh"
 
@@ -264,8 +265,8 @@ __global__ void k_fwd_records(Geometry g, int P, int PT, int nkb, const float* _
 }
 
 // v(i,k,l) = sum over depth groups of the partials (fixed order), optionally
-// turned into the EM ratio y / (v + rbar).
-__global__ void k_fwd_reduce(const float* __restrict__ part, int G, size_t nproj, float* __restrict__ v,
+// turned into the EM ratio y / (v + rbar), whose rows are np long.
+__global__ void k_fwd_reduce(const float* __restrict__ part, int G, size_t nproj, float* __restrict__ v, int nx, int np,
                              const float* __restrict__ em_y, const float* __restrict__ em_rbar)
 {
     const size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -274,21 +275,58 @@ __global__ void k_fwd_reduce(const float* __restrict__ part, int G, size_t nproj
     for (int gq = 0; gq < G; ++gq) s += part[(size_t)gq * nproj + o];
     if (em_y) {
         const float yb = s + (em_rbar ? em_rbar[o] : 0.f);
-        v[o] = yb > 0.f ? em_y[o] / yb : 0.f;
+        v[np == nx ? o : o + o / nx * (np - nx)] = yb > 0.f ? em_y[o] / yb : 0.f;
     } else {
         v[o] = s;
     }
 }
 
-template <int P, bool TILED>
-__global__ void __launch_bounds__(kFusedThreads, 1) k_adj_sep_fused(Geometry g, FusedDims d, int cls_z,
-                                                                     const float* __restrict__ vin,
-                                                                     const float* __restrict__ mubar,
-                                                                     const float* __restrict__ fx_adj,
-                                                                     const float* __restrict__ fz_adj,
-                                                                     float* __restrict__ slab, int l0, int* err)
+// out (rows of np) = v (n rows of nx)
+__global__ void k_pad_rows(const float* __restrict__ v, float* __restrict__ out, size_t n, int nx, int np)
 {
-    adj_sep_body<P, TILED>(g, d, cls_z, vin, mubar, fx_adj, fz_adj, slab, l0, err, blockIdx.x, blockIdx.y, blockIdx.z);
+    const size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (o < n * nx) out[o + o / nx * (np - nx)] = v[o];
+}
+
+cudaError_t launch_pad_rows(const spect_plan_s& P, const float* v, float* out, cudaStream_t st)
+{
+    const size_t rows = (size_t)P.g.nz * P.g.nview, n = rows * P.g.nx;
+    k_pad_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(v, out, rows, P.g.nx, P.g.np);
+    return cudaGetLastError();
+}
+
+// Blur adjoint + attenuation: one block per (column tile, depth group of J planes, view).
+template <int P>
+__global__ void __launch_bounds__(AdjBlock<P>::T, AdjBlock<P>::B)
+    k_adj_sep_fused(const __grid_constant__ CUtensorMap mu_map, const __grid_constant__ CUtensorMap t_map,
+                    const __grid_constant__ CUtensorMap v_map, Geometry g, AdjDims d,
+                    const float* __restrict__ rec, int l0, int mu_l0, int* err)
+{
+    const int grp = blockIdx.x / d.nT;
+    adj_sep_body<P>(g, d, &mu_map, &t_map, &v_map, rec, l0, mu_l0, err, grp, blockIdx.y, blockIdx.x - grp * d.nT);
+}
+
+// Plan time: the tap records of the blur adjoint (layout: AdjRec), one block per PSF plane.
+__global__ void k_adj_records(Geometry g, int P, int PT, int EC, int cls_z, const float* __restrict__ fx_adj,
+                              const float* __restrict__ fz_adj, float* __restrict__ rec)
+{
+    const int row = blockIdx.x, nrow = gridDim.x, C = (P - 1) / 2, ox = (P - g.px) / 2, oz = (P - g.pz) / 2;
+    float* r = rec + (size_t)row * (2 * PT + 4 * EC);
+    auto tap = [&](const float* f, int cls, int p, int off, int a) {  // class cls, padded tap a
+        return a >= off && a < off + p ? f[((size_t)cls * nrow + row) * p + a - off] : 0.f;
+    };
+    for (int a = threadIdx.x; a < PT; a += blockDim.x) {
+        r[a] = tap(fx_adj, 0, g.px, ox, a);
+        r[PT + a] = tap(fz_adj, 0, g.pz, oz, a);
+    }
+    for (int m = threadIdx.x; m < EC; m += blockDim.x) {
+        float* e = r + 2 * PT + m;
+        const bool in = m <= C;
+        e[0] = in ? tap(fx_adj, 1, g.px, ox, C + m) : 0.f;
+        e[EC] = in ? tap(fx_adj, 2, g.px, ox, m) : 0.f;
+        e[2 * EC] = in && cls_z == 3 ? tap(fz_adj, 1, g.pz, oz, C + m) : 0.f;
+        e[3 * EC] = in && cls_z == 3 ? tap(fz_adj, 2, g.pz, oz, m) : 0.f;
+    }
 }
 
 // ============================================================================
@@ -489,7 +527,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_adj_dir_fused(Geometry g, 
     __syncthreads();
     for (int e = tid; e < pln; e += T) {
         const int k = e / nx, i = e - k * nx;
-        Vx[(ZH + k) * d.wp + C + i] = vin[(size_t)l * pln + e];
+        Vx[(ZH + k) * d.wp + C + i] = vin[((size_t)l * nz + k) * g.np + i];
     }
 
     unsigned phases = 0u;
@@ -672,6 +710,30 @@ __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const Adj
     }
 }
 
+namespace {
+cudaError_t encode_3d(CUtensorMap* map, const float* base, const cuuint64_t (&dims)[3], const cuuint64_t (&strides)[2],
+                      cuuint32_t b0, cuuint32_t b1, CUtensorMapSwizzle swizzle)
+{
+    const cuuint32_t box[3] = {b0, b1, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    if (!encode_fn() ||
+        encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return cudaSuccess;
+}
+
+}  // namespace
+
+// Projections v (rows of np) as a tensor map, boxed as the blur adjoint stages them.
+cudaError_t encode_v_map(const Geometry& g, const AdjDims& d, const float* v, CUtensorMap* map)
+{
+    const cuuint64_t dims[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.nz, (cuuint64_t)g.nview};
+    const cuuint64_t strides[2] = {(cuuint64_t)g.np * 4, (cuuint64_t)g.np * g.nz * 4};
+    return encode_3d(map, v, dims, strides, d.vp, d.vrows, CU_TENSOR_MAP_SWIZZLE_NONE);
+}
+
 // ============================================================================
 // host side: dimensioning and launchers
 // ============================================================================
@@ -708,13 +770,16 @@ cudaError_t fwd_launch(const spect_plan_s& Pl, const float* /*xt: the blur reads
 template <int P>
 cudaError_t adj_launch(const spect_plan_s& Pl, const float* v, int l0, int nv, cudaStream_t st)
 {
-    const FusedDims d = dims_for<P>(Pl.g, Pl.adj_J, Pl.adj_nT);
-    const size_t smem = smem_adj<P>(Pl.g, d);
-    auto kern = d.nT > 1 ? k_adj_sep_fused<P, true> : k_adj_sep_fused<P, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const AdjDims d = adj_dims<P>(Pl.g, Pl.adj_J, Pl.adj_nT, (size_t)Pl.smem_optin);
+    const size_t smem = smem_adj<P>(d);
+    CUtensorMap vmap{};
+    cudaError_t e = encode_v_map(Pl.g, d, v, &vmap);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(d.G, nv, d.nT), kFusedThreads, smem, st>>>(Pl.g, d, Pl.cls_z, v, mubar_for(Pl, l0), Pl.fx_adj, Pl.fz_adj,
-                                                           Pl.slab, l0, Pl.err);
+    e = cudaFuncSetAttribute(k_adj_sep_fused<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    // a recomputing plan's factors are those of views l0 .. at chunk-relative positions
+    k_adj_sep_fused<P><<<dim3(d.G * d.nT, nv), d.T, smem, st>>>(Pl.amap_mu, Pl.amap_t, vmap, Pl.g, d, Pl.arec, l0,
+                                                                Pl.recompute ? l0 : 0, Pl.err);
     return cudaGetLastError();
 }
 }  // namespace
@@ -919,31 +984,28 @@ cudaError_t launch_fused_rotate(const spect_plan_s& P, const float* xt, int l0, 
 }
 
 namespace {
-// The plane images of the work slab as a tensor map -- k (nz; zeros beyond) x column
-// (nx) x plane (chunk * ny) -- with the forward blur's tile as its box.
+// The planes of the work slab and of the attenuation factors as tensor maps -- k x column
+// (nx) x plane -- with the blur kernels' tiles as boxes.  The images end at k = nz
+// (zeros beyond); t and the factors at kp.
 template <int P>
-cudaError_t encode_fwd_map(spect_plan_s& Pl)
+cudaError_t encode_maps(spect_plan_s& Pl)
 {
     const Geometry& g = Pl.g;
-    cuuint32_t box[3] = {0, 0, 1};
-    if (Pl.separable) {
-        const FwdDims d = fwd_dims<P>(g, Pl.fused_J, Pl.fwd_nT, (size_t)Pl.smem_optin);
-        box[0] = kWK;
-        box[1] = (cuuint32_t)d.wr;
-    } else {
-        const DirDims d = dir_fwd_dims<P>(g, Pl.fused_J, (size_t)Pl.smem_optin);
-        box[0] = (cuuint32_t)d.wp;
-        box[1] = (cuuint32_t)d.wr;
-    }
-    const cuuint64_t dims[3] = {(cuuint64_t)g.nz, (cuuint64_t)g.nx, (cuuint64_t)Pl.chunk * g.ny};
     const cuuint64_t strides[2] = {(cuuint64_t)g.kp * 4, (cuuint64_t)Pl.ps * 4};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    if (!encode_fn() ||
-        encode_fn()(&Pl.fmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, Pl.slab, dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    return cudaSuccess;
+    const cuuint64_t planes = (cuuint64_t)Pl.chunk * g.ny;
+    const cuuint64_t img[3] = {(cuuint64_t)g.nz, (cuuint64_t)g.nx, planes};
+    if (!Pl.separable) {
+        const DirDims d = dir_fwd_dims<P>(g, Pl.fused_J, (size_t)Pl.smem_optin);
+        return encode_3d(&Pl.fmap, Pl.slab, img, strides, d.wp, d.wr, CU_TENSOR_MAP_SWIZZLE_NONE);
+    }
+    const FwdDims f = fwd_dims<P>(g, Pl.fused_J, Pl.fwd_nT, (size_t)Pl.smem_optin);
+    const AdjDims a = adj_dims<P>(g, Pl.adj_J, Pl.adj_nT, (size_t)Pl.smem_optin);
+    const cuuint64_t t[3] = {(cuuint64_t)g.kp, (cuuint64_t)g.nx, planes};
+    const cuuint64_t mu[3] = {(cuuint64_t)g.kp, (cuuint64_t)g.nx, Pl.recompute ? planes : (cuuint64_t)g.nview * g.ny};
+    cudaError_t e = encode_3d(&Pl.fmap, Pl.slab, img, strides, kWK, f.wr, CU_TENSOR_MAP_SWIZZLE_NONE);
+    if (e == cudaSuccess) e = encode_3d(&Pl.amap_t, Pl.slab, t, strides, 16, a.TI, CU_TENSOR_MAP_SWIZZLE_64B);
+    if (e == cudaSuccess) e = encode_3d(&Pl.amap_mu, Pl.mubar, mu, strides, 16, a.TI, CU_TENSOR_MAP_SWIZZLE_64B);
+    return e;
 }
 }  // namespace
 
@@ -954,56 +1016,112 @@ size_t fwd_records_floats(const spect_plan_s& P)
     return (size_t)P.g.nvp * P.g.ny * (P.separable ? fwd_rec_floats(PT, nkb) : P.bucket * PT);
 }
 
-cudaError_t launch_fwd_records(const spect_plan_s& P, cudaStream_t st)
+namespace {
+int rec_edge(int P) { return ((P - 1) / 2 + 4) & ~3; }  // AdjRec::EC
+}  // namespace
+
+// Floats of the blur adjoint's tap records of a (separable) plan.
+size_t adj_records_floats(const spect_plan_s& P)
 {
-    const int PT = (P.bucket + 3) & ~3, nkb = (P.g.nz + 15) / 16;
-    if (P.separable) k_fwd_records<<<P.g.nvp * P.g.ny, 128, 0, st>>>(P.g, P.bucket, PT, nkb, P.fx, P.fz, P.frec);
-    else k_dir_records<<<P.g.nvp * P.g.ny, 256, 0, st>>>(P.g, P.bucket, PT, P.psf, P.frec);
+    if (!P.separable) return 0;
+    return (size_t)P.g.nvp * P.g.ny * (2 * ((P.bucket + 3) & ~3) + 4 * rec_edge(P.bucket));
+}
+
+cudaError_t launch_records(const spect_plan_s& P, cudaStream_t st)
+{
+    const int PT = (P.bucket + 3) & ~3, nkb = (P.g.nz + 15) / 16, rows = P.g.nvp * P.g.ny;
+    if (P.separable) {
+        k_fwd_records<<<rows, 128, 0, st>>>(P.g, P.bucket, PT, nkb, P.fx, P.fz, P.frec);
+        k_adj_records<<<rows, 64, 0, st>>>(P.g, P.bucket, PT, rec_edge(P.bucket), P.cls_z, P.fx_adj, P.fz_adj, P.arec);
+    } else {
+        k_dir_records<<<rows, 256, 0, st>>>(P.g, P.bucket, PT, P.psf, P.frec);
+    }
     return cudaGetLastError();
 }
 
-cudaError_t build_fwd_map(spect_plan_s& P)
+cudaError_t build_maps(spect_plan_s& P)
 {
-    SPECT_DISPATCH(encode_fwd_map, P)
+    SPECT_DISPATCH(encode_maps, P)
 }
 
-// Default launch shape of the forward blur.  Tiles of 32 columns: a block is then
-// 2 nkb warps, and four to sixteen such blocks share an SM, so one block's
-// barriers, plane loads and set-up are covered by the others' FMAs (128x80, 128 views,
-// 37 taps: 485 us, 542 with 48 columns; 160x96, 120 views, 29 taps: 698 against 846
-// with 48; whole planes in one block of 640 threads took 513 and 880).  J = 8
-// planes per block, fewer when that leaves the chip short of blocks: at 64x32, 64
-// views J = 4 takes 19 us against 21, at 32x16, 32 views J = 2 takes 8.0 against 12.2.
-void default_fwd_shape(spect_plan_s& P)
+namespace {
+// Estimated time (us) of a separable blur launch: `blocks` blocks of J planes and T
+// threads, B of them resident per SM.  Resident warps W share the issue slots, with
+// about four warps' worth lost to latency, so a plane takes W + 4 warp items of
+// 32 P + 100 issue slots; a block's set-up costs about s planes; up to four waves the
+// last one counts whole, beyond that half a block on average.  Against the measured
+// launches (shapes of 16..64 columns and J = 1..16, twelve geometries from 16x8 to
+// 192x128) the shapes it picks are within 4 % of the fastest, 8 % at worst.
+double blur_cost(int P, long long blocks, int J, double s, int T, int B, int sms)
+{
+    const double per_sm = (double)((blocks + sms - 1) / sms);
+    const double res = std::min<double>(B, per_sm);
+    const double w = (double)blocks / (res * sms);
+    const double waves = w <= 4.0 ? std::max(1.0, std::ceil(w - 1e-9)) : w + 0.5;
+    return waves * (J + s) * (res * T / 32.0 + 4.0) * (32.0 * P + 100.0) / 4.0 / 1.92e3;
+}
+
+template <int P>
+void choose_shape(spect_plan_s& Pl)
+{
+    const Geometry& g = Pl.g;
+    const size_t limit = (size_t)Pl.smem_optin;
+    const int nib = (g.nx + 15) / 16, fmin = Pl.fwd_nT, amin = Pl.adj_nT;
+    double fbest = 1e30, abest = 1e30;
+    for (int ti : {32, 48, 64, 16}) {  // 32 columns unless another width is clearly better
+        const int tiles = (nib + ti / 16 - 1) / (ti / 16);
+        for (int J : {8, 4, 6, 10, 12, 16, 7, 5, 3, 2, 1}) {
+            if (J > g.ny) continue;
+            const FwdDims f = fwd_dims<P>(g, J, std::max(tiles, fmin), limit);
+            if (smem_fwd<P>(f) <= limit && (f.racc || ti == 16)) {
+                const int B = blocks_per_sm(smem_fwd<P>(f), f.T, FwdBlock<P>::regs);
+                // + the reduce: G partials written and read
+                const double c = blur_cost(P, (long long)f.G * f.nT * g.nview, J, 1.0, f.T, B, Pl.sms) +
+                                 (double)f.G * g.nx * g.nz * g.nview * 8.0 / 5e6;
+                if (c < 0.98 * fbest) fbest = c, Pl.fused_J = J, Pl.fwd_nT = f.nT;
+            }
+            const AdjDims a = adj_dims<P>(g, J, std::max(tiles, amin), limit);
+            if (smem_adj<P>(a) <= limit) {
+                const int B = blocks_per_sm(smem_adj<P>(a), a.T, AdjBlock<P>::regs);
+                const double c = blur_cost(P, (long long)a.G * a.nT * g.nview, J, 1.0, a.T, B, Pl.sms);
+                if (c < 0.98 * abest) abest = c, Pl.adj_J = J, Pl.adj_nT = a.nT;
+            }
+        }
+    }
+}
+}  // namespace
+
+// Default launch shapes of the blur kernels.  A block is one thread per work item of a
+// column tile, so that several blocks share an SM and one block's barriers, plane
+// loads and set-up are covered by the others' FMAs: forward at 128x80, 128 views, 37
+// taps 485 us with 32 columns, 542 with 48 (whole planes in one block of 640 threads:
+// 513); adjoint 538, 578 with 48; 192x128, 64 views: adjoint 1013 with 32, 952 with 48.
+void default_shape(spect_plan_s& P)
 {
     const Geometry& g = P.g;
     P.fused_J = 8;
-    if (!P.separable) {  // as below, with blocks of the full-PSF kernel
+    P.adj_J = 8;
+    if (!P.separable) {  // blocks of the full-PSF forward kernel
         const long long blocks = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * g.nview;
         if (blocks < 24ll * P.sms) P.fused_J = blocks >= 4ll * P.sms ? 4 : 2;
         return;
     }
-    const int nib = (g.nx + 15) / 16;
-    P.fwd_nT = std::max(P.fwd_nT, (nib + 1) / 2);
-    P.fwd_nT = fwd_tiles(P);
-    const auto blocks = [&](int J) { return (long long)((g.ny + J - 1) / J) * P.fwd_nT * g.nview; };
-    if (blocks(8) < 10ll * P.sms) P.fused_J = blocks(4) >= 4ll * P.sms ? 4 : 2;
+    switch (P.bucket) {
+#define SPECT_CS(B) \
+    case B: choose_shape<B>(P); break;
+        SPECT_CS(3) SPECT_CS(5) SPECT_CS(7) SPECT_CS(9) SPECT_CS(11) SPECT_CS(13) SPECT_CS(15)
+        SPECT_CS(17) SPECT_CS(21) SPECT_CS(25) SPECT_CS(29) SPECT_CS(33) SPECT_CS(37)
+#undef SPECT_CS
+        default: break;
+    }
 }
 
-// Column tiles of the blur adjoint: the fewest, at least adj_nT, that fit with adj_J planes per block.
+// Column tiles of the blur adjoint at its launch shape (what adj_dims makes of the request).
 int adj_tiles(const spect_plan_s& P)
 {
-    auto find = [&](auto tag) -> int {
-        constexpr int B = decltype(tag)::value;
-        for (int t = P.adj_nT; t <= (P.g.nx + 15) / 16; ++t) {
-            const FusedDims d = dims_for<B>(P.g, P.adj_J, t);
-            if (smem_adj<B>(P.g, d) <= (size_t)P.smem_optin) return d.nT;
-        }
-        return P.adj_nT;
-    };
     switch (P.bucket) {
 #define SPECT_AT(B) \
-    case B: return find(std::integral_constant<int, B>());
+    case B: return adj_dims<B>(P.g, P.adj_J, P.adj_nT, (size_t)P.smem_optin).nT;
         SPECT_AT(3) SPECT_AT(5) SPECT_AT(7) SPECT_AT(9) SPECT_AT(11) SPECT_AT(13) SPECT_AT(15)
         SPECT_AT(17) SPECT_AT(21) SPECT_AT(25) SPECT_AT(29) SPECT_AT(33) SPECT_AT(37)
 #undef SPECT_AT
@@ -1043,7 +1161,8 @@ cudaError_t launch_fwd_reduce(const spect_plan_s& P, float* v, const float* em_y
                               cudaStream_t st)
 {
     const size_t nproj = (size_t)P.g.nx * P.g.nz * P.g.nview;
-    k_fwd_reduce<<<(unsigned)((nproj + 255) / 256), 256, 0, st>>>(P.part, fused_groups(P), nproj, v, em_y, em_rbar);
+    k_fwd_reduce<<<(unsigned)((nproj + 255) / 256), 256, 0, st>>>(P.part, fused_groups(P), nproj, v, P.g.nx, P.g.np,
+                                                                  em_y, em_rbar);
     return cudaGetLastError();
 }
 

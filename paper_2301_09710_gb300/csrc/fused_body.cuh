@@ -111,8 +111,6 @@ struct FusedDims {
     int kpu;    // U row pitch (>= nkb*CZ + 2*ZH, multiple of 4, pitch/4 odd)
     int nib, nkb;
     int TI, nT; // tile width in columns (multiple of CX), tiles per plane
-    int wz;     // row pitch of the adjoint's Zb (multiple of 4, wz/4 odd: conflict-free float4 windows)
-    int zarea;  // floats of Zb, nz x wz
     int farea;  // floats of a whole plane with halo columns (bound of the shapes taken, rot_smem_bound)
     int urows;  // rows of U / ACC / MB per tile: min(TI, nx)
     int vrows;  // detector rows a tile's k-adjoint needs: min(nx, TI + 2*C)
@@ -122,12 +120,6 @@ struct FusedDims {
     int ts;     // rotation table block per (view, row): 5*nx rounded up to 4
     int apc;    // accumulator row pitch (>= nkb*CZ, multiple of 4, pitch/4 odd)
 };
-
-__host__ __device__ inline size_t adj_smem_floats(const FusedDims& d, int PT)
-{
-    // Zb | V | MB x2 | taps J x (FX[3],FZ[3]) | 2 mbarriers
-    return (size_t)d.zarea + (size_t)d.vrows * d.kpu + 2 * (size_t)d.marea + 6 * (size_t)PT * d.J + 8;
-}
 
 template <int P>
 __device__ __forceinline__ void load_window_f4(const float* base, float (&win)[Sep<P>::WZ])
@@ -178,43 +170,6 @@ __device__ __forceinline__ void fir(const float* taps, const float (&win)[WN], f
                 for (int c = 0; c < N; ++c) o[c] = fmaf(fv[u], win[c + SIGN * b + OFF], o[c]);
             }
         }
-    }
-}
-
-// sum_b taps[b] w[b + SH] for b = 0..P-1, in that order (one FMA chain)
-template <int P, int SH, int N>
-__device__ __forceinline__ float tap_dot(const float* taps, const float (&w)[N])
-{
-    constexpr int PT = Sep<P>::PT;
-    static_assert(P - 1 + SH < N, "window too short");
-    float s = 0.f;
-#pragma unroll
-    for (int b4 = 0; b4 < PT / 4; ++b4) {
-        const float4 f4 = reinterpret_cast<const float4*>(taps)[b4];
-        const float fv[4] = {f4.x, f4.y, f4.z, f4.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (4 * b4 + u < P) s = fmaf(fv[u], w[4 * b4 + u + SH], s);
-    }
-    return s;
-}
-
-// sum_b taps[b] row[s + b] for b = 0..P-1 (the edge-class output of an adjoint
-// FIR): the samples come in as float4 loads from the aligned position s & ~3
-// (row 16-byte aligned, pitch4odd pitch: conflict-free with lanes over rows)
-// and the shift s & 3 selects a compile-time offset, so no lane issues P
-// dependent scalar loads.  The loads may read up to 3 floats past row[s + P - 1]
-// (still inside the caller's shared memory); those are never used.
-template <int P>
-__device__ __forceinline__ float edge_tap_dot(const float* taps, const float* row, int s)
-{
-    float w[4 * ((P + 3 + 3) / 4)];
-    load_row_f4(row + (s & ~3), w);
-    switch (s & 3) {
-        case 0: return tap_dot<P, 0>(taps, w);
-        case 1: return tap_dot<P, 1>(taps, w);
-        case 2: return tap_dot<P, 2>(taps, w);
-        default: return tap_dot<P, 3>(taps, w);
     }
 }
 
@@ -568,193 +523,255 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FwdDims& d
 }
 
 // ============================================================================
-// Fused transpose of the blur + attenuation, separable PSF.
-//   V   nx rows x kpu: the detector plane, V[i][ZH + k], zero halo columns
-//   Zb  nz rows x wp: k-adjoint of every V row, Zb[k][C + i], zero halo columns
-//   MB  two plane buffers: each receives mubar(:, j, :) by TMA, is overwritten
-//       in place with t = wbar * mubar, and leaves for the slab by a TMA bulk
-//       store; the buffer of plane j+1 is loaded while plane j is computed.
+// Fused transpose of the blur + attenuation, separable PSF: the forward blur's tiles
+// and passes in the same order (the i and k transposes commute), so no detector
+// column is blurred for two tiles.  Per plane of the group:
+//   i-adjoint  U(i,k) = sum_a fx~(a) v(i+a-cx, k), lanes over k, windows along the
+//     rows of V (nz x vp, V[k][ZH + i - i0]), staged once per block as tensor boxes of
+//     the detector plane (zero fill outside);
+//   k-adjoint  wbar(i,k) = sum_b fz~(b) U(i, k+b-cz), lanes over i, 16 k per thread,
+//     times mubar in MB, in place: t.
+// MB is one or two buffers of nkb boxes (16 k x TI columns) that arrive from the
+// attenuation factors and leave for the t slab by TMA, 64-byte swizzled: the 16-byte
+// chunk q of column i sits at q ^ (i / 2 % 4), so the float4 accesses of eight lanes
+// over i are conflict-free.  The first and last detector row and column, where
+// replicate padding folds taps together, take their edge-class taps.
 // ============================================================================
-template <int P, bool TILED>
-__device__ __forceinline__ void adj_sep_body(const Geometry& g, const FusedDims& d, int cls_z,
-                                             const float* __restrict__ vin, const float* __restrict__ mubar,
-                                             const float* __restrict__ fx_adj, const float* __restrict__ fz_adj,
-                                             float* __restrict__ slab, int l0, int* err, const int grp, const int v,
-                                             const int tile)
+struct AdjDims {
+    int TI, nT;        // tile width in columns (multiple of CX), tiles per plane
+    int vp, kpu;       // row pitches of V (pitch4odd(TI + 2ZH) <= 252, a tensor box's width) and U (multiples of 4, /4 odd)
+    int vbox, vrows;   // tensor boxes of V and detector rows per box
+    int varea;         // floats of V, rounded up to 128 bytes
+    int nkb, urows;    // k runs; rows of U: min(TI, nx)
+    int marea, nmb;    // floats of an attenuation buffer (nkb * TI * 16); buffers
+    int J, G, T;       // depth planes per block, depth groups, threads
+};
+
+// Tap record of one PSF plane for the blur adjoint (k_adj_records): FX and FZ of the
+// interior class (PT floats each, zero-padded to P and centred), then the taps of the
+// first and last column and of the first and last row that are not zero (C + 1 each,
+// EC floats): first takes v(0 .. C), last v(n-1-C .. n-1).
+template <int P>
+struct AdjRec {
+    static constexpr int EC = (Sep<P>::C + 4) & ~3;
+    static constexpr int N = 2 * Sep<P>::PT + 4 * EC;
+};
+
+__host__ __device__ inline size_t adj_smem_floats(const AdjDims& d, int rec)
+{
+    // MB x nmb | V | U | tap records of J planes | 3 mbarriers
+    return (size_t)d.nmb * d.marea + (size_t)d.varea + (size_t)d.urows * d.kpu + (size_t)d.J * rec + 8;
+}
+
+// sum_m taps[m] row[s + m], m = 0..N-1 (taps 16-byte aligned): the samples come in as
+// float4 loads from the aligned position s & ~3, the shift s & 3 selects a compile-
+// time offset.  May read up to 3 floats past row[s + N - 1], which are not used.
+template <int N>
+__device__ __forceinline__ float edge_dot(const float* taps, const float* row, int s)
+{
+    float w[4 * ((N + 3 + 3) / 4)], f[(N + 3) & ~3];
+    load_row_f4(row + (s & ~3), w);
+    load_row_f4(taps, f);
+    float acc = 0.f;
+    switch (s & 3) {
+        case 0:
+#pragma unroll
+            for (int m = 0; m < N; ++m) acc = fmaf(f[m], w[m], acc);
+            break;
+        case 1:
+#pragma unroll
+            for (int m = 0; m < N; ++m) acc = fmaf(f[m], w[m + 1], acc);
+            break;
+        case 2:
+#pragma unroll
+            for (int m = 0; m < N; ++m) acc = fmaf(f[m], w[m + 2], acc);
+            break;
+        default:
+#pragma unroll
+            for (int m = 0; m < N; ++m) acc = fmaf(f[m], w[m + 3], acc);
+    }
+    return acc;
+}
+
+// sum_m taps[m] w[m + OFF], m = 0..N-1
+template <int N, int OFF, int WN>
+__device__ __forceinline__ float edge_dot_reg(const float* taps, const float (&w)[WN])
+{
+    static_assert(N - 1 + OFF < WN, "window too short");
+    float f[(N + 3) & ~3], acc = 0.f;
+    load_row_f4(taps, f);
+#pragma unroll
+    for (int m = 0; m < N; ++m) acc = fmaf(f[m], w[m + OFF], acc);
+    return acc;
+}
+
+template <int P>
+__device__ __forceinline__ void adj_sep_body(const Geometry& g, const AdjDims& d, const CUtensorMap* mu_map,
+                                             const CUtensorMap* t_map, const CUtensorMap* v_map,
+                                             const float* __restrict__ rec, int l0, int mu_l0, int* err,
+                                             const int grp, const int v, const int tile)
 {
     using S = Sep<P>;
     constexpr int C = S::C, CX = S::CX, CZ = S::CZ, ZH = S::ZH, WZ = S::WZ, PT = S::PT;
-    extern __shared__ __align__(16) float sm[];
+    constexpr int EC = AdjRec<P>::EC, RN = AdjRec<P>::N;
+    extern __shared__ __align__(1024) float sma[];
     const int nx = g.nx, ny = g.ny, nz = g.nz;
-    float* Zb = sm;
-    float* V = Zb + d.zarea;
-    float* MB = V + (size_t)d.vrows * d.kpu;  // [2][marea]
-    float* TAP = MB + 2 * (size_t)d.marea;    // [J][FX 3 classes | FZ 3 classes] x PT, every plane of the group
-    uint64_t* bar = reinterpret_cast<uint64_t*>(TAP + 6 * PT * (size_t)d.J);
-    const int tid = threadIdx.x;
-    constexpr int T = kFusedThreads;
+    float* MB = sma;                                       // [nmb][nkb][TI][16]
+    float* V = MB + (size_t)d.nmb * d.marea;               // [nz][vp]
+    float* U = V + (size_t)d.varea;                        // [urows][kpu]
+    float* TAP = U + (size_t)d.urows * d.kpu;              // the records of every plane of the group
+    uint64_t* bar = reinterpret_cast<uint64_t*>(TAP + (size_t)d.J * RN);  // buffers, records
+    const int tid = threadIdx.x, T = blockDim.x;
     const int l = l0 + v;
-    // output columns [i0, i0 + ti); their i-adjoint reads detector rows [vlo, vhi)
-    // (untiled: the whole plane, with the constants folded at compile time)
-    const int i0 = TILED ? (int)tile * d.TI : 0;
-    const int ti = TILED ? min(d.TI, nx - i0) : nx;
-    const int vlo = TILED ? max(0, i0 - C) : 0;
-    const int nvr = TILED ? min(nx, i0 + d.TI + C) - vlo : nx;
-    const int nibt = TILED ? (ti + CX - 1) / CX : d.nib;
-    const int zoff = C + vlo - i0;       // Zb column of detector row vlo
-    const int last_col = nx - 1 - i0;    // tile-relative position of column nx-1
-    const bool first_tile = i0 == 0;
-    // attenuation / t tile: columns [i0, i0 + ti) of a plane are one contiguous run
-#define SPECT_MBYTES ((unsigned)(ti * kp) * 4u)
+    const int i0 = tile * d.TI, ti = min(d.TI, nx - i0), nibt = (ti + CX - 1) / CX;
     const int lp = g.nvp == 1 ? 0 : l;
-    const int j_begin = grp * d.J, j_end = min(ny, j_begin + d.J);
-    const int ox = (P - g.px) / 2, oz = (P - g.pz) / 2;
-    const size_t nrow = (size_t)g.nvp * ny;
-    const int pln = nx * nz;
-    const int kp = g.kp;
-    const float* mub = mubar + ((size_t)l * ny) * d.ps + (size_t)i0 * kp;
-    float* tsl = slab + ((size_t)v * ny) * d.ps + (size_t)i0 * kp;
+    const int j_begin = grp * d.J, nj = min(ny - j_begin, d.J);
 
-    // the first plane's attenuation is requested before anything else
+    // swizzled tensor copies want 512-byte aligned shared memory: refuse (error word) rather than fault
+    if ((smem_u32(sma) & 511u) != 0) {
+        if (tid == 0 && err) atomicExch(err, (int)SPECT_ECUDA);
+        return;
+    }
+    auto request = [&](int n) {  // attenuation factors of plane j_begin + n into their buffer
+        const int b = d.nmb == 1 ? 0 : n & 1;
+        float* dst = MB + (size_t)b * d.marea;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar + b)),
+                     "r"((unsigned)d.marea * 4u)
+                     : "memory");
+        for (int q = 0; q < d.nkb; ++q)
+            tma_load_3d(dst + q * d.TI * 16, mu_map, q * 16, i0, (l - mu_l0) * ny + j_begin + n, bar + b);
+    };
     if (tid == 0) {
         mbar_init(bar, 1);
         mbar_init(bar + 1, 1);
+        mbar_init(bar + 2, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        tma_load_1d(MB, mub + (size_t)j_begin * d.ps, SPECT_MBYTES, bar);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar + 2)),
+                     "r"((unsigned)(nj * RN + d.vbox * d.vrows * d.vp) * 4u)
+                     : "memory");
+        tma_copy_1d(TAP, rec + ((size_t)lp * ny + j_begin) * RN, (unsigned)(nj * RN) * 4u, bar + 2);
+        for (int q = 0; q < d.vbox; ++q)
+            tma_load_3d(V + q * d.vrows * d.vp, v_map, i0 - ZH, q * d.vrows, l, bar + 2);
+        request(0);
     }
-    // the detector plane v(:,:,l), transposed, by asynchronous copies issued
-    // next, so their latency overlaps the tap staging and the zeroing below
-    for (int e = tid; e < nz * nvr; e += T) {
-        const int k = e / nvr, r = e - k * nvr;
-        cp_async_4(V + r * d.kpu + ZH + k, vin + (size_t)l * pln + (size_t)k * nx + vlo + r);
+    // zero k-halo columns of U (never written again): [0, ZH) and [ZH + nz, kpu) of each row
+    for (int r = tid; r < d.urows; r += T) {
+        float* ur = U + r * d.kpu;
+#pragma unroll
+        for (int c = 0; c < ZH; c += 4) *reinterpret_cast<float4*>(ur + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+        int c = ZH + nz;
+        for (; c & 3; ++c) ur[c] = 0.f;
+        for (; c < d.kpu; c += 4) *reinterpret_cast<float4*>(ur + c) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    // edge-class taps of every plane of the group (zero-padded to P), also asynchronously
-    for (int e = tid; e < (j_end - j_begin) * 3 * PT; e += T) {
-        const int jj = e / (3 * PT), r3 = e - jj * 3 * PT, c = r3 / PT, a = r3 - c * PT, j = j_begin + jj;
-        const int ax = a - ox, az = a - oz;
-        const bool okx = ax >= 0 && ax < g.px, okz = c < cls_z && az >= 0 && az < g.pz;
-        float* F = TAP + jj * 6 * PT;
-        cp_async_4_or_zero(F + r3, okx ? fx_adj + ((size_t)c * nrow + (size_t)lp * ny + j) * g.px + ax : fx_adj, okx);
-        cp_async_4_or_zero(F + 3 * PT + r3, okz ? fz_adj + ((size_t)c * nrow + (size_t)lp * ny + j) * g.pz + az : fz_adj,
-                           okz);
-    }
-
-    // zero V outside the detector (the halo columns of the staged rows, and
-    // whole rows beyond them) and Zb; then wait for the staged plane and taps
-    const int halo = d.kpu - nz;  // zero columns of a staged row: [0, ZH) and [ZH + nz, kpu)
-    for (int e = tid; e < nvr * halo; e += T) {
-        const int r = e / halo, c = e - r * halo;
-        V[r * d.kpu + (c < ZH ? c : c + nz)] = 0.f;
-    }
-    for (int e = nvr * d.kpu + tid; e < d.vrows * d.kpu; e += T) V[e] = 0.f;
-    for (int e = tid; e < d.zarea; e += T) Zb[e] = 0.f;
-    cp_async_wait_all();
-    __syncthreads();
+    __syncthreads();  // the barriers are initialised and U's halos are zero
+    bool ok = mbar_wait_bounded(bar + 2, 0u);
 
     // the thread's first work item of each pass and the step to its next one
     // (the same for every plane: the divisions stay out of the plane loop)
-    const int ka_kb = tid / nvr, ka_r = tid - ka_kb * nvr;  // k-adjoint: (k run, detector row)
-    const int ka_dkb = T / nvr, ka_dr = T - ka_dkb * nvr;
     const int ia_ib = tid / nz, ia_k = tid - ia_ib * nz;    // i-adjoint: (column run, k)
+    const int ka_kb = tid / ti, ka_i = tid - ka_kb * ti;    // k-adjoint: (k run, column)
     const int ia_dib = T / nz, ia_dk = T - ia_dib * nz;
-    unsigned phases = 0u;  // bit b: parity of buffer b's barrier
-    for (int j = j_begin; j < j_end; ++j) {
-        const int n = j - j_begin, b = n & 1;
-        const float* FX = TAP + n * 6 * PT;
-        const float* FZ = FX + 3 * PT;
-        // k-adjoint: Zb[k][C+i] = sum_b' fz~(b') v(i, k+b'-cz), lanes over i.
-        // The first and last detector rows, where replicate padding folds
-        // taps together, take their edge-class taps instead of the interior ones.
-        int kb = ka_kb, r = ka_r;  // detector row vlo + r
-        for (int it = tid; it < nvr * d.nkb; it += T, kb += ka_dkb, r += ka_dr) {
-            if (r >= nvr) r -= nvr, ++kb;
-            const float* vr = V + r * d.kpu;
-            float win[WZ];
-            load_window_f4<P>(vr + kb * CZ, win);
-            float o[CZ];
-            fir<P, CZ, 1, ZH - C>(FZ, win, o);
-            const int k0 = kb * CZ;
-            if (nz > 1 && k0 == 0) {  // row k = 0
-                const float* f = FZ + PT;
-                float sacc = 0.f;
+    const int ka_dkb = T / ti, ka_di = T - ka_dkb * ti;
+    const int last_col = nx - 1 - i0;  // tile-relative position of column nx-1
+    for (int n = 0; n < nj; ++n) {
+        const int b = d.nmb == 1 ? 0 : n & 1;
+        const float* FX = TAP + n * RN;
+        const float* FZ = FX + PT;
+        const float* FE = FZ + PT;  // edge taps: first column, last column, first row, last row
+        if (ok) {
+            int ib = ia_ib, k = ia_k;
+            for (int it = tid; it < nz * nibt; it += T) {
+                const int li = ib * CX;  // first column of this run, relative to the tile
+                const float* vr = V + k * d.vp;
+                float win[WZ];
+                load_window_f4<P>(vr + li, win);
+                float o[CX];
+                fir<P, CX, 1, ZH - C>(FX, win, o);
+                if (i0 + li == 0) o[0] = edge_dot_reg<C + 1, ZH>(FE, win);
+                const int cl = last_col - li;  // position of column nx-1 in this run
+                float* ur = U + li * d.kpu + ZH + k;
+                if (cl >= CX) {
 #pragma unroll
-                for (int bb = 0; bb < P; ++bb) sacc = fmaf(f[bb], win[bb - C + ZH], sacc);
-                o[0] = sacc;
-            }
-            const int cl = nz - 1 - k0;  // position of row k = nz-1 in this block
-            const bool last = nz > 1 && cl < CZ;
-            const float e_last = last ? edge_tap_dot<P>(FZ + 2 * PT, vr, (nz - 1) - C + ZH) : 0.f;
-            float* zc = Zb + zoff + r;
-            if (k0 + CZ <= nz && !last) {
+                    for (int c = 0; c < CX; ++c) ur[c * d.kpu] = o[c];
+                } else {
+                    const float e_last = edge_dot<C + 1>(FE + EC, vr, li + cl + ZH - C);
 #pragma unroll
-                for (int c = 0; c < CZ; ++c) zc[(k0 + c) * d.wz] = o[c];
-            } else {
-#pragma unroll
-                for (int c = 0; c < CZ; ++c)
-                    if (k0 + c < nz) zc[(k0 + c) * d.wz] = (last && c == cl) ? e_last : o[c];
+                    for (int c = 0; c < CX; ++c)
+                        if (c <= cl) ur[c * d.kpu] = c == cl ? e_last : o[c];
+                }
+                ib += ia_dib;  // next item: it + T
+                k += ia_dk;
+                if (k >= nz) k -= nz, ++ib;
             }
         }
         __syncthreads();
-        // the other buffer: the previous plane's bulk store has had the whole
-        // k-adjoint to read it; it now receives the next plane's attenuation
-        if (tid == 0 && j + 1 < j_end) {
+        // the other buffer: the previous plane's store has had the whole i-adjoint to
+        // read it; it now receives the next plane's attenuation
+        if (d.nmb == 2 && tid == 0 && n + 1 < nj) {
             tma_store_wait_read<0>();
-            tma_load_1d(MB + (b ^ 1) * (size_t)d.marea, mub + (size_t)(j + 1) * d.ps, SPECT_MBYTES, bar + (b ^ 1));
+            request(n + 1);
         }
-
-        // i-adjoint times mubar, in place in MB[b]; lanes over k
-        float* mb = MB + b * (size_t)d.marea;
-        const bool ok = mbar_wait_bounded(bar + b, (phases >> b) & 1u);
-        phases ^= 1u << b;
+        float* mb = MB + (size_t)b * d.marea;
+        ok = mbar_wait_bounded(bar + b, (unsigned)(d.nmb == 1 ? n : n >> 1) & 1u) && ok;
         if (ok) {
-            int ib = ia_ib, k = ia_k;
-            for (int it = tid; it < nz * nibt; it += T, ib += ia_dib, k += ia_dk) {
-                if (k >= nz) k -= nz, ++ib;
-                const int li = ib * CX;  // first column of this run, relative to the tile
-                const float* zr = Zb + k * d.wz + li;
-                float win[4 * ((CX + P - 1 + 3) / 4)];
-                load_row_f4(zr, win);
-                float o[CX];
-                fir<P, CX, 1, 0>(FX, win, o);
-                // first / last detector column: edge-class taps (replicate-padding folds)
-                if (first_tile && li == 0) {
-                    const float* f = FX + PT;
-                    float sacc = 0.f;
+            int kb = ka_kb, i = ka_i;  // i relative to the tile
+            for (int it = tid; it < ti * d.nkb; it += T) {
+                const float* ur = U + i * d.kpu;
+                const int k0 = kb * CZ;
+                float win[WZ];
+                load_window_f4<P>(ur + k0, win);
+                float o[CZ];
+                fir<P, CZ, 1, ZH - C>(FZ, win, o);
+                if (nz > 1 && k0 == 0) o[0] = edge_dot_reg<C + 1, ZH>(FE + 2 * EC, win);
+                const int cl = nz - 1 - k0;  // position of row nz-1 in this run
+                if (nz > 1 && cl < CZ) {
+                    const float e_last = edge_dot<C + 1>(FE + 3 * EC, ur, ZH + nz - 1 - C);
 #pragma unroll
-                    for (int a = 0; a < P; ++a) sacc = fmaf(f[a], win[a], sacc);
-                    o[0] = sacc;
+                    for (int c = 0; c < CZ; ++c)
+                        if (c == cl) o[c] = e_last;
                 }
-                const int cl = last_col - li;  // position of column nx-1 in this run
-                const bool last = cl < CX;
-                const float e_last = last ? edge_tap_dot<P>(FX + 2 * PT, zr - li, li + cl) : 0.f;
-                float* mp = mb + li * kp + k;
-                if (!last) {
+                float4* m4 = reinterpret_cast<float4*>(mb + ((size_t)kb * d.TI + i) * 16);
+                const int sw = (i >> 1) & 3;
 #pragma unroll
-                    for (int c = 0; c < CX; ++c) mp[c * kp] = o[c] * mp[c * kp];
-                } else {
-#pragma unroll
-                    for (int c = 0; c < CX; ++c)
-                        if (c <= cl) mp[c * kp] = (c == cl ? e_last : o[c]) * mp[c * kp];
+                for (int q = 0; q < 4; ++q) {
+                    float4 m = m4[q ^ sw];
+                    m.x *= o[4 * q];
+                    m.y *= o[4 * q + 1];
+                    m.z *= o[4 * q + 2];
+                    m.w *= o[4 * q + 3];
+                    m4[q ^ sw] = m;
                 }
+                kb += ka_dkb;  // next item: it + T
+                i += ka_di;
+                if (i >= ti) i -= ti, ++kb;
             }
         }
         if (__syncthreads_or(!ok)) {
-            if (tid == 0) {
+            if (tid == 0) {  // a last chance for the copies in flight
                 flag_timeout(err);
-                mbar_wait_bounded(bar + b, ((phases >> b) & 1u) ^ 1u);
+                mbar_wait_bounded(bar + 2, 0u);
+                for (int m = n; m < n + d.nmb && m < nj; ++m)
+                    mbar_wait_bounded(bar + (d.nmb == 1 ? 0 : m & 1), (unsigned)(d.nmb == 1 ? m : m >> 1) & 1u);
                 tma_store_wait_all();
             }
             return;
         }
-        // t plane -> slab[v][j]
+        // t tile -> slab[v][j]
         if (tid == 0) {
             fence_proxy_async_smem();
-            tma_store_1d(tsl + (size_t)j * d.ps, mb, SPECT_MBYTES);
+            for (int q = 0; q < d.nkb; ++q)
+                tma_store_3d(t_map, q * 16, i0, v * ny + j_begin + n, mb + q * d.TI * 16);
+            tma_store_commit();
+            if (d.nmb == 1 && n + 1 < nj) {  // the one buffer: the next plane's factors once the store has read it
+                tma_store_wait_read<0>();
+                request(n + 1);
+            }
         }
     }
     if (tid == 0) tma_store_wait_read<0>();  // the writes complete with the grid
-#undef SPECT_MBYTES
 }
+
+cudaError_t encode_v_map(const Geometry& g, const AdjDims& d, const float* v, CUtensorMap* map);
 
 // ---------------------------------------------------------------- host-side dimensioning
 namespace {
@@ -777,8 +794,6 @@ FusedDims dims_for(const Geometry& g, int J, int tiles)
     d.marea = d.urows * g.kp;
     d.wp = pitch4odd(d.TI + 2 * S::C);
     d.warea = (g.nz * d.wp + 3) & ~3;
-    d.wz = pitch4odd(d.TI + 2 * S::C);
-    d.zarea = g.nz * d.wz;
     d.farea = (g.nz * pitch4odd(d.nib * S::CX + 2 * S::C) + 3) & ~3;
     int kpu = d.nkb * S::CZ + 2 * S::ZH;
     kpu = (kpu + 3) & ~3;
@@ -852,18 +867,62 @@ size_t smem_fwd(const FwdDims& d)
     return fwd_smem_floats(d, Sep<P>::PT) * sizeof(float);
 }
 
+// Launch shape of the blur adjoint for `tiles` column tiles (more where a tile would not
+// fit) and J planes per block; threads as the forward blur.  Two attenuation
+// buffers unless one lets more blocks run on an SM.
 template <int P>
-size_t smem_adj(const Geometry& g, const FusedDims& d)
+struct AdjBlock {
+    static constexpr int T = FwdBlock<P>::T, B = FwdBlock<P>::B, regs = FwdBlock<P>::regs;
+};
+
+template <int P>
+AdjDims adj_dims(const Geometry& g, int J, int tiles, size_t smem_limit)
 {
-    (void)g;
-    return adj_smem_floats(d, Sep<P>::PT) * sizeof(float);
+    using S = Sep<P>;
+    constexpr int kT = AdjBlock<P>::T, RN = AdjRec<P>::N;
+    AdjDims d;
+    const int nib = (g.nx + S::CX - 1) / S::CX;
+    d.nkb = (g.nz + S::CZ - 1) / S::CZ;
+    tiles = tiles < 1 ? 1 : (tiles > nib ? nib : tiles);
+    d.TI = ((nib + tiles - 1) / tiles) * S::CX;
+    while (pitch4odd(d.TI + 2 * S::ZH) > 252) d.TI -= S::CX;
+    d.J = J;
+    d.G = (g.ny + J - 1) / J;
+    d.kpu = pitch4odd(d.nkb * S::CZ + 2 * S::ZH);
+    for (;; d.TI -= S::CX) {
+        d.nT = (g.nx + d.TI - 1) / d.TI;
+        d.vp = pitch4odd(d.TI + 2 * S::ZH);
+        // boxes of at most 256 rows; more than one start on 128 bytes (vp is 4 * odd: 8 rows are a multiple)
+        d.vbox = (g.nz + 255) / 256;
+        d.vrows = d.vbox == 1 ? g.nz : ((g.nz + d.vbox - 1) / d.vbox + 7) & ~7;
+        d.varea = (d.vbox * d.vrows * d.vp + 31) & ~31;
+        d.urows = d.TI < g.nx ? d.TI : g.nx;
+        d.marea = d.nkb * d.TI * 16;
+        const int kitems = d.urows * d.nkb, iitems = g.nz * ((d.urows + S::CX - 1) / S::CX);
+        const int want = kitems > iitems ? kitems : iitems;
+        d.T = want <= kT ? (want + 31) & ~31 : kT;
+        d.nmb = 2;
+        const size_t two = adj_smem_floats(d, RN) * sizeof(float);
+        d.nmb = 1;
+        const size_t one = adj_smem_floats(d, RN) * sizeof(float);
+        const int b1 = blocks_per_sm(one, d.T, AdjBlock<P>::regs), b2 = blocks_per_sm(two, d.T, AdjBlock<P>::regs);
+        if (two <= smem_limit && b2 >= 1 && (b1 <= b2 || b2 * d.T >= 768)) d.nmb = 2;
+        if (one <= smem_limit || d.TI == S::CX) return d;
+    }
 }
 
-// The same for the blur adjoint, its attenuation planes counted without their k padding.
+template <int P>
+size_t smem_adj(const AdjDims& d)
+{
+    return adj_smem_floats(d, AdjRec<P>::N) * sizeof(float);
+}
+
+// Part of the bound of the shapes taken: Zb, V, two attenuation tiles and the edge-class taps.
 template <int P>
 size_t smem_adj_bound(const Geometry& g, const FusedDims& d)
 {
-    return smem_adj<P>(g, d) - 2 * ((size_t)d.marea - (((size_t)d.urows * g.nz + 3) & ~(size_t)3)) * sizeof(float);
+    return ((size_t)g.nz * d.wp + (size_t)d.vrows * d.kpu + 2 * (((size_t)d.urows * g.nz + 3) & ~(size_t)3) +
+            6 * (size_t)Sep<P>::PT * d.J + 8) * sizeof(float);
 }
 
 // The geometries and shapes that the fused kernels take: two tile buffers, U,

@@ -25,7 +25,7 @@ namespace {
 struct GroupPlan {
     Geometry g;
     RotDims dr;        // rotation launch shape
-    FusedDims da;      // adjoint launch shape
+    AdjDims da;        // adjoint launch shape
     FwdDims df;        // forward launch shape
     int cls_z;
     const float* rtab;
@@ -34,8 +34,7 @@ struct GroupPlan {
     float* slab;
     const float* frec;
     float* part;
-    const float* fx_adj;
-    const float* fz_adj;
+    const float* arec;
     float* ratio;
     const float* y;
     const float* rbar;
@@ -44,7 +43,8 @@ struct GroupPlan {
 };
 struct GroupPlans {
     GroupPlan p[kGroupMax];
-    CUtensorMap fmap[kGroupMax];  // the slabs' plane images (forward blur)
+    CUtensorMap fmap[kGroupMax];                  // the slabs' plane images (forward blur)
+    CUtensorMap mmap[kGroupMax], tmap[kGroupMax], vmap[kGroupMax];  // factors, t planes, ratios (blur adjoint)
     GroupGrid grid;
 };
 
@@ -74,13 +74,14 @@ __global__ void __launch_bounds__(FwdBlock<P>::T, FwdBlock<P>::B) k_fwd_sep_grp(
     fwd_sep_body<P, RACC>(q.g, q.df, &gp.fmap[w.x], q.frec, q.part, 0, q.err, grp, w.z, w.y - grp * q.df.nT);
 }
 
-template <int P, bool TILED>
-__global__ void __launch_bounds__(kFusedThreads, 1) k_adj_sep_grp(const __grid_constant__ GroupPlans gp)
+template <int P>
+__global__ void __launch_bounds__(AdjBlock<P>::T, AdjBlock<P>::B) k_adj_sep_grp(const __grid_constant__ GroupPlans gp)
 {
     const int4 w = group_item(gp.grid);
     const GroupPlan q = gp.p[w.x];  // by value: the fields live in registers, not re-read from parameter space
-    adj_sep_body<P, TILED>(q.g, q.da, q.cls_z, q.ratio, q.mubar, q.fx_adj, q.fz_adj, q.slab, 0, q.err, w.y, w.z,
-                           w.w);
+    const int grp = w.y / q.da.nT;
+    adj_sep_body<P>(q.g, q.da, &gp.mmap[w.x], &gp.tmap[w.x], &gp.vmap[w.x], q.arec, 0, 0, q.err, grp, w.z,
+                    w.y - grp * q.da.nT);
 }
 
 // v = sum over depth groups (fixed order), then the EM ratio y / (v + rbar): k_fwd_reduce per plan
@@ -94,7 +95,8 @@ __global__ void __launch_bounds__(kReduceThreads) k_fwd_reduce_grp(const __grid_
     float s = 0.f;
     for (int gq = 0; gq < q.df.G; ++gq) s += q.part[(size_t)gq * q.nproj + o];
     const float yb = s + (q.rbar ? q.rbar[o] : 0.f);
-    q.ratio[o] = yb > 0.f ? q.y[o] / yb : 0.f;
+    const int nx = q.g.nx, np = q.g.np;
+    q.ratio[np == nx ? o : o + o / nx * (np - nx)] = yb > 0.f ? q.y[o] / yb : 0.f;
 }
 
 __global__ void k_transpose_grp(const __grid_constant__ GroupTs gt)
@@ -125,14 +127,13 @@ void fill_plan(GroupPlan& q, const spect_plan_s* Pl, const float* y, const float
 {
     q.g = Pl->g;
     q.df = fwd_dims<P>(Pl->g, Pl->fused_J, Pl->fwd_nT, (size_t)Pl->smem_optin);
-    q.da = dims_for<P>(Pl->g, Pl->adj_J, Pl->adj_nT);
+    q.da = adj_dims<P>(Pl->g, Pl->adj_J, Pl->adj_nT, (size_t)Pl->smem_optin);
     q.cls_z = Pl->cls_z;
     q.mubar = Pl->mubar;
     q.slab = Pl->slab;
     q.frec = Pl->frec;
     q.part = Pl->part;
-    q.fx_adj = Pl->fx_adj;
-    q.fz_adj = Pl->fz_adj;
+    q.arec = Pl->arec;
     q.ratio = Pl->ratio;
     q.y = y;
     q.rbar = rbar;
@@ -170,21 +171,19 @@ cudaError_t stage_launches(int stage, const std::vector<int>& idx, const std::ve
                            const float* const* y, const float* const* rbar, GroupedBatch& /*B*/,
                            std::vector<GroupLaunch>& out)
 {
-    // sub-groups by kernel variant: sums in registers (blur), tiled (adjoint)
+    // sub-groups by kernel variant: the forward blur's sums in registers or not
     std::vector<int> var[2];
     for (int i : idx) {
         bool flag = false;
         if (stage == 1)
             flag = fwd_dims<P>(plans[i]->g, plans[i]->fused_J, plans[i]->fwd_nT, (size_t)plans[i]->smem_optin).racc;
-        else
-            flag = dims_for<P>(plans[i]->g, plans[i]->adj_J, plans[i]->adj_nT).nT > 1;
         var[flag ? 1 : 0].push_back(i);
     }
     for (int f = 0; f < 2; ++f) {
         for (const std::vector<int>& ch : chunks_of(var[f], plans)) {
             GroupPlans gp{};
             size_t smem = 0;
-            int thr = 0;  // the forward blur's block: the largest of its plans'
+            int thr = 0;  // threads per block: the largest of the plans'
             for (int m = 0; m < (int)ch.size(); ++m) {
                 const spect_plan_s* Pl = plans[ch[m]];
                 fill_plan<P>(gp.p[m], Pl, y[ch[m]], rbar ? rbar[ch[m]] : nullptr);
@@ -194,9 +193,14 @@ cudaError_t stage_launches(int stage, const std::vector<int>& idx, const std::ve
                     thr = std::max(thr, q.df.T);
                     gp.fmap[m] = Pl->fmap;
                     add_grid(gp.grid, m, q.df.G * q.df.nT, q.g.nview, 1);
-                } else {           // the adjoint's grid: (depth group, view, column tile)
-                    smem = std::max(smem, smem_adj<P>(q.g, q.da));
-                    add_grid(gp.grid, m, q.da.G, q.g.nview, q.da.nT);
+                } else {           // the adjoint's grid: (depth group and column tile, view)
+                    smem = std::max(smem, smem_adj<P>(q.da));
+                    thr = std::max(thr, q.da.T);
+                    gp.mmap[m] = Pl->amap_mu;
+                    gp.tmap[m] = Pl->amap_t;
+                    const cudaError_t e = encode_v_map(Pl->g, q.da, Pl->ratio, &gp.vmap[m]);
+                    if (e != cudaSuccess) return e;
+                    add_grid(gp.grid, m, q.da.G * q.da.nT, q.g.nview, 1);
                 }
             }
             if (ch.empty()) continue;
@@ -204,8 +208,7 @@ cudaError_t stage_launches(int stage, const std::vector<int>& idx, const std::ve
                 out.push_back(f ? make_launch(k_fwd_sep_grp<P, true>, gp, dim3(thr), smem)
                                 : make_launch(k_fwd_sep_grp<P, false>, gp, dim3(thr), smem));
             else
-                out.push_back(f ? make_launch(k_adj_sep_grp<P, true>, gp, dim3(kFusedThreads), smem)
-                                : make_launch(k_adj_sep_grp<P, false>, gp, dim3(kFusedThreads), smem));
+                out.push_back(make_launch(k_adj_sep_grp<P>, gp, dim3(thr), smem));
         }
     }
     return cudaSuccess;

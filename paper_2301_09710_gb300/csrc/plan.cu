@@ -134,7 +134,7 @@ void free_plan(spect_plan_s* P, cudaStream_t st)
     }
     for (cudaEvent_t e : P->evpool) cudaEventDestroy(e);
     void* ptrs[] = {P->mu, P->psf, P->psf_adj, P->fx, P->fz, P->fx_adj, P->fz_adj, P->rot, P->adj_off, P->adj,
-                    P->frec, P->slab, P->e, P->ratio, P->s, P->mubar, P->xt, P->et, P->st, P->part, P->adjf, P->err, P->rtab, P->ut,
+                    P->frec, P->arec, P->slab, P->e, P->ratio, P->s, P->mubar, P->xt, P->et, P->st, P->part, P->adjf, P->err, P->rtab, P->ut,
                     P->gboxes, P->gent, P->rboxes, P->r3_tab, P->mut};
     for (void* p : ptrs) raw_free(P, p, st);
     delete P;
@@ -287,7 +287,7 @@ spect_status from_internal(spect_plan_s* P, const float* xt, float* x, cudaStrea
     return SPECT_OK;
 }
 
-// v = A x_t (x_t internal layout); with y set, v receives the EM ratio y / (A x + rbar)
+// v = A x_t (x_t internal layout); with y set, v receives the EM ratio y / (A x + rbar) in rows of np
 spect_status fast_forward(spect_plan_s* P, const float* xt, float* v, const float* y, const float* rbar,
                           cudaStream_t st)
 {
@@ -309,7 +309,7 @@ spect_status fast_forward(spect_plan_s* P, const float* xt, float* v, const floa
     return SPECT_OK;
 }
 
-// out_t = A' v (internal layout); with em.x set the last chunk applies the EM update instead
+// out_t = A' v (v: rows of np; out_t: internal layout); with em.x set the last chunk applies the EM update instead
 spect_status fast_back(spect_plan_s* P, const float* v, float* out_t, spect::EmArgs em, cudaStream_t st)
 {
     const int nview = P->g.nview;
@@ -336,8 +336,8 @@ spect_status fast_back(spect_plan_s* P, const float* v, float* out_t, spect::EmA
 spect_status ensure_sensitivity(spect_plan_s* P, cudaStream_t st)
 {
     if (P->s_valid) return SPECT_OK;
-    const size_t nproj = (size_t)P->g.nx * P->g.nz * P->g.nview;
-    SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_fill(P->ratio, nproj, 1.f, st); }),
+    const size_t nratio = (size_t)(P->fast ? P->g.np : P->g.nx) * P->g.nz * P->g.nview;
+    SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_fill(P->ratio, nratio, 1.f, st); }),
                    "fill launch");
     spect_status r = P->fast ? fast_back(P, P->ratio, P->st, spect::EmArgs(), st)
                              : run_back(P, P->ratio, P->s, spect::EmArgs(), st);
@@ -401,8 +401,8 @@ size_t plan_bytes_bound(const spect_plan_s& P)
     const size_t budget = P.recompute ? recompute_budget_bytes() : slab_budget_bytes(P.fast);
     const size_t chunk = view_chunk(P, per_view, budget);
     b += per_view * chunk * F;
-    b += (vol + nproj) * F;
-    if (P.fast) b += spect::fwd_records_floats(P) * F;
+    b += (vol + (P.fast ? (size_t)g.np * g.nz * g.nview : nproj)) * F;
+    if (P.fast) b += (spect::fwd_records_floats(P) + spect::adj_records_floats(P)) * F;
     if (P.fast) {
         // attenuation factors of every view, or of one chunk plus mu in the internal layout
         b += P.recompute ? ((size_t)g.ny * P.ps * chunk + volt) * F : (size_t)g.ny * P.ps * g.nview * F;
@@ -441,6 +441,7 @@ spect_status spect_plan_bytes(int nx, int ny, int nz, int nview, int px, int pz,
     g.px = px; g.pz = pz; g.nvp = nview_psf;
     P.separable = separable != 0;
     g.kp = (nz + 3) & ~3;
+    g.np = (nx + 3) & ~3;
     P.ps = nx * g.kp;
     P.ts = (5 * nx + 3) & ~3;
     P.cls_x = 3;
@@ -461,7 +462,7 @@ spect_status spect_plan_bytes(int nx, int ny, int nz, int nview, int px, int pz,
             cudaGetLastError();
             return fail(SPECT_ECUDA, "device query failed");
         }
-        spect::default_fwd_shape(P);
+        spect::default_shape(P);
     }
     *bytes = plan_bytes_bound(P);
     return SPECT_OK;
@@ -507,6 +508,7 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
     g.has_mu = mu != nullptr;
     P->separable = psf_fx && (!psf || (flags & SPECT_PLAN_PREFER_SEPARABLE));
     g.kp = (nz + 3) & ~3;
+    g.np = (nx + 3) & ~3;
     P->ps = nx * g.kp;
     P->ts = (5 * nx + 3) & ~3;
     P->cls_x = 3;
@@ -551,8 +553,7 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         P->fwd_nT = P->adj_nT = 1;
     }
     PLAN_TRY(cudaDeviceGetAttribute(&P->sms, cudaDevAttrMultiProcessorCount, dev), "device query");
-    if (P->fast) spect::default_fwd_shape(*P);
-    if (P->fast && P->separable) P->adj_nT = spect::adj_tiles(*P);
+    if (P->fast) spect::default_shape(*P);
     P->rot3 = (flags & SPECT_PLAN_ROTATION_3PASS) != 0;
     if (P->rot3 && !P->fast) {
         free_plan(P);
@@ -666,15 +667,17 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         PLAN_TRY(cudaStreamSynchronize(st), "adjacency fill");
     }
 
-    // the forward blur's tap records; the factors (or the stack) themselves are not read again
+    // the blur kernels' tap records; the factors (or the stack) themselves are not read again
     if (P->fast) {
         PLAN_ALLOC(P->frec, spect::fwd_records_floats(*P), "tap records");
-        PLAN_TRY(spect::launch_fwd_records(*P, st), "tap record launch");
-        for (float** p : {&P->fx, &P->fz, &P->psf}) {
+        PLAN_ALLOC(P->arec, spect::adj_records_floats(*P), "adjoint tap records");
+        PLAN_TRY(spect::launch_records(*P, st), "tap record launch");
+        for (float** p : {&P->fx, &P->fz, &P->psf, &P->fx_adj, &P->fz_adj}) {
             raw_free(P, *p, st);
             *p = nullptr;
         }
-        P->bytes -= (P->separable ? (size_t)(px + pz) : (size_t)px * pz) * nrows * sizeof(float);
+        P->bytes -= (P->separable ? (size_t)px * 4 + (size_t)pz * (1 + P->cls_z) : (size_t)px * pz) * nrows *
+                    sizeof(float);
     }
 
     // work slab and EM buffers
@@ -684,12 +687,10 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
     P->chunk = view_chunk(*P, per_view, budget);
     PLAN_ALLOC(P->slab, per_view * (size_t)P->chunk, "work slab");
     P->slab_cap = per_view * (size_t)P->chunk;
-    if (P->fast) PLAN_TRY(spect::build_fwd_map(*P), "tensor map of the plane images");
     // fused adjoint: all views of the slab in one pass by default (measured
     // faster than L2-sized passes); SPECT_ADJ_CHUNK sets fewer views per pass,
     // with a depth-group size that keeps about two blocks per SM (tuning)
     P->adj_chunk = P->chunk;
-    P->adj_J = 8;
     if (const char* env = getenv("SPECT_ADJ_CHUNK")) {
         if (atoi(env) > 0) {
             P->adj_chunk_req = atoi(env);
@@ -699,7 +700,7 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         }
     }
     if (!P->fast) PLAN_ALLOC(P->e, vol, "EM accumulator");
-    PLAN_ALLOC(P->ratio, nproj, "EM ratio");
+    PLAN_ALLOC(P->ratio, P->fast ? (size_t)g.np * nz * nview : nproj, "EM ratio");
     PLAN_ALLOC(P->s, vol, "sensitivity");
 
     // fused path: attenuation cache for every view (or for one view chunk,
@@ -708,6 +709,7 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         const int mu_views = P->recompute ? P->chunk : nview;
         PLAN_ALLOC(P->mubar, (size_t)ny * P->ps * mu_views, "attenuation cache");
         P->mubar_cap = (size_t)ny * P->ps * mu_views;
+        PLAN_TRY(spect::build_maps(*P), "tensor maps of the blur kernels");
         PLAN_ALLOC(P->xt, volt, "internal image");
         PLAN_ALLOC(P->et, volt, "internal back-projection");
         PLAN_ALLOC(P->st, volt, "internal sensitivity");
@@ -800,6 +802,11 @@ spect_status spect_back(spect_plan P, const float* v, float* x, spect_stream str
     if (r != SPECT_OK) return r;
     cudaStream_t st = (cudaStream_t)stream;
     if (P->fast) {
+        if (P->g.np != P->g.nx) {  // rows of whole 16-byte units
+            SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_pad_rows(*P, v, P->ratio, st); }),
+                           "row padding launch");
+            v = P->ratio;
+        }
         r = fast_back(P, v, P->et, spect::EmArgs(), st);
         if (r != SPECT_OK) return r;
         return from_internal(P, P->et, x, st);
@@ -1027,10 +1034,10 @@ spect_status realloc_floats(spect_plan_s* P, float** p, size_t* cap, size_t need
     return SPECT_OK;
 }
 
-// The forward blur's tensor map for the plan's present slab, chunk and launch shape.
+// The blur kernels' tensor maps for the plan's present buffers, chunk and launch shapes.
 spect_status refresh_maps(spect_plan_s* P)
 {
-    SPECT_CUDA_TRY(spect::build_fwd_map(*P), "tensor map of the plane images");
+    SPECT_CUDA_TRY(spect::build_maps(*P), "tensor maps of the blur kernels");
     return SPECT_OK;
 }
 
@@ -1174,9 +1181,9 @@ spect_status spect_plan_autotune(spect_plan P, spect_stream stream)
         }
     }
     // inputs of the timed calls: the plan's own scratch (x_t = 1, v = 1)
-    const size_t volt = (size_t)g.nx * g.ny * g.kp, nproj = (size_t)g.nx * g.nz * g.nview;
+    const size_t volt = (size_t)g.nx * g.ny * g.kp;
     if (spect::launch_fill(P->xt, volt, 1.f, st) != cudaSuccess ||
-        spect::launch_fill(P->ratio, nproj, 1.f, st) != cudaSuccess)
+        spect::launch_fill(P->ratio, (size_t)g.np * g.nz * g.nview, 1.f, st) != cudaSuccess)
         return fail(SPECT_ECUDA, "fill launch failed");
     const int prof = P->prof;
     P->prof = 0;

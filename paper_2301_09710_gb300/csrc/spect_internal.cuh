@@ -41,6 +41,7 @@ struct Geometry {
     float cfrac;      // (nx-1)/2 - cint  (0 or 0.5)
     float dy;
     int has_mu;
+    int np;           // row pitch of internal projections (the EM ratio): nx rounded up to 4
     int kp;           // k pitch of the internal [j][i][k] volumes and [i][k] planes: nz rounded up to 4
 };
 
@@ -64,7 +65,8 @@ struct spect_plan_s {
     float* psf_adj = nullptr;    // direct: nvar * px*pz*ny*nvp edge-class variants for A'
     float* fx = nullptr;         // separable: px*ny*nvp
     float* fz = nullptr;         // separable: pz*ny*nvp
-    float* frec = nullptr;       // fused separable: tap records of the forward blur (then fx, fz are not kept)
+    float* frec = nullptr;       // fused: tap records of the forward blur (then fx, fz, psf are not kept)
+    float* arec = nullptr;       // fused: tap records of the blur adjoint (then the edge-class variants are not kept)
     float* fx_adj = nullptr;     // separable: cls_x * px*ny*nvp
     float* fz_adj = nullptr;     // separable: cls_z * pz*ny*nvp
     spect::ViewRot* rot = nullptr;  // nview
@@ -74,7 +76,7 @@ struct spect_plan_s {
     size_t slab_cap = 0;         // floats allocated for slab
     size_t part_cap = 0;         // floats allocated for part
     float* e = nullptr;          // nx*ny*nz  (EM back-projection accumulator)
-    float* ratio = nullptr;      // nx*nz*nview (EM ratio / ones)
+    float* ratio = nullptr;      // nx*nz*nview (EM ratio / ones); fused plans: rows of np
     float* s = nullptr;          // nx*ny*nz  (sensitivity A'1)
     int s_valid = 0;
     int cls_x = 3, cls_z = 3;    // edge classes per axis for A' (1 when the axis has length 1)
@@ -89,7 +91,8 @@ struct spect_plan_s {
     int fused_J = 8;             // depth planes per fused forward block
     int fwd_nT = 1;              // column tiles per plane of the fused forward blur
     int adj_nT = 1;              // column tiles per plane of the fused blur adjoint
-    CUtensorMap fmap;            // the slab's plane images, boxed as the forward blur's tiles (build_fwd_map)
+    CUtensorMap fmap;            // the slab's plane images, boxed as the forward blur's tiles (build_maps)
+    CUtensorMap amap_mu, amap_t; // attenuation factors / t planes, boxed as the blur adjoint's tiles (build_maps)
     int adj_J = 8;               // depth planes per fused adjoint block
     int adj_chunk = 0;           // views per adjoint pass (t slab sized to stay in L2)
     int adj_chunk_req = 0;       // views per adjoint pass asked for (SPECT_ADJ_CHUNK), 0: all
@@ -403,6 +406,18 @@ __device__ __forceinline__ void tma_load_3d(void* dst_smem, const CUtensorMap* m
         : "memory");
 }
 
+// Tiled 3D tensor store (TMA) of the box at (c0, c1, c2) of `map` from shared memory, in
+// the calling thread's current bulk group (parts outside the tensor are not written).
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, int c0, int c1, int c2, const void* src_smem)
+{
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(src_smem))
+                 : "memory");
+}
+
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+
 // Host: cuTensorMapEncodeTiled through the runtime's driver entry point (NULL when unavailable).
 using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -430,13 +445,14 @@ int choose_sep_tile(const Geometry& g, int cls_z, size_t smem_limit);
 // they do not fit; *tiles receives the column-tile count they need.
 int fused_bucket(const Geometry& g, size_t smem_limit, int* tiles);
 int fused_groups(const spect_plan_s& P);
-// (re)encode P.fmap after the slab, the view chunk or the forward launch shape changed
-cudaError_t build_fwd_map(spect_plan_s& P);
+// (re)encode the blur kernels' tensor maps after the slab, the attenuation buffer, the view chunk or a launch shape changed
+cudaError_t build_maps(spect_plan_s& P);
 size_t fwd_records_floats(const spect_plan_s& P);
-cudaError_t launch_fwd_records(const spect_plan_s& P, cudaStream_t st);
+size_t adj_records_floats(const spect_plan_s& P);
+cudaError_t launch_records(const spect_plan_s& P, cudaStream_t st);
 int fwd_tiles(const spect_plan_s& P);
 int adj_tiles(const spect_plan_s& P);
-void default_fwd_shape(spect_plan_s& P);
+void default_shape(spect_plan_s& P);
 // Bucket of the fused full-PSF kernels (untiled planes), 0 when they do not fit.
 int fused_dir_bucket(const Geometry& g, size_t smem_limit);
 bool fused_dir_fit(const Geometry& g, int bucket, int J, int adj_J, size_t smem_limit);
@@ -453,7 +469,10 @@ cudaError_t launch_fused_rotate(const spect_plan_s& P, const float* xt, int l0, 
 int rot3_ts8(int nx);
 cudaError_t build_rot3(spect_plan_s& P, const double* angles, const float* mu_t, float* scratch, cudaStream_t st);
 size_t fused_slab_per_view(const spect_plan_s& P);
+// v: projections with rows of np floats (16-byte aligned rows)
 cudaError_t launch_fused_adjoint(const spect_plan_s& P, const float* v, int l0, int nv, cudaStream_t st);
+// out (rows of np) = v (rows of nx)
+cudaError_t launch_pad_rows(const spect_plan_s& P, const float* v, float* out, cudaStream_t st);
 cudaError_t launch_fwd_reduce(const spect_plan_s& P, float* v, const float* em_y, const float* em_rbar,
                               cudaStream_t st);
 cudaError_t build_gather(spect_plan_s& P, cudaStream_t st);
