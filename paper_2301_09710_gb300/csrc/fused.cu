@@ -271,8 +271,9 @@ __global__ void k_fwd_reduce(const float* __restrict__ part, int G, size_t nproj
 {
     const size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= nproj) return;
-    float s = 0.f;
-    for (int gq = 0; gq < G; ++gq) s += part[(size_t)gq * nproj + o];
+    KSum acc;  // up to ny partials (J = 1): compensated
+    for (int gq = 0; gq < G; ++gq) acc.add(part[(size_t)gq * nproj + o]);
+    const float s = acc.value();
     if (em_y) {
         const float yb = s + (em_rbar ? em_rbar[o] : 0.f);
         v[np == nx ? o : o + o / nx * (np - nx)] = yb > 0.f ? em_y[o] / yb : 0.f;
@@ -341,13 +342,11 @@ __global__ void k_adj_records(Geometry g, int P, int PT, int EC, int cls_z, cons
 //     padding along i is a clamped column index, along k the blocks at the plane's
 //     ends copy its first / last row into their halo; a thread owns 16 k of one
 //     column and keeps their depth sums in registers.
-//   adjoint: the detector plane is staged once per block, zero-padded
-//     (Vx[ZH + k][C + i]); per plane the taps of the k edge class of each
-//     output row are used for the whole run, and the first / last detector
-//     column (the i edge classes) is recomputed with its own variant.
+//   adjoint: the same tiles and FIRs along k on the detector plane, staged once per
+//     block, transposed and zero-padded (V[C + i][ZH + k]); a lane takes the tap rows
+//     of its column's edge class, and the first / last detector row is summed apart
+//     with the C + 1 taps of its class that are not zero.
 // ============================================================================
-__host__ __device__ inline int dir_rows(int nz, int ZH) { return nz + 2 * ZH; }
-
 // Launch shape of the forward full-PSF blur.
 struct DirDims {
     int TI, nT;   // columns per tile, tiles per plane
@@ -363,12 +362,24 @@ __host__ __device__ inline size_t dir_fwd_smem_floats(const DirDims& d, int P, i
     return (size_t)d.nbuf * (d.warea + (((size_t)P * PT + 31) & ~(size_t)31)) + 8;  // + 2 mbarriers
 }
 
-__host__ __device__ inline size_t dir_adj_smem_floats(const FusedDims& d, int nz, int P, int PT, int ZH, int ncls,
-                                                      int nmb)
+// Launch shape of the full-PSF adjoint (TI, KR, wr, wp as the forward's).
+struct DirAdjDims {
+    int TI, nT, KR, nkr, wr, wp;
+    int varea;    // floats of V (rounded up to 128 bytes)
+    int marea;    // floats of the attenuation boxes, KR * TI
+    int nslot;    // tap sets a block may need: interior, and first and / or last column
+    int J, G, T;
+};
+
+// Adjoint tap set of one PSF plane and column class: P rows (a) along k of PT interior
+// taps, then P rows of EC taps of the first and of the last detector row (the C + 1 that
+// are not zero).
+__host__ __device__ inline int dir_set_floats(int P, int PT, int EC) { return P * (PT + 2 * EC); }
+
+__host__ __device__ inline size_t dir_adj_smem_floats(const DirAdjDims& d, int set)
 {
-    const size_t xarea = ((size_t)dir_rows(nz, ZH) * d.wp + 3) & ~(size_t)3;
-    // Vx | MB x nmb | taps ncls x P x PT | 2 mbarriers
-    return xarea + (size_t)nmb * d.marea + (size_t)ncls * P * PT + 8;
+    // MB | V | tap sets | 2 mbarriers
+    return (size_t)d.marea + d.varea + (size_t)d.nslot * set + 8;
 }
 
 // Plan time: the taps of every PSF plane as rows along k, [a][b], zero-padded to
@@ -488,133 +499,164 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_dir_fused(const __grid
     }
 }
 
+// Plan time: the adjoint's tap sets, [plane][column class 0..2][set], from the edge-class
+// variants psf_adj[column class * cls_z + row class][plane][b][a].
+__global__ void k_dir_adj_records(Geometry g, int P, int PT, int EC, int cls_z, const float* __restrict__ psf_adj,
+                                  float* __restrict__ rec)
+{
+    const size_t row = blockIdx.x, nrow = gridDim.x, pp = (size_t)g.px * g.pz;
+    const int ci = blockIdx.y, C = (P - 1) / 2, ox = (P - g.px) / 2, oz = (P - g.pz) / 2;
+    const int set = dir_set_floats(P, PT, EC);
+    float* r = rec + (row * 3 + ci) * set;
+    for (int e = threadIdx.x; e < set; e += blockDim.x) {
+        int a, b, ck;
+        bool in = true;
+        if (e < P * PT) {
+            ck = 0, a = e / PT, b = e % PT;
+        } else {
+            const int f = e - P * PT, h = f % (P * EC), m = h % EC;
+            ck = f < P * EC ? 1 : 2, a = h / EC;
+            b = ck == 1 ? C + m : m;
+            in = m <= C && cls_z == 3;
+        }
+        in = in && a >= ox && a < ox + g.px && b >= oz && b < oz + g.pz;
+        r[e] = in ? psf_adj[((size_t)(ci * cls_z + ck) * nrow + row) * pp + (size_t)(b - oz) * g.px + a - ox] : 0.f;
+    }
+}
+
+// One block per (column tile, k range, depth group of J planes, view).  The attenuation
+// boxes and the tap sets have one buffer each: the factors are needed only after the
+// plane's FIRs, the taps' wait is covered by the other blocks of the SM.
 template <int P>
-__global__ void __launch_bounds__(kFusedThreads, 1) k_adj_dir_fused(Geometry g, FusedDims d, int cls_z, int nmb,
-                                                                     const float* __restrict__ vin,
-                                                                     const float* __restrict__ mubar,
-                                                                     const float* __restrict__ psf_adj,
-                                                                     float* __restrict__ slab, int l0, int* err)
+__global__ void __launch_bounds__(kFusedThreads, 1)
+    k_adj_dir_fused(const __grid_constant__ CUtensorMap mu_map, const __grid_constant__ CUtensorMap t_map, Geometry g,
+                    DirAdjDims d, const float* __restrict__ vin, const float* __restrict__ rec, int l0, int mu_l0,
+                    int* err)
 {
     using S = Sep<P>;
-    constexpr int C = S::C, CX = S::CX, ZH = S::ZH, PT = S::PT;
-    extern __shared__ __align__(16) float sm[];
+    constexpr int C = S::C, CZ = S::CZ, ZH = S::ZH, WZ = S::WZ, PT = S::PT, EC = AdjRec<P>::EC;
+    constexpr int SET = P * (PT + 2 * EC);
+    extern __shared__ __align__(1024) float sma[];
     const int nx = g.nx, ny = g.ny, nz = g.nz;
-    const int xarea = (dir_rows(nz, ZH) * d.wp + 3) & ~3;
-    const int ncls = 3 * cls_z;                    // edge classes (ci, ck)
-    float* Vx = sm;                                // zero-padded detector plane, Vx[ZH + k][C + i]
-    float* MB = Vx + xarea;                        // [nmb][marea]: two, or one where two do not fit
-    float* TAP = MB + (size_t)nmb * d.marea;       // [ci * cls_z + ck][P][PT], this plane
-    uint64_t* bar = reinterpret_cast<uint64_t*>(TAP + (size_t)ncls * P * PT);
-    const int tid = threadIdx.x;
-    constexpr int T = kFusedThreads;
-    const int grp = blockIdx.x, v = blockIdx.y, l = l0 + v;
+    float* MB = sma;                                   // [KR / 16][TI][16], 64-byte swizzled
+    float* V = MB + d.marea;                           // [wr][wp]
+    float* TAP = V + d.varea;                          // [nslot][SET]
+    uint64_t* bar = reinterpret_cast<uint64_t*>(TAP + (size_t)d.nslot * SET);  // factors, taps
+    const int tid = threadIdx.x, T = blockDim.x;
+    int bx = blockIdx.x;
+    const int tile = bx % d.nT;
+    bx /= d.nT;
+    const int k_lo = (bx % d.nkr) * d.KR, grp = bx / d.nkr;
+    const int v = blockIdx.y, l = l0 + v;
+    const int i0 = tile * d.TI, ti = min(d.TI, nx - i0), nkb = (min(d.KR, nz - k_lo) + CZ - 1) / CZ;
     const int lp = g.nvp == 1 ? 0 : l;
-    const int j_begin = grp * d.J, j_end = min(ny, j_begin + d.J);
-    const int ox = (P - g.px) / 2, oz = (P - g.pz) / 2;
-    const size_t nrow = (size_t)g.nvp * ny, pplane = (size_t)g.px * g.pz;
-    const int pln = nx * nz;
-    const float* mub = mubar + ((size_t)l * ny) * d.ps;
-    float* tsl = slab + ((size_t)v * ny) * d.ps;
-    const unsigned mbytes = (unsigned)d.ps * 4u;
+    const int j_begin = grp * d.J, nj = min(ny - j_begin, d.J);
+    const int ox = (P - g.px) / 2;  // tap rows outside [ox, ox + px) are zero
+    const bool first_tile = tile == 0, last_tile = tile == d.nT - 1;
 
-    for (int e = tid; e < xarea; e += T) Vx[e] = 0.f;
+    // swizzled tensor copies want 512-byte aligned shared memory: refuse (error word) rather than fault
+    if ((smem_u32(sma) & 511u) != 0) {
+        if (tid == 0 && err) atomicExch(err, (int)SPECT_ECUDA);
+        return;
+    }
+    auto request_mu = [&](int n) {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
+                     "r"((unsigned)(nkb * d.TI * 16) * 4u)
+                     : "memory");
+        for (int q = 0; q < nkb; ++q)
+            tma_load_3d(MB + q * d.TI * 16, &mu_map, k_lo + q * 16, i0, (l - mu_l0) * ny + j_begin + n, bar);
+    };
+    auto request_taps = [&](int n) {  // the interior set, then those of the first / last column this tile holds
+        const float* src = rec + ((size_t)lp * ny + j_begin + n) * 3 * SET;
+        const int sets = 1 + first_tile + last_tile;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar + 1)),
+                     "r"((unsigned)(sets * SET) * 4u)
+                     : "memory");
+        tma_copy_1d(TAP, src, (unsigned)SET * 4u, bar + 1);
+        if (first_tile) tma_copy_1d(TAP + SET, src + SET, (unsigned)SET * 4u, bar + 1);
+        if (last_tile) tma_copy_1d(TAP + (1 + first_tile) * SET, src + 2 * SET, (unsigned)SET * 4u, bar + 1);
+    };
     if (tid == 0) {
         mbar_init(bar, 1);
         mbar_init(bar + 1, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        tma_load_1d(MB, mub + (size_t)j_begin * d.ps, mbytes, bar);
+        request_taps(0);
+        request_mu(0);
     }
+    // the detector plane, transposed, zero outside the detector: lanes over columns
+    for (int e = tid; e < d.wr * (d.KR + 2 * ZH); e += T) {
+        const int r = e / d.wr, c = e - r * d.wr, k = k_lo - ZH + r, col = i0 - C + c;
+        const bool in = k >= 0 && k < nz && col >= 0 && col < nx;
+        cp_async_4_or_zero(V + c * d.wp + r, in ? vin + ((size_t)l * nz + k) * g.np + col : vin, in);
+    }
+    cp_async_wait_all();
     __syncthreads();
-    for (int e = tid; e < pln; e += T) {
-        const int k = e / nx, i = e - k * nx;
-        Vx[(ZH + k) * d.wp + C + i] = vin[((size_t)l * nz + k) * g.np + i];
-    }
 
-    unsigned phases = 0u;
-    for (int j = j_begin; j < j_end; ++j) {
-        const int b = nmb == 1 ? 0 : (j - j_begin) & 1;
-        // taps of every edge class of this plane
-        for (int e = tid; e < ncls * P * PT; e += T) {
-            const int cls = e / (P * PT), r = e - cls * P * PT, bb = r / PT, a = r - bb * PT;
-            const int ax = a - ox, bz = bb - oz;
-            TAP[e] = (ax >= 0 && ax < g.px && bz >= 0 && bz < g.pz)
-                         ? __ldg(psf_adj + ((size_t)cls * nrow + (size_t)lp * ny + j) * pplane + (size_t)bz * g.px + ax)
-                         : 0.f;
+    const int kb = tid / ti, i = tid - kb * ti;  // the thread's item: 16 k of column i0 + i
+    const bool mine = kb < nkb;
+    const int k0 = k_lo + kb * CZ, cl = nz - 1 - k0;  // position of row nz - 1 in the item
+    const bool top = mine && nz > 1 && k0 == 0, bottom = mine && nz > 1 && cl < CZ;
+    const int slot = i0 + i == 0 ? 1 : (i0 + i == nx - 1 ? 1 + first_tile : 0);
+    const float* TS = TAP + slot * SET;  // this column's tap set
+    const float* TF = TS + P * PT;       // first row, last row
+    const float* TL = TF + P * EC;
+    for (int n = 0; n < nj; ++n) {
+        bool ok = mbar_wait_bounded(bar + 1, (unsigned)n & 1u);
+        float o[CZ], e_first = 0.f, e_last = 0.f;
+        if (ok && mine) {
+#pragma unroll
+            for (int c = 0; c < CZ; ++c) o[c] = 0.f;
+            for (int a = ox; a < ox + g.px; ++a) {
+                const float* vc = V + (i + a) * d.wp;
+                float win[WZ];
+                load_window_f4<P>(vc + kb * CZ, win);
+                float ob[CZ];
+                fir<P, CZ, 1, ZH - C>(TS + a * PT, win, ob);
+#pragma unroll
+                for (int c = 0; c < CZ; ++c) o[c] += ob[c];
+                if (top) e_first += edge_dot_reg<C + 1, ZH>(TF + a * EC, win);
+                if (bottom) e_last += edge_dot<C + 1>(TL + a * EC, vc, ZH + nz - 1 - k_lo - C);
+            }
+            if (top) o[0] = e_first;
+            if (bottom) {
+#pragma unroll
+                for (int c = 0; c < CZ; ++c)
+                    if (c == cl) o[c] = e_last;
+            }
         }
-        __syncthreads();
-        // the other buffer receives the next plane's attenuation once its store has read it
-        if (nmb == 1 && tid == 0 && j > j_begin) {  // the one buffer: this plane's, once the last store has read it
-            tma_store_wait_read<0>();
-            tma_load_1d(MB, mub + (size_t)j * d.ps, mbytes, bar);
-        }
-        if (nmb == 2 && tid == 0 && j + 1 < j_end) {
-            tma_store_wait_read<0>();
-            tma_load_1d(MB + (b ^ 1) * (size_t)d.marea, mub + (size_t)(j + 1) * d.ps, mbytes, bar + (b ^ 1));
-        }
-        float* mb = MB + b * (size_t)d.marea;
-        const bool ok = mbar_wait_bounded(bar + b, (phases >> b) & 1u);
-        phases ^= 1u << b;
-        if (ok) {
-            for (int it = tid; it < nz * d.nib; it += T) {
-                const int ib = it / nz, k = it - ib * nz;
-                const int li = ib * CX;
-                const int ck = nz == 1 ? 0 : (k == 0 ? 1 : (k == nz - 1 ? 2 : 0));
-                const float* TK = TAP + (size_t)ck * P * PT;  // class (ci = interior, ck)
-                float o[CX];
+        ok = mbar_wait_bounded(bar, (unsigned)n & 1u) && ok;
+        if (ok && mine) {
+            float4* m4 = reinterpret_cast<float4*>(MB + ((size_t)kb * d.TI + i) * 16);
+            const int sw = (i >> 1) & 3;
 #pragma unroll
-                for (int c = 0; c < CX; ++c) o[c] = 0.f;
-                for (int bb = 0; bb < P; ++bb) {
-                    const float* vr = Vx + (ZH + k + bb - C) * d.wp + li;
-                    float win[4 * ((CX + P - 1 + 3) / 4)];
-                    load_row_f4(vr, win);
-                    float ob[CX];
-                    fir<P, CX, 1, 0>(TK + bb * PT, win, ob);
-#pragma unroll
-                    for (int c = 0; c < CX; ++c) o[c] += ob[c];
-                }
-                // first / last detector column: their own edge-class variant
-                const int cl = nx - 1 - li;
-                if (li == 0 || cl < CX) {
-                    auto edge = [&](int c, int ci) {
-                        const float* TC = TAP + (size_t)(ci * cls_z + ck) * P * PT;
-                        float acc = 0.f;
-#pragma unroll 2
-                        for (int bb = 0; bb < P; ++bb) {
-                            const float* vr = Vx + (ZH + k + bb - C) * d.wp + li + c;
-                            float rp = 0.f;
-#pragma unroll
-                            for (int a = 0; a < P; ++a) rp = fmaf(TC[bb * PT + a], vr[a], rp);
-                            acc += rp;
-                        }
-                        return acc;
-                    };
-                    if (li == 0) o[0] = edge(0, 1);
-                    if (cl < CX) {
-#pragma unroll
-                        for (int c = 0; c < CX; ++c)
-                            if (c == cl) o[c] = edge(c, nx == 1 ? 0 : 2);
-                    }
-                }
-                float* mp = mb + li * g.kp + k;
-#pragma unroll
-                for (int c = 0; c < CX; ++c)
-                    if (li + c < nx) mp[c * g.kp] = o[c] * mp[c * g.kp];
+            for (int q = 0; q < 4; ++q) {
+                float4 m = m4[q ^ sw];
+                m.x *= o[4 * q];
+                m.y *= o[4 * q + 1];
+                m.z *= o[4 * q + 2];
+                m.w *= o[4 * q + 3];
+                m4[q ^ sw] = m;
             }
         }
         if (__syncthreads_or(!ok)) {
-            if (tid == 0) {
+            if (tid == 0) {  // a last chance for the copies in flight
                 flag_timeout(err);
-                mbar_wait_bounded(bar + b, ((phases >> b) & 1u) ^ 1u);
+                mbar_wait_bounded(bar, (unsigned)n & 1u);
+                mbar_wait_bounded(bar + 1, (unsigned)n & 1u);
                 tma_store_wait_all();
             }
             return;
         }
         if (tid == 0) {
             fence_proxy_async_smem();
-            tma_store_1d(tsl + (size_t)j * d.ps, mb, mbytes);
+            if (n + 1 < nj) request_taps(n + 1);
+            for (int q = 0; q < nkb; ++q)
+                tma_store_3d(&t_map, k_lo + q * 16, i0, v * ny + j_begin + n, MB + q * d.TI * 16);
+            tma_store_commit();
+            tma_store_wait_read<0>();
+            if (n + 1 < nj) request_mu(n + 1);
         }
     }
-    if (tid == 0) tma_store_wait_read<0>();  // the writes complete with the grid
 }
 
 // x_t(q,k) (+)= sum_{v in chunk} sum_{e < MAXE} w_e t[v][p_e][k]
@@ -785,13 +827,22 @@ cudaError_t adj_launch(const spect_plan_s& Pl, const float* v, int l0, int nv, c
 }  // namespace
 
 namespace {
-// The bound of the full-PSF geometries taken: two whole planes with halo rows,
-// accumulators and taps (the forward kernel's tiles need less).
+// The bound of the full-PSF geometries taken, forward: two whole planes with halo
+// rows, accumulators and taps; adjoint: one plane, two attenuation planes and the taps
+// of every edge class (the kernels' tiles need less).
 template <int P>
 size_t dir_smem_fwd_bound(const Geometry& g, const FusedDims& d)
 {
-    const size_t xarea = ((size_t)dir_rows(g.nz, Sep<P>::ZH) * d.wp + 3) & ~(size_t)3;
+    const size_t xarea = ((size_t)(g.nz + 2 * Sep<P>::ZH) * d.wp + 3) & ~(size_t)3;
     return (2 * xarea + (size_t)P * Sep<P>::PT + (size_t)d.urows * d.apc + 8) * sizeof(float);
+}
+
+template <int P>
+size_t dir_smem_adj_bound(const Geometry& g, const FusedDims& d, int cls_z)
+{
+    const size_t xarea = ((size_t)(g.nz + 2 * Sep<P>::ZH) * d.wp + 3) & ~(size_t)3;
+    const size_t marea = ((size_t)d.urows * g.nz + 3) & ~(size_t)3;
+    return (xarea + 2 * marea + 3 * (size_t)cls_z * P * Sep<P>::PT + 8) * sizeof(float);
 }
 
 // Forward launch shape: 32-column tiles, at most 192 k per block (the tensor map's
@@ -822,9 +873,22 @@ DirDims dir_fwd_dims(const Geometry& g, int J, size_t smem_limit)
 }
 
 template <int P>
-size_t dir_smem_adj(const Geometry& g, const FusedDims& d, int cls_z, int nmb)
+DirAdjDims dir_adj_dims(const Geometry& g, int J)
 {
-    return dir_adj_smem_floats(d, g.nz, P, Sep<P>::PT, Sep<P>::ZH, 3 * cls_z, nmb) * sizeof(float);
+    const DirDims f = dir_fwd_dims<P>(g, J, 0);  // the forward's tiles
+    DirAdjDims d;
+    d.TI = f.TI, d.nT = f.nT, d.KR = f.KR, d.nkr = f.nkr, d.wr = f.wr, d.wp = f.wp;
+    d.varea = f.warea;
+    d.marea = d.KR * d.TI;
+    d.nslot = d.nT == 1 ? 3 : 2;
+    d.J = J, d.G = f.G, d.T = f.T;
+    return d;
+}
+
+template <int P>
+size_t dir_smem_adj(const DirAdjDims& d)
+{
+    return dir_adj_smem_floats(d, dir_set_floats(P, Sep<P>::PT, AdjRec<P>::EC)) * sizeof(float);
 }
 
 template <int P>
@@ -832,11 +896,8 @@ bool dir_fits(const Geometry& g, size_t limit, int J, int adj_J)
 {
     const int cls_z = g.nz >= 2 ? 3 : 1;
     const FusedDims df = dims_for<P>(g, J, 1), da = dims_for<P>(g, adj_J, 1);
-    // attenuation planes counted without their k padding: where that leaves no room for
-    // two padded ones, the adjoint runs with one
-    const size_t pad = 2 * ((size_t)da.marea - (((size_t)g.nx * g.nz + 3) & ~(size_t)3)) * sizeof(float);
-    return df.nT == 1 && dir_smem_fwd_bound<P>(g, df) <= limit && dir_smem_adj<P>(g, da, cls_z, 2) - pad <= limit &&
-           dir_smem_adj<P>(g, da, cls_z, 1) <= limit && rot_smem_bound(df) <= limit && (size_t)df.ps * 4 < (1u << 20);
+    return df.nT == 1 && dir_smem_fwd_bound<P>(g, df) <= limit && dir_smem_adj_bound<P>(g, da, cls_z) <= limit &&
+           rot_smem_bound(df) <= limit && (size_t)df.ps * 4 < (1u << 20);
 }
 
 template <int P>
@@ -853,13 +914,12 @@ cudaError_t dir_fwd_launch(const spect_plan_s& Pl, int l0, int nv, cudaStream_t 
 template <int P>
 cudaError_t dir_adj_launch(const spect_plan_s& Pl, const float* v, int l0, int nv, cudaStream_t st)
 {
-    const FusedDims d = dims_for<P>(Pl.g, Pl.adj_J, 1);
-    const int nmb = dir_smem_adj<P>(Pl.g, d, Pl.cls_z, 2) <= (size_t)Pl.smem_optin ? 2 : 1;
-    const size_t smem = dir_smem_adj<P>(Pl.g, d, Pl.cls_z, nmb);
+    const DirAdjDims d = dir_adj_dims<P>(Pl.g, Pl.adj_J);
+    const size_t smem = dir_smem_adj<P>(d);
     cudaError_t e = cudaFuncSetAttribute(k_adj_dir_fused<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_adj_dir_fused<P><<<dim3(d.G, nv), kFusedThreads, smem, st>>>(Pl.g, d, Pl.cls_z, nmb, v, mubar_for(Pl, l0),
-                                                                    Pl.psf_adj, Pl.slab, l0, Pl.err);
+    k_adj_dir_fused<P><<<dim3(d.nT * d.nkr * d.G, nv), d.T, smem, st>>>(Pl.amap_mu, Pl.amap_t, Pl.g, d, v, Pl.arec, l0,
+                                                                        Pl.recompute ? l0 : 0, Pl.err);
     return cudaGetLastError();
 }
 }  // namespace
@@ -994,17 +1054,19 @@ cudaError_t encode_maps(spect_plan_s& Pl)
     const cuuint64_t strides[2] = {(cuuint64_t)g.kp * 4, (cuuint64_t)Pl.ps * 4};
     const cuuint64_t planes = (cuuint64_t)Pl.chunk * g.ny;
     const cuuint64_t img[3] = {(cuuint64_t)g.nz, (cuuint64_t)g.nx, planes};
-    if (!Pl.separable) {
+    cuuint32_t f0 = kWK, f1, at;
+    if (Pl.separable) {
+        f1 = fwd_dims<P>(g, Pl.fused_J, Pl.fwd_nT, (size_t)Pl.smem_optin).wr;
+        at = adj_dims<P>(g, Pl.adj_J, Pl.adj_nT, (size_t)Pl.smem_optin).TI;
+    } else {
         const DirDims d = dir_fwd_dims<P>(g, Pl.fused_J, (size_t)Pl.smem_optin);
-        return encode_3d(&Pl.fmap, Pl.slab, img, strides, d.wp, d.wr, CU_TENSOR_MAP_SWIZZLE_NONE);
+        f0 = d.wp, f1 = d.wr, at = d.TI;
     }
-    const FwdDims f = fwd_dims<P>(g, Pl.fused_J, Pl.fwd_nT, (size_t)Pl.smem_optin);
-    const AdjDims a = adj_dims<P>(g, Pl.adj_J, Pl.adj_nT, (size_t)Pl.smem_optin);
     const cuuint64_t t[3] = {(cuuint64_t)g.kp, (cuuint64_t)g.nx, planes};
     const cuuint64_t mu[3] = {(cuuint64_t)g.kp, (cuuint64_t)g.nx, Pl.recompute ? planes : (cuuint64_t)g.nview * g.ny};
-    cudaError_t e = encode_3d(&Pl.fmap, Pl.slab, img, strides, kWK, f.wr, CU_TENSOR_MAP_SWIZZLE_NONE);
-    if (e == cudaSuccess) e = encode_3d(&Pl.amap_t, Pl.slab, t, strides, 16, a.TI, CU_TENSOR_MAP_SWIZZLE_64B);
-    if (e == cudaSuccess) e = encode_3d(&Pl.amap_mu, Pl.mubar, mu, strides, 16, a.TI, CU_TENSOR_MAP_SWIZZLE_64B);
+    cudaError_t e = encode_3d(&Pl.fmap, Pl.slab, img, strides, f0, f1, CU_TENSOR_MAP_SWIZZLE_NONE);
+    if (e == cudaSuccess) e = encode_3d(&Pl.amap_t, Pl.slab, t, strides, 16, at, CU_TENSOR_MAP_SWIZZLE_64B);
+    if (e == cudaSuccess) e = encode_3d(&Pl.amap_mu, Pl.mubar, mu, strides, 16, at, CU_TENSOR_MAP_SWIZZLE_64B);
     return e;
 }
 }  // namespace
@@ -1020,11 +1082,11 @@ namespace {
 int rec_edge(int P) { return ((P - 1) / 2 + 4) & ~3; }  // AdjRec::EC
 }  // namespace
 
-// Floats of the blur adjoint's tap records of a (separable) plan.
+// Floats of the blur adjoint's tap records of a plan.
 size_t adj_records_floats(const spect_plan_s& P)
 {
-    if (!P.separable) return 0;
-    return (size_t)P.g.nvp * P.g.ny * (2 * ((P.bucket + 3) & ~3) + 4 * rec_edge(P.bucket));
+    const int PT = (P.bucket + 3) & ~3, EC = rec_edge(P.bucket);
+    return (size_t)P.g.nvp * P.g.ny * (P.separable ? 2 * PT + 4 * EC : 3 * dir_set_floats(P.bucket, PT, EC));
 }
 
 cudaError_t launch_records(const spect_plan_s& P, cudaStream_t st)
@@ -1035,6 +1097,8 @@ cudaError_t launch_records(const spect_plan_s& P, cudaStream_t st)
         k_adj_records<<<rows, 64, 0, st>>>(P.g, P.bucket, PT, rec_edge(P.bucket), P.cls_z, P.fx_adj, P.fz_adj, P.arec);
     } else {
         k_dir_records<<<rows, 256, 0, st>>>(P.g, P.bucket, PT, P.psf, P.frec);
+        k_dir_adj_records<<<dim3(rows, 3), 256, 0, st>>>(P.g, P.bucket, PT, rec_edge(P.bucket), P.cls_z, P.psf_adj,
+                                                         P.arec);
     }
     return cudaGetLastError();
 }
@@ -1104,6 +1168,7 @@ void default_shape(spect_plan_s& P)
     if (!P.separable) {  // blocks of the full-PSF forward kernel
         const long long blocks = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * g.nview;
         if (blocks < 24ll * P.sms) P.fused_J = blocks >= 4ll * P.sms ? 4 : 2;
+        P.adj_J = P.fused_J;
         return;
     }
     switch (P.bucket) {

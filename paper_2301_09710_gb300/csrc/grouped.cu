@@ -27,7 +27,6 @@ struct GroupPlan {
     RotDims dr;        // rotation launch shape
     AdjDims da;        // adjoint launch shape
     FwdDims df;        // forward launch shape
-    int cls_z;
     const float* rtab;
     const float* xt;
     const float* mubar;
@@ -92,8 +91,9 @@ __global__ void __launch_bounds__(kReduceThreads) k_fwd_reduce_grp(const __grid_
     const GroupPlan q = gp.p[w.x];  // by value: the fields live in registers, not re-read from parameter space
     const size_t o = (size_t)w.y * kReduceThreads + threadIdx.x;
     if (o >= q.nproj) return;
-    float s = 0.f;
-    for (int gq = 0; gq < q.df.G; ++gq) s += q.part[(size_t)gq * q.nproj + o];
+    KSum acc;
+    for (int gq = 0; gq < q.df.G; ++gq) acc.add(q.part[(size_t)gq * q.nproj + o]);
+    const float s = acc.value();
     const float yb = s + (q.rbar ? q.rbar[o] : 0.f);
     const int nx = q.g.nx, np = q.g.np;
     q.ratio[np == nx ? o : o + o / nx * (np - nx)] = yb > 0.f ? q.y[o] / yb : 0.f;
@@ -128,7 +128,6 @@ void fill_plan(GroupPlan& q, const spect_plan_s* Pl, const float* y, const float
     q.g = Pl->g;
     q.df = fwd_dims<P>(Pl->g, Pl->fused_J, Pl->fwd_nT, (size_t)Pl->smem_optin);
     q.da = adj_dims<P>(Pl->g, Pl->adj_J, Pl->adj_nT, (size_t)Pl->smem_optin);
-    q.cls_z = Pl->cls_z;
     q.mubar = Pl->mubar;
     q.slab = Pl->slab;
     q.frec = Pl->frec;

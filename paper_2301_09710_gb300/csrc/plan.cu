@@ -672,12 +672,12 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         PLAN_ALLOC(P->frec, spect::fwd_records_floats(*P), "tap records");
         PLAN_ALLOC(P->arec, spect::adj_records_floats(*P), "adjoint tap records");
         PLAN_TRY(spect::launch_records(*P, st), "tap record launch");
-        for (float** p : {&P->fx, &P->fz, &P->psf, &P->fx_adj, &P->fz_adj}) {
+        for (float** p : {&P->fx, &P->fz, &P->psf, &P->fx_adj, &P->fz_adj, &P->psf_adj}) {
             raw_free(P, *p, st);
             *p = nullptr;
         }
-        P->bytes -= (P->separable ? (size_t)px * 4 + (size_t)pz * (1 + P->cls_z) : (size_t)px * pz) * nrows *
-                    sizeof(float);
+        P->bytes -= (P->separable ? (size_t)px * 4 + (size_t)pz * (1 + P->cls_z)
+                                  : (size_t)px * pz * (1 + P->cls_x * P->cls_z)) * nrows * sizeof(float);
     }
 
     // work slab and EM buffers
