@@ -80,8 +80,10 @@ enum {
     SPECT_PLAN_PREFER_SEPARABLE = 1u << 0,
     /* Keep device memory O(image + projections): recompute the attenuation
      * per view and stream views through a small work slab, instead of
-     * caching the attenuation factors of every view (nview * nx*ny*nz floats)
-     * and using the fused kernels. */
+     * caching the attenuation factors of every view (nview * nx*ny*nz floats).
+     * Where the fused kernels fit the geometry they run in view chunks small
+     * enough for that (spect_plan_info still reports fused = 0, and the launch
+     * shapes cannot be tuned); wider PSFs take the low-memory kernels. */
     SPECT_PLAN_LOW_MEMORY = 1u << 1,
     /* Rotate the image and the attenuation map by three 1D linear
      * interpolation passes instead of bilinear interpolation (Section II-A
@@ -238,8 +240,9 @@ spect_status spect_sensitivity(spect_plan plan, float* s, spect_stream stream);
 /*
  * spect_plan_info -- describe a plan (host out-pointers; any may be NULL):
  *   separable    1 when the separable-factor kernels are used, else 0.
- *   fused        1 when the fused kernels with the cached attenuation serve
- *                the plan, 0 for the low-memory kernels.
+ *   fused        1 when the fused kernels with the cached attenuation (or, with
+ *                SPECT_PLAN_RECOMPUTE_ATTENUATION, a chunk's) serve the plan, 0 for
+ *                low-memory plans and geometries the fused kernels do not fit.
  *   view_chunk   views processed per pass through the work slab.
  *   device_bytes device memory held by the plan (state + work slab).
  */

@@ -220,14 +220,14 @@ __global__ void __launch_bounds__(kRotThreads, TAPS == 4 ? 5 : 3) k_rot_fwd(Geom
 // Forward blur + depth sum: one block per (column tile, depth group of J planes,
 // view), the tiles of a plane adjacent, so their overlapping boxes hit L2.
 // ----------------------------------------------------------------------------
-template <int P, bool RACC>
-__global__ void __launch_bounds__(FwdBlock<P>::T, FwdBlock<P>::B) k_fwd_sep_fused(const __grid_constant__ CUtensorMap tmap,
+template <int P, bool RACC, bool KS>
+__global__ void __launch_bounds__(FwdBlock<P>::T, KS ? 1 : FwdBlock<P>::B) k_fwd_sep_fused(const __grid_constant__ CUtensorMap tmap,
                                                                      Geometry g, FwdDims d,
                                                                      const float* __restrict__ rec,
                                                                      float* __restrict__ part, int l0, int* err)
 {
     const int grp = blockIdx.x / d.nT;
-    fwd_sep_body<P, RACC>(g, d, &tmap, rec, part, l0, err, grp, blockIdx.y, blockIdx.x - grp * d.nT);
+    fwd_sep_body<P, RACC, KS>(g, d, &tmap, rec, part, l0, err, grp, blockIdx.y, blockIdx.x - grp * d.nT);
 }
 
 // Plan time: the tap records of the forward blur (layout: fwd_rec_floats), one
@@ -396,8 +396,10 @@ __global__ void k_dir_records(Geometry g, int P, int PT, const float* __restrict
 }
 
 // One block per (column tile, k range, depth group of J planes, view).
-template <int P>
-__global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_dir_fused(const __grid_constant__ CUtensorMap tmap,
+constexpr int kDirThreads = 384;  // 32 columns x 192 / 16 k runs
+
+template <int P, bool KS>
+__global__ void __launch_bounds__(kDirThreads, 1) k_fwd_dir_fused(const __grid_constant__ CUtensorMap tmap,
                                                                      Geometry g, DirDims d,
                                                                      const float* __restrict__ rec,
                                                                      float* __restrict__ part, int l0, int* err)
@@ -445,9 +447,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_dir_fused(const __grid
     const int kb = tid / ti, i = tid - kb * ti;  // the thread's item: 16 k of column i0 + i
     const bool mine = kb < nkb;
     const int kz = nz - 1 - k_lo + ZH;           // position of row nz - 1 in a column of W
-    float acc[CZ];
-#pragma unroll
-    for (int c = 0; c < CZ; ++c) acc[c] = 0.f;
+    DepthSum<KS> acc[CZ];
     for (int n = 0; n < nj; ++n) {
         const int b = d.nbuf == 1 ? 0 : n & 1;
         float* W = smf + (size_t)b * (d.warea + TAPS);
@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_dir_fused(const __grid
                 for (int c = 0; c < CZ; ++c) o[c] += ob[c];
             }
 #pragma unroll
-            for (int c = 0; c < CZ; ++c) acc[c] += o[c];
+            for (int c = 0; c < CZ; ++c) acc[c].add(o[c]);
         }
         __syncthreads();  // buffer b and its taps are free
         if (tid == 0 && n + d.nbuf < nj) {
@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_fwd_dir_fused(const __grid
         float* pout = part + ((size_t)grp * g.nview + l) * pln + i0 + i;
 #pragma unroll
         for (int c = 0; c < CZ; ++c)
-            if (k0 + c < nz) pout[(size_t)(k0 + c) * nx] = acc[c];
+            if (k0 + c < nz) pout[(size_t)(k0 + c) * nx] = acc[c].value();
     }
 }
 
@@ -528,7 +528,7 @@ __global__ void k_dir_adj_records(Geometry g, int P, int PT, int EC, int cls_z, 
 // boxes and the tap sets have one buffer each: the factors are needed only after the
 // plane's FIRs, the taps' wait is covered by the other blocks of the SM.
 template <int P>
-__global__ void __launch_bounds__(kFusedThreads, 1)
+__global__ void __launch_bounds__(kDirThreads, 1)
     k_adj_dir_fused(const __grid_constant__ CUtensorMap mu_map, const __grid_constant__ CUtensorMap t_map, Geometry g,
                     DirAdjDims d, const float* __restrict__ vin, const float* __restrict__ rec, int l0, int mu_l0,
                     int* err)
@@ -668,7 +668,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1)
 template <int MAXE>
 __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const AdjEntry* __restrict__ adj,
                                                    const float* __restrict__ slab, int l0, int nv, float* out,
-                                                   int accumulate, EmArgs em)
+                                                   PassState ps_, EmArgs em)
 {
     using VT = float4;
     constexpr int VEC = 4;
@@ -688,7 +688,11 @@ __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const Adj
     const AdjEntry* e = adj + ((size_t)q * g.nview + l0) * MAXE;
     const float* t = slab + k;
     const size_t vstride = (size_t)g.ny * ps;
+    const size_t o = (size_t)q * g.kp + k;
     KSum acc[VEC];
+    if (ps_.resume)  // the sums of the views of earlier passes
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) acc[u].s = out[o + u], acc[u].c = ps_.comp[o + u];
     // four views per step: all entry loads, then all slab loads, are issued
     // before any is used, so the chain of dependent loads is 4x shorter
     constexpr int UV = 4;
@@ -742,11 +746,14 @@ __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const Adj
         e += MAXE;
         t += vstride;
     }
-    const size_t o = (size_t)q * g.kp + k;
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
-        float val = acc[u].value();
-        if (accumulate) val += out[o + u];
+        if (ps_.more) {
+            out[o + u] = acc[u].s;
+            ps_.comp[o + u] = acc[u].c;
+            continue;
+        }
+        const float val = acc[u].value();
         if (em.x) em.x[o + u] = em_update(em.x[o + u], val, em.s[o + u], em.u ? em.u[o + u] : 0.f, em.beta);
         else out[o + u] = val;
     }
@@ -802,7 +809,8 @@ cudaError_t fwd_launch(const spect_plan_s& Pl, const float* /*xt: the blur reads
 {
     const FwdDims d = fwd_dims<P>(Pl.g, Pl.fused_J, Pl.fwd_nT, (size_t)Pl.smem_optin);
     const size_t smem = smem_fwd<P>(d);
-    auto kern = d.racc ? k_fwd_sep_fused<P, true> : k_fwd_sep_fused<P, false>;
+    auto kern = !d.racc ? k_fwd_sep_fused<P, false, false>
+                        : (Pl.low ? k_fwd_sep_fused<P, true, true> : k_fwd_sep_fused<P, true, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3(d.G * d.nT, nv), d.T, smem, st>>>(Pl.fmap, Pl.g, d, Pl.frec, Pl.part, l0, Pl.err);
@@ -905,9 +913,10 @@ cudaError_t dir_fwd_launch(const spect_plan_s& Pl, int l0, int nv, cudaStream_t 
 {
     const DirDims d = dir_fwd_dims<P>(Pl.g, Pl.fused_J, (size_t)Pl.smem_optin);
     const size_t smem = dir_fwd_smem_floats(d, P, Sep<P>::PT) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k_fwd_dir_fused<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = Pl.low ? k_fwd_dir_fused<P, true> : k_fwd_dir_fused<P, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_fwd_dir_fused<P><<<dim3(d.nT * d.nkr * d.G, nv), d.T, smem, st>>>(Pl.fmap, Pl.g, d, Pl.frec, Pl.part, l0, Pl.err);
+    kern<<<dim3(d.nT * d.nkr * d.G, nv), d.T, smem, st>>>(Pl.fmap, Pl.g, d, Pl.frec, Pl.part, l0, Pl.err);
     return cudaGetLastError();
 }
 
@@ -1130,24 +1139,27 @@ void choose_shape(spect_plan_s& Pl)
 {
     const Geometry& g = Pl.g;
     const size_t limit = (size_t)Pl.smem_optin;
-    const int nib = (g.nx + 15) / 16, fmin = Pl.fwd_nT, amin = Pl.adj_nT;
+    const int nib = (g.nx + 15) / 16, nv = Pl.shape_views;
+    // J decides how A's depth sum is grouped: the same whatever the passes (a recomputing
+    // plan's results are bitwise the caching plan's), except for low-memory plans
+    const int keep_J = nv < g.nview && !Pl.low ? Pl.fused_J : 0;
     double fbest = 1e30, abest = 1e30;
     for (int ti : {32, 48, 64, 16}) {  // 32 columns unless another width is clearly better
         const int tiles = (nib + ti / 16 - 1) / (ti / 16);
-        for (int J : {8, 4, 6, 10, 12, 16, 7, 5, 3, 2, 1}) {
+        for (int J : {8, 4, 6, 7, 5, 3, 2, 1}) {  // longer plain depth sums would cost accuracy
             if (J > g.ny) continue;
-            const FwdDims f = fwd_dims<P>(g, J, std::max(tiles, fmin), limit);
-            if (smem_fwd<P>(f) <= limit && (f.racc || ti == 16)) {
+            const FwdDims f = fwd_dims<P>(g, J, std::max(tiles, Pl.min_nT), limit);
+            if (smem_fwd<P>(f) <= limit && (f.racc || ti == 16) && (keep_J == 0 || J == keep_J)) {
                 const int B = blocks_per_sm(smem_fwd<P>(f), f.T, FwdBlock<P>::regs);
                 // + the reduce: G partials written and read
-                const double c = blur_cost(P, (long long)f.G * f.nT * g.nview, J, 1.0, f.T, B, Pl.sms) +
-                                 (double)f.G * g.nx * g.nz * g.nview * 8.0 / 5e6;
+                const double c = blur_cost(P, (long long)f.G * f.nT * nv, J, 1.0, f.T, B, Pl.sms) +
+                                 (double)f.G * g.nx * g.nz * nv * 8.0 / 5e6;
                 if (c < 0.98 * fbest) fbest = c, Pl.fused_J = J, Pl.fwd_nT = f.nT;
             }
-            const AdjDims a = adj_dims<P>(g, J, std::max(tiles, amin), limit);
+            const AdjDims a = adj_dims<P>(g, J, std::max(tiles, Pl.min_nT), limit);
             if (smem_adj<P>(a) <= limit) {
                 const int B = blocks_per_sm(smem_adj<P>(a), a.T, AdjBlock<P>::regs);
-                const double c = blur_cost(P, (long long)a.G * a.nT * g.nview, J, 1.0, a.T, B, Pl.sms);
+                const double c = blur_cost(P, (long long)a.G * a.nT * nv, J, 1.0, a.T, B, Pl.sms);
                 if (c < 0.98 * abest) abest = c, Pl.adj_J = J, Pl.adj_nT = a.nT;
             }
         }
@@ -1163,10 +1175,10 @@ void choose_shape(spect_plan_s& Pl)
 void default_shape(spect_plan_s& P)
 {
     const Geometry& g = P.g;
-    P.fused_J = 8;
-    P.adj_J = 8;
     if (!P.separable) {  // blocks of the full-PSF forward kernel
-        const long long blocks = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * g.nview;
+        if (P.shape_views < g.nview && !P.low) return;  // as choose_shape's keep_J
+        P.fused_J = P.adj_J = 8;
+        const long long blocks = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * P.shape_views;
         if (blocks < 24ll * P.sms) P.fused_J = blocks >= 4ll * P.sms ? 4 : 2;
         P.adj_J = P.fused_J;
         return;
@@ -1231,7 +1243,7 @@ cudaError_t launch_fwd_reduce(const spect_plan_s& P, float* v, const float* em_y
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, int accumulate, EmArgs em,
+cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,
                              cudaStream_t st)
 {
     const size_t n = (size_t)P.g.nx * P.g.ny * (P.g.kp / 4);
@@ -1239,7 +1251,7 @@ cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, 
     const float* src = P.slab;
     switch (P.adj_max) {
 #define SPECT_ADJ(M)                                                                                                 \
-    case M: k_adj_rot_t<M><<<blocks, 256, 0, st>>>(P.g, P.ps, P.adjf, src, l0, nv, out, accumulate, em); break;
+    case M: k_adj_rot_t<M><<<blocks, 256, 0, st>>>(P.g, P.ps, P.adjf, src, l0, nv, out, pass, em); break;
         SPECT_ADJ(1) SPECT_ADJ(2) SPECT_ADJ(3) SPECT_ADJ(4) SPECT_ADJ(5) SPECT_ADJ(6) SPECT_ADJ(7) SPECT_ADJ(8)
 #undef SPECT_ADJ
         default: return cudaErrorInvalidValue;

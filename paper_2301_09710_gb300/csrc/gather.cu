@@ -102,7 +102,7 @@ struct GatherArgs {
 template <int MAXE>
 __device__ __forceinline__ void adj_gather_body(const CUtensorMap* tmap, const GatherArgs& a,
                                                 const int4* __restrict__ boxes, const AdjEntry* __restrict__ pent,
-                                                float* out, int accumulate, const EmArgs& em, int* err,
+                                                float* out, const PassState& pass, const EmArgs& em, int* err,
                                                 const int patch, const int kcb)
 {
     extern __shared__ __align__(128) float sm[];
@@ -173,6 +173,11 @@ __device__ __forceinline__ void adj_gather_body(const CUtensorMap* tmap, const G
     }
 
     KSum acc[4];
+    if (mine && pass.resume) {  // the sums of the views of earlier passes
+        const float4 s = *reinterpret_cast<const float4*>(out + o), c = *reinterpret_cast<const float4*>(pass.comp + o);
+        acc[0].s = s.x, acc[1].s = s.y, acc[2].s = s.z, acc[3].s = s.w;
+        acc[0].c = c.x, acc[1].c = c.y, acc[2].c = c.z, acc[3].c = c.w;
+    }
     bool failed = false;
     for (int v = 0; v < a.nv; ++v) {
         const int s = v % kStages;
@@ -207,11 +212,15 @@ __device__ __forceinline__ void adj_gather_body(const CUtensorMap* tmap, const G
     if (failed || *abort_flag) return;
 
     if (!mine) return;
+    if (pass.more) {
+        *reinterpret_cast<float4*>(out + o) = make_float4(acc[0].s, acc[1].s, acc[2].s, acc[3].s);
+        *reinterpret_cast<float4*>(pass.comp + o) = make_float4(acc[0].c, acc[1].c, acc[2].c, acc[3].c);
+        return;
+    }
     const float xv[4] = {ex.x, ex.y, ex.z, ex.w}, sv4[4] = {es.x, es.y, es.z, es.w}, uv[4] = {eu.x, eu.y, eu.z, eu.w};
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        float val = acc[u].value();
-        if (accumulate) val += out[o + u];
+        const float val = acc[u].value();
         if (em.x) em.x[o + u] = em_update(xv[u], val, sv4[u], uv[u], em.beta);
         else out[o + u] = val;
     }
@@ -221,13 +230,13 @@ template <int MAXE>
 __global__ void __launch_bounds__(kGT + 32) k_adj_gather(const __grid_constant__ CUtensorMap tmap, GatherArgs a,
                                                          const int4* __restrict__ boxes,
                                                          const AdjEntry* __restrict__ pent, float* out,
-                                                         int accumulate, EmArgs em, int* err)
+                                                         PassState pass, EmArgs em, int* err)
 {
     // the k runs of a patch are adjacent blocks, so they run side by side and the
     // patch's entries, which each of them reads, come from DRAM about once
     // (0.246 -> 0.213 ms per 128-view launch against the patch-major order)
     const int patch = (int)blockIdx.x / a.nkc, kcb = (int)blockIdx.x - patch * a.nkc;
-    adj_gather_body<MAXE>(&tmap, a, boxes, pent, out, accumulate, em, err, patch, kcb);
+    adj_gather_body<MAXE>(&tmap, a, boxes, pent, out, pass, em, err, patch, kcb);
 }
 
 
@@ -250,7 +259,6 @@ struct GroupGather {
     const AdjEntry* pent;
     float* out;
     EmArgs em;
-    int accumulate;
     int* err;
 };
 struct GroupGathers {
@@ -263,7 +271,7 @@ __global__ void __launch_bounds__(kGT + 32) k_adj_gather_grp(const __grid_consta
 {
     const int4 w = group_item(gg.grid);
     const GroupGather& q = gg.p[w.x];
-    adj_gather_body<MAXE>(&q.tmap, q.a, q.boxes, q.pent, q.out, q.accumulate, q.em, q.err, w.z, w.y);
+    adj_gather_body<MAXE>(&q.tmap, q.a, q.boxes, q.pent, q.out, PassState(), q.em, q.err, w.z, w.y);
 }
 
 }  // namespace
@@ -379,7 +387,7 @@ cudaError_t gather_setup(const spect_plan_s& P, int l0, int nv, CUtensorMap* map
 }
 }  // namespace
 
-cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, float* out, int accumulate, EmArgs em,
+cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,
                               cudaStream_t st)
 {
     CUtensorMap map;
@@ -394,7 +402,7 @@ cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, float* out,
         cudaError_t e = cudaFuncSetAttribute(k_adj_gather<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
                                              (int)smem);                                                     \
         if (e != cudaSuccess) return e;                                                                      \
-        k_adj_gather<M><<<grid, kGT + 32, smem, st>>>(map, a, P.gboxes, P.gent, out, accumulate, em, P.err); \
+        k_adj_gather<M><<<grid, kGT + 32, smem, st>>>(map, a, P.gboxes, P.gent, out, pass, em, P.err); \
         break;                                                                                               \
     }
         SPECT_G(1) SPECT_G(2) SPECT_G(3) SPECT_G(4) SPECT_G(5) SPECT_G(6) SPECT_G(7) SPECT_G(8)
@@ -435,7 +443,6 @@ cudaError_t build_grouped_gather(const std::vector<spect_plan_s*>& plans, Groupe
                 q.em.s = P.st;
                 q.em.u = nullptr;
                 q.em.beta = 0.f;
-                q.accumulate = 0;
                 q.err = P.err;
                 smem = std::max(smem, gather_smem(q.a.box_floats, q.a.ent_bytes));
                 // the gather's grid: (run of kc depth rows, patch), the k runs of a patch adjacent

@@ -183,6 +183,47 @@ int view_chunk(const spect_plan_s& P, size_t slab_floats_per_view, size_t budget
     return (int)((nview + passes - 1) / passes);
 }
 
+// Budget of a low-memory plan's chunk buffers on the fused kernels: what keeps the
+// plan within the bytes of the low-memory kernels (their slab of at most 256 MiB, the
+// compressed adjacency lists, three volumes), but at least 24 MiB, so that small
+// plans still run in few passes.  SPECT_SLAB_MB overrides.
+size_t low_budget_bytes(const spect_plan_s& P)
+{
+    if (getenv("SPECT_SLAB_MB")) return slab_budget_bytes(false);
+    const Geometry& g = P.g;
+    const double vol = 4.0 * g.nx * g.ny * g.nz, volt = 4.0 * g.nx * g.ny * g.kp, lists = (double)g.nx * g.ny * g.nview;
+    const double held = std::min((double)slab_budget_bytes(false), vol * g.nview) + 36.0 * lists + 3.0 * vol;
+    // rotation tables 20, box-local entries about 40 bytes a list; five internal volumes; partial sums
+    const double fixed = 60.0 * lists + vol + 5.0 * volt + 4.0 * (double)g.nx * g.nz * g.nview * spect::fused_groups(P);
+    return (size_t)std::max(held - fixed, 24.0 * (1 << 20));
+}
+
+// The forward's depth-group partial sums; between the adjoint's passes (adj_chunk views
+// each) the same buffer holds the compensation terms of the view sums.
+size_t part_floats(const spect_plan_s& P, int adj_chunk)
+{
+    const size_t part = (size_t)P.g.nx * P.g.nz * P.g.nview * spect::fused_groups(P);
+    return adj_chunk < P.g.nview ? std::max(part, (size_t)P.g.nx * P.g.ny * P.g.kp) : part;
+}
+
+// Launch shapes and views per pass of a plan: the work slab (and a recomputing plan's
+// factors) within the budget, the blur shapes for that many views.
+void configure_views(spect_plan_s* P)
+{
+    const size_t vol = (size_t)P->g.nx * P->g.ny * P->g.nz;
+    P->shape_views = P->g.nview;
+    if (P->fast) spect::default_shape(*P);
+    const size_t per_view = std::max(vol, P->fast ? spect::fused_slab_per_view(*P) : vol);
+    const size_t budget = P->fast && P->low ? low_budget_bytes(*P)
+                          : P->recompute   ? recompute_budget_bytes()
+                                           : slab_budget_bytes(P->fast);
+    P->chunk = view_chunk(*P, per_view, budget);
+    if (P->fast && P->chunk < P->g.nview) {
+        P->shape_views = P->chunk;
+        spect::default_shape(*P);
+    }
+}
+
 // The patch gather reads its own box-local copy of the adjacency entries, so
 // once it is set up the fixed-length lists were set-up input only: free them.
 void drop_fixed_lists(spect_plan_s* P, cudaStream_t st)
@@ -323,10 +364,16 @@ spect_status fast_back(spect_plan_s* P, const float* v, float* out_t, spect::EmA
                        "fused adjoint launch");
         spect::EmArgs e = em;
         if (!last) e.x = nullptr;
+        spect::PassState pass;
+        pass.resume = l0 > 0;
+        pass.more = !last;
+        pass.comp = P->part;  // free between the depth-group reduce and the next forward blur
+        if ((pass.resume || pass.more) && P->part_cap < (size_t)P->g.nx * P->g.ny * P->g.kp)
+            return fail(SPECT_ECUDA, "several adjoint passes, one planned");
         SPECT_CUDA_TRY(counted(P, SPECT_K_ROTATE_ADJ, st,
                                [&] {
-                                   return P->gather ? spect::launch_adj_gather(*P, l0, nv, out_t, l0 > 0, e, st)
-                                                    : spect::launch_adj_rot_t(*P, l0, nv, out_t, l0 > 0, e, st);
+                                   return P->gather ? spect::launch_adj_gather(*P, l0, nv, out_t, pass, e, st)
+                                                    : spect::launch_adj_rot_t(*P, l0, nv, out_t, pass, e, st);
                                }),
                        "adjoint rotation launch");
     }
@@ -394,12 +441,12 @@ size_t plan_bytes_bound(const spect_plan_s& P)
     if (P.separable) b += ((size_t)g.px * 4 + (size_t)g.pz * (1 + P.cls_z)) * nrows * F;
     else b += (size_t)g.px * g.pz * nrows * (1 + (size_t)P.cls_x * P.cls_z) * F;
     b += (size_t)g.nview * sizeof(ViewRot);
-    const size_t fixed = nlist * 8 * sizeof(spect::AdjEntry);
+    // a low-memory plan's bound leaves out the fixed lists, which are set-up input only
+    const size_t fixed = P.low ? 0 : nlist * 8 * sizeof(spect::AdjEntry);
     const size_t csr = (nlist + 1) * sizeof(int) + 4 * nlist * sizeof(spect::AdjEntry);
-    b += P.fast ? std::max(fixed, csr) : csr;
+    b += P.fast ? (P.low ? 0 : std::max(fixed, csr)) : csr;
     const size_t per_view = std::max(vol, P.fast ? spect::fused_slab_per_view(P) : vol);
-    const size_t budget = P.recompute ? recompute_budget_bytes() : slab_budget_bytes(P.fast);
-    const size_t chunk = view_chunk(P, per_view, budget);
+    const size_t chunk = (size_t)P.chunk;
     b += per_view * chunk * F;
     b += (vol + (P.fast ? (size_t)g.np * g.nz * g.nview : nproj)) * F;
     if (P.fast) b += (spect::fwd_records_floats(P) + spect::adj_records_floats(P)) * F;
@@ -407,7 +454,7 @@ size_t plan_bytes_bound(const spect_plan_s& P)
         // attenuation factors of every view, or of one chunk plus mu in the internal layout
         b += P.recompute ? ((size_t)g.ny * P.ps * chunk + volt) * F : (size_t)g.ny * P.ps * g.nview * F;
         b += 4 * volt * F;
-        b += nproj * (size_t)spect::fused_groups(P) * F + (size_t)g.nview * g.ny * P.ts * F;
+        b += std::max(nproj * (size_t)spect::fused_groups(P), volt) * F + (size_t)g.nview * g.ny * P.ts * F;
         // patch gather: boxes and box-local entries (at most 8 per list)
         const size_t np = (size_t)((g.nx + 7) / 8) * ((g.ny + 7) / 8) * g.nview;
         b += np * 16 + np * 64 * 8 * sizeof(spect::AdjEntry) + np * 16;  // + rotation boxes
@@ -447,23 +494,17 @@ spect_status spect_plan_bytes(int nx, int ny, int nz, int nview, int px, int pz,
     P.cls_x = 3;
     P.cls_z = nz >= 2 ? 3 : 1;
     P.rot3 = (flags & SPECT_PLAN_ROTATION_3PASS) != 0;
-    if (P.separable && !(flags & SPECT_PLAN_LOW_MEMORY)) {
-        P.bucket = spect::fused_bucket(g, (size_t)smem_optin, &P.fwd_nT);
-        P.fast = P.bucket > 0;
-    } else if (!(flags & SPECT_PLAN_LOW_MEMORY)) {
-        P.bucket = spect::fused_dir_bucket(g, (size_t)smem_optin);
-        P.fast = P.bucket > 0;
-        P.fwd_nT = 1;
-    }
-    P.recompute = (flags & SPECT_PLAN_RECOMPUTE_ATTENUATION) != 0 && P.fast && !P.rot3;
+    P.low = (flags & SPECT_PLAN_LOW_MEMORY) != 0;
+    P.bucket = P.separable ? spect::fused_bucket(g, (size_t)smem_optin, &P.min_nT)
+                           : spect::fused_dir_bucket(g, (size_t)smem_optin);
+    P.fast = P.bucket > 0;
+    P.recompute = ((flags & SPECT_PLAN_RECOMPUTE_ATTENUATION) != 0 || P.low) && P.fast && !P.rot3;
     P.smem_optin = smem_optin;
-    if (P.fast) {
-        if (cudaDeviceGetAttribute(&P.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(SPECT_ECUDA, "device query failed");
-        }
-        spect::default_shape(P);
+    if (cudaDeviceGetAttribute(&P.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(SPECT_ECUDA, "device query failed");
     }
+    configure_views(&P);
     *bytes = plan_bytes_bound(P);
     return SPECT_OK;
 }
@@ -542,30 +583,27 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         PLAN_TRY(cudaDeviceGetAttribute(&pools, cudaDevAttrMemoryPoolsSupported, dev), "device query");
         P->pooled = pools != 0;
     }
-    if (P->separable && !(flags & SPECT_PLAN_LOW_MEMORY)) {
-        P->bucket = spect::fused_bucket(g, (size_t)smem_optin, &P->fwd_nT);
-        P->adj_nT = P->fwd_nT;
-        P->fast = P->bucket > 0;
-    } else if (!(flags & SPECT_PLAN_LOW_MEMORY)) {
-        // full PSF: the fused full-PSF blur kernels, untiled planes only
-        P->bucket = spect::fused_dir_bucket(g, (size_t)smem_optin);
-        P->fast = P->bucket > 0;
-        P->fwd_nT = P->adj_nT = 1;
-    }
+    P->low = (flags & SPECT_PLAN_LOW_MEMORY) != 0;
+    P->bucket = P->separable ? spect::fused_bucket(g, (size_t)smem_optin, &P->min_nT)
+                             : spect::fused_dir_bucket(g, (size_t)smem_optin);
+    P->fast = P->bucket > 0;
     PLAN_TRY(cudaDeviceGetAttribute(&P->sms, cudaDevAttrMultiProcessorCount, dev), "device query");
-    if (P->fast) spect::default_shape(*P);
     P->rot3 = (flags & SPECT_PLAN_ROTATION_3PASS) != 0;
-    if (P->rot3 && !P->fast) {
+    if (P->rot3 && (!P->fast || P->low)) {
         free_plan(P);
         return fail(SPECT_EUNSUPPORTED, "the three-pass rotation runs on the fused kernels (not a low-memory plan)");
     }
     P->recompute = (flags & SPECT_PLAN_RECOMPUTE_ATTENUATION) != 0;
-    if (P->recompute && (!P->fast || P->rot3)) {
+    if (P->recompute && (!P->fast || P->rot3 || P->low)) {
         free_plan(P);
         return fail(SPECT_EUNSUPPORTED,
                     "recomputed attenuation runs on the fused kernels with the bilinear rotation (not with a "
                     "low-memory plan, the three-pass rotation, or a geometry the fused kernels do not fit)");
     }
+    // a low-memory plan the fused kernels fit runs them in small view chunks, its
+    // attenuation recomputed (96x96x64, 60 views, 21 taps: EM update 3327 us with the
+    // low-memory kernels); the others keep the low-memory kernels
+    if (P->low && P->fast) P->recompute = 1;
     if (P->separable) {
         P->sep_tk = spect::choose_sep_tile(g, P->cls_z, (size_t)smem_optin);
         if (P->sep_tk < 1) {
@@ -645,7 +683,7 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         PLAN_TRY(e4, "adjacency count");
         if (P->rot3) mx = std::max(mx, 8);  // eight entries per (voxel, view) for the three-pass lists
         P->adj_max = mx;
-        if (P->fast && mx > 8) P->fast = 0;  // fixed-length lists are instantiated up to 8 entries
+        if (P->fast && mx > 8) P->fast = P->recompute = 0;  // fixed-length lists are instantiated up to 8 entries
         if (P->fast) {
             PLAN_ALLOC(P->adjf, nlist * (size_t)std::max(mx, 1), "adjacency lists");
             if (mx < 1) P->adj_max = 1;
@@ -681,10 +719,8 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
     }
 
     // work slab and EM buffers
-    const size_t budget = P->recompute ? recompute_budget_bytes() : slab_budget_bytes(P->fast);
-    // the fused path stores padded planes (rotated image planes or adjoint planes)
+    configure_views(P);
     const size_t per_view = std::max(vol, P->fast ? spect::fused_slab_per_view(*P) : vol);
-    P->chunk = view_chunk(*P, per_view, budget);
     PLAN_ALLOC(P->slab, per_view * (size_t)P->chunk, "work slab");
     P->slab_cap = per_view * (size_t)P->chunk;
     // fused adjoint: all views of the slab in one pass by default (measured
@@ -716,8 +752,8 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         PLAN_ALLOC(P->ut, volt, "internal regulariser target");
         for (float* p : {P->xt, P->et, P->st, P->ut})  // defines their padding
             PLAN_TRY(cudaMemsetAsync(p, 0, volt * sizeof(float), st), "clear internal volume");
-        PLAN_ALLOC(P->part, nproj * (size_t)spect::fused_groups(*P), "depth-group partial sums");
-        P->part_cap = nproj * (size_t)spect::fused_groups(*P);
+        P->part_cap = part_floats(*P, P->adj_chunk);
+        PLAN_ALLOC(P->part, P->part_cap, "depth-group partial sums");
         // mu in the [j][i][k] layout (temporary, the slab serves as scratch)
         PLAN_TRY(spect::launch_transpose(P->mu, P->slab, nz, (int)nxy, (int)nxy, g.kp, st), "mu transpose launch");
         if (P->rot3) {
@@ -981,7 +1017,7 @@ spect_status spect_plan_info(spect_plan P, int* separable, int* fused, int* view
 {
     if (!P) return fail(SPECT_EINVAL, "plan is NULL");
     if (separable) *separable = P->separable;
-    if (fused) *fused = P->fast;
+    if (fused) *fused = P->fast && !P->low;
     if (view_chunk) *view_chunk = P->chunk;
     if (device_bytes) *device_bytes = P->bytes;
     return SPECT_OK;
@@ -1046,7 +1082,7 @@ spect_status refresh_maps(spect_plan_s* P)
 // shape needs more room.
 spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, int adj_tiles, cudaStream_t st)
 {
-    if (!P->fast) return fail(SPECT_EUNSUPPORTED, "launch-shape tuning applies to the fused kernels only");
+    if (!P->fast || P->low) return fail(SPECT_EUNSUPPORTED, "launch-shape tuning applies to the fused kernels only");
     const Geometry& g = P->g;
     if (J < 1 || J > 32 || adj_J < 1 || adj_J > 32 || tiles < 1 || adj_tiles < 1)
         return fail(SPECT_EINVAL, "fused_J and adj_J must be in [1, 32], tiles >= 1");
@@ -1073,9 +1109,10 @@ spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, int adj_t
     const size_t per_view = std::max(vol, spect::fused_slab_per_view(*P));
     const size_t budget = P->recompute ? recompute_budget_bytes() : slab_budget_bytes(true);
     const int chunk = view_chunk(*P, per_view, budget);
+    const int adj_chunk = P->adj_chunk_req > 0 ? std::min(P->adj_chunk_req, chunk) : chunk;
     spect_status r = realloc_floats(P, &P->slab, &P->slab_cap, per_view * (size_t)chunk, st, "work slab");
     if (r == SPECT_OK)
-        r = realloc_floats(P, &P->part, &P->part_cap, nproj * (size_t)spect::fused_groups(*P), st,
+        r = realloc_floats(P, &P->part, &P->part_cap, part_floats(*P, adj_chunk), st,
                            "depth-group partial sums");
     if (r == SPECT_OK && P->recompute)  // the attenuation factors of one chunk
         r = realloc_floats(P, &P->mubar, &P->mubar_cap, (size_t)g.ny * P->ps * chunk, st, "attenuation factors");
@@ -1089,7 +1126,7 @@ spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, int adj_t
         return fail(r, msg);
     }
     P->chunk = chunk;
-    P->adj_chunk = P->adj_chunk_req > 0 ? std::min(P->adj_chunk_req, chunk) : chunk;
+    P->adj_chunk = adj_chunk;
     return refresh_maps(P);
 }
 
@@ -1165,7 +1202,7 @@ spect_status spect_plan_get_tuning(spect_plan P, int* fused_J, int* adj_J, int* 
 spect_status spect_plan_autotune(spect_plan P, spect_stream stream)
 {
     if (!P) return fail(SPECT_EINVAL, "plan is NULL");
-    if (!P->fast) return SPECT_OK;  // the low-memory kernels have no launch shape to choose
+    if (!P->fast || P->low) return SPECT_OK;  // low-memory plans keep their launch shapes
     cudaStream_t st = (cudaStream_t)stream;
     const Geometry& g = P->g;
     int dev = 0;

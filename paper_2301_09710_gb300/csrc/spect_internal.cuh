@@ -87,6 +87,9 @@ struct spect_plan_s {
     int smem_optin = 0;          // shared memory a block may opt in to (bytes)
     int sms = 0;                 // multiprocessors of the device
     int fast = 0;                // 1 when the fused kernels serve this plan
+    int low = 0;                 // SPECT_PLAN_LOW_MEMORY (with fast: the fused kernels in small view chunks)
+    int min_nT = 1;              // fewest column tiles of the blurs (geometry, SPECT_FUSED_TILES)
+    int shape_views = 0;         // views per pass the default launch shapes are chosen for
     int bucket = 0;              // padded tap count of the fused kernels
     int fused_J = 8;             // depth planes per fused forward block
     int fwd_nT = 1;              // column tiles per plane of the fused forward blur
@@ -287,6 +290,13 @@ struct EmArgs {
     float beta = 0.f;
 };
 
+// The view sum of A' over several passes: each resumes the compensated sums (out, comp)
+// that the last one left, so the result does not depend on how the views are split.
+struct PassState {
+    int resume = 0, more = 0;  // earlier passes' sums in out / comp; further passes follow
+    float* comp = nullptr;     // compensation terms (only read or written when resume or more)
+};
+
 // Kahan-compensated accumulator for depth and view sums.
 struct KSum {
     float s = 0.f, c = 0.f;
@@ -452,6 +462,7 @@ size_t adj_records_floats(const spect_plan_s& P);
 cudaError_t launch_records(const spect_plan_s& P, cudaStream_t st);
 int fwd_tiles(const spect_plan_s& P);
 int adj_tiles(const spect_plan_s& P);
+// default launch shapes of the blur kernels for passes of P.shape_views views
 void default_shape(spect_plan_s& P);
 // Bucket of the fused full-PSF kernels (untiled planes), 0 when they do not fit.
 int fused_dir_bucket(const Geometry& g, size_t smem_limit);
@@ -489,9 +500,9 @@ inline const float* mubar_for(const spect_plan_s& P, int l0)
     return reinterpret_cast<const float*>(reinterpret_cast<uintptr_t>(P.mubar) -
                                           (uintptr_t)l0 * P.g.ny * P.ps * sizeof(float));
 }
-cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, float* out, int accumulate, EmArgs em,
+cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,
                               cudaStream_t st);
-cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, int accumulate, EmArgs em,
+cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,
                              cudaStream_t st);
 bool direct_fits(const Geometry& g, size_t smem_limit);
 // grouped launches of a batch of plans (grouped.cu, gather.cu): per stage and

@@ -67,3 +67,58 @@ def test_full_psf_launch_shapes(case):
     assert_close(host(plan.back(dev(yy))), oracle.back(yy, prob.mu, psf, prob.dy, ang), what="A' y")
     plan.check()
     plan.close()
+
+
+@pytest.mark.parametrize("path", ["lowmem", "direct_lowmem"])
+def test_psf_wider_than_the_fused_kernels(path):
+    """A 41-tap PSF: the low-memory kernels (a low-memory plan of up to 37 taps runs the
+    fused kernels in view chunks), A, A' and one EM step."""
+    need_gpu()
+    nx, nz, nview, p = 40, 18, 5, 41
+    prob = synthetic.random_problem(7, nx=nx, nz=nz, nview=nview, px=p, pz=p, mu_scale=0.05)
+    ang = oracle.default_angles(nview)
+    plan = make_plan(prob, ang, path)
+    assert not plan.info()["fused"]
+    psf = oracle.psf_from_factors(prob.fx, prob.fz) if path == "lowmem" else prob.full_psf().astype(np.float64)
+    v_o = oracle.forward(prob.x, prob.mu, psf, prob.dy, ang)
+    assert_close(host(plan.forward(dev(prob.x))), v_o, what="A x")
+    yy = np.random.default_rng(8).uniform(0.5, 1.5, plan.proj_shape).astype(np.float32)
+    assert_close(host(plan.back(dev(yy))), oracle.back(yy, prob.mu, psf, prob.dy, ang), what="A' y")
+    x0 = np.full(prob.x.shape, 0.5, np.float32)
+    xg = dev(x0)
+    plan.em_step(xg, dev(yy), None, niter=1)
+    assert_close(host(xg), oracle.em_step(x0, yy, None, prob.mu, psf, prob.dy, ang), what="EM step")
+    plan.check()
+    plan.close()
+
+
+def test_low_memory_plan_in_view_chunks(monkeypatch):
+    """A low-memory plan of up to 37 taps runs the fused kernels in view chunks: A and A' over
+    several passes, and its memory bound."""
+    need_gpu()
+    from paper_2301_09710_gb300.projector import plan_bytes
+    prob = synthetic.random_problem(9, nx=48, nz=21, nview=14, px=11, pz=9, mu_scale=0.05)
+    ang = oracle.default_angles(14)
+    monkeypatch.setenv("SPECT_SLAB_MB", "2")
+    plan = make_plan(prob, ang, "lowmem")
+    info = plan.info()
+    assert not info["fused"] and 1 <= info["view_chunk"] < 14
+    assert info["device_bytes"] <= plan_bytes(48, 21, 14, 11, 9, low_memory=True)
+    monkeypatch.delenv("SPECT_SLAB_MB")
+    one = make_plan(prob, ang, "lowmem")
+    assert one.info()["view_chunk"] == 14
+    psf = oracle.psf_from_factors(prob.fx, prob.fz)
+    v_o = oracle.forward(prob.x, prob.mu, psf, prob.dy, ang)
+    assert_close(host(plan.forward(dev(prob.x))), v_o, what="A x")
+    yy = np.random.default_rng(9).uniform(0.5, 1.5, plan.proj_shape).astype(np.float32)
+    xb = host(plan.back(dev(yy)))
+    assert_close(xb, oracle.back(yy, prob.mu, psf, prob.dy, ang), what="A' y")
+    # each pass resumes the compensated view sums of the last one
+    assert np.array_equal(xb, host(one.back(dev(yy)))), "A' depends on how the views are split"
+    x0 = np.full(prob.x.shape, 0.5, np.float32)
+    xg = dev(x0)
+    plan.em_step(xg, dev(yy), None, niter=1)
+    assert_close(host(xg), oracle.em_step(x0, yy, None, prob.mu, psf, prob.dy, ang), what="EM step")
+    plan.check()
+    plan.close()
+    one.close()
