@@ -668,7 +668,7 @@ __global__ void __launch_bounds__(kDirThreads, 1)
 template <int MAXE>
 __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const AdjEntry* __restrict__ adj,
                                                    const float* __restrict__ slab, int l0, int nv, float* out,
-                                                   PassState ps_, EmArgs em)
+                                                   PassState ps_, int seglen, EmArgs em)
 {
     using VT = float4;
     constexpr int VEC = 4;
@@ -696,8 +696,9 @@ __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const Adj
     // four views per step: all entry loads, then all slab loads, are issued
     // before any is used, so the chain of dependent loads is 4x shorter
     constexpr int UV = 4;
-    int v = 0;
-    for (; v + UV <= nv; v += UV) {
+    KSum tot[VEC];
+    for (int v_end = min(nv, seglen), v = 0; v < nv; v_end = min(nv, v_end + seglen)) {
+    for (; v + UV <= v_end; v += UV) {
         AdjEntry a[UV][MAXE];
 #pragma unroll
         for (int w = 0; w < UV; ++w)
@@ -725,7 +726,7 @@ __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const Adj
         e += UV * MAXE;
         t += UV * vstride;
     }
-    for (; v < nv; ++v) {
+    for (; v < v_end; ++v) {
         AdjEntry a[MAXE];
 #pragma unroll
         for (int m = 0; m < MAXE; ++m) a[m] = e[m];
@@ -746,6 +747,14 @@ __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const Adj
         e += MAXE;
         t += vstride;
     }
+    if (seglen < nv) {  // the segments of the patch gather, added in order
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) tot[u].merge(acc[u].s, acc[u].c), acc[u] = KSum();
+    }
+    }
+    if (seglen < nv)
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) acc[u] = tot[u];
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
         if (ps_.more) {
@@ -1249,9 +1258,10 @@ cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, 
     const size_t n = (size_t)P.g.nx * P.g.ny * (P.g.kp / 4);
     const unsigned blocks = (unsigned)((n + 255) / 256);
     const float* src = P.slab;
+    const int segs = P.adj_chunk >= P.g.nview ? P.gsegs : 1, seglen = (nv + segs - 1) / segs;  // as the patch gather
     switch (P.adj_max) {
 #define SPECT_ADJ(M)                                                                                                 \
-    case M: k_adj_rot_t<M><<<blocks, 256, 0, st>>>(P.g, P.ps, P.adjf, src, l0, nv, out, pass, em); break;
+    case M: k_adj_rot_t<M><<<blocks, 256, 0, st>>>(P.g, P.ps, P.adjf, src, l0, nv, out, pass, seglen, em); break;
         SPECT_ADJ(1) SPECT_ADJ(2) SPECT_ADJ(3) SPECT_ADJ(4) SPECT_ADJ(5) SPECT_ADJ(6) SPECT_ADJ(7) SPECT_ADJ(8)
 #undef SPECT_ADJ
         default: return cudaErrorInvalidValue;

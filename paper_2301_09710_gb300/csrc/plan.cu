@@ -135,7 +135,7 @@ void free_plan(spect_plan_s* P, cudaStream_t st)
     for (cudaEvent_t e : P->evpool) cudaEventDestroy(e);
     void* ptrs[] = {P->mu, P->psf, P->psf_adj, P->fx, P->fz, P->fx_adj, P->fz_adj, P->rot, P->adj_off, P->adj,
                     P->frec, P->arec, P->slab, P->e, P->ratio, P->s, P->mubar, P->xt, P->et, P->st, P->part, P->adjf, P->err, P->rtab, P->ut,
-                    P->gboxes, P->gent, P->rboxes, P->r3_tab, P->mut};
+                    P->gboxes, P->gent, P->gcount, P->rboxes, P->r3_tab, P->mut};
     for (void* p : ptrs) raw_free(P, p, st);
     delete P;
 }
@@ -198,12 +198,14 @@ size_t low_budget_bytes(const spect_plan_s& P)
     return (size_t)std::max(held - fixed, 24.0 * (1 << 20));
 }
 
-// The forward's depth-group partial sums; between the adjoint's passes (adj_chunk views
-// each) the same buffer holds the compensation terms of the view sums.
+// The forward's depth-group partial sums; in A' the same buffer holds the sums and
+// compensation terms of the view segments, or between its passes (adj_chunk views
+// each) the compensation terms of the view sums.
 size_t part_floats(const spect_plan_s& P, int adj_chunk)
 {
     const size_t part = (size_t)P.g.nx * P.g.nz * P.g.nview * spect::fused_groups(P);
-    return adj_chunk < P.g.nview ? std::max(part, (size_t)P.g.nx * P.g.ny * P.g.kp) : part;
+    const size_t volt = (size_t)P.g.nx * P.g.ny * P.g.kp;
+    return std::max(part, adj_chunk < P.g.nview ? volt : (P.gsegs > 1 ? 2 * P.gsegs * volt : 0));
 }
 
 // Launch shapes and views per pass of a plan: the work slab (and a recomputing plan's
@@ -218,6 +220,7 @@ void configure_views(spect_plan_s* P)
                           : P->recompute   ? recompute_budget_bytes()
                                            : slab_budget_bytes(P->fast);
     P->chunk = view_chunk(*P, per_view, budget);
+    P->gsegs = P->fast ? spect::gather_segments(*P) : 1;
     if (P->fast && P->chunk < P->g.nview) {
         P->shape_views = P->chunk;
         spect::default_shape(*P);
@@ -454,10 +457,12 @@ size_t plan_bytes_bound(const spect_plan_s& P)
         // attenuation factors of every view, or of one chunk plus mu in the internal layout
         b += P.recompute ? ((size_t)g.ny * P.ps * chunk + volt) * F : (size_t)g.ny * P.ps * g.nview * F;
         b += 4 * volt * F;
-        b += std::max(nproj * (size_t)spect::fused_groups(P), volt) * F + (size_t)g.nview * g.ny * P.ts * F;
+        b += std::max(nproj * (size_t)spect::fused_groups(P), 2 * (size_t)P.gsegs * volt) * F +
+             (size_t)g.nview * g.ny * P.ts * F;
         // patch gather: boxes and box-local entries (at most 8 per list)
         const size_t np = (size_t)((g.nx + 7) / 8) * ((g.ny + 7) / 8) * g.nview;
         b += np * 16 + np * 64 * 8 * sizeof(spect::AdjEntry) + np * 16;  // + rotation boxes
+        b += np / g.nview * ((g.kp + 15) / 16) * sizeof(int);           // segment arrivals
         if (P.rot3)  // the eight-tap table
             b += (size_t)g.nview * g.ny * 16 * (size_t)g.nx * F;
     }
@@ -1070,10 +1075,11 @@ spect_status realloc_floats(spect_plan_s* P, float** p, size_t* cap, size_t need
     return SPECT_OK;
 }
 
-// The blur kernels' tensor maps for the plan's present buffers, chunk and launch shapes.
+// The kernels' tensor maps for the plan's present buffers, chunk and launch shapes.
 spect_status refresh_maps(spect_plan_s* P)
 {
     SPECT_CUDA_TRY(spect::build_maps(*P), "tensor maps of the blur kernels");
+    SPECT_CUDA_TRY(spect::build_gather_maps(*P), "tensor maps of the patch gather");
     return SPECT_OK;
 }
 
@@ -1141,7 +1147,13 @@ spect_status single_pass(spect_plan_s* P, cudaStream_t st)
     const size_t vol = (size_t)g.nx * g.ny * g.nz;
     const size_t per_view = std::max(vol, spect::fused_slab_per_view(*P));
     spect_status r = realloc_floats(P, &P->slab, &P->slab_cap, per_view * (size_t)g.nview, st, "work slab");
-    if (r != SPECT_OK) return r;
+    if (r == SPECT_OK)
+        r = realloc_floats(P, &P->part, &P->part_cap, part_floats(*P, g.nview), st, "depth-group partial sums");
+    if (r != SPECT_OK) {
+        const std::string msg = g_err;
+        refresh_maps(P);  // the slab may have moved
+        return fail(r, msg);
+    }
     P->chunk = g.nview;
     P->adj_chunk = g.nview;
     return refresh_maps(P);

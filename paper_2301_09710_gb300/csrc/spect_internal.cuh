@@ -52,6 +52,12 @@ struct AdjEntry {
     float w;
 };
 
+// Tensor maps of the patch gather, one per box size.
+constexpr int kGatherMaps = 6;
+struct GatherMaps {
+    CUtensorMap m[kGatherMaps];
+};
+
 }  // namespace spect
 
 struct spect_plan_s {
@@ -110,9 +116,13 @@ struct spect_plan_s {
     spect::AdjEntry* adjf = nullptr;  // nview*nx*ny*adj_max fixed-length lists
     // patch-staged adjoint gather (gather.cu); gather == 0: the list gather k_adj_rot_t
     int gather = 0;
-    int4* gboxes = nullptr;      // [patch][l] source box (i0, j0, width, height)
+    int4* gboxes = nullptr;      // [patch][l] source box (i0, j0, size, tensor map)
     spect::AdjEntry* gent = nullptr;  // [patch][l][64][adj_max] box-local entries
-    int gbw = 0, gbh = 0, gnpx = 0, gnpy = 0;
+    int gnpx = 0, gnpy = 0;
+    int gnm = 0, gsize[spect::kGatherMaps] = {};  // box sizes, ascending
+    spect::GatherMaps gmaps;     // the slab, boxed at each size (build_gather_maps)
+    int gsegs = 1;               // view segments of A' when the views go in one pass (gather_segments)
+    int* gcount = nullptr;       // [patch][k run] segment arrivals
     // patch-staged forward rotation (rotpatch.cu): available when rotpatch != 0,
     // used instead of k_rot_fwd when rotpatch_on != 0 (chosen by the autotuner)
     int rotpatch = 0;
@@ -307,6 +317,12 @@ struct KSum {
         c = (t - s) - y;
         s = t;
     }
+    // another such sum of s2 - c2
+    __device__ __forceinline__ void merge(float s2, float c2)
+    {
+        add(s2);
+        add(-c2);
+    }
     __device__ __forceinline__ float value() const { return s - c; }
 };
 
@@ -487,6 +503,9 @@ cudaError_t launch_pad_rows(const spect_plan_s& P, const float* v, float* out, c
 cudaError_t launch_fwd_reduce(const spect_plan_s& P, float* v, const float* em_y, const float* em_rbar,
                               cudaStream_t st);
 cudaError_t build_gather(spect_plan_s& P, cudaStream_t st);
+// (re)encode P.gmaps after the slab or the view chunk changed
+cudaError_t build_gather_maps(spect_plan_s& P);
+int gather_segments(const spect_plan_s& P);
 cudaError_t build_rotpatch(spect_plan_s& P, cudaStream_t st);
 cudaError_t launch_rot_patch(const spect_plan_s& P, int l0, int nv, cudaStream_t st);
 // the attenuation factors of views l0 .. l0+nv-1 (recomputing plans: into the chunk buffer)
