@@ -36,14 +36,14 @@ namespace spect {
 // out[c][r] = in[r][c] for an R x C matrix (tiled through shared memory).
 __global__ void k_transpose(const float* __restrict__ in, float* __restrict__ out, int R, int C, int ip, int op)
 {
+    wait_previous_kernel();
     transpose_body(in, out, R, C, ip, op, blockIdx.x, blockIdx.y);
 }
 
 cudaError_t launch_transpose(const float* in, float* out, int R, int C, int ip, int op, cudaStream_t st)
 {
     dim3 grid((C + 31) / 32, (R + 31) / 32);
-    k_transpose<<<grid, dim3(32, 8), 0, st>>>(in, out, R, C, ip, op);
-    return cudaGetLastError();
+    return launch_chained(k_transpose, grid, dim3(32, 8), 0, st, in, out, R, C, ip, op);
 }
 
 // mubar[l][j][i][k] = exp(-dy (mu~(j)/2 + sum_{s>j} mu~(s))), Eq. (1), for every
@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(kRotThreads, TAPS == 4 ? 5 : 3) k_rot_fwd(Geom
                                                                             const float* __restrict__ mubar,
                                                                             float* __restrict__ wsl, int l0)
 {
+    wait_previous_kernel();
     rot_body<TAPS>(g, d, tabs, xt, mubar, wsl, l0, blockIdx.x, blockIdx.y);
 }
 
@@ -226,6 +227,7 @@ __global__ void __launch_bounds__(FwdBlock<P>::T, KS ? 1 : FwdBlock<P>::B) k_fwd
                                                                      const float* __restrict__ rec,
                                                                      float* __restrict__ part, int l0, int* err)
 {
+    wait_previous_kernel();
     const int grp = blockIdx.x / d.nT;
     fwd_sep_body<P, RACC, KS>(g, d, &tmap, rec, part, l0, err, grp, blockIdx.y, blockIdx.x - grp * d.nT);
 }
@@ -269,6 +271,7 @@ __global__ void k_fwd_records(Geometry g, int P, int PT, int nkb, const float* _
 __global__ void k_fwd_reduce(const float* __restrict__ part, int G, size_t nproj, float* __restrict__ v, int nx, int np,
                              const float* __restrict__ em_y, const float* __restrict__ em_rbar)
 {
+    wait_previous_kernel();
     const size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= nproj) return;
     KSum acc;  // up to ny partials (J = 1): compensated
@@ -285,6 +288,7 @@ __global__ void k_fwd_reduce(const float* __restrict__ part, int G, size_t nproj
 // out (rows of np) = v (n rows of nx)
 __global__ void k_pad_rows(const float* __restrict__ v, float* __restrict__ out, size_t n, int nx, int np)
 {
+    wait_previous_kernel();
     const size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (o < n * nx) out[o + o / nx * (np - nx)] = v[o];
 }
@@ -292,8 +296,7 @@ __global__ void k_pad_rows(const float* __restrict__ v, float* __restrict__ out,
 cudaError_t launch_pad_rows(const spect_plan_s& P, const float* v, float* out, cudaStream_t st)
 {
     const size_t rows = (size_t)P.g.nz * P.g.nview, n = rows * P.g.nx;
-    k_pad_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(v, out, rows, P.g.nx, P.g.np);
-    return cudaGetLastError();
+    return launch_chained(k_pad_rows, (unsigned)((n + 255) / 256), 256, 0, st, v, out, rows, P.g.nx, P.g.np);
 }
 
 // Blur adjoint + attenuation: one block per (column tile, depth group of J planes, view).
@@ -407,6 +410,7 @@ __global__ void __launch_bounds__(kDirThreads, 1) k_fwd_dir_fused(const __grid_c
     using S = Sep<P>;
     constexpr int C = S::C, CZ = S::CZ, ZH = S::ZH, WZ = S::WZ, PT = S::PT;
     constexpr int TAPS = (P * PT + 31) & ~31;
+    wait_previous_kernel();
     extern __shared__ __align__(128) float smf[];
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     const int tid = threadIdx.x, T = blockDim.x;
@@ -536,6 +540,7 @@ __global__ void __launch_bounds__(kDirThreads, 1)
     using S = Sep<P>;
     constexpr int C = S::C, CZ = S::CZ, ZH = S::ZH, WZ = S::WZ, PT = S::PT, EC = AdjRec<P>::EC;
     constexpr int SET = P * (PT + 2 * EC);
+    wait_previous_kernel();
     extern __shared__ __align__(1024) float sma[];
     const int nx = g.nx, ny = g.ny, nz = g.nz;
     float* MB = sma;                                   // [KR / 16][TI][16], 64-byte swizzled
@@ -672,6 +677,7 @@ __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const Adj
 {
     using VT = float4;
     constexpr int VEC = 4;
+    wait_previous_kernel();
     const int nxy = g.nx * g.ny;
     const int nzv = g.kp / VEC;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -822,8 +828,7 @@ cudaError_t fwd_launch(const spect_plan_s& Pl, const float* /*xt: the blur reads
                         : (Pl.low ? k_fwd_sep_fused<P, true, true> : k_fwd_sep_fused<P, true, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(d.G * d.nT, nv), d.T, smem, st>>>(Pl.fmap, Pl.g, d, Pl.frec, Pl.part, l0, Pl.err);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3(d.G * d.nT, nv), d.T, smem, st, Pl.fmap, Pl.g, d, Pl.frec, Pl.part, l0, Pl.err);
 }
 
 template <int P>
@@ -837,9 +842,8 @@ cudaError_t adj_launch(const spect_plan_s& Pl, const float* v, int l0, int nv, c
     e = cudaFuncSetAttribute(k_adj_sep_fused<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // a recomputing plan's factors are those of views l0 .. at chunk-relative positions
-    k_adj_sep_fused<P><<<dim3(d.G * d.nT, nv), d.T, smem, st>>>(Pl.amap_mu, Pl.amap_t, vmap, Pl.g, d, Pl.arec, l0,
-                                                                Pl.recompute ? l0 : 0, Pl.err);
-    return cudaGetLastError();
+    return launch_chained(k_adj_sep_fused<P>, dim3(d.G * d.nT, nv), d.T, smem, st, Pl.amap_mu, Pl.amap_t, vmap, Pl.g, d,
+                          Pl.arec, l0, Pl.recompute ? l0 : 0, Pl.err);
 }
 }  // namespace
 
@@ -925,8 +929,8 @@ cudaError_t dir_fwd_launch(const spect_plan_s& Pl, int l0, int nv, cudaStream_t 
     auto kern = Pl.low ? k_fwd_dir_fused<P, true> : k_fwd_dir_fused<P, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(d.nT * d.nkr * d.G, nv), d.T, smem, st>>>(Pl.fmap, Pl.g, d, Pl.frec, Pl.part, l0, Pl.err);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3(d.nT * d.nkr * d.G, nv), d.T, smem, st, Pl.fmap, Pl.g, d, Pl.frec, Pl.part, l0,
+                          Pl.err);
 }
 
 template <int P>
@@ -936,9 +940,8 @@ cudaError_t dir_adj_launch(const spect_plan_s& Pl, const float* v, int l0, int n
     const size_t smem = dir_smem_adj<P>(d);
     cudaError_t e = cudaFuncSetAttribute(k_adj_dir_fused<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_adj_dir_fused<P><<<dim3(d.nT * d.nkr * d.G, nv), d.T, smem, st>>>(Pl.amap_mu, Pl.amap_t, Pl.g, d, v, Pl.arec, l0,
-                                                                        Pl.recompute ? l0 : 0, Pl.err);
-    return cudaGetLastError();
+    return launch_chained(k_adj_dir_fused<P>, dim3(d.nT * d.nkr * d.G, nv), d.T, smem, st, Pl.amap_mu, Pl.amap_t, Pl.g, d,
+                          v, Pl.arec, l0, Pl.recompute ? l0 : 0, Pl.err);
 }
 }  // namespace
 
@@ -1056,9 +1059,8 @@ cudaError_t launch_fused_rotate(const spect_plan_s& P, const float* xt, int l0, 
     if (P.rotpatch && P.rotpatch_on && xt == P.xt) return launch_rot_patch(P, l0, nv, st);
     const RotDims d = rot_dims(P.g, P.ps, P.rot3 ? rot3_ts8(P.g.nx) : P.ts, nv, P.sms);
     const dim3 grid(d.nb * ((P.g.ny + d.JP - 1) / d.JP), nv);
-    if (P.rot3) k_rot_fwd<8><<<grid, kRotThreads, 0, st>>>(P.g, d, P.r3_tab, xt, mubar_for(P, l0), P.slab, l0);
-    else k_rot_fwd<4><<<grid, kRotThreads, 0, st>>>(P.g, d, P.rtab, xt, mubar_for(P, l0), P.slab, l0);
-    return cudaGetLastError();
+    return launch_chained(P.rot3 ? k_rot_fwd<8> : k_rot_fwd<4>, grid, kRotThreads, 0, st, P.g, d,
+                          P.rot3 ? P.r3_tab : P.rtab, xt, mubar_for(P, l0), P.slab, l0);
 }
 
 namespace {
@@ -1247,9 +1249,8 @@ cudaError_t launch_fwd_reduce(const spect_plan_s& P, float* v, const float* em_y
                               cudaStream_t st)
 {
     const size_t nproj = (size_t)P.g.nx * P.g.nz * P.g.nview;
-    k_fwd_reduce<<<(unsigned)((nproj + 255) / 256), 256, 0, st>>>(P.part, fused_groups(P), nproj, v, P.g.nx, P.g.np,
-                                                                  em_y, em_rbar);
-    return cudaGetLastError();
+    return launch_chained(k_fwd_reduce, (unsigned)((nproj + 255) / 256), 256, 0, st, P.part, fused_groups(P), nproj, v,
+                          P.g.nx, P.g.np, em_y, em_rbar);
 }
 
 cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,
@@ -1261,12 +1262,11 @@ cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, 
     const int segs = P.adj_chunk >= P.g.nview ? P.gsegs : 1, seglen = (nv + segs - 1) / segs;  // as the patch gather
     switch (P.adj_max) {
 #define SPECT_ADJ(M)                                                                                                 \
-    case M: k_adj_rot_t<M><<<blocks, 256, 0, st>>>(P.g, P.ps, P.adjf, src, l0, nv, out, pass, seglen, em); break;
+    case M: return launch_chained(k_adj_rot_t<M>, blocks, 256, 0, st, P.g, P.ps, P.adjf, src, l0, nv, out, pass, seglen, em);
         SPECT_ADJ(1) SPECT_ADJ(2) SPECT_ADJ(3) SPECT_ADJ(4) SPECT_ADJ(5) SPECT_ADJ(6) SPECT_ADJ(7) SPECT_ADJ(8)
 #undef SPECT_ADJ
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace spect

@@ -285,6 +285,7 @@ __global__ void __launch_bounds__(16 * KC + 32) k_adj_gather(const __grid_consta
                                                          const AdjEntry* __restrict__ pent, float* out,
                                                          PassState pass, EmArgs em, int* err)
 {
+    wait_previous_kernel();
     // the k runs of a patch are adjacent blocks, so they run side by side and the
     // patch's entries, which each of them reads, come from DRAM about once
     // (0.246 -> 0.213 ms per 128-view launch against the patch-major order)
@@ -526,19 +527,18 @@ cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, float* out,
         cudaError_t e = cudaFuncSetAttribute(k_adj_gather<M, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
                                              (int)smem);                                                        \
         if (e != cudaSuccess) return e;                                                                         \
-        k_adj_gather<M, KC><<<grid, 16 * KC + 32, smem, st>>>(P.gmaps, a, P.gboxes, P.gent, out, pass, em, P.err);  \
+        return launch_chained(k_adj_gather<M, KC>, grid, 16 * KC + 32, smem, st, P.gmaps, a, P.gboxes, P.gent, out, \
+                              pass, em, P.err);                                                                 \
     }
 #define SPECT_G(M)                     \
     case M:                            \
         if (a.kc == 32) SPECT_GK(M, 32) \
-        else SPECT_GK(M, 16)           \
-        break;
+        else SPECT_GK(M, 16)
         SPECT_G(1) SPECT_G(2) SPECT_G(3) SPECT_G(4) SPECT_G(5) SPECT_G(6) SPECT_G(7) SPECT_G(8)
 #undef SPECT_GK
 #undef SPECT_G
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 // The grouped gather of a batch: per adjacency-list length, one launch over

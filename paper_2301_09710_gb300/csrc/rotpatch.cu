@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(kRT) k_rot_patch(const __grid_constant__ CUten
                                                    const float* __restrict__ rtab, const int4* __restrict__ boxes,
                                                    float* __restrict__ wsl, int* err)
 {
+    wait_previous_kernel();
     extern __shared__ __align__(128) float sm[];
     const Geometry& g = a.g;
     uint64_t* bar = reinterpret_cast<uint64_t*>(sm + 2 * (size_t)a.stage_floats);
@@ -241,8 +242,8 @@ cudaError_t launch_rot_patch(const spect_plan_s& P, int l0, int nv, cudaStream_t
     cudaError_t e = cudaFuncSetAttribute(k_rot_patch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int npy = (g.ny + kRP - 1) / kRP;
-    k_rot_patch<<<dim3(a.npx * npy, nv), kRT, smem, st>>>(P.rmap_x, P.rmap_mu, a, P.rtab, P.rboxes, P.slab, P.err);
-    return cudaGetLastError();
+    return launch_chained(k_rot_patch, dim3(a.npx * npy, nv), kRT, smem, st, P.rmap_x, P.rmap_mu, a, P.rtab, P.rboxes,
+                          P.slab, P.err);
 }
 
 }  // namespace spect

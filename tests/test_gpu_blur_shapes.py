@@ -122,3 +122,29 @@ def test_low_memory_plan_in_view_chunks(monkeypatch):
     plan.check()
     plan.close()
     one.close()
+
+
+@pytest.mark.parametrize("path", ["fused", "direct", "lowmem"])
+def test_chained_launches_keep_their_order(path):
+    """Small kernels back to back, each reading what the one before wrote and overwriting what
+    it read: a run of calls queued at once equals the same calls with a wait after each."""
+    need_gpu()
+    import torch
+    prob = synthetic.random_problem(10, nx=25, nz=7, nview=3, px=7, pz=5, mu_scale=0.05)
+    plan = make_plan(prob, oracle.default_angles(3), path)
+    yy = dev(np.random.default_rng(10).uniform(0.5, 1.5, plan.proj_shape).astype(np.float32))
+
+    def run(wait):
+        x, out = dev(np.full(prob.x.shape, 0.5, np.float32)), []
+        for _ in range(8):
+            for f in (lambda: plan.em_step(x, yy, None, niter=2), lambda: plan.forward(x), lambda: plan.back(yy * x.sum())):
+                out.append(f().clone())
+                if wait:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return [host(o) for o in out]
+
+    for a, b in zip(run(False), run(True)):
+        assert np.array_equal(a, b)
+    plan.check()
+    plan.close()
