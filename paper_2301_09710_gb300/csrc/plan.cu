@@ -675,20 +675,23 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         PLAN_TRY(raw_alloc(P, (void**)&d_max, sizeof(int), st), "adjacency max");
         cudaMemsetAsync(d_max, 0, sizeof(int), st);
         cudaError_t e1 = spect::launch_build_adjacency(*P, 0, d_counts, d_max, st);
-        std::vector<int> counts(nlist);
+        std::vector<int> counts;
         int mx = 0;
-        cudaError_t e2 = cudaMemcpyAsync(counts.data(), d_counts, nlist * sizeof(int), cudaMemcpyDeviceToHost, st);
-        cudaError_t e3 = cudaMemcpyAsync(&mx, d_max, sizeof(int), cudaMemcpyDeviceToHost, st);
+        cudaError_t e2 = cudaMemcpyAsync(&mx, d_max, sizeof(int), cudaMemcpyDeviceToHost, st);
+        cudaError_t e4 = cudaStreamSynchronize(st);
+        if (mx > 8) P->fast = P->recompute = 0;  // fixed-length lists are instantiated up to 8 entries
+        if (e2 == cudaSuccess && e4 == cudaSuccess && !P->fast) {  // fixed-length lists need only the longest
+            counts.resize(nlist);
+            e2 = cudaMemcpyAsync(counts.data(), d_counts, nlist * sizeof(int), cudaMemcpyDeviceToHost, st);
+            e4 = cudaStreamSynchronize(st);
+        }
         raw_free(P, d_counts, st);
         raw_free(P, d_max, st);
-        cudaError_t e4 = cudaStreamSynchronize(st);
         PLAN_TRY(e1, "adjacency count launch");
         PLAN_TRY(e2, "adjacency counts download");
-        PLAN_TRY(e3, "adjacency max download");
         PLAN_TRY(e4, "adjacency count");
         if (P->rot3) mx = std::max(mx, 8);  // eight entries per (voxel, view) for the three-pass lists
         P->adj_max = mx;
-        if (P->fast && mx > 8) P->fast = P->recompute = 0;  // fixed-length lists are instantiated up to 8 entries
         if (P->fast) {
             PLAN_ALLOC(P->adjf, nlist * (size_t)std::max(mx, 1), "adjacency lists");
             if (mx < 1) P->adj_max = 1;

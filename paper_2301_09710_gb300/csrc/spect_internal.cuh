@@ -334,8 +334,8 @@ struct KSum {
 // for the previous kernel to have finished and its writes to be visible.  No kernel
 // triggers its successor early: operands read through the read-only path would then be
 // written while the reader is already on the chip.  Bound by launch latency at small
-// sizes; measured: two EM updates of 64x64x32 with 32 views each 172 -> 145 us (12
-// launches), 99x99x37 with 60 views 343 -> 326 (7), 128x128x80 with 128 views 1466 -> 1451.
+// sizes; measured: two EM updates of 64x64x32, 64 views, 172 -> 145 us (12
+// launches), 99x99x53 with 60 views 343 -> 326 (7), 128x128x80 with 128 views 1466 -> 1451.
 __device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class... P, class... A>
