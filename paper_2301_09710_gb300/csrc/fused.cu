@@ -17,9 +17,9 @@
 //    sliding-window passes (i, then k; replicate padding folded into edge
 //    taps), and keeps the group's depth sum in registers; the groups' partials
 //    are added in a fixed order by a small reduce kernel (deterministic, no atomics).
-//  * Transpose: one block per (view, depth group) expands the detector plane
-//    into blurred-adjoint planes times mubar (the t slab, [v][j][i][k]); a
-//    gather kernel then sums sum_l sum_p W_l(p;q) t_l(p,k) per destination voxel
+//  * Transpose: one block per (view, depth group, column tile) expands the detector
+//    plane into blurred-adjoint planes times mubar (the t slab, [v][j][i][k]); a
+//    gather kernel (gather.cu, k_adj_rot_t) then sums sum_l sum_p W_l(p;q) t_l(p,k) per destination voxel
 //    q over fixed-length adjacency lists (weights bitwise those of A).
 #include <algorithm>
 #include <cmath>
@@ -668,8 +668,8 @@ __global__ void __launch_bounds__(kDirThreads, 1)
 // with the EM update (em_update) on the last chunk when em.x is set.  The
 // lists are laid out [q][l][e] so one destination's entries for all views are
 // contiguous; each entry holds the premultiplied offset p*kp of its source
-// column in the slab.  A thread owns four consecutive k of one destination (float4 loads).  Per view the few terms are summed plainly, the views
-// with Kahan compensation.
+// column in the slab.  A thread owns four consecutive k of one destination (float4
+// loads).  Per view the few terms are summed plainly, the views with Kahan compensation.
 template <int MAXE>
 __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const AdjEntry* __restrict__ adj,
                                                    const float* __restrict__ slab, int l0, int nv, float* out,
@@ -802,6 +802,8 @@ cudaError_t encode_v_map(const Geometry& g, const AdjDims& d, const float* v, CU
 // host side: dimensioning and launchers
 // ============================================================================
 namespace {
+// The fewest column tiles with which the bounds of the geometries taken fit `limit`
+// bytes of shared memory; 0 when none does.
 template <int P>
 int tiles_that_fit(const Geometry& g, size_t limit, int min_tiles)
 {
@@ -819,8 +821,7 @@ int tiles_that_fit(const Geometry& g, size_t limit, int min_tiles)
 }
 
 template <int P>
-cudaError_t fwd_launch(const spect_plan_s& Pl, const float* /*xt: the blur reads the work slab*/, int l0, int nv,
-                       cudaStream_t st)
+cudaError_t fwd_launch(const spect_plan_s& Pl, int l0, int nv, cudaStream_t st)
 {
     const FwdDims d = fwd_dims<P>(Pl.g, Pl.fused_J, Pl.fwd_nT, (size_t)Pl.smem_optin);
     const size_t smem = smem_fwd<P>(d);
@@ -1045,12 +1046,12 @@ int fused_groups(const spect_plan_s& P) { return (P.g.ny + P.fused_J - 1) / P.fu
         default: return cudaErrorInvalidValue;         \
     }
 
-cudaError_t launch_fused_forward(const spect_plan_s& P, const float* xt, int l0, int nv, cudaStream_t st)
+cudaError_t launch_fused_forward(const spect_plan_s& P, int l0, int nv, cudaStream_t st)
 {
     if (!P.separable) {
         SPECT_DISPATCH(dir_fwd_launch, P, l0, nv, st)
     }
-    SPECT_DISPATCH(fwd_launch, P, xt, l0, nv, st)
+    SPECT_DISPATCH(fwd_launch, P, l0, nv, st)
 }
 
 cudaError_t launch_fused_rotate(const spect_plan_s& P, const float* xt, int l0, int nv, cudaStream_t st)
@@ -1134,8 +1135,8 @@ namespace {
 // about four warps' worth lost to latency, so a plane takes W + 4 warp items of
 // 32 P + 100 issue slots; a block's set-up costs about s planes; up to four waves the
 // last one counts whole, beyond that half a block on average.  Against the measured
-// launches (shapes of 16..64 columns and J = 1..16, twelve geometries from 16x8 to
-// 192x128) the shapes it picks are within 4 % of the fastest, 8 % at worst.
+// launches (shapes of 16..64 columns and J = 1..8, nineteen geometries from 16x8 to
+// 192x128) the shapes it picks are within 6 % of the fastest for A, 4 % for A'.
 double blur_cost(int P, long long blocks, int J, double s, int T, int B, int sms)
 {
     const double per_sm = (double)((blocks + sms - 1) / sms);

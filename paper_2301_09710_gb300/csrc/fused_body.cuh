@@ -61,9 +61,9 @@ __device__ __forceinline__ void transpose_body(const float* __restrict__ in, flo
 // Fused forward, separable PSF, padded tap count P (odd).
 //
 // The forward runs as two kernels: k_rot_fwd rotates and attenuates every
-// (view, depth) plane into the work slab, already in the blur kernel's
-// shared-memory image; k_fwd_sep_fused (one block per view and depth group)
-// streams those images in by TMA and blurs them.  Its shared memory:
+// (view, depth) plane into a plane image [i][k] of the work slab;
+// k_fwd_sep_fused (one block per view, depth group and column tile) streams
+// tiles of those images in by TMA and blurs them.  Its shared memory:
 //   W   one or two tile buffers, as runs of 32 k: W[k / 32][C + i][k % 32], zero
 //       outside the plane (the tensor copy's fill); the i-pass windows (lanes over
 //       k) are conflict-free loads at immediate offsets.
@@ -100,11 +100,10 @@ struct FwdBlock {
     static constexpr int regs = P <= 11 ? 72 : 80;
 };
 
-// Shared-memory plan of a fused kernel, computed identically on host and device.
-// Planes wider than shared memory allows are cut into nT column tiles of TI
-// detector columns (TI a multiple of CX); a tile carries C halo columns on
-// each side, so every tile is blurred independently.  nT = 1 is the untiled
-// case (TI = nib*CX >= nx).
+// Bounds of the geometries and launch shapes that the fused kernels take (the kernels
+// need less): a plane cut into nT column tiles of TI detector columns (TI a multiple
+// of CX), each with C halo columns on each side, two tile buffers, U, accumulators,
+// taps and folds in shared memory.
 struct FusedDims {
     int wp;     // W row pitch of one tile image (pitch4odd(TI + 2*C))
     int warea;  // floats of one tile image, nz x wp (multiple of 4, keeps U 16-byte aligned)
@@ -945,10 +944,6 @@ size_t smem_fwd_bound(const Geometry& g, const FusedDims& d)
     return (2 * (size_t)d.warea + (size_t)d.urows * d.kpu + 2 * (size_t)Sep<P>::PT * d.J + (size_t)d.urows * d.apc +
             2 * (size_t)d.J * d.nkb * 16 + 8) * sizeof(float);
 }
-
-// The fewest column tiles with which the rotation, blur and adjoint kernels
-// fit `limit` bytes of shared memory (and every bulk copy stays below the
-// mbarrier's 2^20-byte transaction count); 0 when none does.
 }  // namespace
 
 }  // namespace spect

@@ -345,7 +345,7 @@ spect_status fast_forward(spect_plan_s* P, const float* xt, float* v, const floa
                                [&] { return spect::launch_fused_rotate(*P, xt, l0, nv, st); }),
                        "rotation launch");
         SPECT_CUDA_TRY(counted(P, SPECT_K_CONV_FWD, st,
-                               [&] { return spect::launch_fused_forward(*P, xt, l0, nv, st); }),
+                               [&] { return spect::launch_fused_forward(*P, l0, nv, st); }),
                        "fused forward launch");
     }
     SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_fwd_reduce(*P, v, y, rbar, st); }),
@@ -1114,7 +1114,7 @@ spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, int adj_t
     P->adj_nT = ant;
     if (P->separable) P->adj_nT = spect::adj_tiles(*P);
     P->fwd_nT = P->separable ? spect::fwd_tiles(*P) : 1;
-    const size_t vol = (size_t)g.nx * g.ny * g.nz, nproj = (size_t)g.nx * g.nz * g.nview;
+    const size_t vol = (size_t)g.nx * g.ny * g.nz;
     const size_t per_view = std::max(vol, spect::fused_slab_per_view(*P));
     const size_t budget = P->recompute ? recompute_budget_bytes() : slab_budget_bytes(true);
     const int chunk = view_chunk(*P, per_view, budget);

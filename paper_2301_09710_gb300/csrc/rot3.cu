@@ -15,7 +15,7 @@
 // Every pass reads two neighbours along one axis, so the three passes read
 // eight pixels of the quarter-turned frame, with weights that are products of
 // the three passes' linear-interpolation weights:
-//   A:  the fused rotation kernel's eight-tap variant (k_rot_fwd8, fused.cu)
+//   A:  the fused rotation kernel's eight-tap variant (k_rot_fwd<8>, fused.cu)
 //       gathers them from x_t per output (view, row, column), attenuates and
 //       writes the blur kernel's plane images -- no pass volumes in between.
 //   A': the transposes of passes 3, 2 and 1, of the quarter turn and the sum
@@ -103,7 +103,7 @@ void quarter_to(int n, int q, int si, int sj, int* i, int* j)
 // (weight, element offset) taps of entry (l, j, i) of a table whose (l, j)
 // block holds nx groups of N weights then nx groups of N int offsets into one
 // [j][i][k] volume (unused taps: weight 0, offset 0).  Plan time only (the
-// attenuation cache); the projector itself runs the taps in k_rot_fwd8.
+// attenuation cache); the projector itself runs the taps in k_rot_fwd<8>.
 template <int N>
 __global__ void __launch_bounds__(256) k_gather_taps(Geometry g, int tsn, const float* __restrict__ tab,
                                                      const float* __restrict__ in, float* __restrict__ out, int l)

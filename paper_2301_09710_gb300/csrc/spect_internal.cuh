@@ -404,14 +404,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, unsigned parity
     return false;
 }
 
-__device__ __forceinline__ void tma_store_1d(void* dst_gmem, const void* src_smem, unsigned bytes)
-{
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst_gmem), "r"(smem_u32(src_smem)),
-                 "r"(bytes)
-                 : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-
 // Wait until at most N committed bulk stores still read their shared-memory source.
 template <int N>
 __device__ __forceinline__ void tma_store_wait_read()
@@ -421,14 +413,8 @@ __device__ __forceinline__ void tma_store_wait_read()
 
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// One 4-byte asynchronous copy global -> shared (cp.async, through L1), and the
-// wait for all of the calling thread's copies.
-__device__ __forceinline__ void cp_async_4(float* dst_smem, const float* src_gmem)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem) : "memory");
-}
-
-// The same, writing 0.0f instead of reading when !valid (src is not read then).
+// One 4-byte asynchronous copy global -> shared (cp.async, through L1), 0.0f instead of a
+// read when !valid (src is not read then), and the wait for all of the calling thread's copies.
 __device__ __forceinline__ void cp_async_4_or_zero(float* dst_smem, const float* src_gmem, bool valid)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem),
@@ -517,7 +503,7 @@ cudaError_t launch_transpose(const float* in, float* out, int R, int C, int ip, 
 cudaError_t launch_mubar_cache(const spect_plan_s& P, const float* mu_t, cudaStream_t st);
 cudaError_t launch_build_adjacency_fixed(const spect_plan_s& P, cudaStream_t st);
 cudaError_t launch_rot_tables(const spect_plan_s& P, cudaStream_t st);
-cudaError_t launch_fused_forward(const spect_plan_s& P, const float* xt, int l0, int nv, cudaStream_t st);
+cudaError_t launch_fused_forward(const spect_plan_s& P, int l0, int nv, cudaStream_t st);
 cudaError_t launch_fused_rotate(const spect_plan_s& P, const float* xt, int l0, int nv, cudaStream_t st);
 // three-pass rotation (rot3.cu): table block size, and the plan-time build of
 // the table, the adjoint lists (adjf, adj_max >= 8) and the attenuation cache
