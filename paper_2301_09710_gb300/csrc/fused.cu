@@ -47,73 +47,99 @@ cudaError_t launch_transpose(const float* in, float* out, int R, int C, int ip, 
 }
 
 // mubar[l][j][i][k] = exp(-dy (mu~(j)/2 + sum_{s>j} mu~(s))), Eq. (1), for every
-// view.  One block per (row i, view l = l0 + v, run of up to kMuThreads columns k):
-// the block first stages the rotation-table entries of row i for every depth
-// (the forward rotation's bilinear weights and base voxels) in shared memory,
-// then each thread walks one column k from the detector side with a
-// compensated running sum (AttenScan).  Lanes run over k, so the corner loads
-// and the stores are coalesced, and a depth step's loads depend on nothing
-// but the staged table, so the unrolled walk keeps several steps in flight.
-// With nview * nx * nz independent columns this does O(1) work per factor; a
-// warp scan along depth (atten_warp_scan) would do O(log 32) and measured
-// 2.6x slower here.  mu_t is mu in the [j][i][k] layout; planes (l, j) are ps
-// floats apart (16-byte aligned for bulk copies); view l lands at position v.
-constexpr int kMuThreads = 128;
+// view.  A block owns 32 quads of k of a view's columns; its warps take runs of kMuRun
+// depths from the detector side: each rotates its run into registers with the forward
+// rotation's weights and sums it (compensated, AttenScan), the runs' sums are exchanged
+// through shared memory, and each warp walks its run again from the sum of the runs
+// before it.  mu_t is mu in the [j][i][k] layout; planes (l, j) are ps floats apart;
+// view l lands at position v.
+//   Bound by the latency of table entry and gather (four blocks per SM, two depths' loads
+// in flight per thread; longer batches at fewer blocks: 96x64, 20 views of a pass 35 us
+// against 41).  Against one thread walking a whole column: EM update with the factors
+// recomputed, 160x96 in passes of 2 views 8.5 -> 5.3 ms, 128x80 in passes of 43 2.32 ->
+// 2.29, 96x64 in passes of 20 0.522 -> 0.510.
+constexpr int kMuBatch = 2, kMuWarps = 8;
 
-__global__ void __launch_bounds__(kMuThreads) k_mubar_cache(Geometry g, int ps, int ts,
-                                                            const float* __restrict__ rtab,
-                                                            const float* __restrict__ mu_t,
-                                                            float* __restrict__ mubar, int l0)
+__global__ void __launch_bounds__(32 * kMuWarps, 4) k_mubar_cache(Geometry g, int ps, int ts,
+                                                                  const float* __restrict__ rtab,
+                                                                  const float* __restrict__ mu_t,
+                                                                  float* __restrict__ mubar, int l0)
 {
-    extern __shared__ __align__(16) float smu[];
-    float4* TW = reinterpret_cast<float4*>(smu);        // [ny] weights of row i
-    int* TB = reinterpret_cast<int*>(smu + 4 * g.ny);   // [ny] base voxels of row i
-    const int k = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y, v = blockIdx.z, l = l0 + v;
-    const float* tab_l = rtab + (size_t)l * g.ny * ts;
-    for (int j = threadIdx.x; j < g.ny; j += blockDim.x) {
-        const float* tab = tab_l + (size_t)j * ts;
-        TW[j] = __ldg(reinterpret_cast<const float4*>(tab) + i);
-        TB[j] = __ldg(reinterpret_cast<const int*>(tab + 4 * g.nx) + i);
-    }
-    __syncthreads();
-    if (k >= g.kp) return;
-    const size_t rs = (size_t)g.nx * g.kp;
-    float* out = mubar + (size_t)v * g.ny * ps + (size_t)i * g.kp + k;
-    if (k >= g.nz) {  // padding
-        for (int j = 0; j < g.ny; ++j) out[(size_t)j * ps] = 0.f;
-        return;
-    }
-    if (!g.has_mu) {
-        for (int j = 0; j < g.ny; ++j) out[(size_t)j * ps] = 1.f;
-        return;
-    }
-    AttenScan sc;
-#pragma unroll 8
-    for (int j = g.ny - 1; j >= 0; --j) {
-        const float4 w = TW[j];
-        const float* m = mu_t + (size_t)TB[j] * g.kp + k;
-        float mv = 0.f;
-        mv = __fmaf_rn(w.x, __ldg(m), mv);
-        mv = __fmaf_rn(w.y, __ldg(m + g.kp), mv);
-        mv = __fmaf_rn(w.z, __ldg(m + rs), mv);
-        mv = __fmaf_rn(w.w, __ldg(m + rs + g.kp), mv);
-        out[(size_t)j * ps] = sc.step(mv, g.dy);
+    __shared__ float4 run[2][kMuWarps][2][32];  // sums, compensation terms
+    wait_previous_kernel();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int v = blockIdx.y, l = l0 + v, n = g.nx * g.kp, k4 = g.kp >> 2;
+    const int e4 = min((int)blockIdx.x * 32 + lane, g.nx * k4 - 1), i = e4 / k4, k = 4 * (e4 - i * k4);
+    const bool mine = (int)blockIdx.x * 32 + lane < g.nx * k4;
+    const float* m = mu_t + k;
+    const float* tab = rtab + (size_t)l * g.ny * ts;
+    float* out = mubar + (size_t)v * g.ny * ps + 4 * (size_t)e4;
+    AttenScan carry[4];
+    int buf = 0;
+    for (int top = g.ny - 1; top >= 0; top -= nw * kMuRun, buf ^= 1) {
+        const int j0 = top - w * kMuRun;  // this warp's run: j0, j0 - 1, ...
+        float mv[kMuRun][4] = {};
+        AttenScan own[4];
+        if (g.has_mu && j0 >= 0) {  // no branch below: a batch's loads go out together
+#pragma unroll
+            for (int h = 0; h < kMuRun; h += kMuBatch) {
+                float4 t[kMuBatch];
+                const float* b[kMuBatch];
+#pragma unroll
+                for (int q = 0; q < kMuBatch; ++q) {
+                    const float* tj = tab + (size_t)max(j0 - h - q, 0) * ts;
+                    t[q] = __ldg(reinterpret_cast<const float4*>(tj) + i);
+                    b[q] = m + (size_t)__ldg(reinterpret_cast<const int*>(tj + 4 * g.nx) + i) * g.kp;
+                }
+#pragma unroll
+                for (int q = 0; q < kMuBatch; ++q) {
+                    const float4 c0 = __ldg(reinterpret_cast<const float4*>(b[q]));
+                    const float4 c1 = __ldg(reinterpret_cast<const float4*>(b[q] + g.kp));
+                    const float4 c2 = __ldg(reinterpret_cast<const float4*>(b[q] + n));
+                    const float4 c3 = __ldg(reinterpret_cast<const float4*>(b[q] + n + g.kp));
+                    const bool in = j0 - h - q >= 0;
+                    mv[h + q][0] = in ? fmaf(t[q].w, c3.x, fmaf(t[q].z, c2.x, fmaf(t[q].y, c1.x, t[q].x * c0.x))) : 0.f;
+                    mv[h + q][1] = in ? fmaf(t[q].w, c3.y, fmaf(t[q].z, c2.y, fmaf(t[q].y, c1.y, t[q].x * c0.y))) : 0.f;
+                    mv[h + q][2] = in ? fmaf(t[q].w, c3.z, fmaf(t[q].z, c2.z, fmaf(t[q].y, c1.z, t[q].x * c0.z))) : 0.f;
+                    mv[h + q][3] = in ? fmaf(t[q].w, c3.w, fmaf(t[q].z, c2.w, fmaf(t[q].y, c1.w, t[q].x * c0.w))) : 0.f;
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kMuRun; ++q)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) own[c].add(mv[q][c]);
+        run[buf][w][0][lane] = make_float4(own[0].S, own[1].S, own[2].S, own[3].S);
+        run[buf][w][1][lane] = make_float4(own[0].c, own[1].c, own[2].c, own[3].c);
+        __syncthreads();  // the other buffer is rewritten only after the next one
+        AttenScan sc[4];
+        for (int u = 0; u < nw; ++u) {
+            const float4 s4 = run[buf][u][0][lane], r4 = run[buf][u][1][lane];
+            const float ss[4] = {s4.x, s4.y, s4.z, s4.w}, rr[4] = {r4.x, r4.y, r4.z, r4.w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (u == w) sc[c] = carry[c];
+                carry[c].merge({ss[c], rr[c]});
+            }
+        }
+        if (mine)
+#pragma unroll
+            for (int q = 0; q < kMuRun; ++q)
+                if (j0 - q >= 0) {
+                    float o[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) o[c] = k + c < g.nz ? sc[c].step(mv[q][c], g.dy) : 0.f;  // 0: padding
+                    *reinterpret_cast<float4*>(out + (size_t)(j0 - q) * ps) = make_float4(o[0], o[1], o[2], o[3]);
+                }
     }
 }
 
 namespace {
 cudaError_t mubar_launch(const spect_plan_s& P, const float* mu_t, int l0, int nv, cudaStream_t st)
 {
-    const size_t smem = (size_t)P.g.ny * 5 * sizeof(float);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_mubar_cache, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    // a run of columns k per block: kp rounded up to whole warps, at most kMuThreads
-    const int thr = std::min(kMuThreads, (P.g.kp + 31) & ~31);
-    const dim3 grid((P.g.kp + thr - 1) / thr, P.g.nx, nv);
-    k_mubar_cache<<<grid, thr, smem, st>>>(P.g, P.ps, P.ts, P.rtab, mu_t, P.mubar, l0);
-    return cudaGetLastError();
+    const int warps = std::min(kMuWarps, (P.g.ny + kMuRun - 1) / kMuRun);
+    const dim3 grid((P.g.nx * (P.g.kp / 4) + 31) / 32, nv);
+    return launch_chained(k_mubar_cache, grid, 32 * warps, 0, st, P.g, P.ps, P.ts, P.rtab, mu_t, P.mubar, l0);
 }
 }  // namespace
 

@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(256) k_gather_taps(Geometry g, int tsn, const 
 
 // mubar[l][j][i][k] from the rotated map mu~ of view l ([j][i][k], dense):
 // Eq. (1) walked from the detector side with a compensated running sum, one
-// thread per (i, k) column (coalesced), the same arithmetic as the bilinear
-// rotation's attenuation cache (k_mubar_cache).
+// thread per (i, k) column (coalesced), in the runs of depths and so with the
+// arithmetic of the bilinear rotation's attenuation cache (k_mubar_cache).
 __global__ void k_mubar_rotated(Geometry g, int ps, const float* __restrict__ mu_rot, int l,
                                 float* __restrict__ mubar)
 {
@@ -139,10 +139,15 @@ __global__ void k_mubar_rotated(Geometry g, int ps, const float* __restrict__ mu
         return;
     }
     const size_t pln = (size_t)per;
-    AttenScan sc;
-    for (int j = g.ny - 1; j >= 0; --j) {
-        const float m = mu_rot[(size_t)j * pln + idx];
-        mubar[((size_t)l * g.ny + j) * ps + idx] = g.has_mu ? sc.step(m, g.dy) : 1.f;
+    AttenScan carry;
+    for (int j0 = g.ny - 1; j0 >= 0; j0 -= kMuRun) {
+        AttenScan own, sc = carry;
+        for (int j = j0; j > j0 - kMuRun && j >= 0; --j) {
+            const float m = mu_rot[(size_t)j * pln + idx];
+            own.add(m);
+            mubar[((size_t)l * g.ny + j) * ps + idx] = g.has_mu ? sc.step(m, g.dy) : 1.f;
+        }
+        carry.merge(own);
     }
 }
 

@@ -258,19 +258,31 @@ __device__ __forceinline__ float atten_warp_scan(float m, DFloat& carry, float d
     return mb;
 }
 
-// Eq. (1) walked serially from the detector side with a compensated running
-// sum (the low-memory blur adjoints, which visit depths one at a time).
+// Depths per run of the attenuation caches (k_mubar_cache, k_mubar_rotated): a run starts
+// from the merged sums of the runs before it.
+constexpr int kMuRun = 8;
+
+// Eq. (1) walked serially from the detector side with a compensated running sum.
 struct AttenScan {
     float S = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float m)
+    {
+        const float y = m - c;
+        const float t = S + y;
+        c = (t - S) - y;
+        S = t;
+    }
+    __device__ __forceinline__ void merge(const AttenScan& o)
+    {
+        add(o.S);
+        add(-o.c);
+    }
     // mubar(j) = exp(-dy (mu~(j)/2 + S)), then S += mu~(j)
     __device__ __forceinline__ float step(float m, float dy)
     {
         const float half = 0.5f * m - c;
         const float mb = expf(-dy * (S + half));
-        const float y = m - c;
-        const float t = S + y;
-        c = (t - S) - y;
-        S = t;
+        add(m);
         return mb;
     }
 };

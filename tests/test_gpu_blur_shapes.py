@@ -148,3 +148,19 @@ def test_chained_launches_keep_their_order(path):
         assert np.array_equal(a, b)
     plan.check()
     plan.close()
+
+
+@pytest.mark.parametrize("nx,nz", [(8, 5), (9, 1), (65, 3), (130, 4)])
+def test_attenuation_runs_of_depths(nx, nz):
+    """The attenuation factors at the edges of their runs of eight depths and rounds of 64
+    (one plane past a round, a last run of one plane), a strong mu: A and A' against the oracle."""
+    need_gpu()
+    prob = synthetic.random_problem(nx, nx=nx, nz=nz, nview=3, px=3, pz=3, mu_scale=0.2)
+    ang = np.random.default_rng(nx).uniform(0, 2 * np.pi, 3)
+    plan = make_plan(prob, ang, "fused")
+    psf = oracle.psf_from_factors(prob.fx, prob.fz)
+    assert_close(host(plan.forward(dev(prob.x))), oracle.forward(prob.x, prob.mu, psf, prob.dy, ang), what="A x")
+    yy = np.random.default_rng(11).uniform(0, 1, plan.proj_shape).astype(np.float32)
+    assert_close(host(plan.back(dev(yy))), oracle.back(yy, prob.mu, psf, prob.dy, ang), what="A' y")
+    plan.check()
+    plan.close()
