@@ -102,7 +102,7 @@ enum {
      * projection instead of cached for every view: the views go through the
      * fused kernels in chunks, and before each chunk's rotation (A) or blur
      * adjoint (A') the factors of that chunk's views are computed from the
-     * rotated mu-map (the same warp-scan kernel that fills the cache, so A,
+     * rotated mu-map (the same kernel that fills the cache, so A,
      * A' and the EM update are bitwise those of a caching plan).  Device
      * memory then grows with the chunk (work slab and factors of the chunk's
      * views, 512 MiB by default) rather than with nview * nx*ny*nz.  Bilinear
