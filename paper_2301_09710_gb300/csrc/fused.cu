@@ -332,6 +332,7 @@ __global__ void __launch_bounds__(AdjBlock<P>::T, AdjBlock<P>::B)
                     const __grid_constant__ CUtensorMap v_map, Geometry g, AdjDims d,
                     const float* __restrict__ rec, int l0, int mu_l0, int* err)
 {
+    wait_previous_kernel();
     const int grp = blockIdx.x / d.nT;
     adj_sep_body<P>(g, d, &mu_map, &t_map, &v_map, rec, l0, mu_l0, err, grp, blockIdx.y, blockIdx.x - grp * d.nT);
 }

@@ -124,13 +124,16 @@ def test_low_memory_plan_in_view_chunks(monkeypatch):
     one.close()
 
 
+@pytest.mark.parametrize("nx", [25, 24])  # A' begins with the row padding, or with the blur adjoint right behind the caller's kernel
 @pytest.mark.parametrize("path", ["fused", "direct", "lowmem"])
-def test_chained_launches_keep_their_order(path):
+def test_chained_launches_keep_their_order(path, nx):
     """Small kernels back to back, each reading what the one before wrote and overwriting what
-    it read: a run of calls queued at once equals the same calls with a wait after each."""
+    it read: a run of calls queued at once equals the same calls with a wait after each.  (Both
+    runs chain the launches within a call; that each kernel waits for the one before it is read
+    from the sources, test_chained_launches_cpu.py.)"""
     need_gpu()
     import torch
-    prob = synthetic.random_problem(10, nx=25, nz=7, nview=3, px=7, pz=5, mu_scale=0.05)
+    prob = synthetic.random_problem(10, nx=nx, nz=7, nview=3, px=7, pz=5, mu_scale=0.05)
     plan = make_plan(prob, oracle.default_angles(3), path)
     yy = dev(np.random.default_rng(10).uniform(0.5, 1.5, plan.proj_shape).astype(np.float32))
 
