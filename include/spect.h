@@ -81,9 +81,11 @@ enum {
     /* Keep device memory O(image + projections): recompute the attenuation
      * per view and stream views through a small work slab, instead of
      * caching the attenuation factors of every view (nview * nx*ny*nz floats).
-     * Where the fused kernels fit the geometry they run in view chunks small
-     * enough for that (spect_plan_info still reports fused = 0, and the launch
-     * shapes cannot be tuned); wider PSFs take the low-memory kernels. */
+     * Where the fused kernels fit the geometry they run in view chunks with
+     * which the plan, also while it is made, holds no more than the low-memory
+     * kernels would (or 24 MiB; spect_plan_info still reports fused = 0, and the
+     * launch shapes cannot be tuned); wider PSFs, and geometries for which no
+     * chunk is small enough, take the low-memory kernels. */
     SPECT_PLAN_LOW_MEMORY = 1u << 1,
     /* Rotate the image and the attenuation map by three 1D linear
      * interpolation passes instead of bilinear interpolation (Section II-A

@@ -139,7 +139,7 @@ cudaError_t mubar_launch(const spect_plan_s& P, const float* mu_t, int l0, int n
 {
     const int warps = std::min(kMuWarps, (P.g.ny + kMuRun - 1) / kMuRun);
     const dim3 grid((P.g.nx * (P.g.kp / 4) + 31) / 32, nv);
-    return launch_chained(k_mubar_cache, grid, 32 * warps, 0, st, P.g, P.ps, P.ts, P.rtab, mu_t, P.mubar, l0);
+    return launch_chained(k_mubar_cache, grid, 32 * warps, 0, st, P.g, P.ps, P.ts, rtab_for(P, l0), mu_t, P.mubar, l0);
 }
 }  // namespace
 
@@ -154,29 +154,28 @@ cudaError_t launch_mubar_range(const spect_plan_s& P, int l0, int nv, cudaStream
     return mubar_launch(P, P.mut, l0, nv, st);
 }
 
-// Rotation tables of every (view, depth row), the per-plane input of the fused
-// forward: block (l, j) holds nx float4 weights then nx int bases (ts floats,
-// 16-byte aligned), fetched together with the attenuation plane by one TMA
-// transaction.
-__global__ void k_rot_tables(Geometry g, int ts, const ViewRot* __restrict__ rot, float* __restrict__ tab)
+// Rotation tables of views l0 .. l0 + nv - 1, read by the rotation (k_rot_fwd,
+// k_rot_patch) and the attenuation factors (k_mubar_cache): block (v, j) holds nx
+// float4 weights, then nx int bases (ts floats, 16-byte aligned).
+__global__ void k_rot_tables(Geometry g, int ts, const ViewRot* __restrict__ rot, int l0, int nv, float* __restrict__ tab)
 {
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (size_t)g.nview * g.ny * g.nx) return;
+    if (idx >= (size_t)nv * g.ny * g.nx) return;
     const int i = (int)(idx % g.nx);
     const size_t lj = idx / g.nx;
-    const int j = (int)(lj % g.ny), l = (int)(lj / g.ny);
+    const int j = (int)(lj % g.ny), v = (int)(lj / g.ny);
     float4 w;
     int base;
-    rot_table_entry(i, j, rot[l], g, w, base);
+    rot_table_entry(i, j, rot[l0 + v], g, w, base);
     float* blk = tab + lj * ts;
     reinterpret_cast<float4*>(blk)[i] = w;
     reinterpret_cast<int*>(blk + 4 * g.nx)[i] = base;
 }
 
-cudaError_t launch_rot_tables(const spect_plan_s& P, cudaStream_t st)
+cudaError_t launch_rot_tables(const spect_plan_s& P, int l0, int nv, cudaStream_t st)
 {
-    const size_t n = (size_t)P.g.nview * P.g.ny * P.g.nx;
-    k_rot_tables<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(P.g, P.ts, P.rot, P.rtab);
+    const size_t n = (size_t)nv * P.g.ny * P.g.nx;
+    k_rot_tables<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(P.g, P.ts, P.rot, l0, nv, P.rtab);
     return cudaGetLastError();
 }
 
@@ -223,10 +222,12 @@ __global__ void k_build_adjacency_fixed(Geometry g, int ps, const ViewRot* __res
     }
 }
 
-cudaError_t launch_build_adjacency_fixed(const spect_plan_s& P, cudaStream_t st)
+cudaError_t launch_build_adjacency_fixed(const spect_plan_s& P, int l0, int nv, cudaStream_t st)
 {
-    const size_t n = (size_t)P.g.nx * P.g.ny * P.g.nview;
-    k_build_adjacency_fixed<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(P.g, P.ps, P.rot, P.adj_max, P.adjf);
+    Geometry g = P.g;  // the lists of these views alone
+    g.nview = nv;
+    const size_t n = (size_t)g.nx * g.ny * nv;
+    k_build_adjacency_fixed<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g, P.ps, P.rot + l0, P.adj_max, P.adjf);
     return cudaGetLastError();
 }
 
@@ -255,7 +256,7 @@ __global__ void __launch_bounds__(FwdBlock<P>::T, KS ? 1 : FwdBlock<P>::B) k_fwd
 {
     wait_previous_kernel();
     const int grp = blockIdx.x / d.nT;
-    fwd_sep_body<P, RACC, KS>(g, d, &tmap, rec, part, l0, err, grp, blockIdx.y, blockIdx.x - grp * d.nT);
+    fwd_sep_body<P, RACC, KS>(g, d, &tmap, rec, part, l0, gridDim.y, err, grp, blockIdx.y, blockIdx.x - grp * d.nT);
 }
 
 // Plan time: the tap records of the forward blur (layout: fwd_rec_floats), one
@@ -292,8 +293,8 @@ __global__ void k_fwd_records(Geometry g, int P, int PT, int nkb, const float* _
     }
 }
 
-// v(i,k,l) = sum over depth groups of the partials (fixed order), optionally
-// turned into the EM ratio y / (v + rbar), whose rows are np long.
+// v(i,k,l) = sum over depth groups of the partials (fixed order) of the views of a pass
+// (nproj values), optionally turned into the EM ratio y / (v + rbar), whose rows are np long.
 __global__ void k_fwd_reduce(const float* __restrict__ part, int G, size_t nproj, float* __restrict__ v, int nx, int np,
                              const float* __restrict__ em_y, const float* __restrict__ em_rbar)
 {
@@ -523,7 +524,7 @@ __global__ void __launch_bounds__(kDirThreads, 1) k_fwd_dir_fused(const __grid_c
     }
     if (mine) {
         const int k0 = k_lo + kb * CZ;
-        float* pout = part + ((size_t)grp * g.nview + l) * pln + i0 + i;
+        float* pout = part + ((size_t)grp * gridDim.y + v) * pln + i0 + i;
 #pragma unroll
         for (int c = 0; c < CZ; ++c)
             if (k0 + c < nz) pout[(size_t)(k0 + c) * nx] = acc[c].value();
@@ -1088,7 +1089,7 @@ cudaError_t launch_fused_rotate(const spect_plan_s& P, const float* xt, int l0, 
     const RotDims d = rot_dims(P.g, P.ps, P.rot3 ? rot3_ts8(P.g.nx) : P.ts, nv, P.sms);
     const dim3 grid(d.nb * ((P.g.ny + d.JP - 1) / d.JP), nv);
     return launch_chained(P.rot3 ? k_rot_fwd<8> : k_rot_fwd<4>, grid, kRotThreads, 0, st, P.g, d,
-                          P.rot3 ? P.r3_tab : P.rtab, xt, mubar_for(P, l0), P.slab, l0);
+                          P.rot3 ? P.r3_tab : rtab_for(P, l0), xt, mubar_for(P, l0), P.slab, l0);
 }
 
 namespace {
@@ -1273,12 +1274,13 @@ cudaError_t launch_fused_adjoint(const spect_plan_s& P, const float* v, int l0, 
 }
 #undef SPECT_DISPATCH
 
-cudaError_t launch_fwd_reduce(const spect_plan_s& P, float* v, const float* em_y, const float* em_rbar,
+cudaError_t launch_fwd_reduce(const spect_plan_s& P, int l0, int nv, float* v, const float* em_y, const float* em_rbar,
                               cudaStream_t st)
 {
-    const size_t nproj = (size_t)P.g.nx * P.g.nz * P.g.nview;
+    const size_t view = (size_t)P.g.nx * P.g.nz, nproj = view * nv, at = view * l0;
+    v += em_y ? (size_t)P.g.np * P.g.nz * l0 : at;
     return launch_chained(k_fwd_reduce, (unsigned)((nproj + 255) / 256), 256, 0, st, P.part, fused_groups(P), nproj, v,
-                          P.g.nx, P.g.np, em_y, em_rbar);
+                          P.g.nx, P.g.np, em_y ? em_y + at : nullptr, em_rbar ? em_rbar + at : nullptr);
 }
 
 cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,

@@ -351,8 +351,8 @@ struct DepthSum<true> : KSum {};
 // only to read U; otherwise (planes of more than 640 items) they are in ACC.
 template <int P, bool RACC, bool KS>
 __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FwdDims& d, const CUtensorMap* tmap,
-                                             const float* __restrict__ rec, float* __restrict__ part, int l0, int* err,
-                                             const int grp, const int v, const int tile)
+                                             const float* __restrict__ rec, float* __restrict__ part, int l0, int nv,
+                                             int* err, const int grp, const int v, const int tile)
 {
     using S = Sep<P>;
     constexpr int C = S::C, CX = S::CX, CZ = S::CZ, ZH = S::ZH, WZ = S::WZ, PT = S::PT;
@@ -514,8 +514,8 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FwdDims& d
         __syncthreads();
     }
 
-    // partial depth sums of this group: part[grp][l][k][i], this tile's columns
-    float* pout = part + ((size_t)grp * g.nview + l) * pln + i0;
+    // partial depth sums of this group: part[grp][v][k][i] (v of the nv views of the pass), this tile's columns
+    float* pout = part + ((size_t)grp * nv + v) * pln + i0;
     if (RACC) {
         if (tid < ti * d.nkb) {
 #pragma unroll

@@ -38,11 +38,13 @@ namespace {
 constexpr int kPatch = 8;     // destinations per patch side
 constexpr int kStages = 3;    // views in flight per block (measured best: 3 of 3, 4, 6, 8)
 
-// Box of source pixels read by patch `patch` in view l: (i0, j0, width, height).
-__global__ void k_patch_boxes(Geometry g, int ps, int maxe, const AdjEntry* __restrict__ adjf, int npx, int4* boxes)
+// Box of source pixels read by patch `patch` in view l = l0 + blockIdx.y: (i0, j0, width,
+// height).  adjf holds the lists of the gridDim.y views from l0 on.
+__global__ void k_patch_boxes(Geometry g, int ps, int maxe, const AdjEntry* __restrict__ adjf, int l0, int npx,
+                              int4* boxes)
 {
     __shared__ int mn_i, mn_j, mx_i, mx_j;
-    const int patch = blockIdx.x, l = blockIdx.y, t = threadIdx.x;
+    const int patch = blockIdx.x, l = l0 + blockIdx.y, t = threadIdx.x;
     if (t == 0) {
         mn_i = mn_j = INT_MAX;
         mx_i = mx_j = INT_MIN;
@@ -50,7 +52,7 @@ __global__ void k_patch_boxes(Geometry g, int ps, int maxe, const AdjEntry* __re
     __syncthreads();
     const int qi = (patch % npx) * kPatch + (t % kPatch), qj = (patch / npx) * kPatch + (t / kPatch);
     if (qi < g.nx && qj < g.ny) {
-        const AdjEntry* e = adjf + ((size_t)(qj * g.nx + qi) * g.nview + l) * maxe;
+        const AdjEntry* e = adjf + ((size_t)(qj * g.nx + qi) * gridDim.y + blockIdx.y) * maxe;
         for (int m = 0; m < maxe; ++m) {
             if (e[m].w == 0.f) continue;
             const int pj = e[m].p / ps, pi = (e[m].p - pj * ps) / g.kp;
@@ -70,16 +72,16 @@ __global__ void k_patch_boxes(Geometry g, int ps, int maxe, const AdjEntry* __re
 
 // Patch entries [patch][l][64][maxe]: (box-local offset (row*size + col)*KC, weight);
 // zero entries for padding and for destinations outside the image.  boxes: (i0, j0,
-// box size, tensor map).
-__global__ void k_patch_entries(Geometry g, int ps, int maxe, const AdjEntry* __restrict__ adjf, int npx,
+// box size, tensor map).  Views and lists as in k_patch_boxes.
+__global__ void k_patch_entries(Geometry g, int ps, int maxe, const AdjEntry* __restrict__ adjf, int l0, int npx,
                                 const int4* __restrict__ boxes, int kc, AdjEntry* pent)
 {
-    const int patch = blockIdx.x, l = blockIdx.y, t = threadIdx.x;
+    const int patch = blockIdx.x, l = l0 + blockIdx.y, t = threadIdx.x;
     const int qi = (patch % npx) * kPatch + (t % kPatch), qj = (patch / npx) * kPatch + (t / kPatch);
     const int4 b = boxes[(size_t)patch * g.nview + l];
     AdjEntry* out = pent + (((size_t)patch * g.nview + l) * (kPatch * kPatch) + t) * maxe;
     const bool inside = qi < g.nx && qj < g.ny;
-    const AdjEntry* e = adjf + ((size_t)(qj * g.nx + qi) * g.nview + l) * maxe;
+    const AdjEntry* e = adjf + ((size_t)(qj * g.nx + qi) * gridDim.y + blockIdx.y) * maxe;
     for (int m = 0; m < maxe; ++m) {
         AdjEntry o;  // padding and outside destinations: weight 0 on the box's first element
         o.p = 0;
@@ -384,8 +386,21 @@ cudaError_t build_gather(spect_plan_s& P, cudaStream_t st)
     cudaError_t e = P.pooled ? cudaMallocAsync((void**)&boxes, nb * sizeof(int4), st)
                              : cudaMalloc((void**)&boxes, nb * sizeof(int4));
     if (e != cudaSuccess) return e;
-    k_patch_boxes<<<dim3(npx * npy, g.nview), kPatch * kPatch, 0, st>>>(g, P.ps, P.adj_max, P.adjf, npx, boxes);
-    e = cudaGetLastError();
+    // f(l0, nv) for the ranges of views whose lists adjf holds at once
+    auto ranges = [&](auto&& f) {
+        const int lv = P.list_views;
+        cudaError_t er = cudaSuccess;
+        for (int l0 = 0; l0 < g.nview && er == cudaSuccess; l0 += lv) {
+            const int nv = std::min(lv, g.nview - l0);
+            if (lv < g.nview) er = launch_build_adjacency_fixed(P, l0, nv, st);
+            if (er == cudaSuccess) f(l0, nv);
+            if (er == cudaSuccess) er = cudaGetLastError();
+        }
+        return er;
+    };
+    e = ranges([&](int l0, int nv) {
+        k_patch_boxes<<<dim3(npx * npy, nv), kPatch * kPatch, 0, st>>>(g, P.ps, P.adj_max, P.adjf, l0, npx, boxes);
+    });
     std::vector<int4> hb(nb);
     if (e == cudaSuccess) e = cudaMemcpyAsync(hb.data(), boxes, nb * sizeof(int4), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -451,9 +466,10 @@ cudaError_t build_gather(spect_plan_s& P, cudaStream_t st)
         else cudaFree(boxes);
         return e;
     }
-    k_patch_entries<<<dim3(npx * npy, g.nview), kPatch * kPatch, 0, st>>>(g, P.ps, P.adj_max, P.adjf, npx, boxes,
-                                                                         kc, pent);
-    e = cudaGetLastError();
+    e = ranges([&](int l0, int nv) {
+        k_patch_entries<<<dim3(npx * npy, nv), kPatch * kPatch, 0, st>>>(g, P.ps, P.adj_max, P.adjf, l0, npx, boxes, kc,
+                                                                         pent);
+    });
     const size_t ncount = (size_t)npx * npy * ((g.kp + kc - 1) / kc);
     int* count = nullptr;
     if (e == cudaSuccess)
@@ -469,7 +485,7 @@ cudaError_t build_gather(spect_plan_s& P, cudaStream_t st)
     P.gnpx = npx;
     P.gnpy = npy;
     P.gather = e == cudaSuccess;
-    return e == cudaSuccess ? build_gather_maps(P) : e;
+    return e;
 }
 
 // The t slab as 3D tensor maps -- k (kp, contiguous) x i (nx, stride kp) x plane

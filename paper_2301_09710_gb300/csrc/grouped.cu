@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(FwdBlock<P>::T, FwdBlock<P>::B) k_fwd_sep_grp(
     const int4 w = group_item(gp.grid);
     const GroupPlan q = gp.p[w.x];  // by value: the fields live in registers, not re-read from parameter space
     const int grp = w.y / q.df.nT;
-    fwd_sep_body<P, RACC, false>(q.g, q.df, &gp.fmap[w.x], q.frec, q.part, 0, q.err, grp, w.z, w.y - grp * q.df.nT);
+    fwd_sep_body<P, RACC, false>(q.g, q.df, &gp.fmap[w.x], q.frec, q.part, 0, q.g.nview, q.err, grp, w.z, w.y - grp * q.df.nT);
 }
 
 template <int P>

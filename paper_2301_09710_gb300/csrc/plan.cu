@@ -175,53 +175,164 @@ size_t view_bytes(const spect_plan_s& P, size_t slab_floats_per_view)
 
 // Views per pass: what the budget holds, then evened out over the passes, so that
 // no pass is left with a few views (and the buffers are no larger than that takes).
-int view_chunk(const spect_plan_s& P, size_t slab_floats_per_view, size_t budget)
+int view_chunk(int nview, size_t bytes_per_view, size_t budget)
 {
-    const size_t nview = (size_t)P.g.nview;
-    const size_t most = std::max<size_t>(1, std::min<size_t>(nview, budget / view_bytes(P, slab_floats_per_view)));
+    const size_t most = std::max<size_t>(1, std::min<size_t>(nview, budget / bytes_per_view));
     const size_t passes = (nview + most - 1) / most;
     return (int)((nview + passes - 1) / passes);
 }
 
-// Budget of a low-memory plan's chunk buffers on the fused kernels: what keeps the
-// plan within the bytes of the low-memory kernels (their slab of at most 256 MiB, the
-// compressed adjacency lists, three volumes), but at least 24 MiB, so that small
-// plans still run in few passes.  SPECT_SLAB_MB overrides.
-size_t low_budget_bytes(const spect_plan_s& P)
+// Floats of P.part.  In A: the depth-group partial sums of a pass of `chunk` views.
+// In A' the same buffer holds the sums and compensation terms of the view segments, or
+// between its passes (adj_chunk views each) the compensation terms of the view sums.
+size_t part_floats(const spect_plan_s& P, int chunk, int adj_chunk)
 {
-    if (getenv("SPECT_SLAB_MB")) return slab_budget_bytes(false);
-    const Geometry& g = P.g;
-    const double vol = 4.0 * g.nx * g.ny * g.nz, volt = 4.0 * g.nx * g.ny * g.kp, lists = (double)g.nx * g.ny * g.nview;
-    const double held = std::min((double)slab_budget_bytes(false), vol * g.nview) + 36.0 * lists + 3.0 * vol;
-    // rotation tables 20, box-local entries about 40 bytes a list; five internal volumes; partial sums
-    const double fixed = 60.0 * lists + vol + 5.0 * volt + 4.0 * (double)g.nx * g.nz * g.nview * spect::fused_groups(P);
-    return (size_t)std::max(held - fixed, 24.0 * (1 << 20));
-}
-
-// The forward's depth-group partial sums; in A' the same buffer holds the sums and
-// compensation terms of the view segments, or between its passes (adj_chunk views
-// each) the compensation terms of the view sums.
-size_t part_floats(const spect_plan_s& P, int adj_chunk)
-{
-    const size_t part = (size_t)P.g.nx * P.g.nz * P.g.nview * spect::fused_groups(P);
+    const size_t part = (size_t)P.g.nx * P.g.nz * chunk * spect::fused_groups(P);
     const size_t volt = (size_t)P.g.nx * P.g.ny * P.g.kp;
     return std::max(part, adj_chunk < P.g.nview ? volt : (P.gsegs > 1 ? 2 * P.gsegs * volt : 0));
 }
 
-// Launch shapes and views per pass of a plan: the work slab (and a recomputing plan's
-// factors) within the budget, the blur shapes for that many views.
+// Adjacency lists a low-memory plan takes to the fused kernels.  A list holds the samples
+// of the rotated unit lattice in an open 2x2 square: at most five (counted over 1200
+// angles and 201x201 offsets); longer ones come from the rounding of coordinates.
+constexpr int kLowAdjMax = 5;
+
+// Bytes of the fixed-length lists of a low-memory plan while the gather's entries are made
+// from them, a range of views at a time (at least one view's).
+constexpr size_t kLowListBytes = 8u << 20;
+
+int low_list_views(const spect_plan_s& P)
+{
+    const size_t view = (size_t)P.g.nx * P.g.ny * kLowAdjMax * sizeof(spect::AdjEntry);
+    return (int)std::min<size_t>(P.g.nview, std::max<size_t>(1, kLowListBytes / view));
+}
+
+// What a low-memory plan may hold on the fused kernels where the general kernels' plan
+// would be smaller still: such a plan is small whatever its shape.
+constexpr size_t kSmallPlanBytes = 24u << 20;
+
+// Parts of the bounds below, in bytes: PSF factors or stack with their edge-class
+// variants, rotation constants and the error word.
+size_t psf_bytes(const spect_plan_s& P)
+{
+    const Geometry& g = P.g;
+    const size_t nrows = (size_t)g.nvp * g.ny;
+    return (P.separable ? (size_t)g.px * 4 + (size_t)g.pz * (1 + P.cls_z)
+                        : (size_t)g.px * g.pz * (1 + (size_t)P.cls_x * P.cls_z)) * nrows * sizeof(float);
+}
+
+size_t base_bytes(const spect_plan_s& P) { return sizeof(int) + (size_t)P.g.nview * sizeof(ViewRot); }
+
+// Patch gather: boxes, box-local entries and arrivals, with lists of up to `adj` entries.
+size_t gather_bytes(const spect_plan_s& P, int adj)
+{
+    const Geometry& g = P.g;
+    const size_t np = (size_t)((g.nx + 7) / 8) * ((g.ny + 7) / 8);
+    return np * g.nview * (16 + 64 * adj * sizeof(spect::AdjEntry)) + np * ((g.kp + 15) / 16) * sizeof(int);
+}
+
+size_t csr_bytes(const spect_plan_s& P)
+{
+    const size_t nlist = (size_t)P.g.nx * P.g.ny * P.g.nview;
+    return (nlist + 1) * sizeof(int) + 4 * nlist * sizeof(spect::AdjEntry);
+}
+
+// Upper bound of what a plan on the general low-memory kernels holds: mu, the EM
+// accumulator and the sensitivity, the PSF, the compressed lists (four entries per source
+// pixel), the ratio and the work slab.
+size_t general_bytes(const spect_plan_s& P)
+{
+    const Geometry& g = P.g;
+    const size_t vol = (size_t)g.nx * g.ny * g.nz * sizeof(float);
+    const size_t chunk = (size_t)view_chunk(g.nview, vol, slab_budget_bytes(false));
+    return base_bytes(P) + psf_bytes(P) + csr_bytes(P) + vol * (3 + chunk) + (size_t)g.nx * g.nz * g.nview * sizeof(float);
+}
+
+// Upper bound of what a low-memory plan on the fused kernels holds with its present
+// passes, and of what is live while it is made (spect_plan_create): the list lengths,
+// then a range of the fixed-length lists beside the gather's entries, then mu in both
+// layouts and the PSF beside the tap records, then everything that the plan keeps.
+size_t low_bytes(const spect_plan_s& P)
+{
+    const Geometry& g = P.g;
+    const size_t F = sizeof(float), nxy = (size_t)g.nx * g.ny, vol = nxy * g.nz * F, volt = nxy * g.kp * F;
+    const size_t psf = psf_bytes(P), scratch = P.separable ? 0 : (size_t)g.px * g.pz * g.nvp * g.ny * P.cls_x * F;
+    const size_t gather = gather_bytes(P, kLowAdjMax), chunk = (size_t)P.chunk;
+    const size_t records = (spect::fwd_records_floats(P) + spect::adj_records_floats(P)) * F;
+    const size_t lists = nxy * low_list_views(P) * kLowAdjMax * sizeof(spect::AdjEntry);
+    const size_t lengths = (nxy * g.nview + 1) * sizeof(int);
+    const size_t held = records + gather + 5 * volt + vol + (size_t)g.np * g.nz * g.nview * F +
+                        2 * (size_t)g.ny * P.ps * chunk * F + part_floats(P, P.chunk, P.chunk) * F +
+                        (P.tab_pass ? chunk : (size_t)g.nview) * g.ny * P.ts * F;
+    return base_bytes(P) + std::max({psf + vol + std::max(scratch, lengths), psf + vol + lists + gather,
+                                     psf + vol + volt + gather + records, held});
+}
+
+// A low-memory plan runs the fused kernels in the fewest passes with which it is no
+// larger than the general kernels' plan (or kSmallPlanBytes).  20 of its about 60 bytes per
+// (column, view) are rotation tables: where the tables of a pass, made again in each, take
+// less than three quarters of the passes, it holds those only.  Where no number of passes
+// is small enough it takes the general kernels.  SPECT_SLAB_MB sets the passes instead.
+//   EM update, tables of a pass against all: 192x128, 128 views, 37 taps 10.2 against 15.4 ms
+// (43 and 128 passes), 192x16, 128 views 1.11 against 2.07 (7 and 26); 128x80, 128 views 2.60
+// against 2.57 (8 and 10), 64x32, 64 views 0.195 against 0.175 (3 and 4).  192x192x5, 128 views:
+// 267 MB on the general kernels, 258 with the tables of a pass, above 283 with all of them.
+void configure_low(spect_plan_s* P)
+{
+    const int nview = P->g.nview;
+    auto passes_of = [&](int chunk) {
+        P->chunk = P->shape_views = chunk;
+        P->gsegs = chunk < nview ? 1 : spect::gather_segments(*P);
+        spect::default_shape(*P);
+    };
+    P->tab_pass = 0;
+    if (getenv("SPECT_SLAB_MB")) {
+        passes_of(view_chunk(nview, 2 * (size_t)P->g.ny * P->ps * sizeof(float), slab_budget_bytes(false)));
+        return;
+    }
+    const size_t limit = std::max(general_bytes(*P), kSmallPlanBytes);
+    auto fewest_passes = [&](int tab_pass) {  // 0: not within the limit
+        P->tab_pass = tab_pass;
+        for (int passes = 1, last = 0; passes <= nview; ++passes) {
+            const int chunk = (nview + passes - 1) / passes;
+            if (chunk == last) continue;
+            last = chunk;
+            passes_of(chunk);
+            if (low_bytes(*P) <= limit) return passes;
+            P->gsegs = 1;
+            if (low_bytes(*P) <= limit) return passes;
+        }
+        return 0;
+    };
+    const int per_pass = fewest_passes(1), all = fewest_passes(0);
+    if (all > 0 && (per_pass == 0 || 3 * all <= 4 * per_pass)) return;
+    if (per_pass > 0) {
+        fewest_passes(1);
+        return;
+    }
+    P->tab_pass = 0;
+    P->fast = P->recompute = 0;
+}
+
+// Kernels, launch shapes and views per pass of a plan: the work slab (and a recomputing
+// plan's factors) within the budget, the blur shapes for that many views.
 void configure_views(spect_plan_s* P)
 {
-    const size_t vol = (size_t)P->g.nx * P->g.ny * P->g.nz;
-    P->shape_views = P->g.nview;
-    if (P->fast) spect::default_shape(*P);
-    const size_t per_view = std::max(vol, P->fast ? spect::fused_slab_per_view(*P) : vol);
-    const size_t budget = P->fast && P->low ? low_budget_bytes(*P)
-                          : P->recompute   ? recompute_budget_bytes()
-                                           : slab_budget_bytes(P->fast);
-    P->chunk = view_chunk(*P, per_view, budget);
-    P->gsegs = P->fast ? spect::gather_segments(*P) : 1;
-    if (P->fast && P->chunk < P->g.nview) {
+    const Geometry& g = P->g;
+    if (P->fast && P->low) configure_low(P);
+    if (P->fast && P->low) return;
+    P->gsegs = 1;
+    const size_t vol = (size_t)g.nx * g.ny * g.nz;
+    if (!P->fast) {
+        P->chunk = view_chunk(g.nview, vol * sizeof(float), slab_budget_bytes(false));
+        return;
+    }
+    P->shape_views = g.nview;
+    spect::default_shape(*P);
+    const size_t per_view = std::max(vol, spect::fused_slab_per_view(*P));
+    P->chunk = view_chunk(g.nview, view_bytes(*P, per_view), P->recompute ? recompute_budget_bytes() : slab_budget_bytes(true));
+    P->gsegs = spect::gather_segments(*P);
+    if (P->chunk < g.nview) {
         P->shape_views = P->chunk;
         spect::default_shape(*P);
     }
@@ -232,7 +343,7 @@ void configure_views(spect_plan_s* P)
 void drop_fixed_lists(spect_plan_s* P, cudaStream_t st)
 {
     if (!P->gather || !P->adjf) return;
-    const size_t nlist = (size_t)P->g.nx * P->g.ny * P->g.nview;
+    const size_t nlist = (size_t)P->g.nx * P->g.ny * P->list_views;
     raw_free(P, P->adjf, st);
     P->adjf = nullptr;
     P->bytes -= nlist * (size_t)std::max(P->adj_max, 1) * sizeof(spect::AdjEntry);
@@ -338,6 +449,9 @@ spect_status fast_forward(spect_plan_s* P, const float* xt, float* v, const floa
     const int nview = P->g.nview;
     for (int l0 = 0; l0 < nview; l0 += P->chunk) {
         const int nv = std::min(P->chunk, nview - l0);
+        if (P->tab_pass)
+            SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_rot_tables(*P, l0, nv, st); }),
+                           "rotation table launch");
         if (P->recompute)  // Eq. (1) factors of this chunk's views
             SPECT_CUDA_TRY(counted(P, SPECT_K_ROTATE_ATTEN, st, [&] { return spect::launch_mubar_range(*P, l0, nv, st); }),
                            "attenuation launch");
@@ -347,9 +461,10 @@ spect_status fast_forward(spect_plan_s* P, const float* xt, float* v, const floa
         SPECT_CUDA_TRY(counted(P, SPECT_K_CONV_FWD, st,
                                [&] { return spect::launch_fused_forward(*P, l0, nv, st); }),
                        "fused forward launch");
+        SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st,
+                               [&] { return spect::launch_fwd_reduce(*P, l0, nv, v, y, rbar, st); }),
+                       "depth-group reduce launch");
     }
-    SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_fwd_reduce(*P, v, y, rbar, st); }),
-                   "depth-group reduce launch");
     return SPECT_OK;
 }
 
@@ -360,6 +475,9 @@ spect_status fast_back(spect_plan_s* P, const float* v, float* out_t, spect::EmA
     for (int l0 = 0; l0 < nview; l0 += P->adj_chunk) {
         const int nv = std::min(P->adj_chunk, nview - l0);
         const bool last = l0 + nv >= nview;
+        if (P->tab_pass)
+            SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_rot_tables(*P, l0, nv, st); }),
+                           "rotation table launch");
         if (P->recompute)  // Eq. (1) factors of this chunk's views
             SPECT_CUDA_TRY(counted(P, SPECT_K_CONV_ADJ, st, [&] { return spect::launch_mubar_range(*P, l0, nv, st); }),
                            "attenuation launch");
@@ -430,42 +548,30 @@ namespace {
 // of the allocations in spect_plan_create, with the adjacency lists at their
 // largest: 8 fixed entries per list, or 4 entries per source pixel in the
 // compressed form, whichever is larger).  When the fused kernels serve a
-// geometry, their buffers dominate those of the low-memory path it may fall
-// back to, so the fused sizes bound both.
+// geometry, their buffers dominate those of the general kernels it may fall
+// back to, so the fused sizes bound both; a low-memory plan's bound is the larger of the two.
 size_t plan_bytes_bound(const spect_plan_s& P)
 {
+    if (!P.fast) return general_bytes(P);
+    if (P.low) return std::max(low_bytes(P), general_bytes(P));
     const Geometry& g = P.g;
     const size_t F = sizeof(float);
-    const size_t vol = (size_t)g.nx * g.ny * g.nz, nproj = (size_t)g.nx * g.nz * g.nview;
-    const size_t nxy = (size_t)g.nx * g.ny, nrows = (size_t)g.nvp * g.ny, nlist = nxy * g.nview;
+    const size_t vol = (size_t)g.nx * g.ny * g.nz, nxy = (size_t)g.nx * g.ny, nlist = nxy * g.nview;
     const size_t volt = nxy * g.kp;  // an internal volume
-    size_t b = sizeof(int);
-    if (!P.fast) b += 2 * vol * F;  // mu and the EM accumulator in the image layout
-    if (P.separable) b += ((size_t)g.px * 4 + (size_t)g.pz * (1 + P.cls_z)) * nrows * F;
-    else b += (size_t)g.px * g.pz * nrows * (1 + (size_t)P.cls_x * P.cls_z) * F;
-    b += (size_t)g.nview * sizeof(ViewRot);
-    // a low-memory plan's bound leaves out the fixed lists, which are set-up input only
-    const size_t fixed = P.low ? 0 : nlist * 8 * sizeof(spect::AdjEntry);
-    const size_t csr = (nlist + 1) * sizeof(int) + 4 * nlist * sizeof(spect::AdjEntry);
-    b += P.fast ? (P.low ? 0 : std::max(fixed, csr)) : csr;
-    const size_t per_view = std::max(vol, P.fast ? spect::fused_slab_per_view(P) : vol);
+    size_t b = base_bytes(P) + psf_bytes(P) + std::max(nlist * 8 * sizeof(spect::AdjEntry), csr_bytes(P));
+    const size_t per_view = std::max(vol, spect::fused_slab_per_view(P));
     const size_t chunk = (size_t)P.chunk;
     b += per_view * chunk * F;
-    b += (vol + (P.fast ? (size_t)g.np * g.nz * g.nview : nproj)) * F;
-    if (P.fast) b += (spect::fwd_records_floats(P) + spect::adj_records_floats(P)) * F;
-    if (P.fast) {
-        // attenuation factors of every view, or of one chunk plus mu in the internal layout
-        b += P.recompute ? ((size_t)g.ny * P.ps * chunk + volt) * F : (size_t)g.ny * P.ps * g.nview * F;
-        b += 4 * volt * F;
-        b += std::max(nproj * (size_t)spect::fused_groups(P), 2 * (size_t)P.gsegs * volt) * F +
-             (size_t)g.nview * g.ny * P.ts * F;
-        // patch gather: boxes and box-local entries (at most 8 per list)
-        const size_t np = (size_t)((g.nx + 7) / 8) * ((g.ny + 7) / 8) * g.nview;
-        b += np * 16 + np * 64 * 8 * sizeof(spect::AdjEntry) + np * 16;  // + rotation boxes
-        b += np / g.nview * ((g.kp + 15) / 16) * sizeof(int);           // segment arrivals
-        if (P.rot3)  // the eight-tap table
-            b += (size_t)g.nview * g.ny * 16 * (size_t)g.nx * F;
-    }
+    b += (vol + (size_t)g.np * g.nz * g.nview) * F;
+    b += (spect::fwd_records_floats(P) + spect::adj_records_floats(P)) * F;
+    // attenuation factors of every view, or of one chunk plus mu in the internal layout
+    b += P.recompute ? ((size_t)g.ny * P.ps * chunk + volt) * F : (size_t)g.ny * P.ps * g.nview * F;
+    b += 4 * volt * F;
+    b += std::max(part_floats(P, P.chunk, P.chunk), volt) * F + (size_t)g.nview * g.ny * P.ts * F;
+    // patch gather (at most 8 entries per list), rotation boxes
+    b += gather_bytes(P, 8) + (size_t)((g.nx + 7) / 8) * ((g.ny + 7) / 8) * g.nview * 16;
+    if (P.rot3)  // the eight-tap table
+        b += (size_t)g.nview * g.ny * 16 * (size_t)g.nx * F;
     return b;
 }
 
@@ -609,6 +715,7 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
     // attenuation recomputed (96x96x64, 60 views, 21 taps: EM update 3327 us with the
     // low-memory kernels); the others keep the low-memory kernels
     if (P->low && P->fast) P->recompute = 1;
+    configure_views(P);
     if (P->separable) {
         P->sep_tk = spect::choose_sep_tile(g, P->cls_z, (size_t)smem_optin);
         if (P->sep_tk < 1) {
@@ -679,7 +786,10 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         int mx = 0;
         cudaError_t e2 = cudaMemcpyAsync(&mx, d_max, sizeof(int), cudaMemcpyDeviceToHost, st);
         cudaError_t e4 = cudaStreamSynchronize(st);
-        if (mx > 8) P->fast = P->recompute = 0;  // fixed-length lists are instantiated up to 8 entries
+        if (mx > (P->low ? kLowAdjMax : 8) && P->fast) {  // fixed-length lists are instantiated up to 8 entries
+            P->fast = P->recompute = P->tab_pass = 0;
+            configure_views(P);
+        }
         if (e2 == cudaSuccess && e4 == cudaSuccess && !P->fast) {  // fixed-length lists need only the longest
             counts.resize(nlist);
             e2 = cudaMemcpyAsync(counts.data(), d_counts, nlist * sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -693,9 +803,11 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         if (P->rot3) mx = std::max(mx, 8);  // eight entries per (voxel, view) for the three-pass lists
         P->adj_max = mx;
         if (P->fast) {
-            PLAN_ALLOC(P->adjf, nlist * (size_t)std::max(mx, 1), "adjacency lists");
             if (mx < 1) P->adj_max = 1;
-            PLAN_TRY(spect::launch_build_adjacency_fixed(*P, st), "adjacency fill launch");
+            P->list_views = P->low ? low_list_views(*P) : nview;
+            PLAN_ALLOC(P->adjf, nxy * P->list_views * P->adj_max, "adjacency lists");
+            if (P->list_views == nview)
+                PLAN_TRY(spect::launch_build_adjacency_fixed(*P, 0, nview, st), "adjacency fill launch");
         } else {
             std::vector<int> off(nlist + 1);
             size_t tot = 0;
@@ -713,6 +825,29 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         PLAN_TRY(cudaStreamSynchronize(st), "adjacency fill");
     }
 
+    // What is live at once is kept low for the sake of low-memory plans (low_bytes): the
+    // gather's entries replace the lists before the large buffers are made (the three-pass
+    // lists are written later), and the image-layout mu goes as soon as mut is filled.
+    if (P->fast && !P->rot3) {
+        PLAN_TRY(spect::build_gather(*P, st), "patch gather set-up");
+        drop_fixed_lists(P, st);
+        if (P->adjf && P->list_views < nview) {  // the list gather reads the lists of every view
+            raw_free(P, P->adjf, st);
+            P->bytes -= nxy * P->list_views * P->adj_max * sizeof(spect::AdjEntry);
+            P->list_views = nview;
+            PLAN_ALLOC(P->adjf, nxy * nview * P->adj_max, "adjacency lists");
+            PLAN_TRY(spect::launch_build_adjacency_fixed(*P, 0, nview, st), "adjacency fill launch");
+        }
+    }
+    if (P->recompute) {
+        // mu stays in the [j][i][k] layout; the factors are made per view chunk
+        PLAN_ALLOC(P->mut, volt, "attenuation map (internal layout)");
+        PLAN_TRY(spect::launch_transpose(P->mu, P->mut, nz, (int)nxy, (int)nxy, g.kp, st), "mu transpose launch");
+        raw_free(P, P->mu, st);
+        P->mu = nullptr;
+        P->bytes -= vol * sizeof(float);
+    }
+
     // the blur kernels' tap records; the factors (or the stack) themselves are not read again
     if (P->fast) {
         PLAN_ALLOC(P->frec, spect::fwd_records_floats(*P), "tap records");
@@ -727,7 +862,6 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
     }
 
     // work slab and EM buffers
-    configure_views(P);
     const size_t per_view = std::max(vol, P->fast ? spect::fused_slab_per_view(*P) : vol);
     PLAN_ALLOC(P->slab, per_view * (size_t)P->chunk, "work slab");
     P->slab_cap = per_view * (size_t)P->chunk;
@@ -760,10 +894,11 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
         PLAN_ALLOC(P->ut, volt, "internal regulariser target");
         for (float* p : {P->xt, P->et, P->st, P->ut})  // defines their padding
             PLAN_TRY(cudaMemsetAsync(p, 0, volt * sizeof(float), st), "clear internal volume");
-        P->part_cap = part_floats(*P, P->adj_chunk);
+        P->part_cap = part_floats(*P, P->chunk, P->adj_chunk);
         PLAN_ALLOC(P->part, P->part_cap, "depth-group partial sums");
         // mu in the [j][i][k] layout (temporary, the slab serves as scratch)
-        PLAN_TRY(spect::launch_transpose(P->mu, P->slab, nz, (int)nxy, (int)nxy, g.kp, st), "mu transpose launch");
+        if (!P->recompute)
+            PLAN_TRY(spect::launch_transpose(P->mu, P->slab, nz, (int)nxy, (int)nxy, g.kp, st), "mu transpose launch");
         if (P->rot3) {
             // three passes: the eight-tap table of the forward rotation kernel, the
             // eight-entry lists of the adjoint gather (in adjf), and the attenuation
@@ -776,27 +911,21 @@ spect_status spect_plan_create(spect_plan* out, int nx, int ny, int nz, int nvie
             PLAN_TRY(e3, "three-pass rotation set-up");
             PLAN_TRY(spect::build_gather(*P, st), "patch gather set-up");  // boxes of the three-pass lists
             drop_fixed_lists(P, st);
-        } else if (P->recompute) {
-            // mu stays in the [j][i][k] layout; the factors are made per view chunk
-            PLAN_ALLOC(P->mut, volt, "attenuation map (internal layout)");
-            PLAN_TRY(cudaMemcpyAsync(P->mut, P->slab, volt * sizeof(float), cudaMemcpyDeviceToDevice, st),
-                     "attenuation map copy");
-            PLAN_ALLOC(P->rtab, (size_t)nview * ny * P->ts, "rotation tables");
-            PLAN_TRY(spect::launch_rot_tables(*P, st), "rotation table launch");
-            PLAN_TRY(spect::build_gather(*P, st), "patch gather set-up");
-            drop_fixed_lists(P, st);
         } else {
-            PLAN_ALLOC(P->rtab, (size_t)nview * ny * P->ts, "rotation tables");
-            PLAN_TRY(spect::launch_rot_tables(*P, st), "rotation table launch");
-            PLAN_TRY(spect::launch_mubar_cache(*P, P->slab, st), "attenuation cache launch");
-            PLAN_TRY(spect::build_gather(*P, st), "patch gather set-up");
-            drop_fixed_lists(P, st);
-            PLAN_TRY(spect::build_rotpatch(*P, st), "patch rotation set-up");
+            const int tab_views = P->tab_pass ? P->chunk : nview;
+            PLAN_ALLOC(P->rtab, (size_t)tab_views * ny * P->ts, "rotation tables");
+            if (!P->tab_pass) PLAN_TRY(spect::launch_rot_tables(*P, 0, nview, st), "rotation table launch");
+            if (!P->recompute) {
+                PLAN_TRY(spect::launch_mubar_cache(*P, P->slab, st), "attenuation cache launch");
+                PLAN_TRY(spect::build_rotpatch(*P, st), "patch rotation set-up");
+            }
         }
-        // the image-layout map was set-up input only
-        raw_free(P, P->mu, st);
-        P->mu = nullptr;
-        P->bytes -= vol * sizeof(float);
+        PLAN_TRY(spect::build_gather_maps(*P), "tensor maps of the patch gather");
+        if (P->mu) {  // the image-layout map was set-up input only
+            raw_free(P, P->mu, st);
+            P->mu = nullptr;
+            P->bytes -= vol * sizeof(float);
+        }
     }
     PLAN_TRY(cudaStreamSynchronize(st), "plan set-up");
     *out = P;
@@ -1117,11 +1246,11 @@ spect_status reconfigure(spect_plan_s* P, int J, int adj_J, int tiles, int adj_t
     const size_t vol = (size_t)g.nx * g.ny * g.nz;
     const size_t per_view = std::max(vol, spect::fused_slab_per_view(*P));
     const size_t budget = P->recompute ? recompute_budget_bytes() : slab_budget_bytes(true);
-    const int chunk = view_chunk(*P, per_view, budget);
+    const int chunk = view_chunk(g.nview, view_bytes(*P, per_view), budget);
     const int adj_chunk = P->adj_chunk_req > 0 ? std::min(P->adj_chunk_req, chunk) : chunk;
     spect_status r = realloc_floats(P, &P->slab, &P->slab_cap, per_view * (size_t)chunk, st, "work slab");
     if (r == SPECT_OK)
-        r = realloc_floats(P, &P->part, &P->part_cap, part_floats(*P, adj_chunk), st,
+        r = realloc_floats(P, &P->part, &P->part_cap, part_floats(*P, chunk, adj_chunk), st,
                            "depth-group partial sums");
     if (r == SPECT_OK && P->recompute)  // the attenuation factors of one chunk
         r = realloc_floats(P, &P->mubar, &P->mubar_cap, (size_t)g.ny * P->ps * chunk, st, "attenuation factors");
@@ -1151,7 +1280,7 @@ spect_status single_pass(spect_plan_s* P, cudaStream_t st)
     const size_t per_view = std::max(vol, spect::fused_slab_per_view(*P));
     spect_status r = realloc_floats(P, &P->slab, &P->slab_cap, per_view * (size_t)g.nview, st, "work slab");
     if (r == SPECT_OK)
-        r = realloc_floats(P, &P->part, &P->part_cap, part_floats(*P, g.nview), st, "depth-group partial sums");
+        r = realloc_floats(P, &P->part, &P->part_cap, part_floats(*P, g.nview, g.nview), st, "depth-group partial sums");
     if (r != SPECT_OK) {
         const std::string msg = g_err;
         refresh_maps(P);  // the slab may have moved

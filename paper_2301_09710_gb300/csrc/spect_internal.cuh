@@ -113,8 +113,9 @@ struct spect_plan_s {
     float* et = nullptr;         // nx*ny*kp, [j][i][k] back-projection accumulator
     float* st = nullptr;         // nx*ny*kp, [j][i][k] sensitivity
     float* ut = nullptr;         // nx*ny*kp, [j][i][k] regulariser target of the regularised EM
-    float* part = nullptr;       // G * nx*nz*nview forward partial sums
-    spect::AdjEntry* adjf = nullptr;  // nview*nx*ny*adj_max fixed-length lists
+    float* part = nullptr;       // forward partial sums of a pass (G * nx*nz*chunk); sums of A' (part_floats)
+    spect::AdjEntry* adjf = nullptr;  // list_views*nx*ny*adj_max fixed-length lists
+    int list_views = 0;          // views adjf holds (all; low-memory plans: ranges of them, while the gather is built)
     // patch-staged adjoint gather (gather.cu); gather == 0: the list gather k_adj_rot_t
     int gather = 0;
     int4* gboxes = nullptr;      // [patch][l] source box (i0, j0, size, tensor map)
@@ -144,7 +145,8 @@ struct spect_plan_s {
     CUtensorMap rmap_x, rmap_mu; // x_t (k, i, j) and the attenuation cache (k, i, plane)
     int ps = 0;                  // plane stride of the attenuation cache and slab: nx*kp
     int ts = 0;                  // rotation table block per (view, row): 5*nx rounded up to 4
-    float* rtab = nullptr;       // nview*ny*ts rotation tables of the fused forward
+    float* rtab = nullptr;       // rotation tables of the fused forward: nview*ny*ts, or chunk*ny*ts (tab_pass)
+    int tab_pass = 0;            // the tables are made for the views of each pass (low-memory plans)
     int* err = nullptr;          // device error word (SPECT_ETIMEOUT when a bounded wait ran out)
     size_t bytes = 0;
     // launch accounting and optional per-launch event timing
@@ -513,8 +515,10 @@ int fused_tiles_fit(const Geometry& g, int bucket, int J, int adj_J, int tiles, 
 // out[c][r] = in[r][c], R x C; row pitches of in and out (at least C and R)
 cudaError_t launch_transpose(const float* in, float* out, int R, int C, int ip, int op, cudaStream_t st);
 cudaError_t launch_mubar_cache(const spect_plan_s& P, const float* mu_t, cudaStream_t st);
-cudaError_t launch_build_adjacency_fixed(const spect_plan_s& P, cudaStream_t st);
-cudaError_t launch_rot_tables(const spect_plan_s& P, cudaStream_t st);
+// the lists of views l0 .. l0+nv-1 into adjf, [q][nv][adj_max]
+cudaError_t launch_build_adjacency_fixed(const spect_plan_s& P, int l0, int nv, cudaStream_t st);
+// rotation tables of views l0 .. l0+nv-1, at the start of P.rtab
+cudaError_t launch_rot_tables(const spect_plan_s& P, int l0, int nv, cudaStream_t st);
 cudaError_t launch_fused_forward(const spect_plan_s& P, int l0, int nv, cudaStream_t st);
 cudaError_t launch_fused_rotate(const spect_plan_s& P, const float* xt, int l0, int nv, cudaStream_t st);
 // three-pass rotation (rot3.cu): table block size, and the plan-time build of
@@ -526,8 +530,11 @@ size_t fused_slab_per_view(const spect_plan_s& P);
 cudaError_t launch_fused_adjoint(const spect_plan_s& P, const float* v, int l0, int nv, cudaStream_t st);
 // out (rows of np) = v (rows of nx)
 cudaError_t launch_pad_rows(const spect_plan_s& P, const float* v, float* out, cudaStream_t st);
-cudaError_t launch_fwd_reduce(const spect_plan_s& P, float* v, const float* em_y, const float* em_rbar,
+// the depth sums of views l0 .. l0+nv-1 from the partials of their pass
+cudaError_t launch_fwd_reduce(const spect_plan_s& P, int l0, int nv, float* v, const float* em_y, const float* em_rbar,
                               cudaStream_t st);
+// boxes and entries of the patch gather from adjf, or, where it holds fewer views, from their lists made in it
+// range by range (adjf is not read again); the gather's tensor maps come with the slab
 cudaError_t build_gather(spect_plan_s& P, cudaStream_t st);
 // (re)encode P.gmaps after the slab or the view chunk changed
 cudaError_t build_gather_maps(spect_plan_s& P);
@@ -544,6 +551,13 @@ inline const float* mubar_for(const spect_plan_s& P, int l0)
     if (!P.recompute) return P.mubar;
     return reinterpret_cast<const float*>(reinterpret_cast<uintptr_t>(P.mubar) -
                                           (uintptr_t)l0 * P.g.ny * P.ps * sizeof(float));
+}
+// The rotation tables as the kernels index them, rtab + (l ny + j) ts for view l (as mubar_for).
+inline const float* rtab_for(const spect_plan_s& P, int l0)
+{
+    if (!P.tab_pass) return P.rtab;
+    return reinterpret_cast<const float*>(reinterpret_cast<uintptr_t>(P.rtab) -
+                                          (uintptr_t)l0 * P.g.ny * P.ts * sizeof(float));
 }
 cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,
                               cudaStream_t st);

@@ -1,0 +1,72 @@
+"""Low-memory plans: what they hold, and what is live while they are made."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from gpu_helpers import dev, host, need_gpu, torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _gpu():
+    need_gpu()
+
+
+# nx, nz, nview, taps, separable: MB that the bound of a plan on the general low-memory kernels
+# comes to (image, projections, compressed adjacency lists and a slab of at most 256 MiB)
+GENERAL_MB = [
+    (96, 64, 60, 21, True, 170.1),
+    (128, 80, 128, 37, True, 364.0),
+    (160, 96, 120, 29, True, 413.0),
+    (192, 128, 128, 37, True, 503.5),
+    (256, 64, 128, 21, True, 629.3),
+    (512, 64, 120, 11, True, 1618.1),
+    (96, 64, 60, 21, False, 171.7),
+    (64, 32, 64, 11, True, 45.1),
+    (192, 5, 128, 3, True, 267.0),
+]
+
+
+@pytest.mark.parametrize("case", GENERAL_MB, ids=[f"{c[0]}x{c[1]}v{c[2]}p{c[3]}{'' if c[4] else 'full'}" for c in GENERAL_MB])
+def test_low_memory_bound_does_not_exceed_the_general_kernels(case):
+    from paper_2301_09710_gb300.projector import plan_bytes
+    nx, nz, nview, p, separable, mb = case
+    assert plan_bytes(nx, nz, nview, p, p, separable=separable, low_memory=True) <= 1e6 * (mb + 0.05)
+
+
+def _pool_high():
+    """Read and reset the high-water mark of the device's memory pool (bytes in use)."""
+    rt = ctypes.CDLL("libcudart.so.13")
+    pool, high, zero = ctypes.c_void_p(), ctypes.c_uint64(), ctypes.c_uint64(0)
+    assert rt.cudaDeviceGetDefaultMemPool(ctypes.byref(pool), torch.cuda.current_device()) == 0
+    used_now, used_high = 7, 8  # cudaMemPoolAttrUsedMemCurrent, cudaMemPoolAttrUsedMemHigh
+    assert rt.cudaMemPoolGetAttribute(pool, used_high, ctypes.byref(high)) == 0
+    assert rt.cudaMemPoolSetAttribute(pool, used_high, ctypes.byref(zero)) == 0  # to the bytes now in use
+    now = ctypes.c_uint64()
+    assert rt.cudaMemPoolGetAttribute(pool, used_now, ctypes.byref(now)) == 0
+    return high.value, now.value
+
+
+@pytest.mark.parametrize("kind", ["lowmem", "default", "recompute"])
+@pytest.mark.parametrize("nx,nz,nview,p", [(96, 64, 60, 21), (64, 5, 90, 3), (129, 7, 100, 5)])
+def test_plan_creation_stays_within_plan_bytes(kind, nx, nz, nview, p):
+    """The bound covers what is live while the plan is made, not only what it keeps: the pool's
+    high-water mark over creation and one EM update.  Up to 256 bytes per allocation are rounding."""
+    from paper_2301_09710_gb300 import SpectPlan
+    from paper_2301_09710_gb300.projector import plan_bytes
+    kw = {"lowmem": {"low_memory": True}, "default": {}, "recompute": {"recompute_attenuation": True}}[kind]
+    taps = np.full((1, nx, p), 1.0 / p, np.float32)
+    x, y = dev(np.ones((nz, nx, nx))), dev(np.ones((nview, nz, nx)))
+    torch.cuda.synchronize()
+    _, before = _pool_high()
+    plan = SpectPlan(nx, nz, nview, mu=dev(np.full((nz, nx, nx), 0.01)), fx=taps, fz=taps, **kw)
+    plan.em_step(x, y, None, niter=1)
+    torch.cuda.synchronize()
+    high, _ = _pool_high()
+    bound = plan_bytes(nx, nz, nview, p, p, **kw)
+    held = plan.info()["device_bytes"]
+    plan.check()
+    plan.close()
+    assert held <= bound and high - before <= bound + 64 * 256, (held, high - before, bound)
