@@ -294,15 +294,21 @@ __global__ void k_fwd_records(Geometry g, int P, int PT, int nkb, const float* _
 }
 
 // v(i,k,l) = sum over depth groups of the partials (fixed order) of the views of a pass
-// (nproj values), optionally turned into the EM ratio y / (v + rbar), whose rows are np long.
-__global__ void k_fwd_reduce(const float* __restrict__ part, int G, size_t nproj, float* __restrict__ v, int nx, int np,
-                             const float* __restrict__ em_y, const float* __restrict__ em_rbar)
+// (nproj values; comp: the partials' compensation terms, or NULL), optionally turned into
+// the EM ratio y / (v + rbar), whose rows are np long.
+__global__ void k_fwd_reduce(const float* __restrict__ part, const float* __restrict__ comp, int G, size_t nproj,
+                             float* __restrict__ v, int nx, int np, const float* __restrict__ em_y,
+                             const float* __restrict__ em_rbar)
 {
     wait_previous_kernel();
     const size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= nproj) return;
     KSum acc;  // up to ny partials (J = 1): compensated
-    for (int gq = 0; gq < G; ++gq) acc.add(part[(size_t)gq * nproj + o]);
+    for (int gq = 0; gq < G; ++gq) {
+        const float p = part[(size_t)gq * nproj + o];
+        if (comp) acc.merge(p, comp[(size_t)gq * nproj + o]);
+        else acc.add(p);
+    }
     const float s = acc.value();
     if (em_y) {
         const float yb = s + (em_rbar ? em_rbar[o] : 0.f);
@@ -525,9 +531,10 @@ __global__ void __launch_bounds__(kDirThreads, 1) k_fwd_dir_fused(const __grid_c
     if (mine) {
         const int k0 = k_lo + kb * CZ;
         float* pout = part + ((size_t)grp * gridDim.y + v) * pln + i0 + i;
+        const size_t half = (size_t)d.G * gridDim.y * pln;
 #pragma unroll
         for (int c = 0; c < CZ; ++c)
-            if (k0 + c < nz) pout[(size_t)(k0 + c) * nx] = acc[c].value();
+            if (k0 + c < nz) acc[c].store(pout + (size_t)(k0 + c) * nx, half);
     }
 }
 
@@ -1189,12 +1196,15 @@ void choose_shape(spect_plan_s& Pl)
         for (int J : {8, 4, 6, 7, 5, 3, 2, 1}) {  // longer plain depth sums would cost accuracy
             if (J > g.ny) continue;
             const FwdDims f = fwd_dims<P>(g, J, std::max(tiles, Pl.min_nT), limit);
-            if (smem_fwd<P>(f) <= limit && (f.racc || ti == 16) && (keep_J == 0 || J == keep_J)) {
+            // sums in shared memory are plain: one plane per block where they are to be compensated
+            const bool sums = f.racc || (ti == 16 && (!Pl.low || J == 1));
+            if (smem_fwd<P>(f) <= limit && sums && (keep_J == 0 || J == keep_J)) {
                 const int B = blocks_per_sm(smem_fwd<P>(f), f.T, FwdBlock<P>::regs);
-                // + the reduce: G partials written and read
+                const int comp = Pl.low && f.racc;
+                // + the reduce: G partials (and compensation terms) written and read
                 const double c = blur_cost(P, (long long)f.G * f.nT * nv, J, 1.0, f.T, B, Pl.sms) +
-                                 (double)f.G * g.nx * g.nz * nv * 8.0 / 5e6;
-                if (c < 0.98 * fbest) fbest = c, Pl.fused_J = J, Pl.fwd_nT = f.nT;
+                                 (double)f.G * g.nx * g.nz * nv * 8.0 * (1 + comp) / 5e6;
+                if (c < 0.98 * fbest) fbest = c, Pl.fused_J = J, Pl.fwd_nT = f.nT, Pl.part_comp = comp;
             }
             const AdjDims a = adj_dims<P>(g, J, std::max(tiles, Pl.min_nT), limit);
             if (smem_adj<P>(a) <= limit) {
@@ -1216,6 +1226,7 @@ void default_shape(spect_plan_s& P)
 {
     const Geometry& g = P.g;
     if (!P.separable) {  // blocks of the full-PSF forward kernel
+        P.part_comp = P.low;
         if (P.shape_views < g.nview && !P.low) return;  // as choose_shape's keep_J
         P.fused_J = P.adj_J = 8;
         const long long blocks = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * P.shape_views;
@@ -1279,7 +1290,8 @@ cudaError_t launch_fwd_reduce(const spect_plan_s& P, int l0, int nv, float* v, c
 {
     const size_t view = (size_t)P.g.nx * P.g.nz, nproj = view * nv, at = view * l0;
     v += em_y ? (size_t)P.g.np * P.g.nz * l0 : at;
-    return launch_chained(k_fwd_reduce, (unsigned)((nproj + 255) / 256), 256, 0, st, P.part, fused_groups(P), nproj, v,
+    const float* comp = P.part_comp ? P.part + fused_groups(P) * nproj : nullptr;
+    return launch_chained(k_fwd_reduce, (unsigned)((nproj + 255) / 256), 256, 0, st, P.part, comp, fused_groups(P), nproj, v,
                           P.g.nx, P.g.np, em_y ? em_y + at : nullptr, em_rbar ? em_rbar + at : nullptr);
 }
 

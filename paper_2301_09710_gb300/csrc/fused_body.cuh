@@ -333,19 +333,24 @@ __host__ __device__ inline size_t fwd_smem_floats(const FwdDims& d, int PT)
            (d.racc ? 0 : (size_t)d.urows * d.apc) + 8;
 }
 
-// A depth sum: plain, or compensated (KS).
+// A depth sum: plain, or compensated (KS).  store() leaves a group's sum at p, a
+// compensated one's compensation term at p + half, for the reduce to carry on with.
 template <bool KS>
 struct DepthSum {
     float s = 0.f;
     __device__ __forceinline__ void add(float x) { s += x; }
-    __device__ __forceinline__ float value() const { return s; }
+    __device__ __forceinline__ void store(float* p, size_t) const { *p = s; }
 };
 template <>
-struct DepthSum<true> : KSum {};
+struct DepthSum<true> : KSum {
+    __device__ __forceinline__ void store(float* p, size_t half) const { p[0] = s, p[half] = c; }
+};
 
-// KS: low-memory plans, whose depth sums are compensated throughout (5 to 14 % slower;
-// at 96x96x64 the relative error of A is 3.8e-8, with plain sums of 8 planes before the
-// compensated reduce 4.3e-8).
+// KS: low-memory plans, whose depth sums are compensated over all depths, as the general
+// kernels' are.  Relative error of A, with the groups' terms carried on and with each
+// group rounded: 64x32, 11 taps 3.24e-8 and 3.50e-8, 16x600, 3 taps 3.60e-8 and 4.19e-8
+// (general kernels 3.04e-8 and 3.60e-8); 96x96x64, 60 views: 508 and 511 us an EM update.
+// Compensated sums for every plan cost 5 to 14 % of the forward blur.
 // RACC: a thread keeps the depth sums of its one k-pass item (16 k of a column)
 // in registers over all planes of the group, so the k-pass touches shared memory
 // only to read U; otherwise (planes of more than 640 items) they are in ACC.
@@ -516,12 +521,13 @@ __device__ __forceinline__ void fwd_sep_body(const Geometry& g, const FwdDims& d
 
     // partial depth sums of this group: part[grp][v][k][i] (v of the nv views of the pass), this tile's columns
     float* pout = part + ((size_t)grp * nv + v) * pln + i0;
+    const size_t half = (size_t)d.G * nv * pln;
     if (RACC) {
         if (tid < ti * d.nkb) {
 #pragma unroll
             for (int c = 0; c < CZ; ++c) {
                 const int k = kp_kb * CZ + c;
-                if (k < nz) pout[(size_t)k * nx + kp_i] = acc[c].value();
+                if (k < nz) acc[c].store(pout + (size_t)k * nx + kp_i, half);
             }
         }
     } else {

@@ -182,12 +182,13 @@ int view_chunk(int nview, size_t bytes_per_view, size_t budget)
     return (int)((nview + passes - 1) / passes);
 }
 
-// Floats of P.part.  In A: the depth-group partial sums of a pass of `chunk` views.
+// Floats of P.part.  In A: the depth-group partial sums of a pass of `chunk` views, and
+// the compensation terms of low-memory plans' sums.
 // In A' the same buffer holds the sums and compensation terms of the view segments, or
 // between its passes (adj_chunk views each) the compensation terms of the view sums.
 size_t part_floats(const spect_plan_s& P, int chunk, int adj_chunk)
 {
-    const size_t part = (size_t)P.g.nx * P.g.nz * chunk * spect::fused_groups(P);
+    const size_t part = (size_t)P.g.nx * P.g.nz * chunk * spect::fused_groups(P) * (1 + P.part_comp);
     const size_t volt = (size_t)P.g.nx * P.g.ny * P.g.kp;
     return std::max(part, adj_chunk < P.g.nview ? volt : (P.gsegs > 1 ? 2 * P.gsegs * volt : 0));
 }

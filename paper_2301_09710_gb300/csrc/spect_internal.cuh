@@ -82,6 +82,7 @@ struct spect_plan_s {
     float* slab = nullptr;       // chunk * nx*ny*nz
     size_t slab_cap = 0;         // floats allocated for slab
     size_t part_cap = 0;         // floats allocated for part
+    int part_comp = 0;           // part holds compensation terms behind the sums (low-memory plans)
     float* e = nullptr;          // nx*ny*nz  (EM back-projection accumulator)
     float* ratio = nullptr;      // nx*nz*nview (EM ratio / ones); fused plans: rows of np
     float* s = nullptr;          // nx*ny*nz  (sensitivity A'1)

@@ -1,4 +1,5 @@
-"""Low-memory plans: what they hold, and what is live while they are made."""
+"""Low-memory plans: what they hold, what is live while they are made, and the precision of
+their depth sums."""
 import ctypes
 
 import numpy as np
@@ -70,3 +71,22 @@ def test_plan_creation_stays_within_plan_bytes(kind, nx, nz, nview, p):
     plan.check()
     plan.close()
     assert held <= bound and high - before <= bound + 64 * 256, (held, high - before, bound)
+
+
+@pytest.mark.parametrize("path,nx,nz,nview", [("lowmem", 32, 16, 300), ("lowmem", 16, 600, 300), ("direct_lowmem", 32, 16, 3)])
+def test_low_memory_depth_sums_are_compensated_over_all_depths(path, nx, nz, nview):
+    """Planes 2^24, 1, 0 ..., -2^24, 0 ... under a one-tap PSF at angle 0: every term and every
+    compensation term is a whole number that FP32 holds, so the compensated sum over all depths is
+    exact (one per sixteen planes), while a sum that drops the 1, within a group of planes or
+    between groups, gives 0.  16x600: more work items than a block has threads.
+    Enough views that several planes go to a block."""
+    from paper_2301_09710_gb300 import SpectPlan
+    x = np.zeros((nz, nx, nx), np.float32)
+    x[:, 0::16], x[:, 1::16], x[:, 8::16] = 2.0 ** 24, 1.0, -2.0 ** 24
+    one = np.ones((1, nx, 1), np.float32)
+    kw = {"fx": one, "fz": one} if path == "lowmem" else {"psf": one[..., None]}
+    plan = SpectPlan(nx, nz, nview, angles=[0.0] * nview, low_memory=True, **kw)
+    got = host(plan.forward(dev(x)))
+    plan.check()
+    plan.close()
+    assert np.array_equal(got, np.full((nview, nz, nx), nx // 16, np.float64))
