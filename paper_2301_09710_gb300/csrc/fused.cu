@@ -731,9 +731,9 @@ __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const Adj
     const size_t vstride = (size_t)g.ny * ps;
     const size_t o = (size_t)q * g.kp + k;
     KSum acc[VEC];
-    if (ps_.resume)  // the sums of the views of earlier passes
+    if (ps_.resume)  // the sums of the views of earlier launches
 #pragma unroll
-        for (int u = 0; u < VEC; ++u) acc[u].s = out[o + u], acc[u].c = ps_.comp[o + u];
+        for (int u = 0; u < VEC; ++u) acc[u].s = ps_.acc[o + u], acc[u].c = ps_.acc_c[o + u];
     // four views per step: all entry loads, then all slab loads, are issued
     // before any is used, so the chain of dependent loads is 4x shorter
     constexpr int UV = 4;
@@ -798,9 +798,15 @@ __global__ void __launch_bounds__(256) k_adj_rot_t(Geometry g, int ps, const Adj
         for (int u = 0; u < VEC; ++u) acc[u] = tot[u];
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
-        if (ps_.more) {
-            out[o + u] = acc[u].s;
-            ps_.comp[o + u] = acc[u].c;
+        if (ps_.merge) {  // add this segment to the ones before it
+            KSum t;
+            if (ps_.tot_resume) t.s = out[o + u], t.c = ps_.tot_c[o + u];
+            t.merge(acc[u].s, acc[u].c);
+            acc[u] = t;
+        }
+        if (ps_.more || (ps_.merge && ps_.tot_more)) {
+            (ps_.more ? ps_.acc : out)[o + u] = acc[u].s;
+            (ps_.more ? ps_.acc_c : ps_.tot_c)[o + u] = acc[u].c;
             continue;
         }
         const float val = acc[u].value();
@@ -1295,12 +1301,12 @@ cudaError_t launch_fwd_reduce(const spect_plan_s& P, int l0, int nv, float* v, c
                           P.g.nx, P.g.np, em_y ? em_y + at : nullptr, em_rbar ? em_rbar + at : nullptr);
 }
 
-cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,
+cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, int s0, float* out, PassState pass, EmArgs em,
                              cudaStream_t st)
 {
     const size_t n = (size_t)P.g.nx * P.g.ny * (P.g.kp / 4);
     const unsigned blocks = (unsigned)((n + 255) / 256);
-    const float* src = P.slab;
+    const float* src = P.slab + (size_t)s0 * P.g.ny * P.ps;
     const int segs = P.adj_chunk >= P.g.nview ? P.gsegs : 1, seglen = (nv + segs - 1) / segs;  // as the patch gather
     switch (P.adj_max) {
 #define SPECT_ADJ(M)                                                                                                 \

@@ -102,7 +102,7 @@ struct GatherArgs {
     int box_floats;  // floats of the largest box
     int ent_bytes;   // 64 * maxe * 8
     int stage_floats;
-    int l0, nv;      // views [l0, l0 + nv) of the plan; slab view v holds view l0 + v
+    int l0, nv, s0;  // views [l0, l0 + nv) of the plan; slab view s0 + v holds view l0 + v
     int nkc;         // runs of kc depth rows per patch
     int segs, seglen;  // view segments (blocks) per patch and k run, views of one
     float* seg;        // segs > 1: [segs][2][volume] sums and compensation terms of the segments
@@ -162,7 +162,7 @@ __device__ __forceinline__ void adj_gather_body(const CUtensorMap* maps, const G
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(full + s)),
                          "r"((unsigned)(b.z * b.z * KC * 4 + a.ent_bytes))
                          : "memory");
-            tma_load_3d(st, maps + b.w, kc0, b.x, (v0 + v) * g.ny + b.y, full + s);
+            tma_load_3d(st, maps + b.w, kc0, b.x, (a.s0 + v0 + v) * g.ny + b.y, full + s);
             tma_copy_1d(st + a.box_floats, pent + ((size_t)patch * g.nview + l) * (kPatch * kPatch) * MAXE,
                         (unsigned)a.ent_bytes, full + s);
             issued = v + 1;
@@ -189,8 +189,8 @@ __device__ __forceinline__ void adj_gather_body(const CUtensorMap* maps, const G
     }
 
     KSum acc[4];
-    if (mine && pass.resume) {  // the sums of the views of earlier passes
-        const float4 s = *reinterpret_cast<const float4*>(out + o), c = *reinterpret_cast<const float4*>(pass.comp + o);
+    if (mine && pass.resume) {  // the sums of the views of earlier launches
+        const float4 s = *reinterpret_cast<const float4*>(pass.acc + o), c = *reinterpret_cast<const float4*>(pass.acc_c + o);
         acc[0].s = s.x, acc[1].s = s.y, acc[2].s = s.z, acc[3].s = s.w;
         acc[0].c = c.x, acc[1].c = c.y, acc[2].c = c.z, acc[3].c = c.w;
     }
@@ -267,9 +267,20 @@ __device__ __forceinline__ void adj_gather_body(const CUtensorMap* maps, const G
     }
 
     if (!mine) return;
-    if (pass.more) {
-        *reinterpret_cast<float4*>(out + o) = make_float4(acc[0].s, acc[1].s, acc[2].s, acc[3].s);
-        *reinterpret_cast<float4*>(pass.comp + o) = make_float4(acc[0].c, acc[1].c, acc[2].c, acc[3].c);
+    if (pass.merge) {  // add this segment to the ones before it
+        KSum tot[4];
+        if (pass.tot_resume) {
+            const float4 s = *reinterpret_cast<const float4*>(out + o), c = *reinterpret_cast<const float4*>(pass.tot_c + o);
+            tot[0].s = s.x, tot[1].s = s.y, tot[2].s = s.z, tot[3].s = s.w;
+            tot[0].c = c.x, tot[1].c = c.y, tot[2].c = c.z, tot[3].c = c.w;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) tot[u].merge(acc[u].s, acc[u].c), acc[u] = tot[u];
+    }
+    if (pass.more || (pass.merge && pass.tot_more)) {
+        float *s = pass.more ? pass.acc : out, *c = pass.more ? pass.acc_c : pass.tot_c;
+        *reinterpret_cast<float4*>(s + o) = make_float4(acc[0].s, acc[1].s, acc[2].s, acc[3].s);
+        *reinterpret_cast<float4*>(c + o) = make_float4(acc[0].c, acc[1].c, acc[2].c, acc[3].c);
         return;
     }
     const float xv[4] = {ex.x, ex.y, ex.z, ex.w}, sv4[4] = {es.x, es.y, es.z, es.w}, uv[4] = {eu.x, eu.y, eu.z, eu.w};
@@ -357,10 +368,11 @@ int gather_kc(const spect_plan_s& P)
 }
 }  // namespace
 
-// View segments of A' when all views go in one pass: as many as fill one wave of
-// resident blocks, of at least 8 views each (64x32, 64 views: 27 us with one, 21 with
-// four; 24x60, 30 views: 16 and 12).  More than a wave only adds the segments' sums
-// (96x64, 64 views: 52 and 57).  Several passes resume one another instead.
+// View segments of A': as many as fill one wave of resident blocks, of at least 8 views
+// each (64x32, 64 views: 27 us with one, 21 with four; 24x60, 30 views: 16 and 12).  More
+// than a wave only adds the segments' sums (96x64, 64 views: 52 and 57).  One launch takes
+// all segments; where the views go in several passes the launches end at the segments'
+// boundaries (fast_back), so that the order of the sums is the same.
 int gather_segments(const spect_plan_s& P)
 {
     const Geometry& g = P.g;
@@ -509,8 +521,8 @@ cudaError_t build_gather_maps(spect_plan_s& P)
 }
 
 namespace {
-// The gather's arguments for views [l0, l0 + nv).
-void gather_setup(const spect_plan_s& P, int l0, int nv, GatherArgs* a)
+// The gather's arguments for views [l0, l0 + nv), the first at view s0 of the slab.
+void gather_setup(const spect_plan_s& P, int l0, int nv, int s0, GatherArgs* a)
 {
     const Geometry& g = P.g;
     const int kc = gather_kc(P), top = P.gsize[P.gnm - 1];
@@ -522,6 +534,7 @@ void gather_setup(const spect_plan_s& P, int l0, int nv, GatherArgs* a)
     a->stage_floats = stage_floats(a->box_floats, a->ent_bytes);
     a->l0 = l0;
     a->nv = nv;
+    a->s0 = s0;
     a->nkc = (g.kp + kc - 1) / kc;
     a->segs = P.adj_chunk >= g.nview ? P.gsegs : 1;
     a->seglen = (nv + a->segs - 1) / a->segs;
@@ -530,11 +543,11 @@ void gather_setup(const spect_plan_s& P, int l0, int nv, GatherArgs* a)
 }
 }  // namespace
 
-cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,
+cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, int s0, float* out, PassState pass, EmArgs em,
                               cudaStream_t st)
 {
     GatherArgs a;
-    gather_setup(P, l0, nv, &a);
+    gather_setup(P, l0, nv, s0, &a);
     const size_t smem = gather_smem(a.box_floats, a.ent_bytes);
     const dim3 grid(P.gnpx * P.gnpy * a.nkc, a.segs);  // (patch, k run), the k runs of a patch adjacent
     switch (P.adj_max) {
@@ -580,7 +593,7 @@ cudaError_t build_grouped_gather(const std::vector<spect_plan_s*>& plans, Groupe
             for (size_t m = c0; m < c1; ++m) {
                 const spect_plan_s& P = *plans[idx[m]];
                 GroupGather& q = gg.p[m - c0];
-                gather_setup(P, 0, P.g.nview, &q.a);
+                gather_setup(P, 0, P.g.nview, 0, &q.a);
                 q.maps = P.gmaps;
                 q.boxes = P.gboxes;
                 q.pent = P.gent;

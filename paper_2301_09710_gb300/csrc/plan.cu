@@ -184,13 +184,15 @@ int view_chunk(int nview, size_t bytes_per_view, size_t budget)
 
 // Floats of P.part.  In A: the depth-group partial sums of a pass of `chunk` views, and
 // the compensation terms of low-memory plans' sums.
-// In A' the same buffer holds the sums and compensation terms of the view segments, or
-// between its passes (adj_chunk views each) the compensation terms of the view sums.
+// In A' the same buffer holds the sums and compensation terms of the view segments, or,
+// where its passes (adj_chunk views each) are several, those of the present segment and the
+// compensation terms of the segments before it (one segment: compensation terms only).
 size_t part_floats(const spect_plan_s& P, int chunk, int adj_chunk)
 {
     const size_t part = (size_t)P.g.nx * P.g.nz * chunk * spect::fused_groups(P) * (1 + P.part_comp);
     const size_t volt = (size_t)P.g.nx * P.g.ny * P.g.kp;
-    return std::max(part, adj_chunk < P.g.nview ? volt : (P.gsegs > 1 ? 2 * P.gsegs * volt : 0));
+    if (adj_chunk < P.g.nview) return std::max(part, (P.gsegs > 1 ? 3 : 1) * volt);
+    return std::max(part, P.gsegs > 1 ? 2 * P.gsegs * volt : 0);
 }
 
 // Adjacency lists a low-memory plan takes to the fused kernels.  A list holds the samples
@@ -473,9 +475,13 @@ spect_status fast_forward(spect_plan_s* P, const float* xt, float* v, const floa
 spect_status fast_back(spect_plan_s* P, const float* v, float* out_t, spect::EmArgs em, cudaStream_t st)
 {
     const int nview = P->g.nview;
+    const size_t volt = (size_t)P->g.nx * P->g.ny * P->g.kp;
+    const bool split = P->adj_chunk < nview && P->gsegs > 1;  // several passes and several segments
+    const int seglen = (nview + P->gsegs - 1) / P->gsegs;
+    if (P->adj_chunk < nview && P->part_cap < (split ? 3 : 1) * volt)
+        return fail(SPECT_ECUDA, "several adjoint passes, one planned");
     for (int l0 = 0; l0 < nview; l0 += P->adj_chunk) {
         const int nv = std::min(P->adj_chunk, nview - l0);
-        const bool last = l0 + nv >= nview;
         if (P->tab_pass)
             SPECT_CUDA_TRY(counted(P, SPECT_K_OTHER, st, [&] { return spect::launch_rot_tables(*P, l0, nv, st); }),
                            "rotation table launch");
@@ -484,20 +490,30 @@ spect_status fast_back(spect_plan_s* P, const float* v, float* out_t, spect::EmA
                            "attenuation launch");
         SPECT_CUDA_TRY(counted(P, SPECT_K_CONV_ADJ, st, [&] { return spect::launch_fused_adjoint(*P, v, l0, nv, st); }),
                        "fused adjoint launch");
-        spect::EmArgs e = em;
-        if (!last) e.x = nullptr;
-        spect::PassState pass;
-        pass.resume = l0 > 0;
-        pass.more = !last;
-        pass.comp = P->part;  // free between the depth-group reduce and the next forward blur
-        if ((pass.resume || pass.more) && P->part_cap < (size_t)P->g.nx * P->g.ny * P->g.kp)
-            return fail(SPECT_ECUDA, "several adjoint passes, one planned");
-        SPECT_CUDA_TRY(counted(P, SPECT_K_ROTATE_ADJ, st,
-                               [&] {
-                                   return P->gather ? spect::launch_adj_gather(*P, l0, nv, out_t, pass, e, st)
-                                                    : spect::launch_adj_rot_t(*P, l0, nv, out_t, pass, e, st);
-                               }),
-                       "adjoint rotation launch");
+        for (int p0 = l0, n; p0 < l0 + nv; p0 += n) {  // one launch, or one per segment the pass has views of
+            const int s_begin = split ? p0 / seglen * seglen : 0, s_end = split ? std::min(nview, s_begin + seglen) : nview;
+            n = std::min(l0 + nv, s_end) - p0;
+            spect::EmArgs e = em;
+            if (p0 + n < nview) e.x = nullptr;
+            spect::PassState pass;
+            pass.resume = p0 > s_begin;
+            pass.more = p0 + n < s_end;
+            pass.acc = out_t;
+            pass.acc_c = P->part;  // free between the depth-group reduce and the next forward blur
+            if (split) {
+                pass.merge = !pass.more;
+                pass.tot_resume = s_begin > 0;
+                pass.tot_more = s_end < nview;
+                pass.acc = P->part + volt;
+                pass.tot_c = P->part + 2 * volt;
+            }
+            SPECT_CUDA_TRY(counted(P, SPECT_K_ROTATE_ADJ, st,
+                                   [&] {
+                                       return P->gather ? spect::launch_adj_gather(*P, p0, n, p0 - l0, out_t, pass, e, st)
+                                                        : spect::launch_adj_rot_t(*P, p0, n, p0 - l0, out_t, pass, e, st);
+                                   }),
+                           "adjoint rotation launch");
+        }
     }
     return SPECT_OK;
 }
@@ -568,7 +584,7 @@ size_t plan_bytes_bound(const spect_plan_s& P)
     // attenuation factors of every view, or of one chunk plus mu in the internal layout
     b += P.recompute ? ((size_t)g.ny * P.ps * chunk + volt) * F : (size_t)g.ny * P.ps * g.nview * F;
     b += 4 * volt * F;
-    b += std::max(part_floats(P, P.chunk, P.chunk), volt) * F + (size_t)g.nview * g.ny * P.ts * F;
+    b += std::max(part_floats(P, P.chunk, P.chunk), 3 * volt) * F + (size_t)g.nview * g.ny * P.ts * F;
     // patch gather (at most 8 entries per list), rotation boxes
     b += gather_bytes(P, 8) + (size_t)((g.nx + 7) / 8) * ((g.ny + 7) / 8) * g.nview * 16;
     if (P.rot3)  // the eight-tap table

@@ -124,7 +124,7 @@ struct spect_plan_s {
     int gnpx = 0, gnpy = 0;
     int gnm = 0, gsize[spect::kGatherMaps] = {};  // box sizes, ascending
     spect::GatherMaps gmaps;     // the slab, boxed at each size (build_gather_maps)
-    int gsegs = 1;               // view segments of A' when the views go in one pass (gather_segments)
+    int gsegs = 1;               // view segments of A' (gather_segments)
     int* gcount = nullptr;       // [patch][k run] segment arrivals
     // patch-staged forward rotation (rotpatch.cu): available when rotpatch != 0,
     // used instead of k_rot_fwd when rotpatch_on != 0 (chosen by the autotuner)
@@ -316,11 +316,15 @@ struct EmArgs {
     float beta = 0.f;
 };
 
-// The view sum of A' over several passes: each resumes the compensated sums (out, comp)
-// that the last one left, so the result does not depend on how the views are split.
+// The view sum of A' over several launches.  Within a view segment (gather_segments; all
+// views where there is one) each launch resumes the compensated sums that the last one
+// left, and the segments' sums are merged in order, as one launch over all views does it:
+// for a given number of segments the result does not depend on how the views are split.
 struct PassState {
-    int resume = 0, more = 0;  // earlier passes' sums in out / comp; further passes follow
-    float* comp = nullptr;     // compensation terms (only read or written when resume or more)
+    int resume = 0, more = 0;          // earlier launches' sums of this segment in acc / acc_c; further launches follow
+    int merge = 0;                     // one of several segments ends with this launch:
+    int tot_resume = 0, tot_more = 0;  // earlier segments' sums in out / tot_c; further segments follow
+    float *acc = nullptr, *acc_c = nullptr, *tot_c = nullptr;
 };
 
 // Kahan-compensated accumulator for depth and view sums.
@@ -560,9 +564,10 @@ inline const float* rtab_for(const spect_plan_s& P, int l0)
     return reinterpret_cast<const float*>(reinterpret_cast<uintptr_t>(P.rtab) -
                                           (uintptr_t)l0 * P.g.ny * P.ts * sizeof(float));
 }
-cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,
+// the view sum of A' over views l0 .. l0+nv-1, the first at view s0 of the slab
+cudaError_t launch_adj_gather(const spect_plan_s& P, int l0, int nv, int s0, float* out, PassState pass, EmArgs em,
                               cudaStream_t st);
-cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, float* out, PassState pass, EmArgs em,
+cudaError_t launch_adj_rot_t(const spect_plan_s& P, int l0, int nv, int s0, float* out, PassState pass, EmArgs em,
                              cudaStream_t st);
 bool direct_fits(const Geometry& g, size_t smem_limit);
 // grouped launches of a batch of plans (grouped.cu, gather.cu): per stage and

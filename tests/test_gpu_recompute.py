@@ -74,6 +74,34 @@ def test_recomputing_plan_is_bitwise_the_caching_plan(case, monkeypatch):
     cached.close()
 
 
+@pytest.mark.parametrize("gather", ["1", "0"])
+def test_view_sums_do_not_depend_on_the_passes(gather, monkeypatch):
+    """A small volume with enough views that A' sums them in segments: a caching plan of one pass,
+    and caching and recomputing plans whose passes end inside segments, by the patch gather and
+    by the list gather, give the same bits."""
+    monkeypatch.setenv("SPECT_GATHER", gather)
+    nx, nz, nv = 24, 16, 36
+    prob = synthetic.config1(seed=4, nx=nx, nz=nz, nview=nv, psf_size=7)
+    ang = oracle.default_angles(nv)
+    y = np.random.default_rng(4).uniform(0.5, 1.5, (nv, nz, nx)).astype(np.float32)
+    x0 = np.where(prob.body, 1.0, 0.0).astype(np.float32) + 0.05
+    want = None
+    for mb, recompute in ((None, False), ("1", False), ("1", True), (None, True)):
+        if mb:
+            monkeypatch.setenv("SPECT_SLAB_MB", mb)
+        else:
+            monkeypatch.delenv("SPECT_SLAB_MB", raising=False)
+        plan = _plan(prob, ang, recompute)
+        assert (plan.info()["view_chunk"] < nv) == (mb is not None)
+        got = _run(plan, prob, y, np.full_like(y, 0.1), x0)
+        plan.check()
+        plan.close()
+        want = want or got
+        for g, w, what in zip(got, want, ("A x", "A' y", "EM iterates")):
+            assert np.array_equal(g, w), f"{what} depends on the passes (SPECT_SLAB_MB={mb}, recompute={recompute})"
+    assert_close(want[1], oracle.back(y, prob.mu, oracle_psf(prob, "fused"), prob.dy, ang), what="A' y")
+
+
 def test_recomputing_plan_memory_and_bound():
     from paper_2301_09710_gb300.projector import plan_bytes
     prob = synthetic.config2(seed=0)
