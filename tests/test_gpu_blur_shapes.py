@@ -167,3 +167,26 @@ def test_attenuation_runs_of_depths(nx, nz):
     assert_close(host(plan.back(dev(yy))), oracle.back(yy, prob.mu, psf, prob.dy, ang), what="A' y")
     plan.check()
     plan.close()
+
+
+@pytest.mark.parametrize("i,k", [(0, 4), (47, 4), (20, 20)])
+def test_an_infinite_voxel_reaches_only_its_psf(i, k):
+    """Replicate padding multiplies the edge columns by folded taps: an infinity there reaches the
+    outputs that its PSF reaches, not the rest of a run of 16 (at angle 0 the bilinear rotation
+    hands it on to the column before it with weight 0)."""
+    need_gpu()
+    import torch
+    from paper_2301_09710_gb300 import SpectPlan
+    nx, nz, p = 48, 40, 5
+    taps = np.full((1, nx, p), 1.0 / p, np.float32)
+    plan = SpectPlan(nx, nz, 1, fx=taps, fz=taps, angles=[0.0])
+    x = np.ones((nz, nx, nx), np.float32)
+    x[k, 20, i] = np.inf
+    v = plan.forward(dev(x))
+    finite = torch.isfinite(v)[0].cpu().numpy()
+    plan.check()
+    plan.close()
+    ii, kk = np.meshgrid(np.arange(nx), np.arange(nz))
+    reached = (ii >= i - 1 - p // 2) & (ii <= i + p // 2) & (abs(kk - k) <= p // 2)
+    assert finite[~reached].all()
+    assert not finite[(abs(ii - i) <= p // 2) & (abs(kk - k) <= p // 2)].any()
