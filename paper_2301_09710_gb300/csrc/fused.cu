@@ -303,13 +303,7 @@ __global__ void k_fwd_reduce(const float* __restrict__ part, const float* __rest
     wait_previous_kernel();
     const size_t o = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= nproj) return;
-    KSum acc;  // up to ny partials (J = 1): compensated
-    for (int gq = 0; gq < G; ++gq) {
-        const float p = part[(size_t)gq * nproj + o];
-        if (comp) acc.merge(p, comp[(size_t)gq * nproj + o]);
-        else acc.add(p);
-    }
-    const float s = acc.value();
+    const float s = group_sum(part + o, comp ? comp + o : nullptr, G, nproj);  // up to ny partials (J = 1): compensated
     if (em_y) {
         const float yb = s + (em_rbar ? em_rbar[o] : 0.f);
         v[np == nx ? o : o + o / nx * (np - nx)] = yb > 0.f ? em_y[o] / yb : 0.f;

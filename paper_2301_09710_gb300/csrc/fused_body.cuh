@@ -349,6 +349,24 @@ __host__ __device__ inline size_t fwd_smem_floats(const FwdDims& d, int PT)
            (d.racc ? 0 : (size_t)d.urows * d.apc) + 8;
 }
 
+// The compensated sum over depth groups of partials p[q * stride] (comp: their compensation
+// terms, or NULL).  One that is not finite is the plain sum's infinity or NaN (an overflow
+// leaves NaN in the compensation).
+__device__ __forceinline__ float group_sum(const float* __restrict__ p, const float* __restrict__ comp, int G, size_t stride)
+{
+    KSum acc;
+    if (comp)
+        for (int q = 0; q < G; ++q) acc.merge(p[(size_t)q * stride], comp[(size_t)q * stride]);
+    else
+        for (int q = 0; q < G; ++q) acc.add(p[(size_t)q * stride]);
+    float s = acc.value();
+    if (!(fabsf(s) <= FLT_MAX)) {
+        s = 0.f;
+        for (int q = 0; q < G; ++q) s += p[(size_t)q * stride];
+    }
+    return s;
+}
+
 // A depth sum: plain, or compensated (KS).  store() leaves a group's sum at p, a
 // compensated one's compensation term at p + half, for the reduce to carry on with.
 template <bool KS>

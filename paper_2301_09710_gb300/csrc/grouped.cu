@@ -91,9 +91,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_fwd_reduce_grp(const __grid_
     const GroupPlan q = gp.p[w.x];  // by value: the fields live in registers, not re-read from parameter space
     const size_t o = (size_t)w.y * kReduceThreads + threadIdx.x;
     if (o >= q.nproj) return;
-    KSum acc;
-    for (int gq = 0; gq < q.df.G; ++gq) acc.add(q.part[(size_t)gq * q.nproj + o]);
-    const float s = acc.value();
+    const float s = group_sum(q.part + o, nullptr, q.df.G, q.nproj);
     const float yb = s + (q.rbar ? q.rbar[o] : 0.f);
     const int nx = q.g.nx, np = q.g.np;
     q.ratio[np == nx ? o : o + o / nx * (np - nx)] = yb > 0.f ? q.y[o] / yb : 0.f;

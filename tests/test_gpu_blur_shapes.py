@@ -190,3 +190,18 @@ def test_an_infinite_voxel_reaches_only_its_psf(i, k):
     reached = (ii >= i - 1 - p // 2) & (ii <= i + p // 2) & (abs(kk - k) <= p // 2)
     assert finite[~reached].all()
     assert not finite[(abs(ii - i) <= p // 2) & (abs(kk - k) <= p // 2)].any()
+
+
+def test_a_depth_sum_that_overflows_is_infinite():
+    """Partial sums of depth groups that are finite and add up to more than FP32 holds: the
+    projection is +inf, as a plain sum gives it, not NaN."""
+    need_gpu()
+    import torch
+    from paper_2301_09710_gb300 import SpectPlan
+    nx, nz = 64, 8
+    taps = np.full((1, nx, 3), 1.0 / 3, np.float32)
+    plan = SpectPlan(nx, nz, 1, fx=taps, fz=taps, angles=[0.0])
+    v = plan.forward(torch.full((nz, nx, nx), 1e37, device="cuda"))
+    assert torch.isposinf(v).all()
+    plan.check()
+    plan.close()
