@@ -52,7 +52,7 @@ def parse():
     ap.add_argument("--cpu-views", type=int, default=0, help="views in the CPU baseline sample (0: auto)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-autotune", action="store_true", help="keep the plan's default launch shapes")
-    ap.add_argument("--launch-shape", default=None, metavar="J,ADJ_J,TILES",
+    ap.add_argument("--launch-shape", default=None, metavar="J,ADJ_J,TILES[,ADJ_TILES]",
                     help="fix the main plan's launch shape instead of autotuning it (for profiler runs, where the "
                          "autotuner's timings are distorted)")
     ap.add_argument("--serve-requests", type=int, default=160,
@@ -147,7 +147,7 @@ def make_workload(device, path, nview=NVIEW, autotune=True, rotation="bilinear",
         plan = SpectPlan(NX, NZ, nview, mu=prob.mu, dy=prob.dy, fx=prob.fx, fz=prob.fz, device=device,
                          rotation=rotation, low_memory=low_memory, recompute_attenuation=recompute)
         if shape and not low_memory:
-            plan.set_tuning(*shape)
+            plan.set_tuning(*shape[:3], adj_tiles=shape[3] if len(shape) > 3 else None)
         elif autotune and not low_memory:
             plan.autotune()  # the library's launch-shape autotuner (timed on this device, outside the timed region)
     else:

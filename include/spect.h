@@ -349,7 +349,10 @@ spect_status spect_plan_release(spect_plan plan, spect_stream stream);
  * Launch-shape tuning of the fused kernels (the paper has no counterpart).
  * fused_J / adj_J: depth planes per block of the forward / adjoint blur
  * kernels (1..32); tiles: column tiles per plane (>= 1; the kernels use the
- * nearest count that divides the plane into whole 16-column runs).  The plan
+ * nearest count that divides the plane into whole 16-column runs).  The two
+ * kernels may have different tile counts: set_shape and get_shape take and
+ * give both; get_tuning reports the forward's; set_tuning sets both, except
+ * that the count get_tuning reports leaves the adjoint's as it is.  The plan
  * grows its work slab and partial-sum buffer (and, for a plan made with
  * SPECT_PLAN_RECOMPUTE_ATTENUATION, its buffer of one view chunk's
  * attenuation factors) in stream order on `stream` when the shape needs more
@@ -361,6 +364,9 @@ spect_status spect_plan_release(spect_plan plan, spect_stream stream);
  */
 spect_status spect_plan_set_tuning(spect_plan plan, int fused_J, int adj_J, int tiles, spect_stream stream);
 spect_status spect_plan_get_tuning(spect_plan plan, int* fused_J, int* adj_J, int* tiles);
+spect_status spect_plan_set_shape(spect_plan plan, int fused_J, int adj_J, int tiles, int adj_tiles,
+                                  spect_stream stream);
+spect_status spect_plan_get_shape(spect_plan plan, int* fused_J, int* adj_J, int* tiles, int* adj_tiles);
 
 /*
  * spect_plan_autotune -- time the fused kernels' candidate launch shapes

@@ -99,6 +99,10 @@ def load(path: str = LIB_PATH):
         lib.spect_plan_set_tuning.restype = st
         lib.spect_plan_get_tuning.argtypes = [vp, ip, ip, ip]
         lib.spect_plan_get_tuning.restype = st
+        lib.spect_plan_set_shape.argtypes = [vp, i, i, i, i, vp]
+        lib.spect_plan_set_shape.restype = st
+        lib.spect_plan_get_shape.argtypes = [vp, ip, ip, ip, ip]
+        lib.spect_plan_get_shape.restype = st
         lib.spect_plan_autotune.argtypes = [vp, vp]
         lib.spect_plan_autotune.restype = st
         lib.spect_batch_create.argtypes = [ctypes.POINTER(vp), ctypes.POINTER(vp), i]

@@ -1348,7 +1348,23 @@ extern "C" {
 spect_status spect_plan_set_tuning(spect_plan P, int fused_J, int adj_J, int tiles, spect_stream stream)
 {
     if (!P) return fail(SPECT_EINVAL, "plan is NULL");
-    return reconfigure(P, fused_J, adj_J, tiles, tiles, (cudaStream_t)stream);
+    cudaStream_t st = (cudaStream_t)stream;
+    // the count that get_tuning reports leaves the adjoint's own one as it is
+    if (tiles == P->fwd_nT && reconfigure(P, fused_J, adj_J, tiles, P->adj_nT, st) == SPECT_OK) return SPECT_OK;
+    return reconfigure(P, fused_J, adj_J, tiles, tiles, st);
+}
+
+spect_status spect_plan_set_shape(spect_plan P, int fused_J, int adj_J, int tiles, int adj_tiles, spect_stream stream)
+{
+    if (!P) return fail(SPECT_EINVAL, "plan is NULL");
+    return reconfigure(P, fused_J, adj_J, tiles, adj_tiles, (cudaStream_t)stream);
+}
+
+spect_status spect_plan_get_shape(spect_plan P, int* fused_J, int* adj_J, int* tiles, int* adj_tiles)
+{
+    if (!P) return fail(SPECT_EINVAL, "plan is NULL");
+    if (adj_tiles) *adj_tiles = P->adj_nT;
+    return spect_plan_get_tuning(P, fused_J, adj_J, tiles);
 }
 
 spect_status spect_plan_get_tuning(spect_plan P, int* fused_J, int* adj_J, int* tiles)

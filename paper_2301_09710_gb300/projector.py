@@ -279,14 +279,22 @@ class SpectPlan:
     # ------------------------------------------------------------------ launch shapes
     @property
     def tuning(self) -> dict:
-        """fused_J / adj_J: depth planes per forward / adjoint blur block; tiles: column tiles per plane."""
-        a, b, c = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
-        _lib.check(self.lib.spect_plan_get_tuning(self.handle, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)))
-        return {"fused_J": a.value, "adj_J": b.value, "tiles": c.value}
+        """fused_J / adj_J: depth planes per forward / adjoint blur block; tiles / adj_tiles: column tiles per plane."""
+        a, b, c, d = ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
+        _lib.check(self.lib.spect_plan_get_shape(self.handle, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c),
+                                                 ctypes.byref(d)))
+        return {"fused_J": a.value, "adj_J": b.value, "tiles": c.value, "adj_tiles": d.value}
 
-    def set_tuning(self, fused_J: int, adj_J: int, tiles: int, stream=None) -> None:
-        _lib.check(self.lib.spect_plan_set_tuning(self.handle, int(fused_J), int(adj_J), int(tiles),
-                                                  _stream_handle(stream)))
+    def set_tuning(self, fused_J: int, adj_J: int, tiles: int, stream=None,
+                   adj_tiles: int | None = None) -> None:
+        """Set the launch shape; without adj_tiles the adjoint takes the forward's count (or keeps its
+        own, where tiles is the plan's present one)."""
+        if adj_tiles is None:
+            _lib.check(self.lib.spect_plan_set_tuning(self.handle, int(fused_J), int(adj_J), int(tiles),
+                                                      _stream_handle(stream)))
+        else:
+            _lib.check(self.lib.spect_plan_set_shape(self.handle, int(fused_J), int(adj_J), int(tiles),
+                                                     int(adj_tiles), _stream_handle(stream)))
 
     def autotune(self, stream=None) -> dict:
         """Time the candidate launch shapes on this device and keep the fastest (cached per geometry)."""

@@ -205,3 +205,26 @@ def test_a_depth_sum_that_overflows_is_infinite():
     assert torch.isposinf(v).all()
     plan.check()
     plan.close()
+
+
+def test_launch_shape_round_trips():
+    """The two blurs may have different tile counts: what a plan reports, set on it again or on
+    another plan, gives the same shape, also by the call that takes one count."""
+    need_gpu()
+    prob = synthetic.random_problem(12, nx=96, nz=9, nview=3, px=5, pz=5, mu_scale=0.05)
+    ang = oracle.default_angles(3)
+    plan, other = make_plan(prob, ang, "fused"), make_plan(prob, ang, "fused")
+    plan.set_tuning(4, 8, 2, adj_tiles=6)
+    t = plan.tuning
+    assert t == {"fused_J": 4, "adj_J": 8, "tiles": 2, "adj_tiles": 6}
+    plan.set_tuning(4, 8, 2)
+    assert plan.tuning == t
+    other.set_tuning(**t)
+    assert other.tuning == t
+    other.set_tuning(4, 8, 3)
+    assert other.tuning == {"fused_J": 4, "adj_J": 8, "tiles": 3, "adj_tiles": 3}
+    yy = dev(np.random.default_rng(12).uniform(0, 1, plan.proj_shape))
+    assert np.array_equal(host(plan.back(yy)), host(other.back(yy)))
+    for p in (plan, other):
+        p.check()
+        p.close()
