@@ -1170,8 +1170,9 @@ namespace {
 // about four warps' worth lost to latency, so a plane takes W + 4 warp items of
 // 32 P + 100 issue slots; a block's set-up costs about s planes; up to four waves the
 // last one counts whole, beyond that half a block on average.  Against the measured
-// launches (shapes of 16..64 columns and J = 1..8, nineteen geometries from 16x8 to
-// 192x128) the shapes it picks are within 6 % of the fastest for A, 4 % for A'.
+// calls (shapes of 16..64 columns and J = 1..8; 16x8, 20x20, 24x60, 37x100, 48x24, 64x32,
+// 64x64, 64x80, 96x64, 96x96, 99x53, 113x20, 128x32, 128x64, 128x80, 150x75, 160x48, 160x96,
+// 192x128 with 8 to 128 views and 5 to 37 taps) the shapes it picks are within 5 % of the fastest.
 double blur_cost(int P, long long blocks, int J, double s, int T, int B, int sms)
 {
     const double per_sm = (double)((blocks + sms - 1) / sms);
@@ -1226,6 +1227,9 @@ void default_shape(spect_plan_s& P)
 {
     const Geometry& g = P.g;
     if (!P.separable) {  // blocks of the full-PSF forward kernel
+        // J = 2, 4, 8, A and A' in us: 3.4 blocks of 8 planes per SM (64x32, 32 views, 9x9 PSF) 33.2 33.4 35.5 and
+        // 41.0 41.3 45.2; 14 (96x64, 60 views, 21x21) 565 566 579 and 657 636 643; 25 (128x64, 60 views, 11x11)
+        // 419 400 396 and 475 432 422; 54 (128x80, 128 views, 9x9) 964 893 860 and 1038 933 882
         P.part_comp = P.low;
         if (P.shape_views < g.nview && !P.low) return;  // as choose_shape's keep_J
         P.fused_J = P.adj_J = 8;

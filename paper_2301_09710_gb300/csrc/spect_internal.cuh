@@ -355,7 +355,9 @@ struct KSum {
 // triggers its successor early: operands read through the read-only path would then be
 // written while the reader is already on the chip.  Bound by launch latency at small
 // sizes; measured: two EM updates of 64x64x32, 64 views, 172 -> 145 us (12
-// launches), 99x99x53 with 60 views 343 -> 326 (7), 128x128x80 with 128 views 1466 -> 1451.
+// launches), 99x99x53 with 60 views 343 -> 326 (7), 128x128x80 with 128 views 1466 -> 1452.
+// That every chained kernel begins with the wait is read from the sources
+// (tests/test_chained_launches_cpu.py).
 __device__ __forceinline__ void wait_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class... P, class... A>
