@@ -5,7 +5,10 @@ import ctypes
 import numpy as np
 import pytest
 
-from gpu_helpers import dev, host, need_gpu, torch
+import oracle
+from paper_2301_09710_gb300 import synthetic
+
+from gpu_helpers import assert_close, dev, host, make_plan, need_gpu, torch
 
 pytestmark = pytest.mark.gpu
 
@@ -90,3 +93,39 @@ def test_low_memory_depth_sums_are_compensated_over_all_depths(path, nx, nz, nvi
     plan.check()
     plan.close()
     assert np.array_equal(got, np.full((nview, nz, nx), nx // 16, np.float64))
+
+
+def test_flat_low_memory_plan_makes_its_tables_in_each_pass():
+    """160x160x5: one view per pass, the rotation tables of the pass made in it; A, A' and an EM
+    step against the oracle."""
+    prob = synthetic.random_problem(3, nx=160, nz=5, nview=20, px=9, pz=9, mu_scale=0.02)
+    ang = oracle.default_angles(20)
+    plan = make_plan(prob, ang, "lowmem")
+    assert plan.info()["view_chunk"] == 1
+    psf = oracle.psf_from_factors(prob.fx, prob.fz)
+    assert_close(host(plan.forward(dev(prob.x))), oracle.forward(prob.x, prob.mu, psf, prob.dy, ang), what="A x")
+    y = np.random.default_rng(3).uniform(0.5, 1.5, plan.proj_shape).astype(np.float32)
+    assert_close(host(plan.back(dev(y))), oracle.back(y, prob.mu, psf, prob.dy, ang), what="A' y")
+    x0 = np.full(prob.x.shape, 0.5, np.float32)
+    xg = dev(x0)
+    plan.em_step(xg, dev(y), None, niter=1)
+    assert_close(host(xg), oracle.em_step(x0, y, None, prob.mu, psf, prob.dy, ang), what="EM step")
+    plan.check()
+    plan.close()
+
+
+def test_low_memory_plan_that_fits_only_the_general_kernels():
+    """A full PSF of its own for each of 218 views of a tiny volume: the tap records of the fused
+    kernels would take more than the general kernels' plan, which serves it within its bound."""
+    from paper_2301_09710_gb300.projector import plan_bytes
+    nx, nz, nview, px, pz = 8, 2, 218, 9, 31
+    prob = synthetic.random_problem(5, nx=nx, nz=nz, nview=nview, px=px, pz=pz, nview_psf=nview, mu_scale=0.05)
+    ang = oracle.default_angles(nview)
+    plan = make_plan(prob, ang, "direct_lowmem")
+    assert plan.info()["device_bytes"] <= plan_bytes(nx, nz, nview, px, pz, nview, separable=False, low_memory=True)
+    psf = prob.full_psf().astype(np.float64)
+    assert_close(host(plan.forward(dev(prob.x))), oracle.forward(prob.x, prob.mu, psf, prob.dy, ang), what="A x")
+    y = np.random.default_rng(5).uniform(0.5, 1.5, plan.proj_shape).astype(np.float32)
+    assert_close(host(plan.back(dev(y))), oracle.back(y, prob.mu, psf, prob.dy, ang), what="A' y")
+    plan.check()
+    plan.close()
